@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "prox_kernels.cuh"
+#include "prox_pack.cuh"
 #include "prox_fused.cuh"
 #include "prox_batch_mma.cuh"
 #include "prox_batch_umma.cuh"
@@ -124,8 +125,11 @@ void free_packed(prox_ffn* h) {
   h->quantized = false;
 }
 
+// Packing again in the same format (new weights in the same buffers) keeps the buffers.
 prox_status_t alloc_packed(prox_ffn* h, int bits, int group_len) {
   const int D = h->cfg.d_model, F = h->cfg.d_ff;
+  h->quantized = false;
+  if (h->P && h->S && h->s_plain && h->wdt && h->bits == bits && h->group == group_len) return PROX_OK;
   free_packed(h);
   h->bits = bits;
   h->group = group_len;
@@ -138,6 +142,22 @@ prox_status_t alloc_packed(prox_ffn* h, int bits, int group_len) {
   CK(dev_alloc(&h->s_plain, (size_t)2 * F * ngroups));
   CK(dev_alloc(&h->wdt, (size_t)F * D));
   return PROX_OK;
+}
+
+// scales and codes: one pass over the weights with 128-input groups, two with one scale per row
+template <int BITS>
+void launch_pack(prox_ffn* h, cudaStream_t st) {
+  const int D = h->cfg.d_model, F = h->cfg.d_ff;
+  const dim3 grid((F + (BITS == 4 ? 127 : 63)) / (BITS == 4 ? 128 : 64), D / 128);
+  uint32_t* P = reinterpret_cast<uint32_t*>(h->P);
+  if (h->group == 128) {
+    proxy_pack_kernel<BITS, true><<<grid, 256, 0, st>>>(h->wg, h->wu, D, F, h->S, h->s_plain, P);
+  } else {
+    proxy_row_scale_kernel<BITS><<<dim3((F + 7) / 8, 2), 256, 0, st>>>(h->wg, h->wu, D, F, h->S, h->s_plain);
+    h->launches++;
+    proxy_pack_kernel<BITS, false><<<grid, 256, 0, st>>>(h->wg, h->wu, D, F, h->S, h->s_plain, P);
+  }
+  h->launches++;
 }
 
 int nstrips_for(int F, int bits) {
@@ -910,34 +930,15 @@ prox_status_t prox_quantize_proxy(prox_ffn_t* h, int bits, int group_size, void*
     proxy_pack16_kernel<<<(unsigned)((total + bs - 1) / bs), bs, 0, st>>>(h->wg, h->wu, D, F,
                                                                          reinterpret_cast<uint32_t*>(h->P));
     h->launches++;
-    CK(cudaGetLastError());
+  } else if (bits == 4) {
+    launch_pack<4>(h, st);
   } else {
-  {
-    const long long warps = 2ll * F * ngroups;
-    const long long threads = warps * 32;
-    const int bs = 256;
-    proxy_scale_kernel<<<(unsigned)((threads + bs - 1) / bs), bs, 0, st>>>(
-        reinterpret_cast<const __nv_bfloat16*>(h->wg), reinterpret_cast<const __nv_bfloat16*>(h->wu), D,
-        F, G, bits, h->S, h->s_plain);
-    h->launches++;
-    CK(cudaGetLastError());
+    launch_pack<8>(h, st);
   }
-  {
-    const long long total = (long long)(F / ch_per_chunk(bits)) * 4 * D;
-    const int bs = 256;
-    proxy_pack_kernel<<<(unsigned)((total + bs - 1) / bs), bs, 0, st>>>(
-        reinterpret_cast<const __nv_bfloat16*>(h->wg), reinterpret_cast<const __nv_bfloat16*>(h->wu), D,
-        F, G, bits, h->s_plain, reinterpret_cast<uint32_t*>(h->P));
-    h->launches++;
-    CK(cudaGetLastError());
-  }
-  }
-  {
-    dim3 grid((F + 31) / 32, (D + 31) / 32), block(32, 8);
-    transpose_bf16_kernel<<<grid, block, 0, st>>>(h->wd, h->wdt, D, F);
-    h->launches++;
-    CK(cudaGetLastError());
-  }
+  CK(cudaGetLastError());
+  transpose_bf16_kernel<<<dim3(F / 64, D / 64), 256, 0, st>>>(h->wd, h->wdt, D, F);
+  h->launches++;
+  CK(cudaGetLastError());
   h->quantized = true;
   return PROX_OK;
 }

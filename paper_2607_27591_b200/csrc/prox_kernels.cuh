@@ -1,5 +1,6 @@
-// Device kernels of libprox (sm_100a).  One kernel per step of the path:
-//   quantize/pack (offline)  ->  input top-k  ->  proxy GEMV + score
+// Device kernels of libprox (sm_100a).  One kernel per step of the path (the
+// offline packer is in prox_pack.cuh):
+//   input top-k  ->  proxy GEMV + score
 //   ->  channel top-k  ->  gather gate/up + SwiGLU  ->  masked down projection.
 // Paper references are to Sec. 4.1 (two-stage inference), Sec. 4.3
 // (hardware-aware implementation) and the appendix on top-k selection.
@@ -114,119 +115,6 @@ __device__ __forceinline__ void find_kth_bin(const unsigned* hist, unsigned k,
     }
   }
   __syncthreads();
-}
-
-// ----------------------------------------------------------------------------
-// Offline: scales, proxy packing, W_down transpose          (Sec. 4.3)
-// ----------------------------------------------------------------------------
-// Packed proxy layout ("input-major"): row i (one input coordinate) holds all
-// channels; it is cut into 16-byte chunks, chunk c covering CH consecutive
-// channels (CH = 16 for 4-bit, 8 for 8-bit):
-//   words 0,1 : gate codes of channels c*CH .. c*CH+CH-1  (lowest bits first)
-//   words 2,3 : up   codes of the same channels
-// Codes are offset binary: q + 8 (4-bit) or q + 128 (8-bit).
-// Scale layout: [group][chunk][2][CH] fp16 (gate scales then up scales).
-
-// One warp per (channel j, group g): scale = fp16(absmax / qmax).
-__global__ void proxy_scale_kernel(const __nv_bfloat16* __restrict__ wg,
-                                   const __nv_bfloat16* __restrict__ wu, int D, int F, int G,
-                                   int bits, __half* __restrict__ S, float* __restrict__ s_plain) {
-  const int ngroups = D / G;
-  const int CH = (bits == 4) ? 16 : 8;
-  const long long warp_id = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  const long long total = 2ll * F * ngroups;
-  if (warp_id >= total) return;
-  const int which = (int)(warp_id / ((long long)F * ngroups));
-  const long long rem = warp_id % ((long long)F * ngroups);
-  const int j = (int)(rem / ngroups), g = (int)(rem % ngroups);
-  const __nv_bfloat16* w = (which ? wu : wg) + (size_t)j * D + (size_t)g * G;
-  float a = 0.f;
-  for (int i = lane; i < G; i += 32) a = fmaxf(a, fabsf(__bfloat162float(w[i])));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
-  if (lane == 0) {
-    const float qmax = (float)((1 << (bits - 1)) - 1);
-    const __half s = __float2half_rn(__fdiv_rn(a, qmax));
-    const int chunk = j / CH, c = j % CH;
-    const int nchunks = F / CH;
-    S[(((size_t)g * nchunks + chunk) * 2 + which) * CH + c] = s;
-    s_plain[((size_t)which * F + j) * ngroups + g] = __half2float(s);
-  }
-}
-
-// One thread per packed 32-bit word.
-__global__ void proxy_pack_kernel(const __nv_bfloat16* __restrict__ wg,
-                                  const __nv_bfloat16* __restrict__ wu, int D, int F, int G,
-                                  int bits, const float* __restrict__ s_plain,
-                                  uint32_t* __restrict__ P) {
-  const int CH = (bits == 4) ? 16 : 8;
-  const int per_word = (bits == 4) ? 8 : 4;
-  const int nchunks = F / CH;
-  const int ngroups = D / G;
-  const long long words_per_row = (long long)nchunks * 4;
-  // consecutive threads take consecutive input coordinates (coalesced reads of W)
-  const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long total = words_per_row * D;
-  if (tid >= total) return;
-  const int i = (int)(tid % D);
-  const long long wword = tid / D;                 // word index within the row
-  const int chunk = (int)(wword >> 2), word = (int)(wword & 3);
-  const int which = word >> 1;                     // 0 gate, 1 up
-  const int j0 = chunk * CH + (word & 1) * per_word;
-  const __nv_bfloat16* w = which ? wu : wg;
-  const float qmax = (float)((1 << (bits - 1)) - 1);
-  const int g = i / G;
-  uint32_t out = 0;
-  for (int m = 0; m < per_word; ++m) {
-    const int j = j0 + m;
-    const float s = s_plain[((size_t)which * F + j) * ngroups + g];
-    const float v = __bfloat162float(w[(size_t)j * D + i]);
-    int q = 0;
-    if (s != 0.f) {
-      float r = rintf(__fdiv_rn(v, s));
-      r = fminf(fmaxf(r, -qmax), qmax);
-      q = (int)r;
-    }
-    const uint32_t code = (uint32_t)(q + (bits == 4 ? 8 : 128));
-    out |= code << (m * bits);
-  }
-  P[(size_t)i * words_per_row + wword] = out;
-}
-
-// 16-bit "proxies" (ablation A1 of Sec. "Ablation Studies"; also the 16-bit input-sparse GEMV that
-// the cost ratio alpha of Sec. 4.2 is measured against): the original bf16 weights in the proxies'
-// input-major order.  A 16-byte chunk of row i holds 4 channels: words 0,1 gate, words 2,3 up.
-// One thread per 32-bit word (two channels of one matrix).
-__global__ void proxy_pack16_kernel(const uint16_t* __restrict__ wg, const uint16_t* __restrict__ wu,
-                                    int D, int F, uint32_t* __restrict__ P) {
-  const long long words_per_row = (long long)(F / 4) * 4;
-  const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (tid >= words_per_row * D) return;
-  const int i = (int)(tid % D);                    // consecutive threads: consecutive inputs (coalesced reads)
-  const long long wword = tid / D;
-  const int chunk = (int)(wword >> 2), word = (int)(wword & 3);
-  const uint16_t* w = (word >> 1) ? wu : wg;
-  const int j0 = chunk * 4 + (word & 1) * 2;
-  P[(size_t)i * words_per_row + wword] =
-      (uint32_t)w[(size_t)j0 * D + i] | ((uint32_t)w[(size_t)(j0 + 1) * D + i] << 16);
-}
-
-// W_down [D, F] -> channel-major [F, D]  (Sec. 3.1: y = sum_j s_j W_down[j,:]).
-__global__ void transpose_bf16_kernel(const uint16_t* __restrict__ in, uint16_t* __restrict__ out,
-                                      int rows, int cols) {
-  __shared__ uint16_t tile[32][33];
-  int c = blockIdx.x * 32 + threadIdx.x;
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    int rr = blockIdx.y * 32 + r;
-    if (rr < rows && c < cols) tile[r][threadIdx.x] = in[(size_t)rr * cols + c];
-  }
-  __syncthreads();
-  int oc = blockIdx.y * 32 + threadIdx.x;            // output column = input row
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    int orow = blockIdx.x * 32 + r;                  // output row = input column
-    if (orow < cols && oc < rows) out[(size_t)orow * rows + oc] = tile[threadIdx.x][r];
-  }
 }
 
 // ----------------------------------------------------------------------------
