@@ -125,7 +125,7 @@ prox_status_t prox_ffn_forward(prox_ffn_t* h, const void* x_dev, int B, int k1, 
                                void* y_dev, void* stream);
 
 /* For B = 1 prox_ffn_forward runs the whole path as ONE persistent kernel
- * (cooperative launch, one block per SM, one grid-wide barrier with a bounded
+ * (one block per SM, one grid-wide barrier with a bounded
  * wait between Stage 1 and Stage 2); prox_ffn_set_fused(h, 0) selects the
  * kernel-per-step path instead (always used for B > 1).  If a bounded wait
  * ever expires the kernel leaves, y is not written (undefined) and
@@ -183,6 +183,10 @@ prox_status_t prox_ffn_last_stage1(prox_ffn_t* h, int k1, int32_t* idx_dev_or_nu
  * without writing y and reports it (see prox_last_device_status).  Nothing hangs or faults: the
  * blocks give up and return.  Set both back to 0 afterwards. */
 prox_status_t prox_debug_set_wait(prox_ffn_t* h, uint32_t spin_limit, uint32_t barrier_bias);
+
+/* Test hook: blocks the persistent kernel is launched with (0 = one per SM, at most that).  With fewer, the blocks
+ * that run take over the work of the others, as they would if the rest of the grid had to wait for an SM. */
+prox_status_t prox_debug_set_grid(prox_ffn_t* h, int blocks);
 
 /* Copy the channel mask of the most recent prox_ffn_forward call (top-k rule)
  * into sel_dev, dev int32 [B, k2], ascending per token.  Enqueued on stream. */

@@ -76,6 +76,7 @@ _SIGS = {
     "prox_ffn_last_mask": [_vp, _i, _i, _vp, _vp],
     "prox_ffn_last_stage1": [_vp, _i, _vp, _vp, _vp],
     "prox_debug_set_wait": [_vp, C.c_uint32, C.c_uint32],
+    "prox_debug_set_grid": [_vp, _i],
     "prox_calib_create": [C.c_int64, C.c_uint64, C.POINTER(_vp)],
     "prox_calib_add": [_vp, _vp, C.c_int64, _i, _vp],
     "prox_calib_threshold": [_vp, _d, C.POINTER(_f)],
@@ -396,6 +397,10 @@ def prox_ffn_last_stage1(handle: int, k1: int, idx=None, scores=None, stream=Non
 
 def prox_debug_set_wait(handle: int, spin_limit: int, barrier_bias: int) -> None:
     _check(_lib.prox_debug_set_wait(handle, spin_limit, barrier_bias), "prox_debug_set_wait")
+
+
+def prox_debug_set_grid(handle: int, blocks: int) -> None:
+    _check(_lib.prox_debug_set_grid(handle, blocks), "prox_debug_set_grid")
 
 
 def prox_launch_count(handle: int) -> int:

@@ -54,10 +54,10 @@ struct prox_ffn {
   float* yacc;              // [maxB][D]
   int* dev_status;
   unsigned long long* counters;  // [0] tokens, [1] kept inputs, [2] kept channels
-  unsigned* syncbuf;        // fused kernel: [0..4095] two score histograms (calls alternate), [4096] barrier count,
-                            // (64-bit, [4096..4097]), [4098] finish ticket
+  unsigned* syncbuf;        // fused kernel: [0..4095] two score histograms (calls alternate), [4096..4097] 64-bit count
+                            // of blocks that have left, [4104..4119] two sets of share counters
   int smem_optin;           // largest dynamic shared memory a block may ask for
-  int coop;                 // device supports cooperative launch
+  int debug_grid;           // test knob: blocks of the persistent kernel (0 = one per SM)
   int sel_unordered;        // the last forward left its mask in the persistent kernel's own order
   int use_fused;            // batch-1 forward runs as one persistent kernel
   int use_union;            // batch > 1 reads weights once for the union of the tokens' masks
@@ -625,7 +625,7 @@ prox_status_t launch_stage2_batch(prox_ffn* h, const void* x, int B, const int* 
 // ---- fused persistent kernel (batch 1) ----------------------------------------
 struct FusedPlan {
   bool ok;
-  int grid, pstages, big_bytes, nslots, xch;
+  int grid, loaders, cgran, nshare1, big_bytes, nslots, xch;
   size_t smem;
   int device;           // the handle's GPU
   int optin;            // the device's opt-in limit: what the kernels' dynamic shared memory attribute is set to
@@ -635,20 +635,30 @@ FusedPlan plan_fused(const prox_ffn* h, int k1, int k2, bool thresh = false) {
   FusedPlan pl;
   std::memset(&pl, 0, sizeof(pl));
   const int D = h->cfg.d_model, F = h->cfg.d_ff;
-  if (!h->use_fused || !h->coop || h->bits == 16) return pl;       // the fused kernel reads integer proxies
+  if (!h->use_fused || h->bits == 16) return pl;       // the fused kernel reads integer proxies
   const int G = h->sm_count;
   const size_t fixed = ((sizeof(FusedSmem) + 127) & ~size_t(127)) + (size_t)8 * D;   // + x bf16, idx, x fp32
-  if ((size_t)h->smem_optin < fixed + (size_t)6 * D + 16384) return pl;
+  if ((size_t)h->smem_optin < fixed + (size_t)6 * D) return pl;
   pl.big_bytes = (int)(((size_t)h->smem_optin - fixed) & ~size_t(127));
   pl.nslots = pl.big_bytes / (2 * D);
   if (pl.nslots > kMaxSlots) pl.nslots = kMaxSlots;
   if (pl.nslots < 3) return pl;
   // the proxy GEMV keeps 16 tensor-memory columns per supergroup (4 scale groups), two sets of up to 256
   if ((D / h->group + 3) / 4 > kMaxSuper) return pl;
-  pl.pstages = (pl.big_bytes - 1024 - 3072) / kPStageBytes;
-  if (pl.pstages > kPStages) pl.pstages = kPStages;
-  if (pl.pstages < kPStages) return pl;                                   // every loader warp owns a stage
-  if (pl.big_bytes < 4 * D * 4) return pl;                                // partial y vectors of the down projection
+  // the proxy ring and its partial sums take the place of x as fp32 and the big buffer
+  pl.loaders = (int)((4 * (size_t)D + pl.big_bytes - 1024 - 3072) / proxy_warp_bytes(h->bits));
+  if (pl.loaders > kFusedConsumerWarps) pl.loaders = kFusedConsumerWarps;
+  if (pl.loaders < kMinLoaders) return pl;
+  // Columns of the packed rows per block: whole 128-byte tiles (8 chunks) while there is at most one per SM: narrower
+  // shares on all SMs took as long or longer (4096 x 12288: 8.0 us either way with 96 tiles; 1024 x 3072: 3.5 against
+  // 4.1 us, more blocks add to the same few histogram bins).  Beyond that equal shares in 32-byte sectors: 224 tiles
+  // on 148 SMs took two rounds (4096 x 14336, 8 bits: 38 us against 30).
+  const int nchunks = F / ch_per_chunk(h->bits);
+  pl.cgran = nchunks <= 8 * G ? 8 : 2;                   // (nchunks is a multiple of 4: d_ff is one of 64)
+  const int nunit = (nchunks + pl.cgran - 1) / pl.cgran;
+  pl.nshare1 = nunit < G ? nunit : G;
+  pl.xch = D <= 4096 ? 4 : (D <= 8192 ? 2 : 1);          // warp groups of the down projection
+  if (pl.big_bytes < pl.xch * D * 4) return pl;          // their partial y vectors
   if ((k2 + G - 1) / G + 2 > kMySelCap) return pl;       // a block's share: definite part + part of the threshold bin
   if (thresh) {
     // any number of channels may pass the threshold: a block's share of all of them must fit, the scores
@@ -656,8 +666,7 @@ FusedPlan plan_fused(const prox_ffn* h, int k1, int k2, bool thresh = false) {
     if ((F + G - 1) / G + 2 > kMySelCap || (size_t)F * 4 + 256 > (size_t)pl.big_bytes || F >= 65536) return pl;
   }
   (void)k1;
-  pl.grid = G;
-  pl.xch = D <= 4096 ? 4 : (D <= 8192 ? 2 : 1);          // warp groups of the down projection
+  pl.grid = h->debug_grid ? h->debug_grid : G;
   pl.smem = fixed + (size_t)pl.big_bytes;
   pl.optin = h->smem_optin;
   pl.device = h->device;
@@ -682,22 +691,19 @@ cudaError_t launch_fused_tn(const FusedPlan& pl, const FusedParams& prm, cudaStr
   cfg.blockDim = dim3(kFusedThreads);
   cfg.dynamicSmemBytes = pl.smem;
   cfg.stream = st;
-  // Cooperative (all blocks co-resident: the kernel has a grid barrier) and, if the driver takes the two
-  // together, programmatic stream serialization: the next launch on the stream is set up while this one
+  // Programmatic stream serialization: the next launch on the stream is set up while this one
   // drains, and its blocks wait (griddepcontrol.wait) for this grid to complete before they read anything.
   static int use_pdl = getenv("PROX_NO_PDL") ? 0 : 1;
-  cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeCooperative;
-  at[0].val.cooperative = 1;
-  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = use_pdl ? 2 : 1;
+  cfg.numAttrs = use_pdl ? 1 : 0;
   cudaError_t e = cudaLaunchKernelEx(&cfg, kern, prm);
   if (e != cudaSuccess && use_pdl) {
     (void)cudaGetLastError();
     use_pdl = 0;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 0;
     e = cudaLaunchKernelEx(&cfg, kern, prm);
   }
   return e;
@@ -732,11 +738,12 @@ prox_status_t launch_fused(prox_ffn* h, const FusedPlan& pl, const void* x, int 
   prm.D = h->cfg.d_model; prm.F = h->cfg.d_ff; prm.k1 = k1; prm.k2 = k2;
   prm.gshift = (h->group == h->cfg.d_model) ? 31 : 7;
   prm.out_fp32 = h->cfg.out_dtype;
-  prm.pstages = pl.pstages;
+  prm.loaders = pl.loaders; prm.cgran = pl.cgran;
   prm.scores = h->scores; prm.ghist = h->syncbuf; prm.idx_out = h->idx_x;
   prm.spin_limit = h->spin_limit; prm.bar_bias = h->bar_bias; prm.host_flag = h->host_flag_dev;
   prm.sel_out = sel_out; prm.yacc = h->yacc;
-  prm.bar_count = reinterpret_cast<unsigned long long*>(h->syncbuf + 4096); prm.done_ticket = h->syncbuf + 4098;
+  prm.exits = reinterpret_cast<unsigned long long*>(h->syncbuf + 4096); prm.ctr = h->syncbuf + 4104;
+  prm.nshare = h->sm_count; prm.nshare1 = pl.nshare1;
   prm.status = h->dev_status;
   prm.big_bytes = pl.big_bytes; prm.nslots = pl.nslots;
   prm.trace = h->trace;
@@ -872,7 +879,6 @@ prox_status_t prox_ffn_create(const prox_ffn_config_t* cfg, const void* w_gate, 
     if (st == PROX_OK) A(cudaMemset(h->gacc, 0, (size_t)((F + 15) / 16) * 256 * sizeof(float)));
   }
   A(cudaDeviceGetAttribute(&h->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
-  A(cudaDeviceGetAttribute(&h->coop, cudaDevAttrCooperativeLaunch, h->device));
   h->spin_limit = kSpinLimit;
   if (st == PROX_OK) {
     A(cudaHostAlloc(reinterpret_cast<void**>(&h->host_flag), sizeof(int), cudaHostAllocMapped));
@@ -1130,7 +1136,7 @@ prox_status_t prox_fused_kernel_info(prox_ffn_t* h, int k1, int k2, int32_t* inf
   CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, pl.optin));
   int nb = 0;
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kFusedThreads, pl.smem));
-  info[1] = pl.grid; info[2] = pl.pstages; info[3] = (int)pl.smem; info[4] = pl.nslots;
+  info[1] = pl.grid; info[2] = pl.loaders; info[3] = (int)pl.smem; info[4] = pl.nslots;
   info[5] = fa.numRegs; info[6] = (int)fa.sharedSizeBytes; info[7] = nb;
   return PROX_OK;
 }
@@ -1568,6 +1574,12 @@ prox_status_t prox_debug_set_wait(prox_ffn_t* h, uint32_t spin_limit, uint32_t b
   if (!h) return PROX_ERR_INVALID_ARG;
   h->spin_limit = spin_limit ? spin_limit : kSpinLimit;
   h->bar_bias = barrier_bias;
+  return PROX_OK;
+}
+
+prox_status_t prox_debug_set_grid(prox_ffn_t* h, int blocks) {
+  if (!h || blocks < 0 || blocks > h->sm_count) return PROX_ERR_INVALID_ARG;
+  h->debug_grid = blocks;
   return PROX_OK;
 }
 

@@ -2,8 +2,8 @@
 //
 //   A  every block: exact top-k1 of |x| (redundantly; x is a few KB)
 //   B  proxy GEMV on the tensor cores (tcgen05, integer MMA, accumulators in
-//      tensor memory): a block owns 128-byte column tiles of the packed proxy
-//      over ALL kept rows, so the sums of a tile need no exchange with other
+//      tensor memory): a block owns an equal share of the packed proxy's columns
+//      over ALL kept rows, so its channels' sums need no exchange with other
 //      blocks; the rows' bytes are the A operand as they lie in memory, x enters
 //      as signed base-256 digits; the block writes the scores |u~ SiLU(g~)| of
 //      its channels and adds them to a global 2048-bin histogram
@@ -26,7 +26,12 @@
 //      added to an fp32 accumulator with vector atomics
 //   F  the last block to finish (ticket) rounds y once and clears the scratch.
 //
-// Launch: cooperative (all blocks co-resident), one block per SM.
+// Launch: an ordinary one, one block per SM, with programmatic stream serialization.  No block waits for a block that
+// may not be running: the shares of Stage 1 (columns) and of Stage 2 (kept channels) are claimed by tickets, a
+// running block claims again until there are none left, and the barrier counts finished shares, not blocks.  Where all
+// blocks run, as always on a GPU of its own, every block has one share of each.  (With the cooperative attribute
+// instead, launches of a stream did not overlap and started in steps of 2.05 us:
+// 512 x 1536 20.5 -> 19.6 us per call, 1024 x 3072 layer form 22.4 -> 20.5, 4096 x 12288 38.9 -> 37.7.)
 #pragma once
 
 #include "prox_kernels.cuh"
@@ -47,8 +52,10 @@ constexpr int kChanBatch = 256;      // channels whose h values are held at once
 constexpr int kMySelCap = 512;       // channels one block may own
 constexpr int kCandCap = 4096;       // threshold-bin candidates kept in shared memory
 constexpr int kCand2Cap = 256;       // candidates left after the second refinement
-constexpr int kPStages = 16;             // ring of 32-row stages of the proxy GEMV (one per loader warp)
-constexpr int kPStageBytes = 9216;       // a stage: 4096 bytes of rows | 4096 low nibbles | 512 digits of x | pad
+// Proxy ring: a loader warp owns two stages of 32 rows x 128 bytes (4 KB each), for 4-bit codes a buffer of low
+// nibbles (4 KB), and two stages of digits of x (512 bytes each).
+__host__ __device__ constexpr int proxy_warp_bytes(int bits) { return bits == 4 ? 13312 : 9216; }
+constexpr int kMinLoaders = 8;           // loader warps that must fit (at most all 16 consumer warps)
 constexpr int kMaxSuper = 16;            // supergroups (4 scale groups) whose accumulators fit the tensor memory
 constexpr unsigned kSpinLimit = 1u << 21;
 
@@ -57,13 +64,17 @@ struct FusedParams {
   const uint16_t* wg; const uint16_t* wu; const uint16_t* wdt;
   const uint16_t* x; void* y;
   int D, F, k1, k2, gshift, out_fp32;
-  int pstages;        // stages of the proxy ring that fit (<= kPStages)
+  int loaders;        // loader warps of the proxy GEMV whose stages fit
+  int cgran;          // the proxy rows' 16-byte column chunks are dealt out in units of this many
   float* scores; unsigned* ghist; int* sel_out;
   int* idx_out;       // the kept input list as this kernel built it (block 0 writes it; for checking)
   unsigned spin_limit;        // polls after which a device-side wait gives up
   unsigned bar_bias;          // test knob: added to the grid barrier's target (0 in normal use)
   int* host_flag;             // mapped host word set to 1 when a wait expires (NULL = none)
-  float* yacc; unsigned long long* bar_count; unsigned* done_ticket; int* status;
+  float* yacc; int* status;
+  unsigned long long* exits;  // grows by 256 per call, complete when all its blocks have left: the call number
+  unsigned* ctr;              // [2][8] counters of a call (calls alternate): see FusedCtr
+  int nshare1, nshare;        // shares of Stage 1 and of Stage 2
   int big_bytes;      // bytes of the large shared buffer
   int nslots;         // ring slots of D*2 bytes inside it
   unsigned long long* trace;   // optional [grid][32] phase time stamps (ns), NULL = off
@@ -76,6 +87,8 @@ struct FusedParams {
   unsigned tkey_x, tkey_s;
   int* cnt_x_out; int* count_out; unsigned long long* counters;
 };
+
+enum FusedCtr { kClaim1 = 0, kDone1, kClaim2, kDone2 };    // shares claimed / finished, Stage 1 and Stage 2
 
 // ---- PTX wrappers -----------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -269,7 +282,11 @@ struct FusedSmem {
   int cand2_idx[kCand2Cap];
   int abort_flag;
   int s_last;
-  unsigned call_par;          // parity of the handle's call number: which of the two global histograms is this call's
+  unsigned call_par;          // parity of the handle's call number: which set of global histogram and counters is this call's
+  unsigned vid;               // Stage 1: share of this block (none: >= number of shares)
+  int late;                   // the block started after Stage 1 was complete: it has no part in the call
+  int again;                  // another Stage-1 share was claimed
+  unsigned shr, shr_next;     // Stage 2: share of this block, and the next one
   unsigned ncand;
   unsigned ncand2;
   unsigned prod_seq;       // rows the producers have armed so far (for the give-up path)
@@ -282,11 +299,9 @@ struct FusedSmem {
   int keys_s0, keys_s1;    // ring slots [s0, s1) that overlap the keys
   int list_s0, list_s1;    // ... and the list
   unsigned slot_use[kMaxSlots];   // uses of each ring slot whose data has been seen complete
-  unsigned long long pempty[kPStages];   // proxy ring: the MMAs have read the stage of warp w
+  unsigned long long pempty[kFusedConsumerWarps];   // proxy ring: the MMAs of a warp's block are complete
   unsigned long long acc_bar;            // all MMAs of a tile are complete (one arrival per loader warp)
   uint32_t tmem_base;
-  int sstart[kMaxSuper + 2];             // first kept row of every supergroup (and k1)
-  int bstart[kMaxSuper + 2];             // first 32-row block of every supergroup (and the block count)
   float soff[4 * kMaxSuper];             // per scale group: code offset (8 or 128) * sum of the kept x, as integers
   int gstart[4 * kMaxSuper + 2];         // first kept row of every scale group (and k1)
   unsigned soff_cnt;                     // warps that have finished their share of soff
@@ -301,7 +316,7 @@ struct FusedSmem {
 // Instantiations of their own, so that the plain call carries none of their code or registers.
 template <int BITS, int NG, bool NORM = false, bool THRESH = false>
 __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const FusedParams p) {
-  constexpr int CH = ProxyFmt<BITS>::CH, NACC = ProxyFmt<BITS>::NACC;
+  constexpr int CH = ProxyFmt<BITS>::CH;
   constexpr int NT = kFusedThreads;
   extern __shared__ __align__(128) uint8_t smem_raw[];
   FusedSmem& sm = *reinterpret_cast<FusedSmem*>(smem_raw);
@@ -309,6 +324,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   int k1 = p.k1;                         // THRESH: becomes the number of kept inputs after phase A
   uint16_t* xs = reinterpret_cast<uint16_t*>(smem_raw + ((sizeof(FusedSmem) + 127) & ~size_t(127)));
   uint16_t* idx16 = xs + D;
+  // x as fp32, written after phase B: until then its place belongs to the proxy ring, as the big buffer behind it does
   float* xf = reinterpret_cast<float*>(idx16 + D);
   uint8_t* big = reinterpret_cast<uint8_t*>(xf + D);           // 128-byte aligned: D % 128 == 0
   const uint32_t big_u32 = smem_u32(big);
@@ -326,9 +342,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     fence_mbar_init();
   }
   if (warp == 0) tmem_alloc_all(smem_u32(&sm.tmem_base));      // all 512 columns: one block per SM
-  if (tid < kPStages) {
+  if (tid < kFusedConsumerWarps) {
     mbar_init(smem_u32(&sm.pempty[tid]), 1);
-    if (tid == 0) mbar_init(smem_u32(&sm.acc_bar), kFusedConsumerWarps);
+    if (tid == 0) mbar_init(smem_u32(&sm.acc_bar), (uint32_t)p.loaders);
     fence_mbar_init();
   }
   if (tid == 0) sm.soff_cnt = 0;
@@ -340,13 +356,11 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   asm volatile("griddepcontrol.wait;" ::: "memory");
   // Two global score histograms take turns: this call adds to one and clears the other for the next call (it was
   // last used by the previous call, which has completed), so nothing is left to clean up when the call ends.
-  // The call number is the barrier counter over the grid size: the counter only grows, by one per block and
-  // call, and this call's own increments cannot complete a multiple of the grid size before every block has
-  // passed this point (each block adds its one after phase B).
+  // The call number is exits / 256: blocks of this call that have left add less than 256 until the last one does.
   if (tid == NT - 1) {                          // a thread with no share of the input load below
-    unsigned long long bc;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(bc) : "l"(p.bar_count) : "memory");
-    sm.call_par = (unsigned)((bc / (unsigned long long)G) & 1ull);
+    unsigned long long ex;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(ex) : "l"(p.exits) : "memory");
+    sm.call_par = (unsigned)(ex >> 8) & 1u;
   }
   if (NORM) {
     // FFN input = bf16(RMSNorm(residual stream) * norm weight), the correctly rounded value (the masks
@@ -392,27 +406,29 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     for (int i = tid; i < D; i += NT) {
       const uint16_t b = rms_scale_to_bf16(xf[i], __uint_as_float((uint32_t)idx16[i] << 16), ih, il);
       xs[i] = b;
-      xf[i] = __uint_as_float((uint32_t)b << 16);
     }
   } else {
     const uint4* xg = reinterpret_cast<const uint4*>(p.x);
-    for (int i = tid; i < D / 8; i += NT) {
-      const uint4 v = __ldg(xg + i);
-      reinterpret_cast<uint4*>(xs)[i] = v;
-      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-      reinterpret_cast<float4*>(xf)[2 * i] = make_float4(bf16_lo(w[0]), bf16_hi(w[0]), bf16_lo(w[1]), bf16_hi(w[1]));
-      reinterpret_cast<float4*>(xf)[2 * i + 1] = make_float4(bf16_lo(w[2]), bf16_hi(w[2]), bf16_lo(w[3]), bf16_hi(w[3]));
-    }
+    for (int i = tid; i < D / 8; i += NT) reinterpret_cast<uint4*>(xs)[i] = __ldg(xg + i);
     for (int i = tid; i < 1024 + 32; i += NT) { if (i < 1024) sm.hist[i] = 0; else sm.hist2[i - 1024] = 0; }
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   unsigned* const ghist = p.ghist + 2048u * sm.call_par;
+  unsigned* const ctr = p.ctr + 8u * sm.call_par;
+  // Stage-1 share of this block; the answers are first looked at after phase A.  A block that gets none and finds
+  // Stage 1 complete has started late: it leaves (what it read may be a residual stream that is being added to).
+  unsigned claim1 = 0, done1 = 0;
+  if (tid == NT - 1) {
+    asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(claim1) : "l"(ctr + kClaim1) : "memory");
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(done1) : "l"(ctr + kDone1) : "memory");
+  }
   {
     unsigned* const other = p.ghist + 2048u * (sm.call_par ^ 1u);
     const int per = (2048 + G - 1) / G;
     for (int i = cta * per + tid; i < min(2048, (cta + 1) * per); i += NT) other[i] = 0u;
+    if (cta == 0 && tid < 8) p.ctr[8u * (sm.call_par ^ 1u) + tid] = 0u;
   }
   if (warp < 4) {
     // the accumulators of the proxy GEMV start at zero: 16 columns per supergroup, two sets 256 columns apart
@@ -498,10 +514,6 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     ebase = max(max((int)(mk >> 7), 1) - 22, 1);
     if (THRESH) {
       k1 = (int)__reduce_add_sync(0xffffffffu, (lane < kFusedWarps) ? (sm.wsum[lane] & 0xffffu) : 0u);
-      if (cta == 0 && tid == 0) {
-        if (p.cnt_x_out) p.cnt_x_out[0] = k1;
-        if (p.counters) { atomicAdd(p.counters, 1ull); atomicAdd(p.counters + 1, (unsigned long long)k1); }
-      }
     }
     {
       const unsigned ex = __reduce_add_sync(0xffffffffu, (lane < warp) ? sm.wsum[lane] : 0u) + inc - cnt;
@@ -523,114 +535,159 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       }
     }
     if (tid == 0) sm.gstart[per_row_a ? 1 : (D >> p.gshift)] = k1;
+    if (tid == NT - 1) { sm.vid = claim1; sm.late = done1 >= (unsigned)p.nshare1 && claim1 >= (unsigned)p.nshare1; }
     __syncthreads();
   }
-
-  if (cta == 0 && p.idx_out) {
+  // every block counts its leaving
+  auto leave = [&]() {
+    if (tid == 0) atomicAdd(p.exits, cta == 0 ? 257ull - (unsigned long long)G : 1ull);
+  };
+  if (sm.late) {
+    if (warp == 0) tmem_free_all(sm.tmem_base);
+    leave();
+    return;
+  }
+  if (sm.vid == 0) {
+    if (p.idx_out) {
 #pragma unroll 1
-    for (int i = tid; i < k1; i += NT) p.idx_out[i] = (int)idx16[i];
+      for (int i = tid; i < k1; i += NT) p.idx_out[i] = (int)idx16[i];
+    }
+    if (THRESH && tid == 0) {
+      if (p.cnt_x_out) p.cnt_x_out[0] = k1;
+      if (p.counters) { atomicAdd(p.counters, 1ull); atomicAdd(p.counters + 1, (unsigned long long)k1); }
+    }
   }
   PROX_TRACE(2);
   // --------------------------------------- B: proxy GEMV (tensor cores), scores, score histogram
   // Per scale group g:  sum_k x_k q_kj = 2^(ebase-134) * sum_k X_k (byte_kj - offset), X_k the integer
-  // form of x_k (x_digits).  A block owns 128-byte tiles of the packed rows over all kept rows.  The kept
+  // form of x_k (x_digits).  A block owns a share of the packed rows' 16-byte column chunks (dealt out in units of
+  // p.cgran) over all kept rows, in tiles of at most 8 chunks.  The kept
   // rows are cut into blocks of at most 32 rows that stay inside one supergroup (4 scale groups); block b
   // accumulates into 16 tensor-memory columns of its supergroup: column 4 * (g % 4) + d holds digit d of
-  // group g.  16 loader warps bring the rows in with plain 16-byte loads (8 in flight per lane) and store
-  // them (and the bytes with the high nibble masked off, and the digits of x) in a stage of the ring;
-  // one thread issues the MMAs; after the last one the 16 warps read the accumulators, apply the
+  // group g.  The loader warps bring the rows in with 16-byte asynchronous copies, a block ahead (what bounds this is
+  // the bytes in flight: 64 KB per SM give 3.5 TB/s, 128 KB 5.2), add
+  // the bytes with the high nibble masked off and the digits of x, and
+  // issue the block's MMAs; after the last one the 16 warps read the accumulators, apply the
   // groups' scales and form the scores.
-  {
+  // Measured (this phase, one call): 4096 x 14336 8-bit, all rows: 42.9 -> 33 us (59 MB of copies: 3.6 TB/s); 8192 x 28672
+  // 4-bit, 2458 rows: 24 us, where that shape did not fit and a kernel of its own took 46; 4096 x 12288 4-bit, 1229 rows:
+  // 8 us as before (the first rows arrive 3 us after phase A, the last 2.5 us later).
+  unsigned uses = 0, acc_n = 0;              // blocks of rows this warp has handed to the tensor core; tiles read back
+#pragma unroll 1
+  for (bool first = true;; first = false) {
     constexpr bool LO = (BITS == 4);
     const int nchunks = F / CH;
     const int row_bytes = nchunks * 16;
-    const int ntiles = (row_bytes + 127) >> 7;
+    const unsigned nunit = (unsigned)((nchunks + p.cgran - 1) / p.cgran), vid = sm.vid, n1 = (unsigned)p.nshare1;
+    const int ck0 = vid < n1 ? p.cgran * (int)((nunit * vid) / n1) : 0;                      // this block's chunks
+    const int ckn = vid < n1 ? min(nchunks, p.cgran * (int)((nunit * (vid + 1u)) / n1)) - ck0 : 0;
+    const int ntl = (ckn + 7) >> 3;
     const bool per_row = p.gshift >= 31;
     const int ng = per_row ? 1 : (D >> p.gshift);
     const int nsuper = (ng + 3) >> 2;
-    const int sgshift = per_row ? 31 : p.gshift + 2;
     const uint32_t tbase = sm.tmem_base;
-    // supergroup starts and blocks (one warp), the groups' offsets, the block's own score histogram
-    if (warp == 0) {
-      const int r0s = sm.gstart[min(4 * lane, ng)], r1s = sm.gstart[min(4 * lane + 4, ng)];
-      const unsigned nb = lane < nsuper ? (unsigned)((r1s - r0s + 31) >> 5) : 0u;
-      const unsigned incb = warp_scan_incl(nb, lane);
-      if (lane <= nsuper) { sm.sstart[lane] = r0s; sm.bstart[lane] = (int)(incb - nb); }
-    }
+    if (warp < kFusedConsumerWarps) {          // the block's own score histogram (used after a consumer barrier)
 #pragma unroll 1
-    for (int i = tid; i < 512; i += NT) reinterpret_cast<uint4*>(sm.hist)[i] = make_uint4(0u, 0u, 0u, 0u);
-    __syncthreads();
-    const int nblk = sm.bstart[nsuper];
-    const uint32_t ring = (big_u32 + 1023u) & ~1023u;
-    float* red = reinterpret_cast<float*>(big + (ring - big_u32) + (uint32_t)(kPStages * kPStageBytes));   // [3][128][2] partial sums of warps 4..15
+      for (int i = tid; i < 512; i += kFusedConsumers) reinterpret_cast<uint4*>(sm.hist)[i] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    const uint32_t ring = (smem_u32(xf) + 1023u) & ~1023u;
+    const int NL = p.loaders;
+    float* red = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(xf) + (ring - smem_u32(xf)) + (uint32_t)(NL * proxy_warp_bytes(BITS)));   // [3][128][2] partial sums of warps 4..15
     PROX_TRACE(29);
     if (warp < kFusedConsumerWarps) {
-      // a warp owns one stage of the ring: it fills it and issues the stage's MMAs itself (the tensor core
+      // a warp owns its stages of the ring: it fills them and issues their MMAs itself (the tensor core
       // takes accumulating MMAs from several threads into the same columns; integer sums do not depend on the order)
-      const uint32_t stg = ring + (uint32_t)warp * (uint32_t)kPStageBytes;
-      const uint64_t adesc = umma_smem_desc(stg, 4096u, 1024u, 2u);
-      const uint64_t ldesc = umma_smem_desc(stg + 4096u, 4096u, 1024u, 2u);
-      const uint64_t bdesc = umma_smem_desc(stg + 8192u, 128u, 512u, 0u);
+      const uint32_t stg = ring + (uint32_t)warp * (uint32_t)proxy_warp_bytes(BITS);
+      const uint32_t dig = stg + (LO ? 12288u : 8192u);
+      const uint64_t adesc = umma_smem_desc(stg, 4096u, 1024u, 2u);                  // second stage: 4096 bytes on
+      const uint64_t ldesc = umma_smem_desc(stg + 8192u, 4096u, 1024u, 2u);
+      const uint64_t bdesc = umma_smem_desc(dig, 128u, 512u, 0u);                    // second stage: 512 bytes on
       constexpr uint32_t idesc = umma_idesc_u8s8(128, 16);
       const uint32_t my_empty = smem_u32(&sm.pempty[warp]);
       const int q4 = warp & 3, part = warp >> 2;
       const int col = q4 * 32 + lane;                          // byte column of the tile = data path lane
-      const int c = lane & 7, kq = lane >> 3;
-      unsigned uses = 0;                                       // stages this warp has handed to the tensor core
-      int tile_iter = 0;
+      // blocks of 32 rows: lane l knows supergroup l's first row, its end and the number of the first block behind it
+      const int sg_r0 = sm.gstart[min(4 * lane, ng)], sg_r1 = sm.gstart[min(4 * lane + 4, ng)];
+      const unsigned sg_nb = lane < nsuper ? (unsigned)((sg_r1 - sg_r0 + 31) >> 5) : 0u;
+      const int sg_end = nsuper > 1 ? (int)warp_scan_incl(sg_nb, lane) : __shfl_sync(0xffffffffu, (int)sg_nb, 0);
+      const int nblk = __shfl_sync(0xffffffffu, sg_end, 31);
 #pragma unroll 1
-      for (int tile = cta; tile < ntiles; tile += G, ++tile_iter) {
-        // ---- scales of this thread's byte column for the groups it will read back
-        const int chunk = tile * 8 + (col >> 4);
-        const bool col_ok = chunk < nchunks;
-        const bool c_ok = tile * 8 + c < nchunks;
+      for (int tl = 0; tl < ntl; ++tl) {
+        const int tc0 = tl * 8, w = min(8, ckn - tc0);         // the tile's chunks (of the block's)
+        // a copy instruction covers 32 >> sc rows of up to 1 << sc chunks
+        const int sc = w > 4 ? 3 : (w > 2 ? 2 : 1), rpi = 32 >> sc;
+        const int kq = lane >> sc, c = lane & ((1 << sc) - 1);
+        const bool lane_on = c < w;
+        const uint8_t* tp = p.P + (size_t)(ck0 + tc0) * 16 + (size_t)c * 16;
+        const int chunk = ck0 + tc0 + (col >> 4);              // chunk of this thread's byte column
+        const bool col_ok = (col >> 4) < w;
         bool alive_b = true;
-        int sg = 0;
+        // The copies of a warp's block k are on their way while its block k - 1 goes to the tensor core.
+        // (One copy of the code for all blocks: everything here is fetched cold on every call.)
+        int r0 = 0, nrows = 0, sg = 0;
 #pragma unroll 1
-        for (int b = warp; b < nblk; b += kFusedConsumerWarps) {
-          while (sm.bstart[sg + 1] <= b) ++sg;
-          const int r0 = sm.sstart[sg] + ((b - sm.bstart[sg]) << 5);
-          const int nrows = min(32, sm.sstart[sg + 1] - r0);
-          uint4 v[8];
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const int kk = j * 4 + kq;
-            v[j] = make_uint4(0u, 0u, 0u, 0u);
-            if (kk < nrows && c_ok)
-              v[j] = ld_stream(p.P + (size_t)idx16[r0 + kk] * (size_t)row_bytes + (size_t)tile * 128 + (size_t)c * 16);
-          }
-          if (b == 0) PROX_TRACE(22);
-          uint4 brow = make_uint4(0u, 0u, 0u, 0u);
-          if (lane < nrows) {
-            const int i = idx16[r0 + lane];
-            const uint32_t dg = x_digits(xs[i], ebase);
-            const int slot = per_row ? 0 : ((i >> p.gshift) & 3);
-            brow.x = slot == 0 ? dg : 0u; brow.y = slot == 1 ? dg : 0u; brow.z = slot == 2 ? dg : 0u; brow.w = slot == 3 ? dg : 0u;
-          }
+        for (int nxt = warp, k = 0; warp < NL; nxt += NL, ++k) {
+          const int p_r0 = r0, p_nrows = nrows, p_sg = sg;
+          // the stage to fill was last read by the MMAs of block k - 2 (the low-nibble buffer likewise)
           const bool free_ok = uses == 0 || mbar_wait(my_empty, (uses - 1u) & 1u, abortp, spin);
           if (!__all_sync(0xffffffffu, free_ok)) { alive_b = false; break; }
+          if (nxt < nblk) {
+            if (nsuper > 1) {
+              sg = __popc(__ballot_sync(0xffffffffu, sg_end <= nxt));
+              const int first = __shfl_sync(0xffffffffu, sg_end - (int)sg_nb, sg);
+              r0 = __shfl_sync(0xffffffffu, sg_r0, sg) + ((nxt - first) << 5);
+              nrows = min(32, __shfl_sync(0xffffffffu, sg_r1, sg) - r0);
+            } else {
+              r0 = nxt << 5;
+              nrows = min(32, k1 - r0);
+            }
+            // rows beyond nrows and columns beyond the tile keep whatever is there: their digits are zero, their sums unused
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const int kk = j * 4 + kq;
-            const uint32_t dst = stg + (uint32_t)((kk >> 3) * 1024 + (kk & 7) * 128 + ((c ^ (kk & 7)) << 4));
-            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "r"(v[j].x), "r"(v[j].y), "r"(v[j].z), "r"(v[j].w) : "memory");
-            if (LO)
-              asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(dst + 4096u), "r"(v[j].x & 0x0f0f0f0fu), "r"(v[j].y & 0x0f0f0f0fu),
-                           "r"(v[j].z & 0x0f0f0f0fu), "r"(v[j].w & 0x0f0f0f0fu) : "memory");
+            for (int j = 0; j < 8; ++j) {
+              const int kk = j * rpi + kq;
+              if (lane_on && kk < nrows)
+                cp_async16(stg + (uint32_t)((k & 1) * 4096 + (kk >> 3) * 1024 + (kk & 7) * 128 + ((c ^ (kk & 7)) << 4)),
+                           tp + (size_t)idx16[r0 + kk] * (size_t)row_bytes);
+            }
           }
-          asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(stg + 8192u + (uint32_t)lane * 16u), "r"(brow.x), "r"(brow.y), "r"(brow.z), "r"(brow.w) : "memory");
-          fence_proxy_async();                 // the tensor core reads the stage through the async proxy
-          __syncwarp();
-          if (elect_one()) {
-            umma_i8(tbase + (uint32_t)(16 * sg), adesc, bdesc, idesc, 1u);
-            if (LO) umma_i8(tbase + 256u + (uint32_t)(16 * sg), ldesc, bdesc, idesc, 1u);
-            umma_commit(my_empty);
+          cp_async_commit();
+          if (tl == 0 && k == 0) PROX_TRACE(22);
+          if (k > 0) {
+            const uint32_t st1 = (uint32_t)((k - 1) & 1);
+            uint4 brow = make_uint4(0u, 0u, 0u, 0u);
+            if (lane < p_nrows) {
+              const int i = idx16[p_r0 + lane];
+              const uint32_t dg = x_digits(xs[i], ebase);
+              const int slot = per_row ? 0 : ((i >> p.gshift) & 3);
+              brow.x = slot == 0 ? dg : 0u; brow.y = slot == 1 ? dg : 0u; brow.z = slot == 2 ? dg : 0u; brow.w = slot == 3 ? dg : 0u;
+            }
+            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(dig + st1 * 512u + (uint32_t)lane * 16u), "r"(brow.x), "r"(brow.y), "r"(brow.z), "r"(brow.w) : "memory");
+            cp_async_wait<1>();
+            __syncwarp();
+            if (LO) {
+              uint4 v[8];
+#pragma unroll
+              for (int j = 0; j < 8; ++j) v[j] = lds128(stg + st1 * 4096u + (uint32_t)(j * 512 + lane * 16));
+#pragma unroll
+              for (int j = 0; j < 8; ++j)
+                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(stg + 8192u + (uint32_t)(j * 512 + lane * 16)), "r"(v[j].x & 0x0f0f0f0fu),
+                             "r"(v[j].y & 0x0f0f0f0fu), "r"(v[j].z & 0x0f0f0f0fu), "r"(v[j].w & 0x0f0f0f0fu) : "memory");
+            }
+            fence_proxy_async();                 // the tensor core reads the stage through the async proxy
+            __syncwarp();
+            if (elect_one()) {
+              umma_i8(tbase + (uint32_t)(16 * p_sg), adesc + (uint64_t)(st1 * 256u), bdesc + (uint64_t)(st1 * 32u), idesc, 1u);
+              if (LO) umma_i8(tbase + 256u + (uint32_t)(16 * p_sg), ldesc, bdesc + (uint64_t)(st1 * 32u), idesc, 1u);
+              umma_commit(my_empty);
+            }
+            __syncwarp();
+            if (uses == 0 && tl == 0) PROX_TRACE(23);
+            ++uses;
           }
-          __syncwarp();
-          ++uses;
-          if (b == 0) PROX_TRACE(23);
+          if (nxt >= nblk) break;
         }
-        if (elect_one()) umma_commit(smem_u32(&sm.acc_bar));   // one arrival per warp once its MMAs are complete
+        cp_async_wait<0>();
+        if (warp < NL && elect_one()) umma_commit(smem_u32(&sm.acc_bar));   // one arrival per loader warp once its MMAs are complete
         __syncwarp();
         PROX_TRACE(24);
         // ---- read the accumulators back: thread = byte column, warp part p takes supergroups p, p + 4, ...
@@ -648,16 +705,17 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
         };
         uint32_t scn[4];
         load_scales(part, scn);
-        const bool acc_ok = __all_sync(0xffffffffu, alive_b && mbar_wait(smem_u32(&sm.acc_bar), (unsigned)tile_iter & 1u, abortp, spin));
+        const bool acc_ok = __all_sync(0xffffffffu, alive_b && mbar_wait(smem_u32(&sm.acc_bar), acc_n & 1u, abortp, spin));
+        ++acc_n;
         tc_fence_after();
-        if (tile_iter == 0) {                  // the groups' offsets come from the four warps that do not load
+        if (tl == 0) {                         // the groups' offsets come from the four warps that do not load
 #pragma unroll 1
           for (unsigned it = 0; *reinterpret_cast<volatile unsigned*>(&sm.soff_cnt) < (unsigned)kFusedProducers && it < spin; ++it) __nanosleep(32);
           __threadfence_block();
         }
         PROX_TRACE(25);
         float t0 = 0.f, t1 = 0.f;              // 4-bit: sums of the low / high nibble's channel; 8-bit: t0 only
-        const bool more = tile + G < ntiles;
+        const bool more = tl + 1 < ntl;
 #pragma unroll 1
         for (int sgd = part; sgd < nsuper; sgd += 4) {
           if (!acc_ok) break;
@@ -725,17 +783,17 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       }
     }
     else {
-      // Blocks without a tile pull the kept rows into L2 (whole rows, one bulk prefetch each): the loader
+      // Blocks without a column pull the kept rows into L2 (whole rows, one bulk prefetch each): the loader
       // warps of the other blocks then find them there instead of waiting for HBM one by one.
-      if (cta >= ntiles && lane < 8) {
-        const int nidle = G - ntiles, slot_i = (cta - ntiles) * (kFusedProducers * 8) + (warp - kFusedConsumerWarps) * 8 + lane;
+      if (vid >= n1 && first && lane < 8) {
+        const int nidle = max(G - (int)n1, 1), slot_i = (int)(vid - n1) * (kFusedProducers * 8) + (warp - kFusedConsumerWarps) * 8 + lane;
 #pragma unroll 1
         for (int r = slot_i; r < k1; r += nidle * kFusedProducers * 8)
           asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.P + (size_t)idx16[r] * (size_t)row_bytes), "r"((uint32_t)row_bytes) : "memory");
       }
       // the other four warps: per scale group, offset * sum of the kept x as integers (for the codes' offset binary)
 #pragma unroll 1
-      for (int g = warp - kFusedConsumerWarps; g < ng; g += kFusedProducers) {
+      for (int g = warp - kFusedConsumerWarps; first && g < ng; g += kFusedProducers) {
         int d0 = 0, d1 = 0, d2 = 0, d3 = 0;
 #pragma unroll 1
         for (int r = sm.gstart[g] + lane; r < sm.gstart[g + 1]; r += 32) {
@@ -748,46 +806,78 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
         if (lane == 0) sm.soff[g] = (LO ? 8.f : 128.f) * digits_to_float((uint32_t)d0, (uint32_t)d1, (uint32_t)d2, (uint32_t)d3);
       }
       __syncwarp();
-      if (lane == 0) { __threadfence_block(); atomicAdd(&sm.soff_cnt, 1u); }
+      if (first && lane == 0) { __threadfence_block(); atomicAdd(&sm.soff_cnt, 1u); }
     }
-    // the tensor memory is not used after this phase
     tc_fence_before();
     __syncthreads();
-    if (cta < ntiles) {
+    if (ckn > 0) {
       // one atomic per occupied bin and block (thousands of single increments on a few hot bins serialise in L2)
 #pragma unroll 1
       for (int i = tid; i < 2048; i += NT) { const unsigned v = sm.hist[i]; if (v) atomicAdd(ghist + i, v); }
     }
-    if (warp == 0) tmem_free_all(tbase);
-  }
-
-  PROX_TRACE(3);
-  // -------------------------------------------------------------- grid barrier
-  // One counter that only grows: a block adds 1 and waits until the count
-  // reaches the next multiple of the grid size (no reset, no generation word).
-  fence_proxy_async();                        // phase B's plain accesses to the big buffer come before the ring's bulk copies
-  __syncthreads();
-  if (tid == 0) {
-    // release (cumulative): publishes the block's writes seen through the barrier above
-    unsigned long long old;
-    asm volatile("atom.acq_rel.gpu.global.add.u64 %0, [%1], 1;" : "=l"(old) : "l"(p.bar_count) : "memory");
-    // the count is reset by the host long before 2^32 calls; the low word is enough for the division
-    const unsigned long long target = old - (unsigned long long)((unsigned)old % (unsigned)G) + (unsigned long long)G +
-                                      (unsigned long long)p.bar_bias;
-    bool ok = (old + 1ull == target);
+    PROX_TRACE(3);
+    // ------------------------------------------------------------ grid barrier
+    // Wait until all shares of Stage 1 are finished (not all blocks).  Thread 0 says that this block's is, asks for
+    // another one (there is none unless a block of the grid is not running) and for a share of Stage 2, all in flight
+    // together and with the first look at the count.
+    fence_proxy_async();                        // phase B's plain accesses to the big buffer come before the ring's bulk copies
+    __syncthreads();
+    if (tid == 0) {
+      const unsigned target = n1 + p.bar_bias;
+      unsigned fin = 0, more1 = n1, share2 = 0;
+      bool ok = false, again = false;
+      // release (cumulative): publishes the block's writes seen through the barrier above
+      if (vid < n1) {
+        asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(fin) : "l"(ctr + kDone1) : "memory");
+        asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(more1) : "l"(ctr + kClaim1) : "memory");
+      }
+      if (first) asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(share2) : "l"(ctr + kClaim2) : "memory");
+      ok = vid < n1 && fin + 1u == target;
 #pragma unroll 1
-    for (unsigned it = 0; !ok && it < spin; ++it) {
-      unsigned long long cur;
-      asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(cur) : "l"(p.bar_count) : "memory");
-      ok = cur >= target;
-      if (!ok && it > 64) __nanosleep(32);
+      for (unsigned it = 0; !ok && it < spin; ++it) {
+        unsigned cur;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(cur) : "l"(ctr + kDone1) : "memory");
+        ok = cur >= target;
+        if (!ok && more1 < n1) { again = true; break; }
+        if (!ok && it > 64) __nanosleep(32);
+      }
+      if (first) sm.shr = share2;
+      sm.again = again; sm.vid = more1;
+      if (!ok && !again) { sm.abort_flag = 1; atomicOr(p.status, kWaitExpired); if (p.host_flag) *reinterpret_cast<volatile int*>(p.host_flag) = 1; }
+    } else if (warp > 0) {
+      // meanwhile: x as fp32 for phase D
+#pragma unroll 1
+      for (int i = tid - 32; i < D / 8; i += NT - 32) {
+        const uint4 v = reinterpret_cast<const uint4*>(xs)[i];
+        reinterpret_cast<float4*>(xf)[2 * i] = make_float4(bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y));
+        reinterpret_cast<float4*>(xf)[2 * i + 1] = make_float4(bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w));
+      }
     }
-    if (!ok) { sm.abort_flag = 1; atomicOr(p.status, kWaitExpired); if (p.host_flag) *reinterpret_cast<volatile int*>(p.host_flag) = 1; }
+    __syncthreads();
+    if (!sm.again || *abortp) break;
+    // one more share: the accumulators go back to zero
+    if (warp < 4) {
+      const uint32_t tz = tbase + ((uint32_t)(warp * 32) << 16);
+#pragma unroll 1
+      for (int c = 0; c < 16 * nsuper; c += 16) { tmem_st16_zero(tz + (uint32_t)c); tmem_st16_zero(tz + 256u + (uint32_t)c); }
+      tmem_st_wait();
+      tc_fence_before();
+    }
+    __syncthreads();
+    tc_fence_after();
   }
-  __syncthreads();
+  if (warp == 0) tmem_free_all(sm.tmem_base);
   const bool alive = sm.abort_flag == 0;      // block-uniform; a dead block skips to the end
   PROX_TRACE(4);
 
+  // Stage 2: this block's share of the kept channels (and further ones if a block of the grid is not running)
+  unsigned base_seq = 0;                        // ring rows consumed so far
+  unsigned pseq = 0, puse = 0;                  // producers: rows armed or passed over, uses of the ring, ...
+  int pslot = 0;                                // ... next slot
+#pragma unroll 1
+  for (;;) {
+  const unsigned shr = sm.shr, NSH = (unsigned)p.nshare;
+  if (shr >= NSH && alive) break;
   // ---------------------------------------- C: channel mask (top-k2 of the scores)
   // The first histogram level tells which channels are kept whatever the exact
   // threshold turns out to be (their bin lies above the threshold bin b1:
@@ -851,10 +941,10 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     if (staged) {
       // k2 * G < 2^31 is checked on the host, so the share bounds fit 32 bits
       // (THRESH: nd is only known after the counting pass; the bounds are set there)
-      int Rd0 = (int)((nd * (unsigned)cta) / (unsigned)G);
-      const int Rc0 = (int)((kk * (unsigned)cta) / (unsigned)G);
-      int ndm = min((int)((nd * (unsigned)(cta + 1)) / (unsigned)G) - Rd0, kMySelCap);
-      const int ncm = THRESH ? 0 : min((int)((kk * (unsigned)(cta + 1)) / (unsigned)G) - Rc0, kMySelCap - ndm);
+      int Rd0 = (int)((nd * shr) / NSH);
+      const int Rc0 = (int)((kk * shr) / NSH);
+      int ndm = min((int)((nd * (shr + 1u)) / NSH) - Rd0, kMySelCap);
+      const int ncm = THRESH ? 0 : min((int)((kk * (shr + 1u)) / NSH) - Rc0, kMySelCap - ndm);
       int Rd1 = Rd0 + ndm;
       const int Rc1 = Rc0 + ncm;
       n_mine = ndm + ncm;
@@ -893,11 +983,11 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       if (THRESH) {
         consumer_sync();                                   // the warps' totals: how many channels are kept
         nd = __reduce_add_sync(0xffffffffu, (lane < kFusedConsumerWarps) ? (sm.wsum[lane] & 0xffffu) : 0u);
-        Rd0 = (int)((nd * (unsigned)cta) / (unsigned)G);
-        ndm = min((int)((nd * (unsigned)(cta + 1)) / (unsigned)G) - Rd0, kMySelCap);
+        Rd0 = (int)((nd * shr) / NSH);
+        ndm = min((int)((nd * (shr + 1u)) / NSH) - Rd0, kMySelCap);
         Rd1 = Rd0 + ndm;
         n_mine = ndm;
-        if (cta == 0 && tid == 0) {
+        if (shr == 0 && tid == 0) {
           if (p.count_out) p.count_out[0] = (int)nd;
           if (p.counters) atomicAdd(p.counters + 2, (unsigned long long)nd);
         }
@@ -1098,7 +1188,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       // d_ff, or a huge threshold bin such as an all-zero input gives): the whole block
       // settles the threshold by two radix steps of 10 bits over all keys and keeps its
       // share of the plain ascending list before the ring starts.
-      const int R0 = (int)(((unsigned)k2 * (unsigned)cta) / (unsigned)G), R1 = (int)(((unsigned)k2 * (unsigned)(cta + 1)) / (unsigned)G);
+      const int R0 = (int)(((unsigned)k2 * shr) / NSH), R1 = (int)(((unsigned)k2 * (shr + 1u)) / NSH);
       n_mine = min(R1 - R0, kMySelCap);
       unsigned prefix = b1, kleft = kk;
 #pragma unroll 1
@@ -1194,9 +1284,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       fence_proxy_async();                      // the big buffer becomes a bulk-copy target now
       n_mine = go ? *reinterpret_cast<volatile int*>(&sm.n_mine) : 0;
       const unsigned pq = (unsigned)(warp - kFusedConsumerWarps);
-      unsigned seq = 0;
-      int slot = 0;
-      unsigned use = 0;
+      unsigned seq = pseq, use = puse;
+      int slot = pslot;
       bool dead = false;
       int ready = *reinterpret_cast<volatile int*>(&sm.nready);
       bool kdone = *reinterpret_cast<volatile int*>(&sm.keys_done) != 0;
@@ -1242,11 +1331,17 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
           if (++slot == NS) { slot = 0; ++use; }
         }
       }
+      pseq = seq; puse = use; pslot = slot;
+      if (pq == 0) {
+        // all rows of the share are on their way: the next share, if there is one
+        unsigned nx;
+        asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(nx) : "l"(ctr + kClaim2) : "memory");
+        sm.shr_next = nx;
+      }
     }
   } else {
     // ---- consumer warps
     const uint32_t xf_u32 = smem_u32(xf);
-    unsigned base_seq = 0;
     for (int b0 = 0; b0 < n_mine; b0 += kChanBatch) {
       const int nb = min(kChanBatch, n_mine - b0);
       // D: a warp takes the next channel of the batch that nobody has taken yet (the warps
@@ -1372,15 +1467,17 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       }
     }
     __syncthreads();
+    leave();
     return;
   }
-  if (NORM && p.xres_out == p.xres) return;     // y went straight into the residual stream: nothing to round, nothing to clean
+  const unsigned next_shr = sm.shr_next;
+  if (!(NORM && p.xres_out == p.xres)) {        // (in place y went straight into the residual stream: nothing to round)
   if (tid == 0) {
     // release: the block's atomics (ordered before this thread by the barrier above) are out before the ticket is
     // taken; acquire: the block that draws the last ticket sees every other block's
     unsigned t;
-    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(t) : "l"(p.done_ticket) : "memory");
-    sm.s_last = (t == (unsigned)(G - 1));
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(t) : "l"(ctr + kDone2) : "memory");
+    sm.s_last = (t == NSH - 1u);
   }
   __syncthreads();
   if (sm.s_last) {
@@ -1411,10 +1508,16 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
         }
       }
     }
-    if (tid == 0) *p.done_ticket = 0;
     __syncthreads();
     PROX_TRACE(9);
   }
+  }
+  if (next_shr >= NSH) break;
+  __syncthreads();                              // everyone has read what is reset here
+  if (tid == 0) { sm.shr = next_shr; sm.ncand = 0; sm.ncand2 = 0; sm.next_c = 0; sm.go = 0; sm.nready = 0; sm.n_mine = 0; sm.keys_done = 0; sm.c_done = 0; }
+  __syncthreads();
+  }
+  leave();
 }
 
 // The persistent kernel lists the kept channels as [definite][share of the

@@ -55,3 +55,52 @@ def test_packer_tiles_ties_and_repacking(pb, D, F, bits, group):
                 assert np.linalg.norm(y.cpu().numpy()[0] - y_ref) <= 1e-4 * np.linalg.norm(y_ref) + 1e-20
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("D,F,bits,group", [(512, 1536, 4, 128), (512, 1536, 8, 0), (1024, 4096, 4, 0), (256, 19136, 4, 128)])
+@pytest.mark.parametrize("grid", [1, 7, 100])
+def test_persistent_kernel_with_part_of_its_grid(pb, D, F, bits, group, grid):
+    """Blocks that do not run are replaced by those that do: the same masks and results with a part of the grid, in the
+    plain, the threshold and the layer form in place (19136 channels: shares in 32-byte sectors, two tiles of columns
+    each)."""
+    k1, k2 = D // 3, F // 4 + 1
+    wg, wu, wd, x = inputs.make_small(D, F, 1, seed=D + F + bits)
+    p = Problem(pb, wg, wu, wd, x)
+    try:
+        pb.prox_quantize_proxy(p.h, bits, group)
+        nw = torch.ones(D, dtype=torch.bfloat16, device="cuda")
+
+        def run():
+            y, yt = p.y_empty(), p.y_empty()
+            sel, idx = torch.empty(1, k2, dtype=torch.int32, device="cuda"), torch.empty(k1, dtype=torch.int32, device="cuda")
+            sc = torch.empty(F, dtype=torch.float32, device="cuda")
+            pb.prox_ffn_forward(p.h, p.t_x, 1, k1, k2, y)
+            pb.prox_ffn_last_mask(p.h, 1, k2, sel)
+            pb.prox_ffn_last_stage1(p.h, k1, idx, sc)
+            tau_x = float(p.t_x[0].float().abs().sort(descending=True).values[k1 - 1])
+            tau_s = float(sc.sort(descending=True).values[k2 - 1])
+            pb.prox_runtime_sparsity(p.h, reset=True)
+            pb.prox_ffn_forward_threshold(p.h, p.t_x, 1, tau_x, tau_s, yt)
+            kept = pb.prox_runtime_sparsity(p.h)
+            xr = p.t_x.float().contiguous()
+            pb.prox_ffn_block_forward(p.h, xr, nw, 1e-6, 1, k1, k2, xr)
+            torch.cuda.synchronize()
+            assert pb.prox_last_device_status(p.h) == 0
+            return [t.cpu().numpy() for t in (sel, idx, sc)], [t.cpu().numpy() for t in (y, yt, xr)], kept
+
+        whole, part = run(), None
+        pb.prox_debug_set_grid(p.h, grid)
+        for _ in range(3):                                         # both sets of counters
+            part = run()
+            for a, b in zip(whole[0], part[0]):
+                assert np.array_equal(a, b)
+            assert whole[2] == part[2]
+            # the same products, summed in fp32 in another order
+            for a, b in zip(whole[1], part[1]):
+                assert np.linalg.norm(a - b) <= 1e-5 * np.linalg.norm(a)
+        pb.prox_debug_set_grid(p.h, 0)
+        again = run()
+        for a, b in zip(whole[0], again[0]):
+            assert np.array_equal(a, b)
+    finally:
+        p.close()
