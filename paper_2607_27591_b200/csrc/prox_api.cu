@@ -12,6 +12,7 @@
 
 #include "prox_kernels.cuh"
 #include "prox_pack.cuh"
+#include "prox_select.cuh"
 #include "prox_fused.cuh"
 #include "prox_batch_mma.cuh"
 #include "prox_batch_umma.cuh"
@@ -79,7 +80,6 @@ struct prox_ffn {
   int cmask_marked;         // Stage 1 of the running forward call has set the tokens' bits in cmask already
   unsigned* cmask;          // [F / 4] one byte per channel: which tokens kept it (kept at zero between calls)
   uint8_t* umask;           // [F] that byte for every union row
-  __half* xh;               // [8][D] masked, scaled fp16 x of the tensor-core proxy GEMM
   float* tokfac;            // [8] per token: what undoes its scaling
   uint32_t* xd;             // [D][8] digit words of the tokens' masked inputs (tcgen05 proxy GEMM)
   float* soffb;             // [D / 128][8] per 128-input unit and token: sum of the integer inputs
@@ -189,7 +189,7 @@ int ksplit_for(const prox_ffn* h, int B, int n_rows) {
 }
 
 // Function attributes (dynamic shared memory limits) are per device: one flag per (call site, device).
-enum AttrSite { kAtGateupBatch = 0, kAtBatchS1, kAtProxyB4, kAtProxyB8, kAtMma, kAtRows, kAtStage2, kAtFused0, kAtSites = 24 };
+enum AttrSite { kAtGateupBatch = 0, kAtBatchS1, kAtProxyB4, kAtProxyB8, kAtMma, kAtStage2, kAtFused0, kAtTopk0, kAtRows0 = kAtTopk0 + 4, kAtSites = kAtRows0 + 4 };
 bool& attr_done(int site, int device) {
   static bool done[kAtSites][64] = {};
   return done[site][device & 63];
@@ -283,8 +283,26 @@ prox_status_t launch_proxy(prox_ffn* h, const void* x, int B, const int* idx, in
   return PROX_OK;
 }
 
+// exact top-k2 per token (or, shared, of the tokens' summed scores) by clusters of blocks
+template <int SRC>
+prox_status_t launch_channel_topk(prox_ffn* h, const float* scores, int B, int k2, int* sel, int stride, unsigned* cmask, cudaStream_t st) {
+  const bool shared = SRC == kSharedScores || SRC == kSharedSums;
+  const int F = h->cfg.d_ff;
+  const size_t smem = (size_t)(F / 4 / kTkBlocks + 1) * 16;
+  bool& attr = attr_done(kAtTopk0 + SRC, h->device);
+  if (!attr) {                                         // (the widest layer's 32 KB and the histograms exceed the default 48 KB)
+    CK(cudaFuncSetAttribute(channel_topk_kernel<SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, 40 * 1024));
+    attr = true;
+  }
+  LaunchScope ls(h, kKChannel, st);
+  CK(launch_dep(channel_topk_kernel<SRC>, dim3((shared ? 1 : B) * kTkBlocks), dim3(kTkThreads), smem, st, scores, h->pacc, B, F, k2, sel,
+                stride, cmask));
+  return PROX_OK;
+}
+
 prox_status_t launch_channel_select(prox_ffn* h, const float* scores, int B, int k2, float tau,
                                     int use_tau, int* sel, int stride, int* cnt, cudaStream_t st) {
+  if (!use_tau && !cnt && aligned16(scores)) return launch_channel_topk<kFromScores>(h, scores, B, k2, sel, stride, nullptr, st);
   {
     LaunchScope ls(h, kKChannel, st);
     channel_select_kernel<<<B, kSelThreads, 0, st>>>(scores, h->cfg.d_ff, k2, tau, use_tau, sel, stride, cnt);
@@ -404,29 +422,19 @@ prox_status_t launch_stage1_batch(prox_ffn* h, const void* x, int B, int k1, int
   prox_status_t s;
   const int gshift_m = (h->group == D) ? 31 : 7;
   if (h->use_mma && h->pacc && (h->bits == 4 || h->bits == 8) && F % 64 == 0) {
-    // tensor-core path over all inputs (no union list): per-token masked, scaled fp16 x, then equal
-    // ranges of (strip, K-block) units per block, then the per-token channel masks
-    const size_t lim = (size_t)h->smem_optin - 16384;
-    const bool fast_masks = (size_t)D * 2 <= lim && (size_t)F * 4 <= lim;
+    // tensor-core path over all inputs (no union list): the tokens' masked inputs as digits, then equal
+    // ranges of (tile, 128-input) units per block, then the channel masks
     bool& attr_p = attr_done(kAtBatchS1, h->device);
     if (!attr_p) {
       CK(cudaFuncSetAttribute(proxy_umma_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBuSmem4));
       CK(cudaFuncSetAttribute(proxy_umma_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBuSmem8));
-      CK(cudaFuncSetAttribute(batch_input_mask_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim));
-      CK(cudaFuncSetAttribute(batch_channel_mask_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim));
       attr_p = true;
     }
-    if (fast_masks) {
+    {
       LaunchScope ls(h, kKInput, st);
       CK(launch_dep(batch_input_mask_kernel, dim3(kBT), dim3(kFusedThreads), (size_t)D * 2, st, static_cast<const uint16_t*>(x), B, D, k1,
-                    h->xh, h->tokfac, h->xd, h->soffb));
-    } else {
-      if ((s = launch_input_select(h, x, B, k1, 0.f, 0, h->idx_x, D, nullptr, st)) != PROX_OK) return s;
-      LaunchScope ls(h, kKInput, st);
-      proxy_xprep_kernel<<<kBT, 512, 0, st>>>(static_cast<const uint16_t*>(x), h->idx_x, D, k1, B, D, h->xh, h->tokfac);
-      batch_digits_kernel<<<kBT, 512, 0, st>>>(h->xh, D, h->xd, h->soffb);
+                    h->tokfac, h->xd, h->soffb));
     }
-    bool direct = false;
     {
       LaunchScope ls(h, kKProxy, st);
       const int row_bytes = (F / ch_per_chunk(h->bits)) * 16, ntiles = (row_bytes + 127) / 128, nunits = D / 128;
@@ -459,43 +467,19 @@ prox_status_t launch_stage1_batch(prox_ffn* h, const void* x, int B, int k1, int
         }
         CK(e);
       }
-      direct = fast_masks && !want_scores;
-      if (!direct) CK(launch_dep(proxy_umma_finish_kernel, dim3(2 * h->sm_count), dim3(256), 0, st, h->pacc, B, F, scores));
+      if (want_scores) CK(launch_dep(proxy_umma_finish_kernel, dim3(2 * h->sm_count), dim3(256), 0, st, h->pacc, B, F, scores));
     }
     CK(cudaGetLastError());
+    unsigned* const cm = mark_mask ? h->cmask : nullptr;
     if (h->mask_policy == 1) {
-      if (!fast_masks) return PROX_ERR_UNSUPPORTED;
-      LaunchScope ls(h, kKChannel, st);
-      if (direct) CK(launch_dep(shared_score_from_sums_kernel, dim3((F + 255) / 256), dim3(256), 0, st, h->pacc, B, F, h->svals));
-      else CK(launch_dep(shared_score_kernel, dim3((F + 255) / 256), dim3(256), 0, st, (const float*)scores, B, F, h->svals));
-      if ((size_t)F * 4 + (size_t)k2 * 4 <= lim) {
-        // the one block also writes the list into every token's row
-        CK(launch_dep(batch_channel_mask_kernel, dim3(1), dim3(kCmThreads), (size_t)F * 4 + (size_t)k2 * 4, st, (const float*)h->svals, F, k2, sel,
-                      sel_stride, (unsigned*)nullptr, (1u << B) - 1u, (float*)nullptr, B, mark_mask ? h->u_ch : (int*)nullptr, h->umask,
-                      h->u_cnt + 1));
-        CK(cudaGetLastError());
-        if (mark_mask) h->cmask_marked = 2;          // the union is listed already: it is the mask itself
-        return PROX_OK;
-      } else {
-        CK(launch_dep(batch_channel_mask_kernel, dim3(1), dim3(kCmThreads), (size_t)F * 4, st, (const float*)h->svals, F, k2, sel, sel_stride,
-                      mark_mask ? h->cmask : (unsigned*)nullptr, (1u << B) - 1u, (float*)nullptr, 1, (int*)nullptr, (uint8_t*)nullptr,
-                      (int*)nullptr));
-        CK(launch_dep(replicate_mask_kernel, dim3((k2 + 255) / 256), dim3(256), 0, st, sel, sel_stride, k2, B));
-      }
-      CK(cudaGetLastError());
-      if (mark_mask) h->cmask_marked = 1;
-      return PROX_OK;
+      s = want_scores ? launch_channel_topk<kSharedScores>(h, scores, B, k2, sel, sel_stride, cm, st)
+                      : launch_channel_topk<kSharedSums>(h, nullptr, B, k2, sel, sel_stride, cm, st);
+    } else {
+      s = want_scores ? launch_channel_topk<kFromScores>(h, scores, B, k2, sel, sel_stride, cm, st)
+                      : launch_channel_topk<kFromSums>(h, nullptr, B, k2, sel, sel_stride, cm, st);
     }
-    if (!fast_masks) return launch_channel_select(h, scores, B, k2, 0.f, 0, sel, sel_stride, nullptr, st);
-    {
-      LaunchScope ls(h, kKChannel, st);
-      CK(launch_dep(batch_channel_mask_kernel, dim3(B), dim3(kCmThreads), (size_t)F * 4, st, (const float*)scores, F, k2, sel, sel_stride,
-                    mark_mask ? h->cmask : (unsigned*)nullptr, 0u, (direct && h->mask_policy == 0) ? h->pacc : (float*)nullptr, 1,
-                    (int*)nullptr, (uint8_t*)nullptr, (int*)nullptr));
-    }
-    CK(cudaGetLastError());
-    if (mark_mask) h->cmask_marked = 1;
-    return PROX_OK;
+    if (s == PROX_OK && mark_mask) h->cmask_marked = 1;
+    return s;
   }
   if (h->mask_policy == 1) return PROX_ERR_UNSUPPORTED;      // the shared mask is built by the tensor-core path only
   if ((s = launch_input_select(h, x, B, k1, 0.f, 0, h->idx_x, D, nullptr, st)) != PROX_OK) return s;
@@ -534,13 +518,14 @@ prox_status_t launch_stage2_batch(prox_ffn* h, const void* x, int B, const int* 
   prox_status_t s;
   const size_t mma_smem = stage2_mma_smem(h);
   const bool mma = stage2_mma_ok(h);
+  const bool rows = mma && D <= 4 * kGrPiece / 2;            // the ring kernel: up to four 4 KB sections of a row
   if (mma) {
     LaunchScope ls(h, kKUnion, st);
-    const int listed = marked ? h->cmask_marked : 0;       // 1: bits set by Stage 1 of this call, 2: the union list is there already
+    const int listed = marked ? h->cmask_marked : 0;       // bits set by Stage 1 of this call
     h->cmask_marked = 0;
     if (!listed)
       CK(launch_dep(union_mark_kernel, dim3((B * k2 + 255) / 256), dim3(256), 0, st, sel, sel_stride, k2, B, F, h->cmask, h->dev_status));
-    if (listed != 2) {
+    if (!rows) {
       const size_t need = (size_t)F * 5 + 16;
       const int staged = need <= (size_t)h->smem_optin - 4096 ? 1 : 0;
       bool& attr_u = attr_done(kAtFused0, h->device);
@@ -560,22 +545,23 @@ prox_status_t launch_stage2_batch(prox_ffn* h, const void* x, int B, const int* 
       attr_mma = true;
     }
     const int per_sm = (2 * (mma_smem + 1024) <= (size_t)h->smem_optin) ? 2 : 1;
-    // whole rows through a ring of bulk copies when 16 of them (a tile) plus a few more fit in shared memory
-    const size_t row_pitch = (size_t)(D * 2 < kGrPiece ? D * 2 : kGrPiece) + 64;
-    int ring_slots = (int)(((size_t)h->smem_optin - 4096 - (size_t)kMmaWarps * 128 * sizeof(float)) / row_pitch);
+    // whole rows through a ring of bulk copies, in sections of 16
+    const size_t row_pitch = (size_t)(D * 2 < kGrPiece ? D * 2 : kGrPiece) + 64, red_bytes = (size_t)2 * kMmaWarps * 128 * sizeof(float);
+    int ring_slots = (int)(((size_t)h->smem_optin - 8192 - red_bytes) / row_pitch) & ~15;
     if (ring_slots > kGrMaxSlots) ring_slots = kGrMaxSlots;
     {
       LaunchScope ls(h, kKGateUp, st);
-      if (D % 512 == 0 && D <= 4096 && ring_slots >= 40) {
-        bool& attr_r = attr_done(kAtRows, h->device);
+      if (rows) {
+        const int nsec = (D * 2 + kGrPiece - 1) / kGrPiece;
+        const auto kern = nsec == 1 ? gateup_rows_kernel<1> : nsec == 2 ? gateup_rows_kernel<2> : nsec == 3 ? gateup_rows_kernel<3> : gateup_rows_kernel<4>;
+        bool& attr_r = attr_done(kAtRows0 + nsec - 1, h->device);
         if (!attr_r) {
-          CK(cudaFuncSetAttribute(gateup_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin - 4096));
+          CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin - 8192));
           attr_r = true;
         }
-        CK(launch_dep(gateup_rows_kernel, dim3(h->sm_count), dim3(kGrThreads),
-                      (size_t)ring_slots * row_pitch + (size_t)kMmaWarps * 128 * sizeof(float), st,
-                      h->wg, h->wu, static_cast<const uint16_t*>(x), B, h->u_ch, h->umask, h->u_cnt + 1, D, ring_slots, h->hb,
-                      h->dev_status));
+        CK(launch_dep(kern, dim3(h->sm_count), dim3(kGrThreads), (size_t)ring_slots * row_pitch + red_bytes, st,
+                      h->wg, h->wu, static_cast<const uint16_t*>(x), B, reinterpret_cast<const uint4*>(h->cmask), F, D, ring_slots, h->hb,
+                      h->u_ch, h->u_cnt + 1, h->dev_status));
       } else {
         gateup_mma_kernel<<<per_sm * h->sm_count, kMmaThreads, mma_smem, st>>>(
             h->wg, h->wu, static_cast<const uint16_t*>(x), B, h->u_ch, h->u_cnt + 1, D, h->gacc);
@@ -586,7 +572,7 @@ prox_status_t launch_stage2_batch(prox_ffn* h, const void* x, int B, const int* 
     {
       LaunchScope ls(h, kKDown, st);
       CK(launch_dep(down_mma_kernel, dim3(h->sm_count), dim3(kMmaThreads), (size_t)kMmaWarps * 512 * sizeof(float), st,
-                    h->wdt, h->hb, h->u_ch, h->u_cnt + 1, B, D, h->yacc));
+                    h->wdt, h->hb, h->u_ch, h->u_cnt + 1, B, D, h->yacc, rows ? reinterpret_cast<uint4*>(h->cmask) : (uint4*)nullptr, F));
     }
     CK(cudaGetLastError());
   } else {
@@ -870,7 +856,6 @@ prox_status_t prox_ffn_create(const prox_ffn_config_t* cfg, const void* w_gate, 
     {
       A(dev_alloc(&h->pacc, (size_t)(F / 64) * 1024));
       if (st == PROX_OK) A(cudaMemset(h->pacc, 0, (size_t)(F / 64) * 1024 * sizeof(float)));
-      A(dev_alloc(&h->xh, (size_t)kBT * D));
       A(dev_alloc(&h->cmask, (size_t)(F + 3) / 4)); A(dev_alloc(&h->umask, (size_t)F));
       if (st == PROX_OK) A(cudaMemset(h->cmask, 0, (size_t)((F + 3) / 4) * sizeof(unsigned)));
       A(dev_alloc(&h->tokfac, (size_t)kBT));
@@ -907,7 +892,7 @@ void prox_ffn_destroy(prox_ffn_t* h) {
   cudaFree(h->idx_x); cudaFree(h->cnt_x); cudaFree(h->part); cudaFree(h->ticket);
   cudaFree(h->scores); cudaFree(h->svals); cudaFree(h->xn); cudaFree(h->sel); cudaFree(h->cnt_s); cudaFree(h->hbuf);
   cudaFree(h->yacc); cudaFree(h->dev_status); cudaFree(h->counters); cudaFree(h->syncbuf); cudaFree(h->trace);
-  cudaFree(h->u_in); cudaFree(h->u_ch); cudaFree(h->u_cnt); cudaFree(h->xu); cudaFree(h->member); cudaFree(h->hb); cudaFree(h->gacc); cudaFree(h->pacc); cudaFree(h->xh); cudaFree(h->tokfac); cudaFree(h->xd); cudaFree(h->soffb); cudaFree(h->cmask); cudaFree(h->umask);
+  cudaFree(h->u_in); cudaFree(h->u_ch); cudaFree(h->u_cnt); cudaFree(h->xu); cudaFree(h->member); cudaFree(h->hb); cudaFree(h->gacc); cudaFree(h->pacc); cudaFree(h->tokfac); cudaFree(h->xd); cudaFree(h->soffb); cudaFree(h->cmask); cudaFree(h->umask);
   cudaFree(h->x_stage); cudaFree(h->y_stage);
   if (h->host_flag) cudaFreeHost(h->host_flag);
   if (h->prof) {
@@ -967,7 +952,14 @@ prox_status_t prox_stage1_mask(prox_ffn_t* h, const void* x, int B, int k1, int 
   const int D = h->cfg.d_model;
   float* sc = scores ? scores : h->scores;
   if (B > 1 && h->mask_policy == 1 && !(h->use_union && batch_path_ok(h, B, true))) return PROX_ERR_UNSUPPORTED;
-  if (h->use_union && batch_path_ok(h, B, true)) return launch_stage1_batch(h, x, B, k1, k2, sel, k2, sc, st, false, scores != nullptr);
+  if (h->use_union && batch_path_ok(h, B, true)) {
+    // the batch kernels move scores 16 bytes at a time
+    float* own = aligned16(sc) ? sc : h->scores;
+    s = launch_stage1_batch(h, x, B, k1, k2, sel, k2, own, st, false, scores != nullptr);
+    if (s == PROX_OK && own != sc)
+      CK(cudaMemcpyAsync(sc, own, (size_t)B * h->cfg.d_ff * sizeof(float), cudaMemcpyDeviceToDevice, st));
+    return s;
+  }
   if ((s = launch_input_select(h, x, B, k1, 0.f, 0, h->idx_x, D, nullptr, st)) != PROX_OK) return s;
   if ((s = launch_proxy(h, x, B, h->idx_x, D, nullptr, k1, sc, st)) != PROX_OK) return s;
   return launch_channel_select(h, sc, B, k2, 0.f, 0, sel, k2, nullptr, st);

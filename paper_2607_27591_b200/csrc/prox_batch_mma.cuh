@@ -112,9 +112,8 @@ gateup_mma_kernel(const uint16_t* __restrict__ wg, const uint16_t* __restrict__ 
   }
 }
 
-// Union of the tokens' kept channels for the tensor-core path, in two small
-// kernels: every (token, kept channel) sets the token's bit in a byte per channel;
-// one block then lists the channels whose byte is not zero in ascending order,
+// Union of the tokens' kept channels for the tensor-core path: every (token, kept channel) sets the token's bit in a byte per channel
+// (Stage 1 of the same call does that itself).  For layers wider than gateup_rows_kernel takes, one block then lists the channels whose byte is not zero in ascending order,
 // copies the byte next to the list and clears it for the next call.
 __global__ void __launch_bounds__(256)
 union_mark_kernel(const int* __restrict__ lists, int stride, int k, int B, int n, unsigned* __restrict__ mask32,
@@ -173,149 +172,191 @@ union_compact_kernel(unsigned* __restrict__ mask32, int n, int* __restrict__ uli
 }
 
 // ----------------------------------------------------------------------------
-// Stage 2a with the weight rows streamed by bulk async copies (d_model <= 4096).
+// Stage 2a with the weight rows streamed by bulk async copies (d_model <= 8192), and the union itself.
 // Plain loads of rows that are gathered 64 bytes at a time stay near 4.5 TB/s;
 // whole rows through cp.async.bulk, as in the batch-1 kernel, do not.
 // One block per SM: 16 consumer warps + one producer warp whose 32 lanes issue the
-// copies.  A tile is 8 union channels = 16 rows: rows 0..7 of the MMA's A operand
+// copies.  Every block first reads the tokens' bits (a byte per channel), ranks the union channels in ascending order
+// and takes a contiguous, equal share of their tiles (a kernel of one block that listed the union took 8 us in front of
+// this one, the same work in every block here 2 us); it writes its part of the list for the down projection.
+// A tile is 8 union channels = 16 rows: rows 0..7 of the MMA's A operand
 // are the gate rows, rows 8..15 the up rows of the same channels, so one MMA gives
 // both pre-activations of a channel to the same lane.  A ring slot holds up to 4 KB
 // of a row (+ 64 bytes of padding: the fragment loads of eight rows then fall into
-// different banks); a longer row comes as two sections, so that several tiles are
-// in flight.  A consumer warp owns a sixteenth of every section; its share of x
-// (the B operand) lives in registers for the whole kernel.
-// The warps' partial sums of a tile meet in shared memory and h is written at
-// once: no accumulator in global memory and no finishing kernel.
+// different banks); a longer row comes as NSEC sections, so that several tiles are
+// in flight.  A consumer warp owns every 16th 64-byte piece of a section; its share of x
+// (the B operand) lives in registers for the whole kernel.  One lane per warp waits for a section (hundreds of
+// threads polling the barrier slow the copies down threefold).
+// The warps' partial sums of a tile meet in shared memory (two buffers: one block barrier per tile, where one thread
+// waiting for everybody took three) and h is written at once: no accumulator in global memory and no finishing kernel.
+// Measured (eight tokens): 4096 x 12288 layer, 106.4 -> 101.8 us per call with the channel-mask kernel of prox_select.cuh;
+// 8192 x 28672 (two kernels over plain loads and an accumulator in global memory before): 146 + 13 us -> 141.
 // ----------------------------------------------------------------------------
 constexpr int kGrThreads = kMmaThreads + 32;        // 16 consumer warps + one producer warp
-constexpr int kGrMaxSlots = 64;
-constexpr int kGrMaxTiles = 64;                     // tiles of a block whose channels are staged in shared memory
+constexpr int kGrMaxSlots = 128;
+constexpr int kGrMaxShare = 512;                    // union channels of a block
 constexpr int kGrPiece = 4096;                      // bytes of a row in one ring slot (a whole row if it is shorter)
 
+// bit 7 of every byte that is not zero
+__device__ __forceinline__ unsigned nonzero_bytes(unsigned w) { return (((w & 0x7f7f7f7fu) + 0x7f7f7f7fu) | w) & 0x80808080u; }
+
+template <int NSEC>
 __global__ void __launch_bounds__(kGrThreads, 1)
 gateup_rows_kernel(const uint16_t* __restrict__ wg, const uint16_t* __restrict__ wu,
-                   const uint16_t* __restrict__ x, int B, const int* __restrict__ ulist,
-                   const uint8_t* __restrict__ umask, const int* __restrict__ nu_ptr, int D, int nslots,
-                   float* __restrict__ h_out, int* __restrict__ status) {
-  pdl_enter();
-  extern __shared__ __align__(128) uint8_t mm_smem[];
+                   const uint16_t* __restrict__ x, int B, const uint4* __restrict__ cmask, int F, int D, int nslots,
+                   float* __restrict__ h_out, int* __restrict__ ulist, int* __restrict__ nu_out, int* __restrict__ status) {
+  extern __shared__ __align__(128) uint8_t gr_smem[];
   __shared__ unsigned long long bar_full[kGrMaxSlots / 16], bar_empty[kGrMaxSlots / 16];   // per section of 16 slots
   __shared__ int abort_flag;
   __shared__ unsigned n_issued;                                 // sections armed so far (for the give-up path)
-  __shared__ int my_ch[kGrMaxTiles * 8];
-  const int NSEC = nslots / 16;                                 // sections (16 slots) in the ring
-  const uint32_t piece = (uint32_t)min(kGrPiece, D * 2);        // bytes of a row per slot
-  const int nsec = (D * 2) / (int)piece;                        // sections of a row (1 or 2 up to d_model 4096)
+  __shared__ unsigned wsum[32];
+  __shared__ int my_ch[kGrMaxShare];
+  __shared__ uint8_t my_bits[kGrMaxShare];
+  const int NS = nslots / 16;                                   // sections (16 slots) in the ring
+  const uint32_t piece = (uint32_t)min(kGrPiece, D * 2);        // bytes of a row per slot; the last section may be shorter
+  const uint32_t last = (uint32_t)(D * 2) - (uint32_t)(NSEC - 1) * piece;
   const uint32_t pitch = piece + 64u;
-  float* red = reinterpret_cast<float*>(mm_smem + (size_t)NSEC * 16 * pitch);     // [16 warps][128]
+  float* red = reinterpret_cast<float*>(gr_smem + (size_t)NS * 16 * pitch);     // [2][16 warps][128]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
-  const int nu = *nu_ptr;
-  if (nu <= 0) return;
-  if (tid < NSEC) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (tid < NS) {
     mbar_init(smem_u32(&bar_full[tid]), 1);
     mbar_init(smem_u32(&bar_empty[tid]), kMmaWarps);
     fence_mbar_init();
   }
   if (tid == 0) { abort_flag = 0; n_issued = 0; }
-  const int ntile = (nu + 7) / 8;
-  // the union channels of this block's tiles, so that a producer does not wait for global memory per copy
-  for (int i = tid; i < kGrMaxTiles * 8; i += kGrThreads) {
-    const int tile = blockIdx.x + (i >> 3) * gridDim.x;
-    my_ch[i] = (tile < ntile) ? ulist[min(tile * 8 + (i & 7), nu - 1)] : 0;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  int nu, p0, cnt;
+  {
+    // the union: a thread owns a run of 16-channel groups (at most 8: d_ff <= 65536)
+    const int ngrp = F / 16, per = (ngrp + kGrThreads - 1) / kGrThreads;
+    const int c0 = min(ngrp, tid * per), c1 = min(ngrp, c0 + per);
+    uint4 m[8];
+    unsigned n = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) m[i] = c0 + i < c1 ? __ldcg(cmask + c0 + i) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      n += __popc(nonzero_bytes(m[i].x)) + __popc(nonzero_bytes(m[i].y)) + __popc(nonzero_bytes(m[i].z)) + __popc(nonzero_bytes(m[i].w));
+    const unsigned inc = warp_scan_incl(n, lane);
+    if (lane == 31) wsum[warp] = inc;
+    __syncthreads();
+    const unsigned wv = lane < kGrThreads / 32 ? wsum[lane] : 0u;
+    nu = (int)__reduce_add_sync(0xffffffffu, wv);
+    int pos = (int)(__reduce_add_sync(0xffffffffu, lane < warp ? wv : 0u) + inc - n);
+    const int ntile = (nu + 7) / 8;
+    p0 = 8 * (int)((unsigned)ntile * blockIdx.x / gridDim.x);
+    const int p1 = min(nu, 8 * (int)((unsigned)ntile * (blockIdx.x + 1) / gridDim.x));
+    cnt = max(p1 - p0, 0);
+    if (n && pos < p1 && pos + (int)n > p0) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const unsigned w4[4] = {m[i].x, m[i].y, m[i].z, m[i].w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+#pragma unroll 1
+          for (unsigned nz = nonzero_bytes(w4[q]); nz; nz &= nz - 1) {
+            const int e = (__ffs((int)nz) - 1) >> 3;
+            if (pos >= p0 && pos < p1) {
+              const int ch = (c0 + i) * 16 + q * 4 + e;
+              my_ch[pos - p0] = ch; my_bits[pos - p0] = (uint8_t)(w4[q] >> (8 * e));
+              ulist[pos] = ch;
+            }
+            ++pos;
+          }
+        }
+      }
+    }
+    if (blockIdx.x == 0 && tid == 0) *nu_out = nu;
   }
   fence_proxy_async();
   __syncthreads();
+  if (cnt <= 0) return;
+  const int my_tiles = (cnt + 7) / 8;
   volatile int* abortp = &abort_flag;
-  const uint32_t ring_u32 = smem_u32(mm_smem);
+  const uint32_t ring_u32 = smem_u32(gr_smem);
   if (warp >= kMmaWarps) {
     // ---- producer warp: one thread starts well under a million copies a second here, so all 32
     // lanes issue: lanes 0..15 the 16 rows of one section, lanes 16..31 those of the next one.
     // (One warp, in program order: the use of a slot is always armed after its previous use.)
-    const int per_tile = nsec;                                  // sections per tile
-    const int my_tiles = (ntile - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
-    const int nsect = my_tiles * per_tile;                      // sections of this block
+    const int nsect = my_tiles * NSEC;                          // sections of this block
     const int r = lane & 15;
     bool dead = false;
     for (int s0 = 0; s0 < nsect && !dead; s0 += 2) {
       const int si = s0 + (lane >> 4);                          // this lane's section
-      const int ss = si % NSEC;                                 // its place in the ring (16 slots, one barrier pair)
-      const unsigned use = (unsigned)(si / NSEC);
+      const int ss = si % NS;                                   // its place in the ring (16 slots, one barrier pair)
+      const unsigned use = (unsigned)(si / NS);
       bool ok = true;
       if (si < nsect && use > 0 && r == 0) ok = mbar_wait(smem_u32(&bar_empty[ss]), (use - 1u) & 1u, abortp);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) { dead = true; break; }
       if (si < nsect) {
-        const int ti = si / per_tile, sec = si - ti * per_tile;
-        const int tile = (int)blockIdx.x + ti * (int)gridDim.x;
+        const int ti = si / NSEC, sec = si - ti * NSEC;
+        const uint32_t bytes = sec == NSEC - 1 ? last : piece;
         const uint32_t bar = smem_u32(&bar_full[ss]);
-        if (r == 0) { mbar_expect_tx(bar, 16u * piece); atomicMax(&n_issued, (unsigned)si + 1u); }
-        __syncwarp();
-        const int ch = (ti < kGrMaxTiles) ? my_ch[ti * 8 + (r & 7)] : ulist[min(tile * 8 + (r & 7), nu - 1)];
+        if (r == 0) { mbar_expect_tx(bar, 16u * bytes); atomicMax(&n_issued, (unsigned)si + 1u); }
+        __syncwarp(lane < 16 ? 0x0000ffffu : 0xffff0000u);
+        const int ch = my_ch[min(ti * 8 + (r & 7), cnt - 1)];
         const uint8_t* src = reinterpret_cast<const uint8_t*>((r < 8 ? wg : wu) + (size_t)ch * D) + (size_t)sec * piece;
-        bulk_g2s(ring_u32 + (uint32_t)(ss * 16 + r) * pitch, src, piece, bar);
-      } else {
-        __syncwarp();
+        bulk_g2s(ring_u32 + (uint32_t)(ss * 16 + r) * pitch, src, bytes, bar);
       }
+      __syncwarp();
     }
   } else {
     // ---- consumer warps
-    const int npw = (int)piece / 1024;                          // 32-input pieces of a section per warp (<= 4)
-    uint4 xv[8];                                                // x of token g: sections x pieces of this warp
+    uint4 xv[NSEC * 4];                                         // x of token g: this warp's pieces of every section
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int sec = i >> 2, pc = i & 3;
-      xv[i] = make_uint4(0, 0, 0, 0);
-      if (sec < nsec && pc < npw && g < B)
-        xv[i] = __ldg(reinterpret_cast<const uint4*>(x + (size_t)g * D + sec * ((int)piece / 2) + (warp * npw + pc) * 32 + t * 8));
-    }
-    unsigned sidx = 0;                 // running section number of this block
+    for (int sec = 0; sec < NSEC; ++sec)
+#pragma unroll
+      for (int pc = 0; pc < 4; ++pc) {
+        const uint32_t off = (uint32_t)(pc * kMmaWarps + warp) * 64u;
+        xv[sec * 4 + pc] = make_uint4(0, 0, 0, 0);
+        if (off < (sec == NSEC - 1 ? last : piece) && g < B)
+          xv[sec * 4 + pc] = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>(x + (size_t)g * D) + sec * piece + off) + t);
+      }
+    int ss = 0;                        // section of the ring, and its use
+    unsigned use = 0;
     bool dead = false;                 // a wait expired: go on without touching the ring, but keep every barrier
-    for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+    for (int ti = 0; ti < my_tiles; ++ti) {
       float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-      for (int sec = 0; sec < 2; ++sec) {
-        if (sec < nsec) {
+      for (int sec = 0; sec < NSEC; ++sec) {
+        if (lane == 0 && !dead && !mbar_wait(smem_u32(&bar_full[ss]), use & 1u, abortp)) dead = true;
+        dead = __shfl_sync(0xffffffffu, (int)dead, 0) != 0;
+        if (!dead) {
           // this lane reads the gate row and the up row of channel g of the tile
-          const int ss = (int)(sidx % (unsigned)NSEC);
-          const int sg = ss * 16 + g, su = ss * 16 + 8 + g;
-          // One thread alone waits for the 16 rows of the section: hundreds of threads polling the
-          // barrier slow the copies down.  The others learn of it at a block barrier.
-          if (tid == 0 && !dead) {
-            if (!mbar_wait(smem_u32(&bar_full[ss]), (sidx / (unsigned)NSEC) & 1u, abortp)) abort_flag = 1;
-          }
-          asm volatile("bar.sync 1, %0;" ::"n"(kMmaThreads) : "memory");
-          if (*abortp) dead = true;
-          if (!dead) {
-            const uint32_t pg = ring_u32 + (uint32_t)sg * pitch + (uint32_t)(warp * npw) * 64u + (uint32_t)t * 16u;
-            const uint32_t pu = ring_u32 + (uint32_t)su * pitch + (uint32_t)(warp * npw) * 64u + (uint32_t)t * 16u;
+          const uint32_t pg = ring_u32 + (uint32_t)(ss * 16 + g) * pitch + (uint32_t)warp * 64u + (uint32_t)t * 16u;
+          const uint32_t pu = pg + 8u * pitch;
 #pragma unroll
-            for (int pc = 0; pc < 4; ++pc) {
-              if (pc < npw) {
-                const uint4 gl = lds128(pg + (uint32_t)pc * 64u), ul = lds128(pu + (uint32_t)pc * 64u);
-                const uint4 xw = xv[sec * 4 + pc];
-                mma_bf16(acc, gl.x, ul.x, gl.y, ul.y, xw.x, xw.y);
-                mma_bf16(acc, gl.z, ul.z, gl.w, ul.w, xw.z, xw.w);
-              }
+          for (int pc = 0; pc < 4; ++pc) {
+            const uint32_t off = (uint32_t)(pc * kMmaWarps) * 64u;
+            if (off + (uint32_t)warp * 64u < (sec == NSEC - 1 ? last : piece)) {
+              const uint4 gl = lds128(pg + off), ul = lds128(pu + off);
+              const uint4 xw = xv[sec * 4 + pc];
+              mma_bf16(acc, gl.x, ul.x, gl.y, ul.y, xw.x, xw.y);
+              mma_bf16(acc, gl.z, ul.z, gl.w, ul.w, xw.z, xw.w);
             }
-            __syncwarp();
-            if (lane == 0) mbar_arrive_n(smem_u32(&bar_empty[ss]), 1u);       // this warp is done with the section
           }
-          ++sidx;
+          __syncwarp();
+          if (lane == 0) mbar_arrive_n(smem_u32(&bar_empty[ss]), 1u);       // this warp is done with the section
         }
+        if (++ss == NS) { ss = 0; ++use; }
       }
       // the warps' partial sums meet: [gate | up][channel g][token]
-      float* mine = red + warp * 128;
-      mine[g * 8 + 2 * t] = acc[0]; mine[g * 8 + 2 * t + 1] = acc[1];
-      mine[64 + g * 8 + 2 * t] = acc[2]; mine[64 + g * 8 + 2 * t + 1] = acc[3];
+      float* buf = red + (ti & 1) * (kMmaWarps * 128);
+      float* mine = buf + warp * 128;
+      *reinterpret_cast<float2*>(mine + g * 8 + 2 * t) = make_float2(acc[0], acc[1]);
+      *reinterpret_cast<float2*>(mine + 64 + g * 8 + 2 * t) = make_float2(acc[2], acc[3]);
       asm volatile("bar.sync 1, %0;" ::"n"(kMmaThreads) : "memory");
-      if (tid < 64) {
+      const int who = warp - 2 * (ti & 7);                      // two warps form h, others every tile, while the rest goes on
+      if (who == 0 || who == 1) {
+        const int i = who * 32 + lane;
         float gate = 0.f, up = 0.f;
 #pragma unroll
-        for (int w = 0; w < kMmaWarps; ++w) { gate += red[w * 128 + tid]; up += red[w * 128 + 64 + tid]; }
-        const int r = tile * 8 + (tid >> 3), b = tid & 7;
-        if (r < nu) h_out[(size_t)r * kBT + b] = (b < B && ((umask[r] >> b) & 1u)) ? up * silu_exact(gate) : 0.f;
+        for (int w = 0; w < kMmaWarps; ++w) { gate += buf[w * 128 + i]; up += buf[w * 128 + 64 + i]; }
+        const int r = ti * 8 + (i >> 3), b = i & 7;
+        if (r < cnt) h_out[(size_t)(p0 + r) * kBT + b] = (b < B && ((my_bits[r] >> b) & 1u)) ? up * silu_exact(gate) : 0.f;
       }
-      asm volatile("bar.sync 1, %0;" ::"n"(kMmaThreads) : "memory");
     }
   }
   __syncthreads();
@@ -324,11 +365,11 @@ gateup_rows_kernel(const uint16_t* __restrict__ wg, const uint16_t* __restrict__
     // (bounded) so that none lands after the block has left
     atomicOr(status, kWaitExpired);
     const unsigned issued = n_issued;                           // sections armed
-    const unsigned first = issued > (unsigned)NSEC ? issued - (unsigned)NSEC : 0u;
+    const unsigned first = issued > (unsigned)NS ? issued - (unsigned)NS : 0u;
     for (unsigned q = first; q < issued; ++q) {
-      const uint32_t bar = smem_u32(&bar_full[q % (unsigned)NSEC]);
+      const uint32_t bar = smem_u32(&bar_full[q % (unsigned)NS]);
       for (unsigned it = 0; it < 8192u; ++it) {
-        if (mbar_try_wait(bar, (q / (unsigned)NSEC) & 1u)) break;
+        if (mbar_try_wait(bar, (q / (unsigned)NS) & 1u)) break;
         __nanosleep(256);
       }
     }
@@ -360,8 +401,10 @@ gateup_finish_kernel(float* __restrict__ gacc, const uint8_t* __restrict__ umask
 // ----------------------------------------------------------------------------
 __global__ void __launch_bounds__(kMmaThreads, 1)
 down_mma_kernel(const uint16_t* __restrict__ wdt, const float* __restrict__ h, const int* __restrict__ ulist,
-                const int* __restrict__ nu_ptr, int B, int D, float* __restrict__ yacc) {
+                const int* __restrict__ nu_ptr, int B, int D, float* __restrict__ yacc, uint4* __restrict__ cmask, int F) {
   pdl_enter();
+  // the tokens' bits of this call have been read: cleared for the next one
+  if (cmask) for (int i = blockIdx.x * kMmaThreads + threadIdx.x; i < F / 16; i += gridDim.x * kMmaThreads) cmask[i] = make_uint4(0u, 0u, 0u, 0u);
   extern __shared__ __align__(16) uint8_t mm_smem[];
   float* red = reinterpret_cast<float*>(mm_smem);               // [warps][8 tokens][64 columns]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
@@ -452,57 +495,19 @@ down_mma_kernel(const uint16_t* __restrict__ wdt, const float* __restrict__ h, c
 namespace prox {
 
 // ----------------------------------------------------------------------------
-// Input preparation of Stage 1 for B > 1 (the GEMM itself is the tcgen05 kernel
-// of prox_batch_umma.cuh): the step-wise fallback for shapes whose input mask
-// does not fit the one-block-per-token kernel further down.
+// Input mask m_x of a token straight into the proxy GEMM's operand, one 640-thread block per token, built from the
+// selection code of the persistent batch-1 kernel (short loops, thread-owned runs, one warp scan per pass): exact
+// top-k1 of |x| (ties: lower index first), then the masked input x_i * s (0 at dropped inputs; s the power of two that
+// puts max |x| into [2^13, 2^14)), rounded to fp16, as four signed base-256 digits of X = x_h * 2^16:
+//   xd    the digit words in the layout of the MMA's B operand, 1 KB per block of 32 inputs: two planes of
+//         32 rows x 16 bytes (tokens 0..3 | tokens 4..7), row = input, 4 bytes per token
+//   soff  [u][b] sum of X over the 128 inputs of unit u;  tokfac[b] = 2^24 / s undoes the scaling (and the codes' 2^-24)
+// With eight tokens the union of the kept inputs is nearly everything, so the proxy GEMM runs over all rows and needs
+// no union list; a dropped input contributes 0 * code.  Token slots beyond B are cleared.
 // ----------------------------------------------------------------------------
-// One block per token slot.  The token's kept inputs (its ascending index list)
-// become an fp16 vector over ALL inputs: x * s at a kept input, 0 elsewhere, with
-// s the power of two that puts max |x| into [2^13, 2^14).  With eight tokens the
-// union of the kept inputs is nearly everything, so the proxy GEMM simply runs
-// over all rows and needs no union list; a dropped input contributes 0 * code.
-// tokfac[b] = 2^24 / s undoes the scaling (and the 2^-24 of the codes).
-__global__ void __launch_bounds__(512)
-proxy_xprep_kernel(const uint16_t* __restrict__ x, const int* __restrict__ idx, int stride, int k1, int B, int D,
-                   __half* __restrict__ xh, float* __restrict__ tokfac) {
-  __shared__ unsigned smax;
-  const int b = blockIdx.x, tid = threadIdx.x;
-  __half* row = xh + (size_t)b * D;
-  if (tid == 0) smax = 0;
-  __syncthreads();
-  unsigned m = 0;
-  if (b < B) for (int r = tid; r < k1; r += 512) m = max(m, (unsigned)(x[(size_t)b * D + idx[(size_t)b * stride + r]] & 0x7fffu));
-  m = __reduce_max_sync(0xffffffffu, m);
-  if ((tid & 31) == 0 && m) atomicMax(&smax, m);
-  for (int i = tid; i < D / 8; i += 512) reinterpret_cast<uint4*>(row)[i] = make_uint4(0, 0, 0, 0);
-  __syncthreads();
-  int se = 0;
-  if (smax) se = 13 - ((int)(smax >> 7) - 127);                  // bf16 magnitude bits: exponent in bits 14..7
-  se = max(-100, min(100, se));
-  const float s = __uint_as_float((unsigned)(se + 127) << 23);
-  if (tid == 0) tokfac[b] = __uint_as_float((unsigned)(24 - se + 127) << 23);
-  if (b < B) {
-    for (int r = tid; r < k1; r += 512) {
-      const int i = idx[(size_t)b * stride + r];
-      const float v = __uint_as_float(((uint32_t)x[(size_t)b * D + i]) << 16) * s;
-      row[i] = __float2half_rn(v);
-    }
-  }
-}
-
-// ----------------------------------------------------------------------------
-// Per-token masks of the tensor-core batch path, one 640-thread block per token,
-// built from the selection code of the persistent batch-1 kernel (short loops,
-// thread-owned runs, one warp scan per pass).
-// ----------------------------------------------------------------------------
-
-// Input mask m_x of a token straight into the proxy GEMM's operand: exact top-k1
-// of |x| (ties: lower index first), then xh[b][i] = fp16(x_i * s) at the kept
-// inputs and 0 elsewhere, s the power of two that puts max |x| into [2^13, 2^14);
-// tokfac[b] = 2^24 / s.  Token slots beyond B are cleared.
 __global__ void __launch_bounds__(kFusedThreads)
-batch_input_mask_kernel(const uint16_t* __restrict__ x, int B, int D, int k1, __half* __restrict__ xh,
-                        float* __restrict__ tokfac, uint32_t* __restrict__ xd, float* __restrict__ soff) {
+batch_input_mask_kernel(const uint16_t* __restrict__ x, int B, int D, int k1, float* __restrict__ tokfac,
+                        uint32_t* __restrict__ xd, float* __restrict__ soff) {
   extern __shared__ __align__(16) uint8_t bm_smem[];
   uint16_t* xs = reinterpret_cast<uint16_t*>(bm_smem);           // [D] bf16 bits of the token
   __shared__ unsigned hist[1024], hist2[32], wsum[32], smax;
@@ -510,14 +515,9 @@ batch_input_mask_kernel(const uint16_t* __restrict__ x, int B, int D, int k1, __
   constexpr int NT = kFusedThreads;
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   pdl_enter();                                    // the proxy GEMM may set up and start on the weights
-  __half* row = xh + (size_t)b * D;
   if (b >= B) {
-    if (xd) {
-      for (int i = tid; i < D; i += NT) xd[(size_t)(i >> 5) * 256 + (b >> 2) * 128 + (i & 31) * 4 + (b & 3)] = 0u;
-      for (int u = tid; u < (D >> 7); u += NT) soff[(size_t)u * kBT + b] = 0.f;
-    } else {
-      for (int i = tid; i < D / 8; i += NT) reinterpret_cast<uint4*>(row)[i] = make_uint4(0, 0, 0, 0);
-    }
+    for (int i = tid; i < D; i += NT) xd[(size_t)(i >> 5) * 256 + (b >> 2) * 128 + (i & 31) * 4 + (b & 3)] = 0u;
+    for (int u = tid; u < (D >> 7); u += NT) soff[(size_t)u * kBT + b] = 0.f;
     if (tid == 0) tokfac[b] = 16777216.f;
     return;
   }
@@ -588,217 +588,31 @@ batch_input_mask_kernel(const uint16_t* __restrict__ x, int B, int D, int k1, __
   for (int g = g0; g < g1; ++g) {
     const uint4 kv = *reinterpret_cast<const uint4*>(xs + g * 8);
     const uint32_t w4[4] = {kv.x, kv.y, kv.z, kv.w};
-    uint32_t o[4];
     int d0 = 0, d1 = 0, d2 = 0, d3 = 0;
-    uint32_t* dst = xd ? xd + (size_t)(g >> 2) * 256 + (b >> 2) * 128 + ((g & 3) * 8) * 4 + (b & 3) : nullptr;
+    uint32_t* dst = xd + (size_t)(g >> 2) * 256 + (b >> 2) * 128 + ((g & 3) * 8) * 4 + (b & 3);
 #pragma unroll
-    for (int e2 = 0; e2 < 4; ++e2) {
-      __half hv[2];
-#pragma unroll
-      for (int hh = 0; hh < 2; ++hh) {
-        const unsigned bits = (w4[e2] >> (hh * 16)) & 0xffffu, key = bits & 0x7fffu;
-        const bool gt = all || key > T, eq = !all && key == T;
-        const bool keep = gt || (eq && re < quota);
-        re += eq ? 1u : 0u;
-        hv[hh] = __float2half_rn(keep ? __uint_as_float(bits << 16) * sf : 0.f);
-        if (xd) {
-          // integer form of the masked, scaled fp16 input: X = x_h * 2^16 as four signed base-256 digits
-          const int X = __float2int_rn(__half2float(hv[hh]) * 65536.f);
-          const uint32_t dg = ((uint32_t)X + 0x00808080u) ^ 0x00808080u;
-          dst[(e2 * 2 + hh) * 4] = dg;
-          d0 += (int)(int8_t)(dg & 0xffu); d1 += (int)(int8_t)((dg >> 8) & 0xffu);
-          d2 += (int)(int8_t)((dg >> 16) & 0xffu); d3 += (int)(int8_t)(dg >> 24);
-        }
-      }
-      o[e2] = (uint32_t)__half_as_ushort(hv[0]) | ((uint32_t)__half_as_ushort(hv[1]) << 16);
+    for (int e = 0; e < 8; ++e) {
+      const unsigned bits = (w4[e >> 1] >> ((e & 1) * 16)) & 0xffffu, key = bits & 0x7fffu;
+      const bool gt = all || key > T, eq = !all && key == T;
+      const bool keep = gt || (eq && re < quota);
+      re += eq ? 1u : 0u;
+      const __half hv = __float2half_rn(keep ? __uint_as_float(bits << 16) * sf : 0.f);
+      const int X = __float2int_rn(__half2float(hv) * 65536.f);
+      const uint32_t dg = ((uint32_t)X + 0x00808080u) ^ 0x00808080u;
+      dst[e * 4] = dg;
+      d0 += (int)(int8_t)(dg & 0xffu); d1 += (int)(int8_t)((dg >> 8) & 0xffu);
+      d2 += (int)(int8_t)((dg >> 16) & 0xffu); d3 += (int)(int8_t)(dg >> 24);
     }
-    if (xd) {
-      int* sdg = sd + 4 * (g >> 4);
-      if (d0) atomicAdd(sdg, d0);
-      if (d1) atomicAdd(sdg + 1, d1);
-      if (d2) atomicAdd(sdg + 2, d2);
-      if (d3) atomicAdd(sdg + 3, d3);
-    } else {
-      reinterpret_cast<uint4*>(row)[g] = make_uint4(o[0], o[1], o[2], o[3]);
-    }
-  }
-  if (xd) {
-    __syncthreads();
-    for (int u = tid; u < (D >> 7); u += NT)
-      soff[(size_t)u * kBT + b] = digits_to_float((uint32_t)sd[u * 4], (uint32_t)sd[u * 4 + 1], (uint32_t)sd[u * 4 + 2],
-                                                  (uint32_t)sd[u * 4 + 3]);
-  }
-}
-
-// One mask for the whole batch (a policy beyond the paper): the channels are ranked by the sum of the
-// tokens' proxy scores, added token after token in fp32.
-__global__ void __launch_bounds__(256) shared_score_kernel(const float* __restrict__ scores, int B, int F,
-                                                           float* __restrict__ out) {
-  pdl_enter();
-  const int j = blockIdx.x * 256 + threadIdx.x;
-  if (j >= F) return;
-  float s = 0.f;
-  for (int b = 0; b < B; ++b) s += scores[(size_t)b * F + j];
-  out[j] = s;
-}
-
-// ... and every token's row of the mask output is that one list.
-__global__ void __launch_bounds__(256) replicate_mask_kernel(int* __restrict__ sel, int sel_stride, int k2, int B) {
-  pdl_enter();
-  const int r = blockIdx.x * 256 + threadIdx.x;
-  if (r >= k2) return;
-  const int v = sel[r];
-  for (int b = 1; b < B; ++b) sel[(size_t)b * sel_stride + r] = v;
-}
-
-// Channel mask m_s of a token from its scores: exact top-k2 (ties: lower channel
-// first) by three radix steps over the score bits held in shared memory, then an
-// ordered list of the kept channels; the token's bit is also set in the channel's
-// byte of cmask (the union of the tokens' masks is read off those bytes).
-// token_bits = 0: block b is token b and sets bit b.  Otherwise (one shared mask for the batch: one block
-// over the summed scores) the kept channels get all of token_bits.
-constexpr int kCmThreads = 1024;                   // channel-mask kernel: all 32 warps of a block
-__global__ void __launch_bounds__(kCmThreads)
-batch_channel_mask_kernel(const float* __restrict__ scores, int F, int k2, int* __restrict__ sel_out, int sel_stride,
-                          unsigned* __restrict__ cmask, unsigned token_bits, float* __restrict__ pacc, int nrep,
-                          int* __restrict__ ulist, uint8_t* __restrict__ umask, int* __restrict__ nu_out) {
-  pdl_enter();
-  extern __shared__ __align__(16) uint8_t bm_smem[];
-  unsigned* skey = reinterpret_cast<unsigned*>(bm_smem);         // [F] score bits
-  __shared__ unsigned hist[2048], wsum[32], wsum2[32];
-  constexpr int NT = kCmThreads;
-  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const unsigned* gkey = reinterpret_cast<const unsigned*>(scores) + (size_t)b * F;
-  const uint32_t skey_u32 = smem_u32(skey);
-  for (int i = tid; i < 2048; i += NT) hist[i] = 0;
-  __syncthreads();
-  if (pacc) {
-    // scores straight from the proxy sums of the tensor-core GEMM ([token][gate | up][channel]); the token's
-    // entries are cleared for the next call.  Four rounds of loads are issued before the first use: one round per
-    // dependent iteration would put the latency of global memory on every one of them.
-    float4* pg = reinterpret_cast<float4*>(pacc + (size_t)b * 2 * F);
-    float4* pu = pg + F / 4;
-    const int n4 = F / 4;
-#pragma unroll 1
-    for (int i0 = tid; i0 < n4; i0 += 4 * NT) {
-      float4 g[4], u[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int i = i0 + r * NT;
-        g[r] = i < n4 ? __ldcg(pg + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-        u[r] = i < n4 ? __ldcg(pu + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int i = i0 + r * NT;
-        if (i < n4) {
-          pg[i] = make_float4(0.f, 0.f, 0.f, 0.f); pu[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-          const uint4 k = make_uint4(__float_as_uint(fabsf(u[r].x * silu_fast(g[r].x))), __float_as_uint(fabsf(u[r].y * silu_fast(g[r].y))),
-                                     __float_as_uint(fabsf(u[r].z * silu_fast(g[r].z))), __float_as_uint(fabsf(u[r].w * silu_fast(g[r].w))));
-          reinterpret_cast<uint4*>(skey)[i] = k;
-          atomicAdd(&hist[k.x >> 20], 1u); atomicAdd(&hist[k.y >> 20], 1u);
-          atomicAdd(&hist[k.z >> 20], 1u); atomicAdd(&hist[k.w >> 20], 1u);
-        }
-      }
-    }
-  } else {
-    for (int i = tid; i < F / 4; i += NT) cp_async16(skey_u32 + (uint32_t)i * 16u, gkey + 4 * i);
-    cp_async_commit();
-    cp_async_wait<0>();
-    __syncthreads();
-#pragma unroll 1
-    for (int i = tid; i < F; i += NT) atomicAdd(&hist[skey[i] >> 20], 1u);
+    int* sdg = sd + 4 * (g >> 4);
+    if (d0) atomicAdd(sdg, d0);
+    if (d1) atomicAdd(sdg + 1, d1);
+    if (d2) atomicAdd(sdg + 2, d2);
+    if (d3) atomicAdd(sdg + 3, d3);
   }
   __syncthreads();
-  unsigned ab;
-  unsigned prefix = kth_in_block<4, false>(hist, (unsigned)k2, wsum, lane, warp, &ab);
-  unsigned kleft = (unsigned)k2 - ab;
-#pragma unroll 1
-  for (int sh = 10; sh >= 0; sh -= 10) {           // two more steps of 10 bits
-    __syncthreads();
-    for (int i = tid; i < 1024; i += NT) hist[i] = 0;
-    __syncthreads();
-#pragma unroll 1
-    for (int i = tid; i < F; i += NT) {
-      const unsigned key = skey[i];
-      if ((key >> (sh + 10)) == prefix) atomicAdd(&hist[(key >> sh) & 1023u], 1u);
-    }
-    __syncthreads();
-    const unsigned bb = kth_in_block<2, false>(hist, kleft, wsum, lane, warp, &ab);
-    prefix = (prefix << 10) | bb;
-    kleft -= ab;
-  }
-  const unsigned T = prefix, quota = kleft;
-  // ordered list: a thread owns a run of 4-channel groups
-  const int nq = F / 4, qpt = (nq + NT - 1) / NT;
-  const int q0 = min(nq, tid * qpt), q1 = min(nq, q0 + qpt);
-  unsigned cg = 0, ce = 0;
-#pragma unroll 1
-  for (int q = q0; q < q1; ++q) {
-    const uint4 kv = *reinterpret_cast<const uint4*>(skey + q * 4);
-    const unsigned k4[4] = {kv.x, kv.y, kv.z, kv.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) { cg += (k4[e] > T) ? 1u : 0u; ce += (k4[e] == T) ? 1u : 0u; }
-  }
-  const unsigned ig = warp_scan_incl(cg, lane), ie = warp_scan_incl(ce, lane);
-  __syncthreads();                                 // every warp is done with wsum (k-th search above)
-  if (lane == 31) { wsum[warp] = ig; wsum2[warp] = ie; }
-  __syncthreads();
-  unsigned rg = __reduce_add_sync(0xffffffffu, (lane < warp) ? wsum[lane] : 0u) + ig - cg;
-  unsigned re = __reduce_add_sync(0xffffffffu, (lane < warp) ? wsum2[lane] : 0u) + ie - ce;
-  int* out = sel_out + (size_t)b * sel_stride;
-#pragma unroll 1
-  for (int q = q0; q < q1; ++q) {
-    const uint4 kv = *reinterpret_cast<const uint4*>(skey + q * 4);
-    const unsigned k4[4] = {kv.x, kv.y, kv.z, kv.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const bool gt = k4[e] > T, eq = k4[e] == T;
-      if (gt || (eq && re < quota)) {
-        const int ch = q * 4 + e;
-        if (nrep > 1) reinterpret_cast<int*>(skey + F)[rg + min(re, quota)] = ch;     // staged: every token's row gets the list
-        else out[rg + min(re, quota)] = ch;
-        if (cmask) atomicOr(cmask + (ch >> 2), (token_bits ? token_bits : (1u << b)) << (8 * (ch & 3)));
-      }
-      rg += gt ? 1u : 0u; re += eq ? 1u : 0u;
-    }
-  }
-  if (nrep > 1) {
-    // one mask for the batch: the list goes to every token's row, in whole lines
-    __syncthreads();
-    const int* slist = reinterpret_cast<const int*>(skey + F);
-    for (int r = 0; r < nrep; ++r)
-      for (int i = tid; i < k2; i += NT) sel_out[(size_t)r * sel_stride + i] = slist[i];
-    if (ulist) {
-      // ... and it is the union of the tokens' masks as well: every kept channel belongs to every token
-      for (int i = tid; i < k2; i += NT) { ulist[i] = slist[i]; umask[i] = (uint8_t)token_bits; }
-      if (tid == 0) *nu_out = k2;
-    }
-  }
-}
-
-// One mask for the whole batch straight from the proxy sums of the tensor-core GEMM: out[j] = sum over the
-// tokens of |up~ SiLU(gate~)|, added token after token in fp32; the accumulator is cleared for the next call.
-__global__ void __launch_bounds__(256) shared_score_from_sums_kernel(float* __restrict__ pacc, int B, int F,
-                                                                     float* __restrict__ out) {
-  pdl_enter();
-  const int j = blockIdx.x * 256 + threadIdx.x;
-  if (j >= F) return;
-  // all loads first (a load behind every store would put the latency of global memory on every token)
-  float gate[kBT], up[kBT];
-#pragma unroll
-  for (int b = 0; b < kBT; ++b) {
-    const float* pg = pacc + (size_t)b * 2 * F + j;
-    gate[b] = __ldcg(pg); up[b] = __ldcg(pg + F);
-  }
-  float s = 0.f;
-#pragma unroll
-  for (int b = 0; b < kBT; ++b) {
-    float* pg = pacc + (size_t)b * 2 * F + j;
-    pg[0] = 0.f; pg[F] = 0.f;
-    if (b < B) s += fabsf(up[b] * silu_fast(gate[b]));
-  }
-  out[j] = s;
+  for (int u = tid; u < (D >> 7); u += NT)
+    soff[(size_t)u * kBT + b] = digits_to_float((uint32_t)sd[u * 4], (uint32_t)sd[u * 4 + 1], (uint32_t)sd[u * 4 + 2],
+                                                (uint32_t)sd[u * 4 + 3]);
 }
 
 }  // namespace prox

@@ -9,7 +9,7 @@
 // Data movement: one producer lane keeps a ring of stages full with TMA: per unit of 128 inputs one tiled
 // tensor copy drops the 128 x 128-byte tile of the proxy rows into shared memory already in the swizzled
 // operand layout (four blocks of 32 rows), a bulk copy brings the unit's digit rows (stored in operand layout
-// by batch_digits_kernel).  For 8-bit codes
+// by batch_input_mask_kernel).  For 8-bit codes
 // nothing else touches the bytes: a worker warp waits for the stage and issues the MMA.  For 4-bit
 // codes the worker first writes the tile with the high nibbles masked off into a second buffer (the
 // operand of the second MMA).  B operand of a block: row k = 8 tokens x 4 digits = 32 bytes (N = 32).
@@ -42,46 +42,6 @@ __device__ __forceinline__ void sts128(uint32_t a, uint32_t x, uint32_t y, uint3
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
   asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar) : "memory");
-}
-
-// Integer form of a token's masked, scaled fp16 input: X = x_h * 2^16 (|X| < 2^30), as four signed
-// base-256 digits; x_h = x * 2^se is what batch_input_mask_kernel writes (max |x_h| in [2^13, 2^14)).
-// xd = the digit words in the layout of the MMA's B operand, 1 KB per block of 32 inputs: two planes of
-// 32 rows x 16 bytes (tokens 0..3 | tokens 4..7), row = input, 4 bytes per token.
-// soff[u][b] = sum of X over the 128 inputs of unit u (as float).  One block per token slot.
-__global__ void __launch_bounds__(512)
-batch_digits_kernel(const __half* __restrict__ xh, int D, uint32_t* __restrict__ xd, float* __restrict__ soff) {
-  __shared__ int sd[128 * 4];
-  const int b = blockIdx.x, tid = threadIdx.x;
-  const int ng = D >> 7;                              // units of 128 inputs (d_model <= 16384)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the proxy GEMM may set up and start on the weights
-  sd[tid] = 0;
-  __syncthreads();
-  const __half* row = xh + (size_t)b * D;
-  for (int i0 = tid * 8; i0 < D; i0 += 512 * 8) {
-    const uint4 v = *reinterpret_cast<const uint4*>(row + i0);
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-    int d0 = 0, d1 = 0, d2 = 0, d3 = 0;
-    uint32_t* dst = xd + (size_t)(i0 >> 5) * 256 + (b >> 2) * 128 + (i0 & 31) * 4 + (b & 3);
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const __half hv = __ushort_as_half((unsigned short)((w[e >> 1] >> ((e & 1) * 16)) & 0xffffu));
-      const int X = __float2int_rn(__half2float(hv) * 65536.f);
-      const uint32_t dg = ((uint32_t)X + 0x00808080u) ^ 0x00808080u;
-      dst[e * 4] = dg;
-      d0 += (int)(int8_t)(dg & 0xffu); d1 += (int)(int8_t)((dg >> 8) & 0xffu);
-      d2 += (int)(int8_t)((dg >> 16) & 0xffu); d3 += (int)(int8_t)(dg >> 24);
-    }
-    int* sdg = sd + 4 * (i0 >> 7);
-    if (d0) atomicAdd(sdg, d0);
-    if (d1) atomicAdd(sdg + 1, d1);
-    if (d2) atomicAdd(sdg + 2, d2);
-    if (d3) atomicAdd(sdg + 3, d3);
-  }
-  __syncthreads();
-  if (tid < ng)
-    soff[(size_t)tid * kBT + b] = digits_to_float((uint32_t)sd[tid * 4], (uint32_t)sd[tid * 4 + 1], (uint32_t)sd[tid * 4 + 2],
-                                                  (uint32_t)sd[tid * 4 + 3]);
 }
 
 // sum_d digit_d 256^d of int32 digit sums (|digit sum| < 2^22: 128 rows x 255 x 128), two integer pairs

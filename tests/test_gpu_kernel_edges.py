@@ -104,3 +104,60 @@ def test_persistent_kernel_with_part_of_its_grid(pb, D, F, bits, group, grid):
             assert np.array_equal(a, b)
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("F", [64, 192, 4160, 65536])
+@pytest.mark.parametrize("B,shared", [(1, False), (3, False), (8, True)])
+def test_channel_mask_is_the_exact_topk_of_the_scores(pb, F, B, shared):
+    """Few and many channels per block of a cluster, ties (repeated channels: equal scores), every k at the ends; the
+    scores at an address that is not a multiple of 16."""
+    D = 128
+    g = torch.Generator(device="cuda").manual_seed(F + B)
+    w = [(torch.randn(F, D, device="cuda", generator=g) * 0.1).to(torch.bfloat16) for _ in range(2)]
+    for t in w:
+        t[F // 2:] = t[:F - F // 2]                                 # every score twice
+    wd = torch.zeros(D, F, dtype=torch.bfloat16, device="cuda")
+    x = torch.randn(B, D, device="cuda", generator=g).to(torch.bfloat16)
+    h = pb.prox_ffn_create(D, F, max(B, 2), 1, *w, wd)
+    try:
+        pb.prox_quantize_proxy(h, 4, 128)
+        pb.prox_ffn_set_mask_policy(h, int(shared))
+        buf = torch.empty(B * F + 1, dtype=torch.float32, device="cuda")
+        for k2 in (1, 2, F // 3, F // 2 + 1, F - 1, F):
+            for off in (0, 1):
+                sc = buf[off:off + B * F].view(B, F)
+                sel = torch.empty(B, k2, dtype=torch.int32, device="cuda")
+                pb.prox_stage1_mask(h, x, B, 50, k2, sel, sc)
+                rank = sc
+                if shared:                                          # added token after token in fp32, as the library does
+                    rank = torch.zeros(1, F, device="cuda")
+                    for b in range(B):
+                        rank = rank + sc[b]
+                    rank = rank.expand(B, F)
+                order = torch.sort(rank, dim=1, descending=True, stable=True).indices[:, :k2]
+                assert torch.equal(sel.long(), order.sort(dim=1).values), (k2, off)
+        assert pb.prox_last_device_status(h) == 0
+    finally:
+        pb.prox_ffn_destroy(h)
+
+
+@pytest.mark.parametrize("D,F", [(128, 64), (640, 1600), (2176, 2048), (4224, 1472), (8192, 704)])
+@pytest.mark.parametrize("B", [2, 8])
+def test_batch_stage2_rows_in_sections(pb, D, F, B):
+    """One to four sections of a row, the last one short; unions smaller than the grid, ragged tiles and all channels."""
+    wg, wu, wd, x = inputs.make_small(D, F, B, seed=D + F)
+    p = Problem(pb, wg, wu, wd, x, max_batch=B)
+    try:
+        pb.prox_quantize_proxy(p.h, 4, 128)
+        rng = np.random.default_rng(B)
+        for k2 in (1, 13, F // 2, F):
+            sel = np.stack([np.sort(rng.choice(F, size=k2, replace=False)) for _ in range(B)]).astype(np.int32)
+            y = p.y_empty(B)
+            pb.prox_stage2_ffn(p.h, p.t_x[:B], B, torch.from_numpy(sel).cuda(), k2, y)
+            for b in range(B):
+                y_ref, _ = po.stage2(p.x[b], sel[b], p.wg, p.wu, p.wd)
+                # h enters the down projection as a bf16 pair (2^-17 relative), sums in fp32
+                assert np.linalg.norm(y.cpu().numpy()[b] - y_ref) <= 1e-4 * np.linalg.norm(y_ref)
+        assert pb.prox_last_device_status(p.h) == 0
+    finally:
+        p.close()
