@@ -541,7 +541,7 @@ prox_status_t launch_stage2_batch(prox_ffn* h, const void* x, int B, const int* 
     bool& attr_mma = attr_done(kAtMma, h->device);
     if (!attr_mma) {
       CK(cudaFuncSetAttribute(gateup_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin - 4096));
-      CK(cudaFuncSetAttribute(down_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin - 4096));
+      CK(cudaFuncSetAttribute(down_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDnSmem));
       attr_mma = true;
     }
     const int per_sm = (2 * (mma_smem + 1024) <= (size_t)h->smem_optin) ? 2 : 1;
@@ -571,7 +571,7 @@ prox_status_t launch_stage2_batch(prox_ffn* h, const void* x, int B, const int* 
     CK(cudaGetLastError());
     {
       LaunchScope ls(h, kKDown, st);
-      CK(launch_dep(down_mma_kernel, dim3(h->sm_count), dim3(kMmaThreads), (size_t)kMmaWarps * 512 * sizeof(float), st,
+      CK(launch_dep(down_mma_kernel, dim3(h->sm_count), dim3(kMmaThreads), (size_t)kDnSmem, st,
                     h->wdt, h->hb, h->u_ch, h->u_cnt + 1, B, D, h->yacc, rows ? reinterpret_cast<uint4*>(h->cmask) : (uint4*)nullptr, F));
     }
     CK(cudaGetLastError());

@@ -392,102 +392,144 @@ gateup_finish_kernel(float* __restrict__ gacc, const uint8_t* __restrict__ umask
 
 // ----------------------------------------------------------------------------
 // Stage 2b: y[b] += sum over union rows of h[r][b] * W_downT[j_r, :].
-// Unit = (64 output columns, 16 union rows).  A = h (M = token, rows 8..15 are
-// zero), B = W_downT rows (K = union row, N = output column).  A K-pair of B
-// comes from two different rows of W_downT: one byte permute per register.
-// h is fed as a bf16 pair hi + lo (two MMAs), which keeps ~16 bits of it.
-// A lane loads columns 8g..8g+7, so MMA number i of a unit covers the columns
-// {8c + i}: accumulator (i, c0) is column 8 * 2t + i, (i, c1) column 8 * (2t+1) + i.
+// Unit = (64 output columns, 32 union rows); a block takes an equal, contiguous range of units, its warps every 16th of
+// them.  A = h (M: rows 0..7 the high, rows 8..15 the low part of h of the tokens, a bf16 pair that keeps ~16 bits of
+// it), B = W_downT rows (K = union row, N = output column).  Bound by the weight stream: a warp owns three stages of
+// 32 rows x 128 bytes, filled by 16-byte asynchronous copies two units ahead (128 KB in flight per SM; with two units of
+// plain loads in registers, 64 KB, a 4096 x 12288 layer with
+// eight tokens took 28 us, now 20: 5.2 TB/s after the start-up; per call 102 -> 94, 8192 x 28672 333 -> 308), read by transposing ldmatrix (16-byte chunks xor-ed with the row: no
+// bank conflicts).
 // ----------------------------------------------------------------------------
+constexpr int kDnStages = 3, kDnStage = 4096;
+constexpr int kDnSmem = kMmaWarps * kDnStages * kDnStage + kMmaWarps * 512 * (int)sizeof(float);
+
+__device__ __forceinline__ void ldsm_x4_trans(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+
 __global__ void __launch_bounds__(kMmaThreads, 1)
 down_mma_kernel(const uint16_t* __restrict__ wdt, const float* __restrict__ h, const int* __restrict__ ulist,
                 const int* __restrict__ nu_ptr, int B, int D, float* __restrict__ yacc, uint4* __restrict__ cmask, int F) {
   pdl_enter();
   // the tokens' bits of this call have been read: cleared for the next one
   if (cmask) for (int i = blockIdx.x * kMmaThreads + threadIdx.x; i < F / 16; i += gridDim.x * kMmaThreads) cmask[i] = make_uint4(0u, 0u, 0u, 0u);
-  extern __shared__ __align__(16) uint8_t mm_smem[];
-  float* red = reinterpret_cast<float*>(mm_smem);               // [warps][8 tokens][64 columns]
+  extern __shared__ __align__(128) uint8_t dn_smem[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+  float* red = reinterpret_cast<float*>(dn_smem + kMmaWarps * kDnStages * kDnStage);          // [warps][8 tokens][64 columns]
+  const uint32_t ring = smem_u32(dn_smem) + (uint32_t)(warp * kDnStages * kDnStage);
   const int nu = *nu_ptr;
   if (nu <= 0) return;
-  const int nkb = (nu + 15) / 16, ncol = D / 64;
+  const int nkb = (nu + 31) / 32, ncol = D / 64;
   const long long total = (long long)ncol * nkb;
-  long long u = total * blockIdx.x / gridDim.x;
-  const long long u1 = total * (blockIdx.x + 1) / gridDim.x;
-  while (u < u1) {
-    const int ct = (int)(u / nkb), a = (int)(u - (long long)ct * nkb);
-    const int b = (int)min((long long)nkb, a + (u1 - u));
+  const long long u0 = total * blockIdx.x / gridDim.x, u1 = total * (blockIdx.x + 1) / gridDim.x;
+  if (u0 >= u1) return;
+  const int ct0 = (int)(u0 / nkb), kb0 = (int)(u0 - (long long)ct0 * nkb);
+  const int ct1 = (int)((u1 - 1) / nkb), kbe = (int)(u1 - (long long)ct1 * nkb);              // last column tile, its end
+  // the warp's units in order: (column tile, 32-row block)
+  auto first_of = [&](int ct) -> int { return (ct == ct0 ? kb0 : 0) + warp; };
+  auto end_of = [&](int ct) -> int { return ct == ct1 ? kbe : nkb; };
+  auto settle = [&](int& ct, int& kb) {                         // past a tile's end: on to the next one
+    while (ct <= ct1 && kb >= end_of(ct)) { ++ct; kb = ct <= ct1 ? first_of(ct) : 0; }
+  };
+  auto row_id = [&](int ct, int kb) -> int { return ct <= ct1 ? __ldg(ulist + min(kb * 32 + lane, nu - 1)) : 0; };
+  auto copy_unit = [&](int ct, int stage, int j) {
+    if (ct <= ct1) {
+      const uint32_t dst = ring + (uint32_t)(stage * kDnStage);
+      const uint16_t* src = wdt + (size_t)ct * 64 + (lane & 7) * 8;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int row = i * 4 + (lane >> 3);
+        const int jr = __shfl_sync(0xffffffffu, j, row);
+        cp_async16(dst + (uint32_t)(row * 128 + (((lane & 7) ^ (row & 7)) << 4)), src + (size_t)jr * D);
+      }
+    }
+    cp_async_commit();
+  };
+  auto load_h = [&](int ct, int kb, float (&hv)[8]) {           // k = 16 q + {2t, 2t+1, 2t+8, 2t+9} of token g
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int r = kb * 32 + (q >> 2) * 16 + 2 * t + (q & 1) + ((q >> 1) & 1) * 8;
+      hv[q] = (ct <= ct1 && r < nu) ? __ldg(h + (size_t)r * kBT + g) : 0.f;
+    }
+  };
+  int pct = ct0, pkb = first_of(ct0);                           // next unit to copy
+  settle(pct, pkb);
+  int ct = pct, kb = pkb;                                       // next unit to compute
+  int j = row_id(pct, pkb);
+  float hn[8];
+  load_h(ct, kb, hn);
+#pragma unroll 1
+  for (int s = 0; s < kDnStages; ++s) {
+    int nct = pct, nkbi = pkb + kMmaWarps;
+    settle(nct, nkbi);
+    const int jn = row_id(nct, nkbi);
+    copy_unit(pct, s, j);
+    pct = nct; pkb = nkbi; j = jn;
+  }
+  int stage = 0;
+#pragma unroll 1
+  for (int c = ct0; c <= ct1; ++c) {
     float acc[8][4];
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-    const uint16_t* colp = wdt + (size_t)ct * 64 + g * 8;
-    auto rows_of = [&](int kb, int (&j)[4]) {                  // W_downT rows of the unit's four K slots
-      const int c0 = kb * 16 + 2 * t;
-      const int cr[4] = {c0, c0 + 1, c0 + 8, c0 + 9};
+      for (int q = 0; q < 4; ++q) acc[i][q] = 0.f;
+#pragma unroll 1
+    while (ct == c) {
+      float hv[8];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) j[q] = __ldg(ulist + min(cr[q], nu - 1));
-    };
-    auto load_unit = [&](int kb, const int (&j)[4], uint4 (&w)[4], float (&hv)[4]) {
-      const int c0 = kb * 16 + 2 * t;
-      const int cr[4] = {c0, c0 + 1, c0 + 8, c0 + 9};
+      for (int q = 0; q < 8; ++q) hv[q] = hn[q];
+      int nct = ct, nkbi = kb + kMmaWarps;
+      settle(nct, nkbi);
+      load_h(nct, nkbi, hn);
+      cp_async_wait<kDnStages - 1>();
+      __syncwarp();
+      const uint32_t st = ring + (uint32_t)(stage * kDnStage);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        w[q] = ld_stream(colp + (size_t)j[q] * D);
-        hv[q] = (cr[q] < nu) ? __ldg(h + (size_t)cr[q] * kBT + g) : 0.f;
+      for (int ks = 0; ks < 2; ++ks) {
+        uint32_t hi[2], lo[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const float a = hv[ks * 4 + 2 * q], d = hv[ks * 4 + 2 * q + 1];
+          const __nv_bfloat16 h0 = __float2bfloat16_rn(a), h1 = __float2bfloat16_rn(d);
+          const __nv_bfloat16 l0 = __float2bfloat16_rn(a - __bfloat162float(h0)), l1 = __float2bfloat16_rn(d - __bfloat162float(h1));
+          hi[q] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
+          lo[q] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
+        }
+        const int k = ks * 16 + ((lane >> 3) & 1) * 8 + (lane & 7);
+#pragma unroll
+        for (int c2 = 0; c2 < 4; ++c2) {
+          uint32_t bf[4];
+          ldsm_x4_trans(bf, st + (uint32_t)(k * 128 + (((2 * c2 + (lane >> 4)) ^ (k & 7)) << 4)));
+          mma_bf16(acc[2 * c2], hi[0], lo[0], hi[1], lo[1], bf[0], bf[1]);
+          mma_bf16(acc[2 * c2 + 1], hi[0], lo[0], hi[1], lo[1], bf[2], bf[3]);
+        }
       }
-    };
-    auto mma_unit = [&](const uint4 (&w)[4], const float (&hv)[4]) {
-      uint32_t ahi[2], alo[2];
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const __nv_bfloat16 h0 = __float2bfloat16_rn(hv[2 * q]), h1 = __float2bfloat16_rn(hv[2 * q + 1]);
-        const __nv_bfloat16 l0 = __float2bfloat16_rn(hv[2 * q] - __bfloat162float(h0));
-        const __nv_bfloat16 l1 = __float2bfloat16_rn(hv[2 * q + 1] - __bfloat162float(h1));
-        ahi[q] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
-        alo[q] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
-      }
-      const uint32_t w0[4] = {w[0].x, w[0].y, w[0].z, w[0].w}, w1[4] = {w[1].x, w[1].y, w[1].z, w[1].w};
-      const uint32_t w2[4] = {w[2].x, w[2].y, w[2].z, w[2].w}, w3[4] = {w[3].x, w[3].y, w[3].z, w[3].w};
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const uint32_t be0 = __byte_perm(w0[q], w1[q], 0x5410), be1 = __byte_perm(w2[q], w3[q], 0x5410);
-        const uint32_t bo0 = __byte_perm(w0[q], w1[q], 0x7632), bo1 = __byte_perm(w2[q], w3[q], 0x7632);
-        mma_bf16(acc[2 * q], ahi[0], 0u, ahi[1], 0u, be0, be1);
-        mma_bf16(acc[2 * q], alo[0], 0u, alo[1], 0u, be0, be1);
-        mma_bf16(acc[2 * q + 1], ahi[0], 0u, ahi[1], 0u, bo0, bo1);
-        mma_bf16(acc[2 * q + 1], alo[0], 0u, alo[1], 0u, bo0, bo1);
-      }
-    };
-    int ja[4], jb[4];
-    if (a + warp < b) rows_of(a + warp, ja);
-    if (a + warp + kMmaWarps < b) rows_of(a + warp + kMmaWarps, jb);
-    for (int kb = a + warp; kb < b; kb += 2 * kMmaWarps) {      // two units in flight per warp
-      uint4 wa[4], wb[4];
-      float ha[4], hb[4];
-      const bool two = kb + kMmaWarps < b;
-      load_unit(kb, ja, wa, ha);
-      if (two) load_unit(kb + kMmaWarps, jb, wb, hb);
-      if (kb + 2 * kMmaWarps < b) rows_of(kb + 2 * kMmaWarps, ja);
-      if (kb + 3 * kMmaWarps < b) rows_of(kb + 3 * kMmaWarps, jb);
-      mma_unit(wa, ha);
-      if (two) mma_unit(wb, hb);
+      __syncwarp();                                             // every lane has read the stage: it is filled again
+      int qct = pct, qkb = pkb + kMmaWarps;
+      settle(qct, qkb);
+      const int jn = row_id(qct, qkb);
+      copy_unit(pct, stage, j);
+      pct = qct; pkb = qkb; j = jn;
+      if (++stage == kDnStages) stage = 0;
+      ct = nct; kb = nkbi;
     }
-    float* mine = red + warp * 512 + g * 64;                    // token g
+    float* mine = red + warp * 512 + g * 64;                    // token g: the high and the low part's sums
 #pragma unroll
-    for (int i = 0; i < 8; ++i) { mine[8 * (2 * t) + i] = acc[i][0]; mine[8 * (2 * t + 1) + i] = acc[i][1]; }
+    for (int i = 0; i < 8; ++i)
+      *reinterpret_cast<float2*>(mine + 8 * i + 2 * t) = make_float2(acc[i][0] + acc[i][2], acc[i][1] + acc[i][3]);
     __syncthreads();
     {
       float s = 0.f;
 #pragma unroll
-      for (int w2i = 0; w2i < kMmaWarps; ++w2i) s += red[w2i * 512 + tid];
+      for (int w = 0; w < kMmaWarps; ++w) s += red[w * 512 + tid];
       const int tok = tid >> 6, col = tid & 63;
-      if (tok < B) atomicAdd(yacc + (size_t)tok * D + (size_t)ct * 64 + col, s);
+      if (tok < B) atomicAdd(yacc + (size_t)tok * D + (size_t)c * 64 + col, s);
     }
     __syncthreads();
-    u += b - a;
   }
+  cp_async_wait<0>();
 }
 
 }  // namespace prox
