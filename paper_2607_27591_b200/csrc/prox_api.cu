@@ -437,12 +437,8 @@ prox_status_t launch_stage1_batch(prox_ffn* h, const void* x, int B, int k1, int
     }
     {
       LaunchScope ls(h, kKProxy, st);
-      const int row_bytes = (F / ch_per_chunk(h->bits)) * 16, ntiles = (row_bytes + 127) / 128, nunits = D / 128;
-      int usplit = (2 * h->sm_count + ntiles - 1) / ntiles;
-      if (usplit > nunits) usplit = nunits;
-      if (usplit < 1) usplit = 1;
-      const int nitems = ntiles * usplit;
-      const int grid = nitems < h->sm_count ? nitems : h->sm_count;
+      const int row_bytes = (F / ch_per_chunk(h->bits)) * 16, ntiles = (row_bytes + 127) / 128, units = ntiles * (D / 128);
+      const int grid = units < h->sm_count ? units : h->sm_count;
       const size_t smem = (size_t)(h->bits == 4 ? kBuSmem4 : kBuSmem8);
       if ((s = ensure_pmap(h, row_bytes)) != PROX_OK) return s;
       {
@@ -456,8 +452,8 @@ prox_status_t launch_stage1_batch(prox_ffn* h, const void* x, int B, int k1, int
         at[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = at; cfg.numAttrs = use_pdl ? 1 : 0;
         const __half* Sp = h->S; const uint32_t* xdp = h->xd; const float* sop = h->soffb; const float* tfp = h->tokfac;
-        int Dv = D, Fv = F, gs = gshift_m, us = usplit; float* pa = h->pacc; int* stp = h->dev_status;
-        void* args[] = {&h->pmap, &Sp, &xdp, &sop, &tfp, &Dv, &Fv, &gs, &us, &pa, &stp};
+        int Dv = D, Fv = F, gs = gshift_m; float* pa = h->pacc; int* stp = h->dev_status;
+        void* args[] = {&h->pmap, &Sp, &xdp, &sop, &tfp, &Dv, &Fv, &gs, &pa, &stp};
         const void* fn = h->bits == 4 ? reinterpret_cast<const void*>(&proxy_umma_kernel<4>) : reinterpret_cast<const void*>(&proxy_umma_kernel<8>);
         cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
         if (e != cudaSuccess && use_pdl) {              // attribute not accepted here: plain launch from now on

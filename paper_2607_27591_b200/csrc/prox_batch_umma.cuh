@@ -16,8 +16,11 @@
 // A unit = 128 consecutive inputs (4 blocks): its MMAs accumulate into one of four 64-column sets of
 // tensor memory (32 columns for the bytes, 32 for the low nibbles; a unit's first MMA overwrites them); two groups
 // of eight read-back warps take turns on the units and apply their scales while the workers already fill
-// the other sets.  Items = (128-byte tile of the rows, range of units); an item's partial sums are added to an fp32 accumulator in global memory, a small kernel forms
-// the scores.
+// the other sets.  Items = (128-byte tile of the rows, range of units); an item's partial sums
+// are added to an fp32 accumulator in global memory, from which the channel-mask kernel forms the scores.  Every block has
+// the same number of units, to one: with items of equal size dealt out in turn some blocks had 4 where 3.03 was the mean
+// (eight tokens, kernel alone: 4096 x 12288 4-bit 20.8 -> 19.8 us, 4096 x 14336 4-bit 24.2 -> 21.4 and 8-bit 27.3 -> 24.8,
+// 8192 x 28672 4-bit 69.3 -> 53.9: 4.5 TB/s).  A second producer lane changed nothing.
 #pragma once
 
 #include <cuda.h>
@@ -54,7 +57,7 @@ __device__ __forceinline__ float digits4_to_float(int d0, int d1, int d2, int d3
 template <int BITS>
 __global__ void __launch_bounds__(kBuThreads, 1)
 proxy_umma_kernel(const __grid_constant__ CUtensorMap pmap, const __half* __restrict__ S, const uint32_t* __restrict__ xd,
-                  const float* __restrict__ soff, const float* __restrict__ tokfac, int D, int F, int gshift, int usplit,
+                  const float* __restrict__ soff, const float* __restrict__ tokfac, int D, int F, int gshift,
                   float* __restrict__ pacc, int* __restrict__ status) {
   constexpr bool LO = BITS == 4;
   constexpr int CH = LO ? 16 : 8;
@@ -87,7 +90,19 @@ proxy_umma_kernel(const __grid_constant__ CUtensorMap pmap, const __half* __rest
   tc_fence_after();
   const uint32_t tbase = tmem_base_s;
   const int rb = warp - 1 - kBuWorkers;               // read-back warp: set rb / 8, tokens 4 * (rb / 4 % 2) .., lanes 32 * (warp % 4) ..
-  const int nitems = ntiles * usplit;
+  // Work of a block: whole tiles in rounds while there is one for every block, then an equal range of the units of
+  // the tiles that are left (two or three items in all; equal to a unit).
+  const unsigned G = gridDim.x, rounds = (unsigned)ntiles / G, rest = ((unsigned)ntiles - rounds * G) * (unsigned)nunits;
+  const unsigned lo = (unsigned)((unsigned long long)rest * blockIdx.x / G), hi = (unsigned)((unsigned long long)rest * (blockIdx.x + 1) / G);
+  struct Item { int tile, u0, u1; unsigned round, at; };
+  auto next_item = [&](Item& it) -> bool {
+    if (it.round < rounds) { it.tile = (int)(it.round * G + blockIdx.x); it.u0 = 0; it.u1 = nunits; ++it.round; return true; }
+    if (it.at >= hi) return false;
+    const unsigned t = it.at / (unsigned)nunits;
+    it.tile = (int)(rounds * G + t); it.u0 = (int)(it.at - t * (unsigned)nunits); it.u1 = min(nunits, it.u0 + (int)(hi - it.at));
+    it.at += (unsigned)(it.u1 - it.u0);
+    return true;
+  };
   if (tid != 0) asm volatile("griddepcontrol.wait;" ::: "memory");   // thread 0 (the producer) first requests weights
   unsigned gseq = 0;                                  // units this CTA has started (unit number modulo 4 = accumulator set)
   if (warp == 0) {
@@ -97,15 +112,16 @@ proxy_umma_kernel(const __grid_constant__ CUtensorMap pmap, const __half* __rest
       // produce this call's digits have finished (programmatic dependent launch); the digits follow
       bool early = true;
       int first_u0 = 0;
+      bool first_item = true;
+      Item it = {0, 0, 0, 0u, lo};
 #pragma unroll 1
-      for (int item = blockIdx.x; item < nitems && !*abortp; item += gridDim.x) {
-        const int tile = item % ntiles, part = item / ntiles;
-        const int u0 = (int)(((long long)nunits * part) / usplit), u1 = (int)(((long long)nunits * (part + 1)) / usplit);
-        if (item == (int)blockIdx.x) first_u0 = u0;
+      while (!*abortp && next_item(it)) {
+        const int tile = it.tile, u0 = it.u0, u1 = it.u1;
+        if (gseq == 0) first_u0 = u0; else first_item = false;
 #pragma unroll 1
         for (int u = u0; u < u1; ++u, ++gseq) {
           const unsigned s = gseq % kBuStages, use = gseq / kBuStages;
-          if (early && (use > 0 || item != (int)blockIdx.x)) {
+          if (early && (use > 0 || !first_item)) {
             // the ring is full (or the first item has ended): now the digits of what was requested
             asm volatile("griddepcontrol.wait;" ::: "memory");
             for (unsigned k = 0; k < gseq; ++k)
@@ -149,10 +165,10 @@ proxy_umma_kernel(const __grid_constant__ CUtensorMap pmap, const __half* __rest
     unsigned mine = 0, s_prev = 0, use_prev = 0;
     bool bad = false;                                 // a wait of this warp gave up; the group leaves together
     if (LO || wj == 0) {
+      Item it = {0, 0, 0, 0u, lo};
 #pragma unroll 1
-      for (int item = blockIdx.x; item < nitems; item += gridDim.x) {
-        const int part = item / ntiles;
-        const int u0 = (int)(((long long)nunits * part) / usplit), u1 = (int)(((long long)nunits * (part + 1)) / usplit);
+      while (next_item(it)) {
+        const int u0 = it.u0, u1 = it.u1;
         bool dead = false;
 #pragma unroll 1
         for (int ul = (int)(((unsigned)grp + gseq) & 1u); ul < u1 - u0; ul += 2) {
@@ -232,10 +248,10 @@ proxy_umma_kernel(const __grid_constant__ CUtensorMap pmap, const __half* __rest
     float tf[4];
 #pragma unroll
     for (int b = 0; b < 4; ++b) tf[b] = tokfac[half * 4 + b] * 9.094947017729282e-13f;   // * 2^-40
+    Item it = {0, 0, 0, 0u, lo};
 #pragma unroll 1
-    for (int item = blockIdx.x; item < nitems; item += gridDim.x) {
-      const int tile = item % ntiles, part = item / ntiles;
-      const int u0 = (int)(((long long)nunits * part) / usplit), u1 = (int)(((long long)nunits * (part + 1)) / usplit);
+    while (next_item(it)) {
+      const int tile = it.tile, u0 = it.u0, u1 = it.u1;
       const int nu = u1 - u0;
       const int chunk = tile * 8 + (col >> 4);
       const bool col_ok = chunk < nchunks;
@@ -298,8 +314,8 @@ proxy_umma_kernel(const __grid_constant__ CUtensorMap pmap, const __half* __rest
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
           float* dst = pacc + ((size_t)(half * 4 + b) * 2 + which) * F + ch;
-          atomicAdd(dst, t0[b] * tf[b]);
-          if (LO) atomicAdd(dst + 1, t1[b] * tf[b]);
+          if (LO) atomicAdd(reinterpret_cast<float2*>(dst), make_float2(t0[b] * tf[b], t1[b] * tf[b]));
+          else atomicAdd(dst, t0[b] * tf[b]);
         }
       }
       gseq += (unsigned)nu;
