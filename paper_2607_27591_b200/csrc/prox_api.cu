@@ -613,11 +613,11 @@ struct FusedPlan {
   int optin;            // the device's opt-in limit: what the kernels' dynamic shared memory attribute is set to
 };
 
-FusedPlan plan_fused(const prox_ffn* h, int k1, int k2, bool thresh = false) {
+FusedPlan plan_fused(const prox_ffn* h, int k1, int k2, bool thresh = false, int mode = kWhole) {
   FusedPlan pl;
   std::memset(&pl, 0, sizeof(pl));
   const int D = h->cfg.d_model, F = h->cfg.d_ff;
-  if (!h->use_fused || h->bits == 16) return pl;       // the fused kernel reads integer proxies
+  if (!h->use_fused || (h->bits == 16 && mode != kGivenList)) return pl;       // phase B reads integer proxies
   const int G = h->sm_count;
   const size_t fixed = ((sizeof(FusedSmem) + 127) & ~size_t(127)) + (size_t)8 * D;   // + x bf16, idx, x fp32
   if ((size_t)h->smem_optin < fixed + (size_t)6 * D) return pl;
@@ -626,11 +626,11 @@ FusedPlan plan_fused(const prox_ffn* h, int k1, int k2, bool thresh = false) {
   if (pl.nslots > kMaxSlots) pl.nslots = kMaxSlots;
   if (pl.nslots < 3) return pl;
   // the proxy GEMV keeps 16 tensor-memory columns per supergroup (4 scale groups), two sets of up to 256
-  if ((D / h->group + 3) / 4 > kMaxSuper) return pl;
+  if ((D / h->group + 3) / 4 > kMaxSuper && mode != kGivenList) return pl;
   // the proxy ring and its partial sums take the place of x as fp32 and the big buffer
   pl.loaders = (int)((4 * (size_t)D + pl.big_bytes - 1024 - 3072) / proxy_warp_bytes(h->bits));
   if (pl.loaders > kFusedConsumerWarps) pl.loaders = kFusedConsumerWarps;
-  if (pl.loaders < kMinLoaders) return pl;
+  if (pl.loaders < kMinLoaders && mode != kGivenList) return pl;
   // Columns of the packed rows per block: whole 128-byte tiles (8 chunks) while there is at most one per SM: narrower
   // shares on all SMs took as long or longer (4096 x 12288: 8.0 us either way with 96 tiles; 1024 x 3072: 3.5 against
   // 4.1 us, more blocks add to the same few histogram bins).  Beyond that equal shares in 32-byte sectors: 224 tiles
@@ -645,7 +645,8 @@ FusedPlan plan_fused(const prox_ffn* h, int k1, int k2, bool thresh = false) {
   if (thresh) {
     // any number of channels may pass the threshold: a block's share of all of them must fit, the scores
     // must fit in shared memory (no radix fallback in this form), counts are kept in 16 bits
-    if ((F + G - 1) / G + 2 > kMySelCap || (size_t)F * 4 + 256 > (size_t)pl.big_bytes || F >= 65536) return pl;
+    if ((F + G - 1) / G + 2 > kMySelCap) return pl;
+    if (mode == kWhole && ((size_t)F * 4 + 256 > (size_t)pl.big_bytes || F >= 65536)) return pl;
   }
   (void)k1;
   pl.grid = h->debug_grid ? h->debug_grid : G;
@@ -656,10 +657,10 @@ FusedPlan plan_fused(const prox_ffn* h, int k1, int k2, bool thresh = false) {
   return pl;
 }
 
-template <int BITS, int NG, bool NORM, bool THRESH>
+template <int BITS, int NG, bool NORM, bool THRESH, int MODE = kWhole>
 cudaError_t launch_fused_tn(const FusedPlan& pl, const FusedParams& prm, cudaStream_t st) {
   static bool attr_dev[64] = {};     // per instantiation and device: the attribute belongs to the function on a device
-  auto kern = prox_fused_kernel<BITS, NG, NORM, THRESH>;
+  auto kern = prox_fused_kernel<BITS, NG, NORM, THRESH, MODE>;
   bool& attr_set = attr_dev[pl.device & 63];
   if (!attr_set) {
     // the limit, not this plan's size: another handle's shape may need a few bytes more
@@ -712,16 +713,18 @@ RmsConst rms_const(int D, double eps) {
 prox_status_t launch_fused(prox_ffn* h, const FusedPlan& pl, const void* x, int k1, int k2, void* y,
                            int* sel_out, cudaStream_t st, const float* xres = nullptr,
                            const uint16_t* norm_w = nullptr, double eps = 0.0, float* xres_out = nullptr,
-                           const float* taus = nullptr) {
+                           const float* taus = nullptr, int mode = kWhole, float* scores = nullptr,
+                           const int* sel_in = nullptr, const int* sel_cnt = nullptr) {
   FusedParams prm;
   std::memset(&prm, 0, sizeof(prm));
+  prm.sel_in = sel_in; prm.sel_cnt = sel_cnt;
   prm.P = h->P; prm.S = h->S; prm.wg = h->wg; prm.wu = h->wu; prm.wdt = h->wdt;
   prm.x = static_cast<const uint16_t*>(x); prm.y = y;
   prm.D = h->cfg.d_model; prm.F = h->cfg.d_ff; prm.k1 = k1; prm.k2 = k2;
   prm.gshift = (h->group == h->cfg.d_model) ? 31 : 7;
   prm.out_fp32 = h->cfg.out_dtype;
-  prm.loaders = pl.loaders; prm.cgran = pl.cgran;
-  prm.scores = h->scores; prm.ghist = h->syncbuf; prm.idx_out = h->idx_x;
+  prm.loaders = pl.loaders > 0 ? pl.loaders : 1; prm.cgran = pl.cgran;
+  prm.scores = scores ? scores : h->scores; prm.ghist = h->syncbuf; prm.idx_out = h->idx_x;
   prm.spin_limit = h->spin_limit; prm.bar_bias = h->bar_bias; prm.host_flag = h->host_flag_dev;
   prm.sel_out = sel_out; prm.yacc = h->yacc;
   prm.exits = reinterpret_cast<unsigned long long*>(h->syncbuf + 4096); prm.ctr = h->syncbuf + 4104;
@@ -737,12 +740,18 @@ prox_status_t launch_fused(prox_ffn* h, const FusedPlan& pl, const void* x, int 
     std::memcpy(&bx, &tx, 4); std::memcpy(&bs, &ts, 4);
     prm.tkey_x = (bx >> 16) + ((bx & 0xffffu) ? 1u : 0u);
     prm.tkey_s = bs;
-    prm.cnt_x_out = h->cnt_x; prm.count_out = h->cnt_s; prm.counters = h->counters;
+    prm.cnt_x_out = h->cnt_x; prm.count_out = h->cnt_s; prm.counters = mode == kWhole ? h->counters : nullptr;
   }
   cudaError_t e;
   {
     LaunchScope ls(h, kKFused, st);
-    if (h->bits == 4) {
+    if (mode == kScoresOnly) {
+      e = h->bits == 4 ? (taus ? launch_fused_tn<4, 4, false, true, kScoresOnly>(pl, prm, st) : launch_fused_tn<4, 4, false, false, kScoresOnly>(pl, prm, st))
+                       : (taus ? launch_fused_tn<8, 4, false, true, kScoresOnly>(pl, prm, st) : launch_fused_tn<8, 4, false, false, kScoresOnly>(pl, prm, st));
+    } else if (mode == kGivenList) {                     // (the proxies are not used)
+      e = pl.xch == 4 ? launch_fused_tn<8, 4, false, false, kGivenList>(pl, prm, st)
+        : pl.xch == 2 ? launch_fused_tn<8, 2, false, false, kGivenList>(pl, prm, st) : launch_fused_tn<8, 1, false, false, kGivenList>(pl, prm, st);
+    } else if (h->bits == 4) {
       e = pl.xch == 4 ? launch_fused_t<4, 4>(pl, prm, st)
         : pl.xch == 2 ? launch_fused_t<4, 2>(pl, prm, st) : launch_fused_t<4, 1>(pl, prm, st);
     } else {
@@ -956,6 +965,17 @@ prox_status_t prox_stage1_mask(prox_ffn_t* h, const void* x, int B, int k1, int 
       CK(cudaMemcpyAsync(sc, own, (size_t)B * h->cfg.d_ff * sizeof(float), cudaMemcpyDeviceToDevice, st));
     return s;
   }
+  if (B == 1) {
+    // input mask and proxy scores by the persistent kernel (up to its barrier)
+    const FusedPlan pl = plan_fused(h, k1, 1, false, kScoresOnly);
+    if (pl.ok) {
+      float* own = aligned16(sc) ? sc : h->scores;
+      if ((s = launch_fused(h, pl, x, k1, 1, nullptr, nullptr, st, nullptr, nullptr, 0.0, nullptr, nullptr, kScoresOnly, own)) != PROX_OK) return s;
+      if ((s = launch_channel_select(h, own, 1, k2, 0.f, 0, sel, k2, nullptr, st)) != PROX_OK) return s;
+      if (own != sc) CK(cudaMemcpyAsync(sc, own, (size_t)h->cfg.d_ff * sizeof(float), cudaMemcpyDeviceToDevice, st));
+      return PROX_OK;
+    }
+  }
   if ((s = launch_input_select(h, x, B, k1, 0.f, 0, h->idx_x, D, nullptr, st)) != PROX_OK) return s;
   if ((s = launch_proxy(h, x, B, h->idx_x, D, nullptr, k1, sc, st)) != PROX_OK) return s;
   return launch_channel_select(h, sc, B, k2, 0.f, 0, sel, k2, nullptr, st);
@@ -970,6 +990,12 @@ prox_status_t prox_stage2_ffn(prox_ffn_t* h, const void* x, int B, const int32_t
   if (!h->quantized) return PROX_ERR_NOT_QUANTIZED;
   if (h->use_union && batch_path_ok(h, B))
     return launch_stage2_batch(h, x, B, sel, k2, k2, y, static_cast<cudaStream_t>(stream));
+  if (B == 1) {
+    const FusedPlan pl = plan_fused(h, 1, k2, false, kGivenList);
+    if (pl.ok)
+      return launch_fused(h, pl, x, 1, k2, y, nullptr, static_cast<cudaStream_t>(stream), nullptr, nullptr, 0.0, nullptr, nullptr, kGivenList,
+                          nullptr, sel);
+  }
   return launch_stage2(h, x, B, sel, k2, nullptr, k2, y, static_cast<cudaStream_t>(stream));
 }
 
@@ -1339,8 +1365,14 @@ prox_status_t prox_stage1_mask_threshold(prox_ffn_t* h, const void* x, int B, fl
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int D = h->cfg.d_model, F = h->cfg.d_ff;
   float* sc = scores ? scores : h->scores;
-  if ((s = launch_input_select(h, x, B, 0, tau_x, 1, h->idx_x, D, h->cnt_x, st)) != PROX_OK) return s;
-  if ((s = launch_proxy(h, x, B, h->idx_x, D, h->cnt_x, D, sc, st)) != PROX_OK) return s;
+  const FusedPlan pl = plan_fused(h, D, 1, true, kScoresOnly);
+  if (B == 1 && pl.ok && tau_x < INFINITY && aligned16(sc)) {
+    const float taus[2] = {tau_x, 0.f};
+    if ((s = launch_fused(h, pl, x, D, 1, nullptr, nullptr, st, nullptr, nullptr, 0.0, nullptr, taus, kScoresOnly, sc)) != PROX_OK) return s;
+  } else {
+    if ((s = launch_input_select(h, x, B, 0, tau_x, 1, h->idx_x, D, h->cnt_x, st)) != PROX_OK) return s;
+    if ((s = launch_proxy(h, x, B, h->idx_x, D, h->cnt_x, D, sc, st)) != PROX_OK) return s;
+  }
   if ((s = launch_channel_select(h, sc, B, 0, tau_s, 1, sel, F, count, st)) != PROX_OK) return s;
   count_accum_kernel<<<1, 32, 0, st>>>(h->cnt_x, count, B, h->counters);
   h->launches++;
@@ -1354,6 +1386,12 @@ prox_status_t prox_stage2_ffn_var(prox_ffn_t* h, const void* x, int B, const int
   if (s != PROX_OK) return s;
   if (!sel || !count || !y || !aligned16(y)) return PROX_ERR_INVALID_ARG;
   if (!h->quantized) return PROX_ERR_NOT_QUANTIZED;
+  if (B == 1) {
+    const FusedPlan pl = plan_fused(h, 1, 1, true, kGivenList);
+    if (pl.ok)
+      return launch_fused(h, pl, x, 1, 1, y, nullptr, static_cast<cudaStream_t>(stream), nullptr, nullptr, 0.0, nullptr, nullptr, kGivenList,
+                          nullptr, sel, count);
+  }
   return launch_stage2(h, x, B, sel, h->cfg.d_ff, count, h->cfg.d_ff, y, static_cast<cudaStream_t>(stream));
 }
 

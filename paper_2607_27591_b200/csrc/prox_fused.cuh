@@ -59,7 +59,10 @@ constexpr int kMinLoaders = 8;           // loader warps that must fit (at most 
 constexpr int kMaxSuper = 16;            // supergroups (4 scale groups) whose accumulators fit the tensor memory
 constexpr unsigned kSpinLimit = 1u << 21;
 
+enum FusedMode { kWhole = 0, kScoresOnly, kGivenList };   // whole path; A and B; D to F for the caller's channels
+
 struct FusedParams {
+  const int* sel_in; const int* sel_cnt;   // kGivenList: the channels, and how many (NULL: k2)
   const uint8_t* P; const __half* S;
   const uint16_t* wg; const uint16_t* wu; const uint16_t* wdt;
   const uint16_t* x; void* y;
@@ -314,7 +317,8 @@ struct FusedSmem {
 // NORM = layer sub-block form (RMSNorm in the prologue, residual add at the end); THRESH = threshold
 // form of the two masks (Sec. 4.1 indicators with calibrated thresholds; no k-th element search at all).
 // Instantiations of their own, so that the plain call carries none of their code or registers.
-template <int BITS, int NG, bool NORM = false, bool THRESH = false>
+// MODE: instantiations of their own for the two stages called alone (as a run-time switch it cost the whole path 1 %).
+template <int BITS, int NG, bool NORM = false, bool THRESH = false, int MODE = kWhole>
 __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const FusedParams p) {
   constexpr int CH = ProxyFmt<BITS>::CH;
   constexpr int NT = kFusedThreads;
@@ -420,7 +424,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   // Stage-1 share of this block; the answers are first looked at after phase A.  A block that gets none and finds
   // Stage 1 complete has started late: it leaves (what it read may be a residual stream that is being added to).
   unsigned claim1 = 0, done1 = 0;
-  if (tid == NT - 1) {
+  if (tid == NT - 1 && MODE != kGivenList) {
     asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(claim1) : "l"(ctr + kClaim1) : "memory");
     asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(done1) : "l"(ctr + kDone1) : "memory");
   }
@@ -430,7 +434,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     for (int i = cta * per + tid; i < min(2048, (cta + 1) * per); i += NT) other[i] = 0u;
     if (cta == 0 && tid < 8) p.ctr[8u * (sm.call_par ^ 1u) + tid] = 0u;
   }
-  if (warp < 4) {
+  if (warp < 4 && MODE != kGivenList) {
     // the accumulators of the proxy GEMV start at zero: 16 columns per supergroup, two sets 256 columns apart
     const int ngz = (p.gshift >= 31) ? 1 : (D >> p.gshift);
     const uint32_t tz = sm.tmem_base + ((uint32_t)(warp * 32) << 16);
@@ -441,6 +445,25 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   }
   PROX_TRACE(1);
 
+  // every block counts its leaving
+  auto leave = [&]() {
+    if (tid == 0) atomicAdd(p.exits, cta == 0 ? 257ull - (unsigned long long)G : 1ull);
+  };
+  auto widen_x = [&](int t0) {                  // x as fp32 for phase D, by the threads from t0 on
+#pragma unroll 1
+    for (int i = tid - t0; i < D / 8; i += NT - t0) {
+      const uint4 v = reinterpret_cast<const uint4*>(xs)[i];
+      reinterpret_cast<float4*>(xf)[2 * i] = make_float4(bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y));
+      reinterpret_cast<float4*>(xf)[2 * i + 1] = make_float4(bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w));
+    }
+  };
+  if (MODE == kGivenList) {
+    unsigned share2 = 0;
+    if (tid == 0) asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(share2) : "l"(ctr + kClaim2) : "memory");
+    widen_x(0);
+    if (tid == 0) sm.shr = share2;
+    __syncthreads();
+  } else {
   // ------------------------------------------------- A: input mask (top-k1 of |x|)
   int ebase = 1;
   const bool per_row_a = p.gshift >= 31;
@@ -538,10 +561,6 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     if (tid == NT - 1) { sm.vid = claim1; sm.late = done1 >= (unsigned)p.nshare1 && claim1 >= (unsigned)p.nshare1; }
     __syncthreads();
   }
-  // every block counts its leaving
-  auto leave = [&]() {
-    if (tid == 0) atomicAdd(p.exits, cta == 0 ? 257ull - (unsigned long long)G : 1ull);
-  };
   if (sm.late) {
     if (warp == 0) tmem_free_all(sm.tmem_base);
     leave();
@@ -831,8 +850,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
         asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(fin) : "l"(ctr + kDone1) : "memory");
         asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(more1) : "l"(ctr + kClaim1) : "memory");
       }
-      if (first) asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(share2) : "l"(ctr + kClaim2) : "memory");
+      if (first && MODE == kWhole) asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(share2) : "l"(ctr + kClaim2) : "memory");
       ok = vid < n1 && fin + 1u == target;
+      if (MODE == kScoresOnly) { again = more1 < n1; ok = true; }      // nobody waits
 #pragma unroll 1
       for (unsigned it = 0; !ok && it < spin; ++it) {
         unsigned cur;
@@ -845,13 +865,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       sm.again = again; sm.vid = more1;
       if (!ok && !again) { sm.abort_flag = 1; atomicOr(p.status, kWaitExpired); if (p.host_flag) *reinterpret_cast<volatile int*>(p.host_flag) = 1; }
     } else if (warp > 0) {
-      // meanwhile: x as fp32 for phase D
-#pragma unroll 1
-      for (int i = tid - 32; i < D / 8; i += NT - 32) {
-        const uint4 v = reinterpret_cast<const uint4*>(xs)[i];
-        reinterpret_cast<float4*>(xf)[2 * i] = make_float4(bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y));
-        reinterpret_cast<float4*>(xf)[2 * i + 1] = make_float4(bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w));
-      }
+      widen_x(32);                              // meanwhile
     }
     __syncthreads();
     if (!sm.again || *abortp) break;
@@ -866,10 +880,16 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     __syncthreads();
     tc_fence_after();
   }
+  }
   if (warp == 0) tmem_free_all(sm.tmem_base);
   const bool alive = sm.abort_flag == 0;      // block-uniform; a dead block skips to the end
   PROX_TRACE(4);
 
+  if (MODE == kScoresOnly) {
+    if (!alive && tid == 0) { atomicOr(p.status, kWaitExpired); if (p.host_flag) *reinterpret_cast<volatile int*>(p.host_flag) = 1; }
+    leave();
+    return;
+  }
   // Stage 2: this block's share of the kept channels (and further ones if a block of the grid is not running)
   unsigned base_seq = 0;                        // ring rows consumed so far
   unsigned pseq = 0, puse = 0;                  // producers: rows armed or passed over, uses of the ring, ...
@@ -887,7 +907,26 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   // is known after two passes over the scores, so its weight rows start to stream
   // while the consumer warps still settle the threshold inside b1.
   int n_mine = 0;
-  if (alive && warp < kFusedConsumerWarps) {          // the producer warps wait at the ring for the go flag
+  if (MODE == kGivenList) {
+    if (warp < kFusedConsumerWarps) {
+      const unsigned n = (unsigned)(p.sel_cnt ? min(max(__ldcg(p.sel_cnt), 0), F) : k2);
+      const int R0 = (int)((n * shr) / NSH);
+      n_mine = min((int)((n * (shr + 1u)) / NSH) - R0, kMySelCap);
+#pragma unroll 1
+      for (int i = tid; i < n_mine; i += kFusedConsumers) {
+        const int j = p.sel_in[R0 + i];
+        if (j < 0 || j >= F) atomicOr(p.status, kBadChannel);
+        sm.mysel[i] = (j < 0 || j >= F) ? -1 : j;
+      }
+      if (tid == 0) {
+        sm.keys_s0 = sm.keys_s1 = sm.list_s0 = sm.list_s1 = 0;
+        sm.n_mine = n_mine; sm.nready = n_mine; sm.keys_done = 1; sm.c_done = 1;
+      }
+      __threadfence_block();
+      consumer_sync();
+      if (tid == 0) *reinterpret_cast<volatile int*>(&sm.go) = 1;
+    }
+  } else if (alive && warp < kFusedConsumerWarps) {          // the producer warps wait at the ring for the go flag
     // Shared-memory plan: the keys (score bits) sit at the END of the big buffer (the ring fills
     // from slot 0 and reaches those slots last); the ascending list of b1's members goes where
     // the input index list was (free since phase B), or in front of the keys if it is long.
@@ -1317,9 +1356,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
             if (use > 0 && !mbar_wait(smem_u32(&sm.mbar_empty[slot]), (use - 1u) & 1u, abortp, spin)) { dead = true; break; }
             const uint16_t* src;
             if (q < 2 * nb) {
-              src = ((q & 1) ? p.wu : p.wg) + (size_t)sm.mysel[mi] * D;
+              src = ((q & 1) ? p.wu : p.wg) + (size_t)max(sm.mysel[mi], 0) * D;
             } else {
-              src = p.wdt + (size_t)sm.mysel[mi] * D;
+              src = p.wdt + (size_t)max(sm.mysel[mi], 0) * D;
             }
             const uint32_t bar = smem_u32(&sm.mbar_full[slot]);
             if (seq == 0) PROX_TRACE_AT(28, tid);

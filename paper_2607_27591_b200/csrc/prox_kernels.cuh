@@ -628,8 +628,8 @@ down_kernel(const uint16_t* __restrict__ wdt, const float* __restrict__ h, int h
   }
   if (e < D && c1 > c0) {
     float* yp = yacc + (size_t)b * D + e;
-#pragma unroll
-    for (int m = 0; m < 8; ++m) atomicAdd(yp + m, acc[m]);
+    atomicAdd(reinterpret_cast<float4*>(yp), make_float4(acc[0], acc[1], acc[2], acc[3]));
+    atomicAdd(reinterpret_cast<float4*>(yp) + 1, make_float4(acc[4], acc[5], acc[6], acc[7]));
   }
 }
 

@@ -141,7 +141,7 @@ def test_channel_mask_is_the_exact_topk_of_the_scores(pb, F, B, shared):
         pb.prox_ffn_destroy(h)
 
 
-@pytest.mark.parametrize("D,F", [(128, 64), (640, 1600), (2176, 2048), (4224, 1472), (8192, 704)])
+@pytest.mark.parametrize("D,F", [(128, 64), (640, 1600), (2176, 2048), (3584, 1472), (4224, 1472), (8192, 704)])
 @pytest.mark.parametrize("B", [2, 8])
 def test_batch_stage2_rows_in_sections(pb, D, F, B):
     """One to four sections of a row, the last one short; unions smaller than the grid, ragged tiles and all channels."""
@@ -159,5 +159,41 @@ def test_batch_stage2_rows_in_sections(pb, D, F, B):
                 # h enters the down projection as a bf16 pair (2^-17 relative), sums in fp32
                 assert np.linalg.norm(y.cpu().numpy()[b] - y_ref) <= 1e-4 * np.linalg.norm(y_ref)
         assert pb.prox_last_device_status(p.h) == 0
+    finally:
+        p.close()
+
+
+@pytest.mark.parametrize("D,F,bits,group", [(128, 64, 4, 0), (640, 4992, 8, 128), (8192, 704, 4, 128), (10240, 192, 4, 128), (1024, 2048, 16, 0)])
+def test_stages_one_by_one(pb, D, F, bits, group):
+    """The stages called alone (persistent kernel up to its barrier, and on a given list; wider layers and 16-bit proxies:
+    step-wise kernels) against the whole path on the same masks, with repeated calls; bad channel ids are skipped."""
+    wg, wu, wd, x = inputs.make_small(D, F, 2, seed=D + F)
+    p = Problem(pb, wg, wu, wd, x)
+    try:
+        pb.prox_quantize_proxy(p.h, bits, group)
+        for k1, k2 in ((D // 3, F // 3), (1, 1), (D, F)):
+            for t in (0, 1, 0):
+                y, y1 = p.y_empty(), p.y_empty()
+                sel, sel1 = (torch.empty(1, k2, dtype=torch.int32, device="cuda") for _ in range(2))
+                sc, sc1 = (torch.empty(F, dtype=torch.float32, device="cuda") for _ in range(2))
+                pb.prox_ffn_forward(p.h, p.t_x[t], 1, k1, k2, y)
+                pb.prox_ffn_last_mask(p.h, 1, k2, sel)
+                pb.prox_ffn_last_stage1(p.h, k1, None, sc)
+                pb.prox_stage1_mask(p.h, p.t_x[t], 1, k1, k2, sel1, sc1)
+                pb.prox_stage2_ffn(p.h, p.t_x[t], 1, sel1, k2, y1)
+                torch.cuda.synchronize()
+                assert torch.equal(sc, sc1) and torch.equal(sel, sel1)
+                # the same products in another order of summation
+                assert float((y - y1).norm()) <= 1e-5 * float(y.norm())
+        n = min(F, 40)
+        ids = torch.arange(F, dtype=torch.int32, device="cuda").view(1, F).contiguous()
+        cnt = torch.tensor([n], dtype=torch.int32, device="cuda")
+        y, y1 = p.y_empty(), p.y_empty()
+        pb.prox_stage2_ffn_var(p.h, p.t_x, 1, ids, cnt, y)
+        assert pb.prox_last_device_status(p.h) == 0
+        bad = torch.cat([ids[0, :n], torch.tensor([F, -1], dtype=torch.int32, device="cuda")]).view(1, -1).contiguous()
+        pb.prox_stage2_ffn(p.h, p.t_x, 1, bad, n + 2, y1)
+        assert pb.prox_last_device_status(p.h) == 1
+        assert float((y - y1).norm()) <= 1e-5 * float(y.norm())
     finally:
         p.close()
