@@ -657,10 +657,10 @@ FusedPlan plan_fused(const prox_ffn* h, int k1, int k2, bool thresh = false, int
   return pl;
 }
 
-template <int BITS, int NG, bool NORM, bool THRESH, int MODE = kWhole>
+template <int BITS, int NG, bool NORM, bool THRESH, int MODE = kWhole, bool TRACE = false>
 cudaError_t launch_fused_tn(const FusedPlan& pl, const FusedParams& prm, cudaStream_t st) {
   static bool attr_dev[64] = {};     // per instantiation and device: the attribute belongs to the function on a device
-  auto kern = prox_fused_kernel<BITS, NG, NORM, THRESH, MODE>;
+  auto kern = prox_fused_kernel<BITS, NG, NORM, THRESH, MODE, TRACE>;
   bool& attr_set = attr_dev[pl.device & 63];
   if (!attr_set) {
     // the limit, not this plan's size: another handle's shape may need a few bytes more
@@ -692,13 +692,19 @@ cudaError_t launch_fused_tn(const FusedPlan& pl, const FusedParams& prm, cudaStr
   return e;
 }
 
+template <int BITS, int NG, bool NORM, bool THRESH>
+cudaError_t launch_fused_tr(const FusedPlan& pl, const FusedParams& prm, cudaStream_t st) {
+  return prm.trace ? launch_fused_tn<BITS, NG, NORM, THRESH, kWhole, true>(pl, prm, st)
+                   : launch_fused_tn<BITS, NG, NORM, THRESH>(pl, prm, st);
+}
+
 template <int BITS, int NG>
 cudaError_t launch_fused_t(const FusedPlan& pl, const FusedParams& prm, cudaStream_t st) {
   if (prm.count_out)                                                                   // threshold form
-    return prm.xres ? launch_fused_tn<BITS, NG, true, true>(pl, prm, st)
-                    : launch_fused_tn<BITS, NG, false, true>(pl, prm, st);
-  return prm.xres ? launch_fused_tn<BITS, NG, true, false>(pl, prm, st)
-                  : launch_fused_tn<BITS, NG, false, false>(pl, prm, st);
+    return prm.xres ? launch_fused_tr<BITS, NG, true, true>(pl, prm, st)
+                    : launch_fused_tr<BITS, NG, false, true>(pl, prm, st);
+  return prm.xres ? launch_fused_tr<BITS, NG, true, false>(pl, prm, st)
+                  : launch_fused_tr<BITS, NG, false, false>(pl, prm, st);
 }
 
 // 1/d_model and eps as pairs of floats for the device-side RMSNorm

@@ -151,8 +151,8 @@ __device__ __forceinline__ unsigned long long global_ns() {
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
   return t;
 }
-#define PROX_TRACE_AT(k, who) do { if (p.trace && tid == (who)) p.trace[(size_t)cta * 32 + (k)] = global_ns(); } while (0)
-#define PROX_TRACE(k) do { if (p.trace && tid == 0) p.trace[(size_t)cta * 32 + (k)] = global_ns(); } while (0)
+#define PROX_TRACE_AT(k, who) do { if (TRACE && tid == (who)) p.trace[(size_t)cta * 32 + (k)] = global_ns(); } while (0)
+#define PROX_TRACE(k) do { if (TRACE && tid == 0) p.trace[(size_t)cta * 32 + (k)] = global_ns(); } while (0)
 __device__ __forceinline__ bool elect_one() {          // the same lane every time for a full warp
   uint32_t pred;
   asm volatile("{\n\t.reg .pred P1;\n\telect.sync _|P1, 0xffffffff;\n\tselp.u32 %0, 1, 0, P1;\n\t}" : "=r"(pred));
@@ -313,12 +313,36 @@ struct FusedSmem {
   float ninv[2];                  // ... and 1 / sqrt(mean + eps) (hi, lo)
 };
 
+// k-th largest (k >= 1) over a histogram held in registers: thread t < 512 has the counts of N bins in descending order,
+// the first of them bin `top`; the threads' runs follow each other downwards (threads from 512 on: zeros).  One scan and two
+// barriers where reading the bins segment by segment took three passes over shared memory (0.8 -> 0.4 us for 1024 bins,
+// 1.1 -> 0.6 for 2048).  res[0..2] = bin, elements above it, elements inside.
+template <int N, bool CONSUMERS_ONLY>
+__device__ __forceinline__ void find_kth(FusedSmem& sm, const unsigned (&c)[N], int top, unsigned k, int lane, int warp) {
+  unsigned s = 0;
+#pragma unroll
+  for (int j = 0; j < N; ++j) s += c[j];
+  const unsigned inc = warp_scan_incl(s, lane);
+  if (lane == 31) sm.wsum[warp] = inc;
+  if (CONSUMERS_ONLY) consumer_sync(); else __syncthreads();
+  unsigned run = __reduce_add_sync(0xffffffffu, (lane < warp) ? sm.wsum[lane] : 0u) + inc - s;
+  if (run < k && k <= run + s) {
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      if (run < k && k <= run + c[j]) { sm.res[0] = (unsigned)(top - j); sm.res[1] = run; sm.res[2] = c[j]; }
+      run += c[j];
+    }
+  }
+  if (CONSUMERS_ONLY) consumer_sync(); else __syncthreads();
+}
+
 // NG = warp groups of the down projection (4: d_model <= 4096, 2: <= 8192, 1: <= 16384)
 // NORM = layer sub-block form (RMSNorm in the prologue, residual add at the end); THRESH = threshold
 // form of the two masks (Sec. 4.1 indicators with calibrated thresholds; no k-th element search at all).
 // Instantiations of their own, so that the plain call carries none of their code or registers.
+// TRACE: with time stamps (the tests for them cost the plain kernel up to 4 %: code that runs once is fetched cold).
 // MODE: instantiations of their own for the two stages called alone (as a run-time switch it cost the whole path 1 %).
-template <int BITS, int NG, bool NORM = false, bool THRESH = false, int MODE = kWhole>
+template <int BITS, int NG, bool NORM = false, bool THRESH = false, int MODE = kWhole, bool TRACE = false>
 __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const FusedParams p) {
   constexpr int CH = ProxyFmt<BITS>::CH;
   constexpr int NT = kFusedThreads;
@@ -483,8 +507,10 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       }
       __syncthreads();
       PROX_TRACE(10);
-      unsigned above1;
-      const unsigned bin1 = kth_in_block<2, false>(sm.hist, (unsigned)k1, sm.wsum, lane, warp, &above1);
+      unsigned hb[2] = {0u, 0u};
+      if (tid < 512) { const uint2 v = reinterpret_cast<const uint2*>(sm.hist)[511 - tid]; hb[0] = v.y; hb[1] = v.x; }
+      find_kth<2, false>(sm, hb, 1023 - 2 * tid, (unsigned)k1, lane, warp);
+      const unsigned bin1 = sm.res[0], above1 = sm.res[1];
       PROX_TRACE(11);
       // Inputs whose magnitude lies in a bin above the threshold bin are kept whatever the exact threshold:
       // their packed proxy rows are pulled into L2 now (every block a share of them, one bulk prefetch per
@@ -943,23 +969,22 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     auto key4_at = [&](int i) -> uint4 {                  // i % 4 == 0
       return in_smem ? lds128(skey_u32 + (uint32_t)i * 4u) : __ldcg(reinterpret_cast<const uint4*>(gkey + i));
     };
-    if (!THRESH && tid < 512) cp_async16(smem_u32(sm.hist) + (uint32_t)tid * 16u, ghist + tid * 4);
-    cp_async_commit();
+    uint4 hv = make_uint4(0u, 0u, 0u, 0u);
+    if (!THRESH) hv = __ldcg(reinterpret_cast<const uint4*>(ghist) + (511 - tid));
     if (in_smem) {
 #pragma unroll 1
       for (int i = tid; i < F / 4; i += kFusedConsumers) cp_async16(skey_u32 + (uint32_t)i * 16u, gkey + 4 * i);
     }
     cp_async_commit();
     if (tid < 256) sm.hist2[tid] = 0;
-    cp_async_wait<1>();                                    // the histogram (the keys may still be on their way)
-    consumer_sync();
     PROX_TRACE(16);
     unsigned nd = 0;                                       // channels above bin b1 (THRESH: at or above tau_s)
     unsigned b1 = 0, kk = 0, nb1 = 0;
     if (!THRESH) {
-      b1 = kth_in_block<4, true>(sm.hist, (unsigned)k2, sm.wsum, lane, warp, &nd);
+      const unsigned hb[4] = {hv.w, hv.z, hv.y, hv.x};
+      find_kth<4, true>(sm, hb, 2047 - 4 * tid, (unsigned)k2, lane, warp);       // (the keys are on their way meanwhile)
+      b1 = sm.res[0]; nd = sm.res[1]; nb1 = sm.res[2];
       kk = (unsigned)k2 - nd;                              // members of b1 to keep (>= 1)
-      nb1 = sm.hist[b1];
     }
     uint32_t list_u32 = smem_u32(idx16);                   // 2 * D bytes: room for D / 4 members
     uint32_t list_off = 0;                                 // offset in the big buffer when it has to go there
