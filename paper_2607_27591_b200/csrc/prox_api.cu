@@ -49,6 +49,8 @@ struct prox_ffn {
   uint16_t* xn;             // [maxB][D] bf16 FFN input of the layer sub-block form (step-wise path)
   const float* fin_resid;   // while a layer sub-block call is enqueued: the residual stream to add ...
   float* fin_out;           // ... and where the sum goes
+  const uint16_t* norm_w;   // ... and, where the batch Stage 1 forms the norm itself, its weight
+  RmsConst norm_rc;
   int* sel;                 // [maxB][F]
   int* cnt_s;               // [maxB]
   float* hbuf;              // [maxB][F]
@@ -363,6 +365,9 @@ bool batch_path_ok(const prox_ffn* h, int B, bool stage1 = false) {
   return xs_bytes <= lim && red_bytes <= lim && ubits <= lim;
 }
 
+// Stage 1 for several tokens on the tensor cores
+bool batch_umma_ok(const prox_ffn* h) { return h->use_mma && h->pacc && (h->bits == 4 || h->bits == 8); }
+
 prox_status_t launch_union(prox_ffn* h, const int* lists, int stride, const int* cnt, int k, int B, int n,
                            const void* x, int* ulist, int* nu, float* val, cudaStream_t st) {
   const size_t smem = (size_t)(B + 2) * ((n + 31) / 32) * sizeof(unsigned);
@@ -421,7 +426,7 @@ prox_status_t launch_stage1_batch(prox_ffn* h, const void* x, int B, int k1, int
   const int D = h->cfg.d_model, F = h->cfg.d_ff;
   prox_status_t s;
   const int gshift_m = (h->group == D) ? 31 : 7;
-  if (h->use_mma && h->pacc && (h->bits == 4 || h->bits == 8) && F % 64 == 0) {
+  if (batch_umma_ok(h)) {
     // tensor-core path over all inputs (no union list): the tokens' masked inputs as digits, then equal
     // ranges of (tile, 128-input) units per block, then the channel masks
     bool& attr_p = attr_done(kAtBatchS1, h->device);
@@ -432,8 +437,17 @@ prox_status_t launch_stage1_batch(prox_ffn* h, const void* x, int B, int k1, int
     }
     {
       LaunchScope ls(h, kKInput, st);
-      CK(launch_dep(batch_input_mask_kernel, dim3(kBT), dim3(kFusedThreads), (size_t)D * 2, st, static_cast<const uint16_t*>(x), B, D, k1,
-                    h->tokfac, h->xd, h->soffb));
+      const NormIn nin = {h->fin_resid, h->norm_w, h->xn, h->norm_rc};
+      const uint16_t* xp = static_cast<const uint16_t*>(x);
+      if (h->norm_w) {
+        // An ordinary launch: behind the down projection of the layer before, set up early like the others, this kernel
+        // and the proxy GEMM behind it took SMs from that one's last blocks (four layers, four tokens: 391 us against 352).
+        batch_input_mask_kernel<true><<<kBT, kFusedThreads, (size_t)D * 2, st>>>(xp, nin, B, D, k1, h->tokfac, h->xd, h->soffb);
+        CK(cudaGetLastError());
+      } else {
+        CK(launch_dep(batch_input_mask_kernel<false>, dim3(kBT), dim3(kFusedThreads), (size_t)D * 2, st, xp, nin, B, D, k1, h->tokfac,
+                      h->xd, h->soffb));
+      }
     }
     {
       LaunchScope ls(h, kKProxy, st);
@@ -514,6 +528,8 @@ prox_status_t launch_stage2_batch(prox_ffn* h, const void* x, int B, const int* 
   prox_status_t s;
   const size_t mma_smem = stage2_mma_smem(h);
   const bool mma = stage2_mma_ok(h);
+  // layer form in place: y is added straight to the residual stream (Stage 1 of this call has read it)
+  const bool in_place = mma && marked && h->fin_resid && h->fin_resid == h->fin_out;
   const bool rows = mma && D <= 4 * kGrPiece / 2;            // the ring kernel: up to four 4 KB sections of a row
   if (mma) {
     LaunchScope ls(h, kKUnion, st);
@@ -568,7 +584,7 @@ prox_status_t launch_stage2_batch(prox_ffn* h, const void* x, int B, const int* 
     {
       LaunchScope ls(h, kKDown, st);
       CK(launch_dep(down_mma_kernel, dim3(h->sm_count), dim3(kMmaThreads), (size_t)kDnSmem, st,
-                    h->wdt, h->hb, h->u_ch, h->u_cnt + 1, B, D, h->yacc, rows ? reinterpret_cast<uint4*>(h->cmask) : (uint4*)nullptr, F));
+                    h->wdt, h->hb, h->u_ch, h->u_cnt + 1, B, D, in_place ? h->fin_out : h->yacc, rows ? reinterpret_cast<uint4*>(h->cmask) : (uint4*)nullptr, F));
     }
     CK(cudaGetLastError());
   } else {
@@ -594,6 +610,7 @@ prox_status_t launch_stage2_batch(prox_ffn* h, const void* x, int B, const int* 
   }
   CK(cudaGetLastError());
   }
+  if (in_place) return PROX_OK;
   const int n = B * D;
   {
     LaunchScope ls(h, kKFinalize, st);
@@ -736,7 +753,7 @@ prox_status_t launch_fused(prox_ffn* h, const FusedPlan& pl, const void* x, int 
   prm.exits = reinterpret_cast<unsigned long long*>(h->syncbuf + 4096); prm.ctr = h->syncbuf + 4104;
   prm.nshare = h->sm_count; prm.nshare1 = pl.nshare1;
   prm.status = h->dev_status;
-  prm.big_bytes = pl.big_bytes; prm.nslots = pl.nslots;
+  prm.big_bytes = pl.big_bytes; prm.nslots = pl.nslots; prm.nslots_rcp = (unsigned)((1ull << 32) / (unsigned)pl.nslots + 1ull);
   prm.trace = h->trace;
   prm.xres = xres; prm.norm_w = norm_w; prm.rc = rms_const(h->cfg.d_model, eps); prm.xres_out = xres_out;
   if (taus) {
@@ -1039,12 +1056,17 @@ prox_status_t prox_ffn_block_forward(prox_ffn_t* h, const float* x_res, const vo
                           static_cast<const uint16_t*>(norm_w), eps, x_res_out);
     }
   }
-  rmsnorm_kernel<<<B, 256, 0, st>>>(x_res, static_cast<const uint16_t*>(norm_w), rms_const(D, eps), D, h->xn);
-  h->launches++;
-  CK(cudaGetLastError());
+  if (h->use_union && batch_path_ok(h, B, true) && batch_umma_ok(h)) {
+    h->norm_w = static_cast<const uint16_t*>(norm_w);      // the kernel that masks the inputs forms the norm
+    h->norm_rc = rms_const(D, eps);
+  } else {
+    rmsnorm_kernel<<<B, 256, 0, st>>>(x_res, static_cast<const uint16_t*>(norm_w), rms_const(D, eps), D, h->xn);
+    h->launches++;
+    CK(cudaGetLastError());
+  }
   h->fin_resid = x_res; h->fin_out = x_res_out;          // the last kernel adds the residual stream
   s = forward_kernels(h, h->xn, B, k1, k2, nullptr, st);
-  h->fin_resid = nullptr; h->fin_out = nullptr;
+  h->fin_resid = nullptr; h->fin_out = nullptr; h->norm_w = nullptr;
   return s;
 }
 

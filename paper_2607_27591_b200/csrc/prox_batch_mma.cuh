@@ -546,9 +546,14 @@ namespace prox {
 //   soff  [u][b] sum of X over the 128 inputs of unit u;  tokfac[b] = 2^24 / s undoes the scaling (and the codes' 2^-24)
 // With eight tokens the union of the kept inputs is nearly everything, so the proxy GEMM runs over all rows and needs
 // no union list; a dropped input contributes 0 * code.  Token slots beyond B are cleared.
+// NORM (layer sub-block form): x is bf16(RMSNorm(xres) * norm_w), formed here and written to xn for Stage 2 (a kernel of
+// its own in front of this one took 6.6 us).
 // ----------------------------------------------------------------------------
+struct NormIn { const float* xres; const uint16_t* w; uint16_t* xn; RmsConst rc; };
+
+template <bool NORM>
 __global__ void __launch_bounds__(kFusedThreads)
-batch_input_mask_kernel(const uint16_t* __restrict__ x, int B, int D, int k1, float* __restrict__ tokfac,
+batch_input_mask_kernel(const uint16_t* __restrict__ x, NormIn nin, int B, int D, int k1, float* __restrict__ tokfac,
                         uint32_t* __restrict__ xd, float* __restrict__ soff) {
   extern __shared__ __align__(16) uint8_t bm_smem[];
   uint16_t* xs = reinterpret_cast<uint16_t*>(bm_smem);           // [D] bf16 bits of the token
@@ -568,12 +573,48 @@ batch_input_mask_kernel(const uint16_t* __restrict__ x, int B, int D, int k1, fl
   for (int i = tid; i < 1024 + 32; i += NT) { if (i < 1024) hist[i] = 0; else hist2[i - 1024] = 0; }
   __syncthreads();
   unsigned m = 0;
-  for (int i = tid; i < D / 8; i += NT) {
-    const uint4 v = __ldg(reinterpret_cast<const uint4*>(x + (size_t)b * D) + i);
-    reinterpret_cast<uint4*>(xs)[i] = v;
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  if (NORM) {
+    // the correctly rounded value (the masks depend on it): sum of squares and 1 / rms as pairs of floats
+    __shared__ float nsum[kFusedWarps][2], ninv[2];
+    const float4* x4 = reinterpret_cast<const float4*>(nin.xres + (size_t)b * D);
+    const uint2* w2 = reinterpret_cast<const uint2*>(nin.w);
+    float hi = 0.f, lo = 0.f;
+    for (int i0 = tid; i0 < D / 4; i0 += 4 * NT) {
+      float4 v[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) m = max(m, max(w[e] & 0x7fffu, (w[e] >> 16) & 0x7fffu));
+      for (int r = 0; r < 4; ++r) v[r] = i0 + r * NT < D / 4 ? __ldcg(x4 + i0 + r * NT) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int r = 0; r < 4; ++r) { f2_add_square(hi, lo, v[r].x); f2_add_square(hi, lo, v[r].y); f2_add_square(hi, lo, v[r].z); f2_add_square(hi, lo, v[r].w); }
+    }
+    f2_warp_sum(hi, lo);
+    if (lane == 0) { nsum[warp][0] = hi; nsum[warp][1] = lo; }
+    __syncthreads();
+    if (warp == 0) {
+      hi = lane < kFusedWarps ? nsum[lane][0] : 0.f;
+      lo = lane < kFusedWarps ? nsum[lane][1] : 0.f;
+      f2_warp_sum(hi, lo);
+      if (lane == 0) rms_inverse(hi, lo, nin.rc, ninv[0], ninv[1]);
+    }
+    __syncthreads();
+    const float ih = ninv[0], il = ninv[1];
+    for (int i = tid; i < D / 4; i += NT) {
+      const float4 v = __ldcg(x4 + i);
+      const uint2 w = __ldg(w2 + i);
+      const uint32_t a = rms_scale_to_bf16(v.x, bf16_lo(w.x), ih, il), c = rms_scale_to_bf16(v.y, bf16_hi(w.x), ih, il);
+      const uint32_t d = rms_scale_to_bf16(v.z, bf16_lo(w.y), ih, il), e = rms_scale_to_bf16(v.w, bf16_hi(w.y), ih, il);
+      const uint2 o = make_uint2(a | (c << 16), d | (e << 16));
+      reinterpret_cast<uint2*>(xs)[i] = o;
+      reinterpret_cast<uint2*>(nin.xn + (size_t)b * D)[i] = o;
+      m = max(m, max(max(a & 0x7fffu, c & 0x7fffu), max(d & 0x7fffu, e & 0x7fffu)));
+    }
+  } else {
+    for (int i = tid; i < D / 8; i += NT) {
+      const uint4 v = __ldg(reinterpret_cast<const uint4*>(x + (size_t)b * D) + i);
+      reinterpret_cast<uint4*>(xs)[i] = v;
+      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) m = max(m, max(w[e] & 0x7fffu, (w[e] >> 16) & 0x7fffu));
+    }
   }
   m = __reduce_max_sync(0xffffffffu, m);
   if (lane == 0 && m) atomicMax(&smax, m);

@@ -80,6 +80,7 @@ struct FusedParams {
   int nshare1, nshare;        // shares of Stage 1 and of Stage 2
   int big_bytes;      // bytes of the large shared buffer
   int nslots;         // ring slots of D*2 bytes inside it
+  unsigned nslots_rcp;   // ceil(2^32 / nslots): __umulhi(q, it) = q / nslots for q < 2^27
   unsigned long long* trace;   // optional [grid][32] phase time stamps (ns), NULL = off
   // Layer sub-block form (all NULL / 0 otherwise): the input is bf16(RMSNorm(xres) * norm_w) and the
   // result is xres + y, written as fp32 to xres_out (which may be xres itself).
@@ -1416,8 +1417,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
         c = __shfl_sync(0xffffffffu, c, 0);
         if (c >= nb) break;
         const unsigned sq = base_seq + 2u * (unsigned)c;
-        const int sg = (int)(sq % (unsigned)NS), su = (int)((sq + 1u) % (unsigned)NS);
-        const unsigned ug = sq / (unsigned)NS, uu = (sq + 1u) / (unsigned)NS;
+        const unsigned ug = __umulhi(sq, p.nslots_rcp);
+        const int sg = (int)(sq - ug * (unsigned)NS), su = sg + 1 == NS ? 0 : sg + 1;
+        const unsigned uu = ug + (su == 0 ? 1u : 0u);
         const bool ok1 = slot_wait(smem_u32(&sm.mbar_full[sg]), &sm.slot_use[sg], ug, abortp, spin);
         const bool ok2 = slot_wait(smem_u32(&sm.mbar_full[su]), &sm.slot_use[su], uu, abortp, spin);
         float ag = 0.f, au = 0.f, ag2 = 0.f, au2 = 0.f;
@@ -1456,8 +1458,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
         const int gq = tid / TG, tg = tid % TG;
         for (int c = gq; c < nb; c += NG) {
           const unsigned sq = base_seq + 2u * (unsigned)nb + (unsigned)c;
-          const int sd = (int)(sq % (unsigned)NS);
-          const unsigned ud = sq / (unsigned)NS;
+          const unsigned ud = __umulhi(sq, p.nslots_rcp);
+          const int sd = (int)(sq - ud * (unsigned)NS);
           const bool ok = slot_wait(smem_u32(&sm.mbar_full[sd]), &sm.slot_use[sd], ud, abortp, spin);
           if (ok) {
             const float hv = sm.hval[c];
