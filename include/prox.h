@@ -145,8 +145,8 @@ prox_status_t prox_ffn_set_mask_policy(prox_ffn_t* h, int policy);
  * weights are read once per call for the UNION of the tokens' kept inputs and of
  * their kept channels; a token contributes zero outside its own masks, so its
  * result is the one it would get alone.  With the union, the exact Stage 2
- * runs as warp-level bf16 tensor-core tiles (16 channels x 8 tokens x 16 inputs)
- * with fp32 accumulation; in the down projection h enters as a bf16 pair
+ * runs as warp-level bf16 tensor-core tiles (8 channels x (gate, up) x 8 tokens x
+ * 16 inputs; 16 channels for d_model > 8192) with fp32 accumulation; in the down projection h enters as a bf16 pair
  * hi + lo.  prox_ffn_set_union(h, 1) keeps the union but computes with plain fp32
  * FMAs, prox_ffn_set_union(h, 0) selects the older path that runs the
  * single-token kernels once per token; any other value (the default) selects the
@@ -154,8 +154,8 @@ prox_status_t prox_ffn_set_mask_policy(prox_ffn_t* h, int policy);
 prox_status_t prox_ffn_set_union(prox_ffn_t* h, int on);
 
 /* Launch plan of the persistent kernel for budgets (k1, k2), for diagnostics:
- * info[8] (host) = {usable, grid blocks, row split, dynamic shared bytes, ring
- * slots, registers per thread, static shared bytes, co-resident blocks per SM}. */
+ * info[8] (host) = {usable, grid blocks, loader warps of the proxy GEMV,
+ * dynamic shared bytes, ring slots, registers per thread, static shared bytes, co-resident blocks per SM}. */
 prox_status_t prox_fused_kernel_info(prox_ffn_t* h, int k1, int k2, int32_t* info_host);
 
 /* Debug aid: with on != 0 every block of the persistent kernel records time

@@ -624,7 +624,7 @@ prox_status_t launch_stage2_batch(prox_ffn* h, const void* x, int B, const int* 
 // ---- fused persistent kernel (batch 1) ----------------------------------------
 struct FusedPlan {
   bool ok;
-  int grid, loaders, cgran, nshare1, big_bytes, nslots, xch;
+  int grid, loaders, plines, pleft0, ppart, pmore, cgran, nshare1, big_bytes, nslots, xch;
   size_t smem;
   int device;           // the handle's GPU
   int optin;            // the device's opt-in limit: what the kernels' dynamic shared memory attribute is set to
@@ -648,14 +648,19 @@ FusedPlan plan_fused(const prox_ffn* h, int k1, int k2, bool thresh = false, int
   pl.loaders = (int)((4 * (size_t)D + pl.big_bytes - 1024 - 3072) / proxy_warp_bytes(h->bits));
   if (pl.loaders > kFusedConsumerWarps) pl.loaders = kFusedConsumerWarps;
   if (pl.loaders < kMinLoaders && mode != kGivenList) return pl;
-  // Columns of the packed rows per block: whole 128-byte tiles (8 chunks) while there is at most one per SM: narrower
-  // shares on all SMs took as long or longer (4096 x 12288: 8.0 us either way with 96 tiles; 1024 x 3072: 3.5 against
-  // 4.1 us, more blocks add to the same few histogram bins).  Beyond that equal shares in 32-byte sectors: 224 tiles
-  // on 148 SMs took two rounds (4096 x 14336, 8 bits: 38 us against 30).
+  // Columns of the packed rows per block: whole 128-byte lines (8 chunks); narrower shares on all SMs where there is less
+  // than one line per SM took as long or longer (4096 x 12288: 8.0 us either way with 96 lines; 1024 x 3072: 3.5 against
+  // 4.1 us, more blocks add to the same few histogram bins).  The lines that do not go round are dealt out in halves if
+  // that gives about one to a block, otherwise whole (224 lines on 148 SMs, 8 bits: 125.2 us for two calls with halves,
+  // 126.9 with whole lines, 143.5 with all 224 cut into equal shares of 32-byte sectors).
   const int nchunks = F / ch_per_chunk(h->bits);
-  pl.cgran = nchunks <= 8 * G ? 8 : 2;                   // (nchunks is a multiple of 4: d_ff is one of 64)
-  const int nunit = (nchunks + pl.cgran - 1) / pl.cgran;
-  pl.nshare1 = nunit < G ? nunit : G;
+  pl.nshare1 = std::min(G, (nchunks + 7) / 8);           // (nchunks is a multiple of 4: d_ff is one of 64)
+  pl.plines = nchunks / 8 / pl.nshare1;
+  pl.pleft0 = pl.plines * pl.nshare1 * 8;
+  pl.cgran = pl.plines == 0 || nchunks - pl.pleft0 > 5 * pl.nshare1 ? 8 : 4;
+  const int nunit = (nchunks - pl.pleft0 + pl.cgran - 1) / pl.cgran;
+  pl.ppart = nunit / pl.nshare1 * pl.cgran;
+  pl.pmore = nunit % pl.nshare1;
   pl.xch = D <= 4096 ? 4 : (D <= 8192 ? 2 : 1);          // warp groups of the down projection
   if (pl.big_bytes < pl.xch * D * 4) return pl;          // their partial y vectors
   if ((k2 + G - 1) / G + 2 > kMySelCap) return pl;       // a block's share: definite part + part of the threshold bin
@@ -746,7 +751,8 @@ prox_status_t launch_fused(prox_ffn* h, const FusedPlan& pl, const void* x, int 
   prm.D = h->cfg.d_model; prm.F = h->cfg.d_ff; prm.k1 = k1; prm.k2 = k2;
   prm.gshift = (h->group == h->cfg.d_model) ? 31 : 7;
   prm.out_fp32 = h->cfg.out_dtype;
-  prm.loaders = pl.loaders > 0 ? pl.loaders : 1; prm.cgran = pl.cgran;
+  prm.loaders = pl.loaders > 0 ? pl.loaders : 1;
+  prm.plines = pl.plines; prm.pleft0 = pl.pleft0; prm.ppart = pl.ppart; prm.pmore = pl.pmore; prm.cgran = pl.cgran;
   prm.scores = scores ? scores : h->scores; prm.ghist = h->syncbuf; prm.idx_out = h->idx_x;
   prm.spin_limit = h->spin_limit; prm.bar_bias = h->bar_bias; prm.host_flag = h->host_flag_dev;
   prm.sel_out = sel_out; prm.yacc = h->yacc;

@@ -68,7 +68,9 @@ struct FusedParams {
   const uint16_t* x; void* y;
   int D, F, k1, k2, gshift, out_fp32;
   int loaders;        // loader warps of the proxy GEMV whose stages fit
-  int cgran;          // the proxy rows' 16-byte column chunks are dealt out in units of this many
+  // a share of Stage 1: plines whole 128-byte lines of the proxy rows, and of the chunks from pleft0 on an equal part:
+  // ppart, in the first pmore shares cgran more
+  int plines, pleft0, ppart, pmore, cgran;
   float* scores; unsigned* ghist; int* sel_out;
   int* idx_out;       // the kept input list as this kernel built it (block 0 writes it; for checking)
   unsigned spin_limit;        // polls after which a device-side wait gives up
@@ -606,8 +608,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   PROX_TRACE(2);
   // --------------------------------------- B: proxy GEMV (tensor cores), scores, score histogram
   // Per scale group g:  sum_k x_k q_kj = 2^(ebase-134) * sum_k X_k (byte_kj - offset), X_k the integer
-  // form of x_k (x_digits).  A block owns a share of the packed rows' 16-byte column chunks (dealt out in units of
-  // p.cgran) over all kept rows, in tiles of at most 8 chunks.  The kept
+  // form of x_k (x_digits).  A block owns a share of the packed rows' 16-byte column chunks over all kept rows: whole
+  // 128-byte lines, and half a line or a line of what is left over; a tile is a line or half of one.  The kept
   // rows are cut into blocks of at most 32 rows that stay inside one supergroup (4 scale groups); block b
   // accumulates into 16 tensor-memory columns of its supergroup: column 4 * (g % 4) + d holds digit d of
   // group g.  The loader warps bring the rows in with 16-byte asynchronous copies, a block ahead (what bounds this is
@@ -615,19 +617,21 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   // the bytes with the high nibble masked off and the digits of x, and
   // issue the block's MMAs; after the last one the 16 warps read the accumulators, apply the
   // groups' scales and form the scores.
-  // Measured (this phase, one call): 4096 x 14336 8-bit, all rows: 42.9 -> 33 us (59 MB of copies: 3.6 TB/s); 8192 x 28672
-  // 4-bit, 2458 rows: 24 us, where that shape did not fit and a kernel of its own took 46; 4096 x 12288 4-bit, 1229 rows:
-  // 8 us as before (the first rows arrive 3 us after phase A, the last 2.5 us later).
+  // Measured (this phase, one call): 4096 x 14336 8-bit, all rows: 30 us, the lines of the first pass at 6.7 TB/s, the half
+  // lines of the second at 3.5 (42.9 at first; 38 with shares of six 32-byte sectors, cut without regard to the lines: a
+  // segment over two lines costs two requests, and 155 MB of whole lines took less time than 116 MB of those shares);
+  // 8192 x 28672 4-bit, 2458 rows: 24 us; 4096 x 12288 4-bit, 1229 rows: 8 us (the first rows arrive 3 us after phase A,
+  // the last 2.5 us later).
   unsigned uses = 0, acc_n = 0;              // blocks of rows this warp has handed to the tensor core; tiles read back
 #pragma unroll 1
   for (bool first = true;; first = false) {
     constexpr bool LO = (BITS == 4);
     const int nchunks = F / CH;
     const int row_bytes = nchunks * 16;
-    const unsigned nunit = (unsigned)((nchunks + p.cgran - 1) / p.cgran), vid = sm.vid, n1 = (unsigned)p.nshare1;
-    const int ck0 = vid < n1 ? p.cgran * (int)((nunit * vid) / n1) : 0;                      // this block's chunks
-    const int ckn = vid < n1 ? min(nchunks, p.cgran * (int)((nunit * (vid + 1u)) / n1)) - ck0 : 0;
-    const int ntl = (ckn + 7) >> 3;
+    const unsigned vid = sm.vid, n1 = (unsigned)p.nshare1;
+    const int lk0 = p.pleft0 + (int)vid * p.ppart + min((int)vid, p.pmore) * p.cgran;       // this block's part of the rest
+    const int lk1 = min(nchunks, lk0 + p.ppart + ((int)vid < p.pmore ? p.cgran : 0));
+    const int ntl = vid >= n1 ? 0 : p.plines + (lk1 > lk0 ? ((lk1 + 7) >> 3) - (lk0 >> 3) : 0);
     const bool per_row = p.gshift >= 31;
     const int ng = per_row ? 1 : (D >> p.gshift);
     const int nsuper = (ng + 3) >> 2;
@@ -659,13 +663,14 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       const int nblk = __shfl_sync(0xffffffffu, sg_end, 31);
 #pragma unroll 1
       for (int tl = 0; tl < ntl; ++tl) {
-        const int tc0 = tl * 8, w = min(8, ckn - tc0);         // the tile's chunks (of the block's)
-        // a copy instruction covers 32 >> sc rows of up to 1 << sc chunks
-        const int sc = w > 4 ? 3 : (w > 2 ? 2 : 1), rpi = 32 >> sc;
+        const int ln = (tl < p.plines ? (int)vid * p.plines : (lk0 >> 3) - p.plines) + tl;    // the tile's line
+        const int tc0 = tl < p.plines ? ln * 8 : max(lk0, ln * 8);                            // and its chunks
+        const int w = (tl < p.plines ? ln * 8 + 8 : min(lk1, ln * 8 + 8)) - tc0;
+        // (8 or 4 of them)  a copy instruction covers 32 >> sc rows of 1 << sc chunks
+        const int sc = w > 4 ? 3 : 2, rpi = 32 >> sc;
         const int kq = lane >> sc, c = lane & ((1 << sc) - 1);
-        const bool lane_on = c < w;
-        const uint8_t* tp = p.P + (size_t)(ck0 + tc0) * 16 + (size_t)c * 16;
-        const int chunk = ck0 + tc0 + (col >> 4);              // chunk of this thread's byte column
+        const uint8_t* tp = p.P + (size_t)tc0 * 16 + (size_t)c * 16;
+        const int chunk = tc0 + (col >> 4);                    // chunk of this thread's byte column
         const bool col_ok = (col >> 4) < w;
         bool alive_b = true;
         // The copies of a warp's block k are on their way while its block k - 1 goes to the tensor core.
@@ -691,7 +696,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
               const int kk = j * rpi + kq;
-              if (lane_on && kk < nrows)
+              if (kk < nrows)
                 cp_async16(stg + (uint32_t)((k & 1) * 4096 + (kk >> 3) * 1024 + (kk & 7) * 128 + ((c ^ (kk & 7)) << 4)),
                            tp + (size_t)idx16[r0 + kk] * (size_t)row_bytes);
             }
@@ -856,7 +861,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     }
     tc_fence_before();
     __syncthreads();
-    if (ckn > 0) {
+    if (ntl > 0) {
       // one atomic per occupied bin and block (thousands of single increments on a few hot bins serialise in L2)
 #pragma unroll 1
       for (int i = tid; i < 2048; i += NT) { const unsigned v = sm.hist[i]; if (v) atomicAdd(ghist + i, v); }

@@ -8,6 +8,7 @@ import __graft_entry__ as entry
 from oracle import prox_oracle as po
 from paper_2607_27591_b200 import inputs
 from tests.gpu_common import Problem, dev_bf16
+from tests.test_gpu_parity import _check_fused_stage1
 
 pytestmark = pytest.mark.gpu
 
@@ -61,8 +62,8 @@ def test_packer_tiles_ties_and_repacking(pb, D, F, bits, group):
 @pytest.mark.parametrize("grid", [1, 7, 100])
 def test_persistent_kernel_with_part_of_its_grid(pb, D, F, bits, group, grid):
     """Blocks that do not run are replaced by those that do: the same masks and results with a part of the grid, in the
-    plain, the threshold and the layer form in place (19136 channels: shares in 32-byte sectors, two tiles of columns
-    each)."""
+    plain, the threshold and the layer form in place (19136 channels: a line and sometimes half a line of the proxy
+    rows each)."""
     k1, k2 = D // 3, F // 4 + 1
     wg, wu, wd, x = inputs.make_small(D, F, 1, seed=D + F + bits)
     p = Problem(pb, wg, wu, wd, x)
@@ -106,7 +107,21 @@ def test_persistent_kernel_with_part_of_its_grid(pb, D, F, bits, group, grid):
         p.close()
 
 
-@pytest.mark.parametrize("F", [64, 192, 4160, 65536])
+@pytest.mark.parametrize("F,bits", [(9536, 4), (19008, 4), (28672, 4), (38016, 4), (9472, 8), (9536, 8), (14336, 8), (15872, 8)])
+def test_shares_of_the_proxy_columns(pb, F, bits):
+    """Proxy scores with less than a 128-byte line of the packed rows per SM, with one or two lines and halves or wholes of
+    the lines left over, with a last line that is half a line, against the oracle."""
+    p = Problem(pb, *inputs.make_small(256, F, 2, seed=F + bits))
+    try:
+        p.quantize(bits, 128)
+        for t, k1 in ((0, 85), (1, 256)):
+            _check_fused_stage1(pb, p, p.t_x[t], p.x[t], k1, F // 4)
+        assert pb.prox_last_device_status(p.h) == 0
+    finally:
+        p.close()
+
+
+@pytest.mark.parametrize("F", [64, 192, 2048, 4160, 65536])
 @pytest.mark.parametrize("B,shared", [(1, False), (3, False), (8, True)])
 def test_channel_mask_is_the_exact_topk_of_the_scores(pb, F, B, shared):
     """Few and many channels per block of a cluster, ties (repeated channels: equal scores), every k at the ends; the
@@ -136,6 +151,9 @@ def test_channel_mask_is_the_exact_topk_of_the_scores(pb, F, B, shared):
                     rank = rank.expand(B, F)
                 order = torch.sort(rank, dim=1, descending=True, stable=True).indices[:, :k2]
                 assert torch.equal(sel.long(), order.sort(dim=1).values), (k2, off)
+            # nothing but ties: the first k2 channels
+            pb.prox_stage1_mask(h, torch.zeros_like(x), B, 50, k2, sel, sc)
+            assert torch.equal(sel, torch.arange(k2, dtype=torch.int32, device="cuda").expand(B, k2))
         assert pb.prox_last_device_status(h) == 0
     finally:
         pb.prox_ffn_destroy(h)
