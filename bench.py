@@ -588,6 +588,8 @@ def run_prox(args):
 
             levels = (0.0, 0.10, 0.55, 0.70)
             res = {}
+            for h in handles:
+                pb.prox_ffn_set_fused(h, 0)                      # Stage 1 of integer proxies by the step-wise kernel too
             for fmt in (PROXY, (16, 0)):
                 for h in handles:
                     pb.prox_quantize_proxy(h, *fmt)
@@ -600,6 +602,7 @@ def run_prox(args):
                                          "stage1_us_one_row": base_whole}
             for h in handles:
                 pb.prox_quantize_proxy(h, *PROXY)
+                pb.prox_ffn_set_fused(h, 1)
             torch.cuda.synchronize()
             alpha = {"proxy": f"int{PROXY[0]} group-{PROXY[1]}", "against": "bf16 input-major rows, same kernel template",
                      "levels": []}
