@@ -68,7 +68,6 @@ channel_topk_kernel(const float* __restrict__ scores, float* __restrict__ pacc, 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = blockIdx.x / kTkBlocks, rank = blockIdx.x % kTkBlocks;
   const int nq = F / 4, q0 = (int)((long long)nq * rank / kTkBlocks), n = (int)((long long)nq * (rank + 1) / kTkBlocks) - q0;
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   for (int i = tid; i < 1024; i += NT) reinterpret_cast<uint4*>(hist)[i] = make_uint4(0u, 0u, 0u, 0u);
   asm volatile("griddepcontrol.wait;" ::: "memory");
   __syncthreads();
@@ -104,6 +103,9 @@ channel_topk_kernel(const float* __restrict__ scores, float* __restrict__ pacc, 
     skey[i] = k;
     atomicAdd(&hist[k.x >> 20], 1u); atomicAdd(&hist[k.y >> 20], 1u); atomicAdd(&hist[k.z >> 20], 1u); atomicAdd(&hist[k.w >> 20], 1u);
   }
+  // Only now: blocks of the next kernel that start earlier take issue slots from the histograms (one mask for eight
+  // tokens, two calls: 146.4 -> 145.1 us; stages one by one, two layers: 91.8 -> 90.8; the other batch cases equal).
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   cl.sync();
   unsigned prefix, kleft = (unsigned)k2;
   {
