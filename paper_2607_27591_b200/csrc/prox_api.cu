@@ -440,10 +440,8 @@ prox_status_t launch_stage1_batch(prox_ffn* h, const void* x, int B, int k1, int
       const NormIn nin = {h->fin_resid, h->norm_w, h->xn, h->norm_rc};
       const uint16_t* xp = static_cast<const uint16_t*>(x);
       if (h->norm_w) {
-        // An ordinary launch: behind the down projection of the layer before, set up early like the others, this kernel
-        // and the proxy GEMM behind it took SMs from that one's last blocks (four layers, four tokens: 391 us against 352).
-        batch_input_mask_kernel<true><<<kBT, kFusedThreads, (size_t)D * 2, st>>>(xp, nin, B, D, k1, h->tokfac, h->xd, h->soffb);
-        CK(cudaGetLastError());
+        CK(launch_dep(batch_input_mask_kernel<true>, dim3(kBT), dim3(kFusedThreads), (size_t)D * 2, st, xp, nin, B, D, k1, h->tokfac,
+                      h->xd, h->soffb));
       } else {
         CK(launch_dep(batch_input_mask_kernel<false>, dim3(kBT), dim3(kFusedThreads), (size_t)D * 2, st, xp, nin, B, D, k1, h->tokfac,
                       h->xd, h->soffb));
@@ -528,8 +526,6 @@ prox_status_t launch_stage2_batch(prox_ffn* h, const void* x, int B, const int* 
   prox_status_t s;
   const size_t mma_smem = stage2_mma_smem(h);
   const bool mma = stage2_mma_ok(h);
-  // layer form in place: y is added straight to the residual stream (Stage 1 of this call has read it)
-  const bool in_place = mma && marked && h->fin_resid && h->fin_resid == h->fin_out;
   const bool rows = mma && D <= 4 * kGrPiece / 2;            // the ring kernel: up to four 4 KB sections of a row
   if (mma) {
     LaunchScope ls(h, kKUnion, st);
@@ -584,7 +580,7 @@ prox_status_t launch_stage2_batch(prox_ffn* h, const void* x, int B, const int* 
     {
       LaunchScope ls(h, kKDown, st);
       CK(launch_dep(down_mma_kernel, dim3(h->sm_count), dim3(kMmaThreads), (size_t)kDnSmem, st,
-                    h->wdt, h->hb, h->u_ch, h->u_cnt + 1, B, D, in_place ? h->fin_out : h->yacc, rows ? reinterpret_cast<uint4*>(h->cmask) : (uint4*)nullptr, F));
+                    h->wdt, h->hb, h->u_ch, h->u_cnt + 1, B, D, h->yacc, rows ? reinterpret_cast<uint4*>(h->cmask) : (uint4*)nullptr, F));
     }
     CK(cudaGetLastError());
   } else {
@@ -610,7 +606,9 @@ prox_status_t launch_stage2_batch(prox_ffn* h, const void* x, int B, const int* 
   }
   CK(cudaGetLastError());
   }
-  if (in_place) return PROX_OK;
+  // Layer form: the residual stream is added here, once per element, in place as well.  (The down projection's partial sums
+  // added straight to it were rounded at the stream's magnitude one by one: relative error 2.4e-8 -> 4.3e-8 at 4096
+  // columns, 9.5e-8 at 256, with a stream a thousand times y, for 1 us less per layer of 90.)
   const int n = B * D;
   {
     LaunchScope ls(h, kKFinalize, st);

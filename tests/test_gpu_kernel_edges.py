@@ -215,3 +215,32 @@ def test_stages_one_by_one(pb, D, F, bits, group):
         assert float((y - y1).norm()) <= 1e-5 * float(y.norm())
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("D,F,B", [(128, 512, 2), (256, 768, 8), (1024, 3072, 5), (4224, 1472, 3), (9216, 320, 8)])
+def test_batch_layer_form_rounds_the_residual_stream_once(pb, D, F, B):
+    """x_res + y with one rounding to fp32 per element, in place or not, few or many blocks per column tile: a residual
+    stream a thousand times y, against the y that the plain call gives for the same normalised input."""
+    wg, wu, wd, x = inputs.make_small(D, F, B, seed=D + F)
+    p = Problem(pb, wg, wu, wd, x, max_batch=B)
+    try:
+        pb.prox_quantize_proxy(p.h, 4, 128)
+        k1, k2 = D // 2, F // 2
+        nw = torch.ones(D, dtype=torch.bfloat16, device="cuda")
+        xr = (p.t_x[:B].float() * 1e3 + 1.0).contiguous()
+        xn = torch.empty(B, D, dtype=torch.bfloat16, device="cuda")
+        pb.prox_rmsnorm(p.h, xr, nw, 1e-6, B, xn)
+        y, out = p.y_empty(B), torch.empty_like(xr)
+        pb.prox_ffn_forward(p.h, xn, B, k1, k2, y)
+        for again in range(2):                                     # the accumulator is back at zero
+            pb.prox_ffn_block_forward(p.h, xr, nw, 1e-6, B, k1, k2, out)
+            inplace = xr.clone()
+            pb.prox_ffn_block_forward(p.h, inplace, nw, 1e-6, B, k1, k2, inplace)
+            exact = xr.double().cpu().numpy() + y.double().cpu().numpy()
+            # half a unit in the last place, and what two orders of y's fp32 sums differ by
+            bound = 0.5 * np.spacing(np.abs(exact).astype(np.float32)).astype(np.float64) + 1e-5 * float(y.double().pow(2).mean().sqrt())
+            for got in (out, inplace):
+                assert np.all(np.abs(got.double().cpu().numpy() - exact) <= bound)
+        assert pb.prox_last_device_status(p.h) == 0
+    finally:
+        p.close()
