@@ -185,7 +185,8 @@ prox_status_t prox_ffn_last_stage1(prox_ffn_t* h, int k1, int32_t* idx_dev_or_nu
 prox_status_t prox_debug_set_wait(prox_ffn_t* h, uint32_t spin_limit, uint32_t barrier_bias);
 
 /* Test hook: blocks the persistent kernel is launched with (0 = one per SM, at most that).  With fewer, the blocks
- * that run take over the work of the others, as they would if the rest of the grid had to wait for an SM. */
+ * that run take over the work of the others, as they would if the rest of the grid had to wait for an SM.  The gate/up
+ * kernel of the batch path (d_model <= 8192) takes the same number, as on a GPU with that many SMs. */
 prox_status_t prox_debug_set_grid(prox_ffn_t* h, int blocks);
 
 /* Copy the channel mask of the most recent prox_ffn_forward call (top-k rule)

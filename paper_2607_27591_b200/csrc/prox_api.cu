@@ -60,7 +60,7 @@ struct prox_ffn {
   unsigned* syncbuf;        // fused kernel: [0..4095] two score histograms (calls alternate), [4096..4097] 64-bit count
                             // of blocks that have left, [4104..4119] two sets of share counters
   int smem_optin;           // largest dynamic shared memory a block may ask for
-  int debug_grid;           // test knob: blocks of the persistent kernel (0 = one per SM)
+  int debug_grid;           // test knob: blocks of the persistent kernel and of the batch gate/up ring kernel (0 = one per SM)
   int sel_unordered;        // the last forward left its mask in the persistent kernel's own order
   int use_fused;            // batch-1 forward runs as one persistent kernel
   int use_union;            // batch > 1 reads weights once for the union of the tokens' masks
@@ -567,7 +567,9 @@ prox_status_t launch_stage2_batch(prox_ffn* h, const void* x, int B, const int* 
           CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin - 8192));
           attr_r = true;
         }
-        CK(launch_dep(kern, dim3(h->sm_count), dim3(kGrThreads), (size_t)ring_slots * row_pitch + red_bytes, st,
+        // One block per SM, but as many as it takes for a block's share of the union to fit (65536 channels: 128 blocks).
+        const int blocks = std::max(h->debug_grid ? h->debug_grid : h->sm_count, (F + kGrMaxShare - 1) / kGrMaxShare);
+        CK(launch_dep(kern, dim3(blocks), dim3(kGrThreads), (size_t)ring_slots * row_pitch + red_bytes, st,
                       h->wg, h->wu, static_cast<const uint16_t*>(x), B, reinterpret_cast<const uint4*>(h->cmask), F, D, ring_slots, h->hb,
                       h->u_ch, h->u_cnt + 1, h->dev_status));
       } else {
@@ -634,6 +636,7 @@ FusedPlan plan_fused(const prox_ffn* h, int k1, int k2, bool thresh = false, int
   const int D = h->cfg.d_model, F = h->cfg.d_ff;
   if (!h->use_fused || (h->bits == 16 && mode != kGivenList)) return pl;       // phase B reads integer proxies
   const int G = h->sm_count;
+  if (G > 256) return pl;                                // `exits` grows by 256 per call, with up to 256 blocks
   const size_t fixed = ((sizeof(FusedSmem) + 127) & ~size_t(127)) + (size_t)8 * D;   // + x bf16, idx, x fp32
   if ((size_t)h->smem_optin < fixed + (size_t)6 * D) return pl;
   pl.big_bytes = (int)(((size_t)h->smem_optin - fixed) & ~size_t(127));

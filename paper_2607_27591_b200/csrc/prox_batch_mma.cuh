@@ -194,7 +194,7 @@ union_compact_kernel(unsigned* __restrict__ mask32, int n, int* __restrict__ uli
 // ----------------------------------------------------------------------------
 constexpr int kGrThreads = kMmaThreads + 32;        // 16 consumer warps + one producer warp
 constexpr int kGrMaxSlots = 128;
-constexpr int kGrMaxShare = 512;                    // union channels of a block
+constexpr int kGrMaxShare = 512;                    // union channels of a block (64 tiles): the grid has d_ff / 512 blocks at least
 constexpr int kGrPiece = 4096;                      // bytes of a row in one ring slot (a whole row if it is shorter)
 
 // bit 7 of every byte that is not zero

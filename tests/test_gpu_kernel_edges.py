@@ -244,3 +244,30 @@ def test_batch_layer_form_rounds_the_residual_stream_once(pb, D, F, B):
         assert pb.prox_last_device_status(p.h) == 0
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("D,F", [(128, 12288), (640, 3136), (128, 65536)])
+@pytest.mark.parametrize("grid", [1, 18, 56])
+def test_batch_gateup_on_fewer_sms(pb, D, F, grid):
+    """A block's share of the union is bounded whatever the number of SMs: every channel in the union, fewer blocks than
+    a share's bound allows for."""
+    B = 2
+    g = torch.Generator(device="cuda").manual_seed(F)
+    w = [torch.empty(s, dtype=torch.bfloat16, device="cuda").normal_(0.0, 0.1, generator=g) for s in ((F, D), (F, D), (D, F))]
+    x = torch.randn(B, D, device="cuda", generator=g).to(torch.bfloat16)
+    h = pb.prox_ffn_create(D, F, B, 1, *w)
+    try:
+        pb.prox_quantize_proxy(h, 4, 128)
+        sel = torch.arange(F, dtype=torch.int32, device="cuda").repeat(B, 1)
+        whole, part = (torch.empty(B, D, device="cuda") for _ in range(2))
+        pb.prox_stage2_ffn(h, x, B, sel, F, whole)
+        pb.prox_debug_set_grid(h, grid)
+        pb.prox_stage2_ffn(h, x, B, sel, F, part)
+        y64 = [(lambda gt, up: w[2].double() @ (up * gt / (1 + torch.exp(-gt))))(w[0].double() @ x[b].double(), w[1].double() @ x[b].double())
+               for b in range(B)]
+        for b in range(B):                                         # h enters the down projection as a bf16 pair: 2^-17
+            for y in (whole, part):
+                assert float((y[b].double() - y64[b]).norm()) <= 1e-4 * float(y64[b].norm())
+        assert pb.prox_last_device_status(h) == 0
+    finally:
+        pb.prox_ffn_destroy(h)
