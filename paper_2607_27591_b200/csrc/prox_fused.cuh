@@ -74,7 +74,7 @@ struct FusedParams {
   float* scores; unsigned* ghist; int* sel_out;
   int* idx_out;       // the kept input list as this kernel built it (block 0 writes it; for checking)
   unsigned spin_limit;        // polls after which a device-side wait gives up
-  unsigned bar_bias;          // test knob: added to the grid barrier's target (0 in normal use)
+  unsigned bar_bias;          // test knob (0 in normal use): added to the grid barrier's target; bit 31: see prox_debug_set_wait
   int* host_flag;             // mapped host word set to 1 when a wait expires (NULL = none)
   float* yacc; int* status;
   unsigned long long* exits;  // grows by 256 per call, complete when all its blocks have left: the call number
@@ -756,12 +756,15 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
         };
         uint32_t scn[4];
         load_scales(part, scn);
-        const bool acc_ok = __all_sync(0xffffffffu, alive_b && mbar_wait(smem_u32(&sm.acc_bar), acc_n & 1u, abortp, spin));
+        bool acc_ok = __all_sync(0xffffffffu, alive_b && mbar_wait(smem_u32(&sm.acc_bar), acc_n & 1u, abortp, spin));
         ++acc_n;
         tc_fence_after();
         if (tl == 0) {                         // the groups' offsets come from the four warps that do not load
+          const unsigned want = (unsigned)kFusedProducers + (vid == 0 ? p.bar_bias >> 31 : 0u);       // (test knob)
+          volatile unsigned* const cnt = &sm.soff_cnt;
 #pragma unroll 1
-          for (unsigned it = 0; *reinterpret_cast<volatile unsigned*>(&sm.soff_cnt) < (unsigned)kFusedProducers && it < spin; ++it) __nanosleep(32);
+          for (unsigned it = 0; *cnt < want && it < spin; ++it) __nanosleep(32);
+          if (!__all_sync(0xffffffffu, *cnt >= want)) { acc_ok = false; *abortp = 1; }
           __threadfence_block();
         }
         PROX_TRACE(25);
@@ -874,7 +877,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     fence_proxy_async();                        // phase B's plain accesses to the big buffer come before the ring's bulk copies
     __syncthreads();
     if (tid == 0) {
-      const unsigned target = n1 + p.bar_bias;
+      const unsigned target = n1 + (p.bar_bias & 0x7fffffffu);
       unsigned fin = 0, more1 = n1, share2 = 0;
       bool ok = false, again = false;
       // release (cumulative): publishes the block's writes seen through the barrier above

@@ -271,3 +271,42 @@ def test_batch_gateup_on_fewer_sms(pb, D, F, grid):
         assert pb.prox_last_device_status(h) == 0
     finally:
         pb.prox_ffn_destroy(h)
+
+
+@pytest.mark.parametrize("bits,group", [(4, 128), (8, 0)])
+def test_expired_wait_inside_stage1_is_reported(pb, bits, group):
+    """The wait for the code offsets runs out in one block, in Stage 1 called alone and in the whole path: the status says
+    so (the scores of that block are not valid), y is untouched, and the next calls are ordinary."""
+    D, F, k1, k2 = 512, 1536, 200, 300
+    p = Problem(pb, *inputs.make_small(D, F, 1, seed=3))
+    try:
+        pb.prox_quantize_proxy(p.h, bits, group)
+
+        def stage1(tau=False):
+            sel, cnt = torch.empty(1, F if tau else k2, dtype=torch.int32, device="cuda"), torch.empty(1, dtype=torch.int32, device="cuda")
+            sc = torch.empty(F, device="cuda")
+            if tau:
+                pb.prox_stage1_mask_threshold(p.h, p.t_x, 1, 0.5, 0.1, sel, cnt, sc)
+            else:
+                pb.prox_stage1_mask(p.h, p.t_x, 1, k1, k2, sel, sc)
+            return sc
+
+        y = p.y_empty()
+        good = [stage1().cpu(), stage1(True).cpu()]
+        pb.prox_debug_set_wait(p.h, 500, 1 << 31)
+        try:
+            for tau in (False, True):
+                stage1(tau)
+                status, code = pb.prox_last_device_status_raw(p.h)
+                assert status == 6 and code == 4          # PROX_ERR_TIMEOUT
+            y.fill_(7.0)
+            pb.prox_ffn_forward(p.h, p.t_x, 1, k1, k2, y)
+            status, code = pb.prox_last_device_status_raw(p.h)
+            assert status == 6 and code == 4 and torch.all(y == 7.0)
+        finally:
+            pb.prox_debug_set_wait(p.h, 0, 0)
+        assert torch.equal(stage1().cpu(), good[0]) and torch.equal(stage1(True).cpu(), good[1])
+        pb.prox_ffn_forward(p.h, p.t_x, 1, k1, k2, y)
+        assert pb.prox_last_device_status(p.h) == 0 and not torch.any(y == 7.0)
+    finally:
+        p.close()
