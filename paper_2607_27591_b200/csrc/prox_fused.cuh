@@ -880,8 +880,11 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       const unsigned target = n1 + (p.bar_bias & 0x7fffffffu);
       unsigned fin = 0, more1 = n1, share2 = 0;
       bool ok = false, again = false;
+      // A block that has given up does not finish its share: without it no block gets past the barrier, and the call ends
+      // before anything is written to y or to the residual stream.
+      const bool gave_up = *abortp != 0;
       // release (cumulative): publishes the block's writes seen through the barrier above
-      if (vid < n1) {
+      if (vid < n1 && !gave_up) {
         asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(fin) : "l"(ctr + kDone1) : "memory");
         asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(more1) : "l"(ctr + kClaim1) : "memory");
       }
@@ -889,7 +892,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       ok = vid < n1 && fin + 1u == target;
       if (MODE == kScoresOnly) { again = more1 < n1; ok = true; }      // nobody waits
 #pragma unroll 1
-      for (unsigned it = 0; !ok && it < spin; ++it) {
+      for (unsigned it = 0; !ok && !gave_up && it < spin; ++it) {
         unsigned cur;
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(cur) : "l"(ctr + kDone1) : "memory");
         ok = cur >= target;

@@ -303,6 +303,12 @@ def test_expired_wait_inside_stage1_is_reported(pb, bits, group):
             pb.prox_ffn_forward(p.h, p.t_x, 1, k1, k2, y)
             status, code = pb.prox_last_device_status_raw(p.h)
             assert status == 6 and code == 4 and torch.all(y == 7.0)
+            nw, xr = torch.ones(D, dtype=torch.bfloat16, device="cuda"), p.t_x.float().contiguous()
+            for form in (lambda: pb.prox_ffn_block_forward(p.h, xr, nw, 1e-6, 1, k1, k2, xr),
+                         lambda: pb.prox_ffn_block_forward_threshold(p.h, xr, nw, 1e-6, 1, 0.5, 0.1, xr)):
+                form()                                    # in place: nothing of the call has reached the residual stream
+                status, code = pb.prox_last_device_status_raw(p.h)
+                assert status == 6 and code == 4 and torch.equal(xr, p.t_x.float())
         finally:
             pb.prox_debug_set_wait(p.h, 0, 0)
         assert torch.equal(stage1().cpu(), good[0]) and torch.equal(stage1(True).cpu(), good[1])
