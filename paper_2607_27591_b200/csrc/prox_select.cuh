@@ -98,6 +98,10 @@ channel_topk_kernel(const float* __restrict__ scores, float* __restrict__ pacc, 
         const float4 v = __ldcg(reinterpret_cast<const float4*>(scores + (size_t)t * F) + q);
         s[0] += v.x; s[1] += v.y; s[2] += v.z; s[3] += v.w;
       }
+      // (scores are magnitudes; whatever a Stage 1 that gave up has left in the buffer must order like one too, or more
+      // or fewer than k2 channels would pass)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) s[e] = fabsf(s[e]);
     }
     const uint4 k = make_uint4(__float_as_uint(s[0]), __float_as_uint(s[1]), __float_as_uint(s[2]), __float_as_uint(s[3]));
     skey[i] = k;

@@ -316,3 +316,28 @@ def test_expired_wait_inside_stage1_is_reported(pb, bits, group):
         assert pb.prox_last_device_status(p.h) == 0 and not torch.any(y == 7.0)
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("stale", [-1.0, float("nan"), float("-inf")])
+def test_topk_of_a_stage1_that_gave_up_stays_in_its_list(pb, stale):
+    """One block, which gives up in its first share: most scores are whatever the caller's buffer held.  The call reports
+    it, and the list still has k2 valid channels and nothing behind them."""
+    D, F, k1, k2 = 512, 12288, 200, 1000
+    p = Problem(pb, *inputs.make_small(D, F, 1, seed=5))
+    try:
+        pb.prox_quantize_proxy(p.h, 4, 128)
+        sc = torch.full((F,), stale, device="cuda")
+        sel = torch.full((F,), -7, dtype=torch.int32, device="cuda")
+        pb.prox_debug_set_grid(p.h, 1)
+        pb.prox_debug_set_wait(p.h, 500, 1 << 31)
+        try:
+            pb.prox_stage1_mask(p.h, p.t_x, 1, k1, k2, sel, sc)
+            status, code = pb.prox_last_device_status_raw(p.h)
+        finally:
+            pb.prox_debug_set_wait(p.h, 0, 0)
+            pb.prox_debug_set_grid(p.h, 0)
+        assert status == 6 and code == 4
+        got = sel.cpu().numpy()
+        assert np.all(got[k2:] == -7) and np.all(got[1:k2] > got[:k2 - 1]) and got[0] >= 0 and got[k2 - 1] < F
+    finally:
+        p.close()
