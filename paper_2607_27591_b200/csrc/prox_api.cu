@@ -464,8 +464,8 @@ prox_status_t launch_stage1_batch(prox_ffn* h, const void* x, int B, int k1, int
         at[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = at; cfg.numAttrs = use_pdl ? 1 : 0;
         const __half* Sp = h->S; const uint32_t* xdp = h->xd; const float* sop = h->soffb; const float* tfp = h->tokfac;
-        int Dv = D, Fv = F, gs = gshift_m; float* pa = h->pacc; int* stp = h->dev_status;
-        void* args[] = {&h->pmap, &Sp, &xdp, &sop, &tfp, &Dv, &Fv, &gs, &pa, &stp};
+        int Bv = B, Dv = D, Fv = F, gs = gshift_m; float* pa = h->pacc; int* stp = h->dev_status;
+        void* args[] = {&h->pmap, &Sp, &xdp, &sop, &tfp, &Bv, &Dv, &Fv, &gs, &pa, &stp};
         const void* fn = h->bits == 4 ? reinterpret_cast<const void*>(&proxy_umma_kernel<4>) : reinterpret_cast<const void*>(&proxy_umma_kernel<8>);
         cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
         if (e != cudaSuccess && use_pdl) {              // attribute not accepted here: plain launch from now on

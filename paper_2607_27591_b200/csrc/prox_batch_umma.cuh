@@ -52,12 +52,12 @@ __device__ __forceinline__ float digits4_to_float(int d0, int d1, int d2, int d3
   return fmaf((float)(d2 + d3 * 256), 65536.f, (float)(d0 + d1 * 256));
 }
 
-// pacc[(token * 2 + which) * F + channel] += partial proxy sums (gate: which = 0, up: 1), already scaled.
+// pacc[(token * 2 + which) * F + channel] += partial proxy sums of the B tokens (gate: which = 0, up: 1), already scaled.
 // pmap: the packed proxy as a 2-D byte tensor [D rows][row bytes], box 128 bytes x 128 rows, 128-byte swizzle.
 template <int BITS>
 __global__ void __launch_bounds__(kBuThreads, 1)
 proxy_umma_kernel(const __grid_constant__ CUtensorMap pmap, const __half* __restrict__ S, const uint32_t* __restrict__ xd,
-                  const float* __restrict__ soff, const float* __restrict__ tokfac, int D, int F, int gshift,
+                  const float* __restrict__ soff, const float* __restrict__ tokfac, int B, int D, int F, int gshift,
                   float* __restrict__ pacc, int* __restrict__ status) {
   constexpr bool LO = BITS == 4;
   constexpr int CH = LO ? 16 : 8;
@@ -313,6 +313,9 @@ proxy_umma_kernel(const __grid_constant__ CUtensorMap pmap, const __half* __rest
         const int ch = LO ? chunk * 16 + 2 * (col & 7) : chunk * 8 + (col & 7);
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
+          // (nothing for tokens that are not there: their sums are 0 times a scale, not a number where a scale has
+          // overflowed, and only the tokens of a call are cleared behind it)
+          if (half * 4 + b >= B) break;
           float* dst = pacc + ((size_t)(half * 4 + b) * 2 + which) * F + ch;
           if (LO) atomicAdd(reinterpret_cast<float2*>(dst), make_float2(t0[b] * tf[b], t1[b] * tf[b]));
           else atomicAdd(dst, t0[b] * tf[b]);

@@ -341,3 +341,31 @@ def test_topk_of_a_stage1_that_gave_up_stays_in_its_list(pb, stale):
         assert np.all(got[k2:] == -7) and np.all(got[1:k2] > got[:k2 - 1]) and got[0] >= 0 and got[k2 - 1] < F
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("shared", [0, 1])
+@pytest.mark.parametrize("bits", [4, 8])
+def test_overflowed_scales_leave_nothing_behind(pb, bits, shared):
+    """Finite weights whose scale overflows fp16 in one channel (its scores are not numbers), a call with two tokens; then
+    ordinary weights and a call with eight: the masks are those of a handle that never saw the first weights."""
+    D, F, k1, k2 = 256, 512, 100, 200
+    wg, wu, wd, x = inputs.make_small(D, F, 8, seed=11)
+    p, fresh = Problem(pb, wg, wu, wd, x, max_batch=8), Problem(pb, wg, wu, wd, x, max_batch=8)
+    try:
+        good = p.t_wg[17].clone()
+        p.t_wg[17] = 3e38
+        for q in (p, fresh):
+            pb.prox_ffn_set_mask_policy(q.h, shared)
+            pb.prox_quantize_proxy(q.h, bits, 128)
+        y = p.y_empty(8)
+        pb.prox_ffn_forward(p.h, p.t_x, 2, k1, k2, y)
+        p.t_wg[17] = good
+        pb.prox_quantize_proxy(p.h, bits, 128)
+        sel = [torch.empty(8, k2, dtype=torch.int32, device="cuda") for _ in range(2)]
+        for q, s in zip((p, fresh), sel):
+            pb.prox_ffn_forward(q.h, q.t_x, 8, k1, k2, y)
+            pb.prox_ffn_last_mask(q.h, 8, k2, s)
+        assert torch.equal(sel[0], sel[1])
+    finally:
+        p.close()
+        fresh.close()
