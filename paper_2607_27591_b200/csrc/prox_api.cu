@@ -191,7 +191,7 @@ int ksplit_for(const prox_ffn* h, int B, int n_rows) {
 }
 
 // Function attributes (dynamic shared memory limits) are per device: one flag per (call site, device).
-enum AttrSite { kAtGateupBatch = 0, kAtBatchS1, kAtProxyB4, kAtProxyB8, kAtMma, kAtStage2, kAtFused0, kAtTopk0, kAtRows0 = kAtTopk0 + 4, kAtSites = kAtRows0 + 4 };
+enum AttrSite { kAtGateupBatch = 0, kAtBatchS1, kAtProxyB4, kAtProxyB8, kAtMma, kAtStage2, kAtFused0, kAtTopk0, kAtRows0 = kAtTopk0 + 3, kAtSites = kAtRows0 + 4 };
 bool& attr_done(int site, int device) {
   static bool done[kAtSites][64] = {};
   return done[site][device & 63];
@@ -287,8 +287,8 @@ prox_status_t launch_proxy(prox_ffn* h, const void* x, int B, const int* idx, in
 
 // exact top-k2 per token (or, shared, of the tokens' summed scores) by clusters of blocks
 template <int SRC>
-prox_status_t launch_channel_topk(prox_ffn* h, const float* scores, int B, int k2, int* sel, int stride, unsigned* cmask, cudaStream_t st) {
-  const bool shared = SRC == kSharedScores || SRC == kSharedSums;
+prox_status_t launch_channel_topk(prox_ffn* h, float* scores, int B, int k2, int* sel, int stride, unsigned* cmask, cudaStream_t st) {
+  const bool shared = SRC == kSharedSums;
   const int F = h->cfg.d_ff;
   const size_t smem = (size_t)(F / 4 / kTkBlocks + 1) * 16;
   bool& attr = attr_done(kAtTopk0 + SRC, h->device);
@@ -302,7 +302,7 @@ prox_status_t launch_channel_topk(prox_ffn* h, const float* scores, int B, int k
   return PROX_OK;
 }
 
-prox_status_t launch_channel_select(prox_ffn* h, const float* scores, int B, int k2, float tau,
+prox_status_t launch_channel_select(prox_ffn* h, float* scores, int B, int k2, float tau,
                                     int use_tau, int* sel, int stride, int* cnt, cudaStream_t st) {
   if (!use_tau && !cnt && aligned16(scores)) return launch_channel_topk<kFromScores>(h, scores, B, k2, sel, stride, nullptr, st);
   {
@@ -475,17 +475,12 @@ prox_status_t launch_stage1_batch(prox_ffn* h, const void* x, int B, int k1, int
         }
         CK(e);
       }
-      if (want_scores) CK(launch_dep(proxy_umma_finish_kernel, dim3(2 * h->sm_count), dim3(256), 0, st, h->pacc, B, F, scores));
     }
     CK(cudaGetLastError());
     unsigned* const cm = mark_mask ? h->cmask : nullptr;
-    if (h->mask_policy == 1) {
-      s = want_scores ? launch_channel_topk<kSharedScores>(h, scores, B, k2, sel, sel_stride, cm, st)
-                      : launch_channel_topk<kSharedSums>(h, nullptr, B, k2, sel, sel_stride, cm, st);
-    } else {
-      s = want_scores ? launch_channel_topk<kFromScores>(h, scores, B, k2, sel, sel_stride, cm, st)
-                      : launch_channel_topk<kFromSums>(h, nullptr, B, k2, sel, sel_stride, cm, st);
-    }
+    float* const out = want_scores ? scores : nullptr;
+    s = h->mask_policy == 1 ? launch_channel_topk<kSharedSums>(h, out, B, k2, sel, sel_stride, cm, st)
+                            : launch_channel_topk<kFromSums>(h, out, B, k2, sel, sel_stride, cm, st);
     if (s == PROX_OK && mark_mask) h->cmask_marked = 1;
     return s;
   }

@@ -330,17 +330,4 @@ proxy_umma_kernel(const __grid_constant__ CUtensorMap pmap, const __half* __rest
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tbase), "r"(256u) : "memory");
 }
 
-// score[b][ch] = |up~ * SiLU(gate~)| from the accumulated sums; the accumulator is cleared for the next call.
-__global__ void __launch_bounds__(256)
-proxy_umma_finish_kernel(float* __restrict__ pacc, int B, int F, float* __restrict__ scores) {
-  pdl_enter();
-  for (int i = blockIdx.x * 256 + threadIdx.x; i < kBT * F; i += gridDim.x * 256) {
-    const int b = i / F, ch = i - b * F;
-    float* pg = pacc + (size_t)b * 2 * F + ch;
-    const float gate = pg[0], up = pg[F];
-    pg[0] = 0.f; pg[F] = 0.f;
-    if (b < B) scores[(size_t)b * F + ch] = fabsf(up * silu_fast(gate));
-  }
-}
-
 }  // namespace prox

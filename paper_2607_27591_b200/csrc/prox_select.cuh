@@ -45,20 +45,22 @@ __device__ __forceinline__ void kth_of_counts(const unsigned (&c)[N], unsigned k
   __syncthreads();
 }
 
-enum ScoreSource { kFromScores = 0, kFromSums, kSharedScores, kSharedSums };
+enum ScoreSource { kFromScores = 0, kFromSums, kSharedSums };
 
 // Cluster b of the grid is token b.  SRC: where the scores come from
 //   kFromScores    scores[b][F]
 //   kFromSums      |up~ SiLU(gate~)| of the proxy sums pacc [token][gate | up][F], which are cleared for the next call
-//   kSharedScores, kSharedSums   one mask for the batch: the scores are added token after token in fp32 (one cluster);
-//                  the list goes to every token's row
+//   kSharedSums    one mask for the batch: these scores added token after token in fp32 (one cluster); the list goes to
+//                  every token's row
+// From the sums, the tokens' scores are also written to scores[b][F] if that is given.  (A kernel of its own that formed
+// and wrote them, in front of this one: 44 us for Stage 1 of eight tokens with scores at 4096 x 12288 against 32.)
 // cmask: a byte per channel with the tokens' bits (NULL: not wanted).  Dynamic shared memory: the block's scores.
 template <int SRC>
 __global__ void __cluster_dims__(kTkBlocks, 1, 1) __launch_bounds__(kTkThreads)
-channel_topk_kernel(const float* __restrict__ scores, float* __restrict__ pacc, int B, int F, int k2, int* __restrict__ sel_out,
+channel_topk_kernel(float* __restrict__ scores, float* __restrict__ pacc, int B, int F, int k2, int* __restrict__ sel_out,
                     int sel_stride, unsigned* __restrict__ cmask) {
   constexpr int NT = kTkThreads;
-  constexpr bool SHARED = SRC == kSharedScores || SRC == kSharedSums, SUMS = SRC == kFromSums || SRC == kSharedSums;
+  constexpr bool SHARED = SRC == kSharedSums, SUMS = SRC != kFromScores;
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   extern __shared__ __align__(16) uint8_t tk_smem[];
@@ -89,19 +91,17 @@ channel_topk_kernel(const float* __restrict__ scores, float* __restrict__ pacc, 
         if (b0 + t < b1) {
           float4* pg = reinterpret_cast<float4*>(pacc + (size_t)(b0 + t) * 2 * F) + q;
           pg[0] = make_float4(0.f, 0.f, 0.f, 0.f); pg[F / 4] = make_float4(0.f, 0.f, 0.f, 0.f);
-          s[0] += fabsf(u[t].x * silu_fast(g[t].x)); s[1] += fabsf(u[t].y * silu_fast(g[t].y));
-          s[2] += fabsf(u[t].z * silu_fast(g[t].z)); s[3] += fabsf(u[t].w * silu_fast(g[t].w));
+          const float4 v = make_float4(fabsf(u[t].x * silu_fast(g[t].x)), fabsf(u[t].y * silu_fast(g[t].y)),
+                                       fabsf(u[t].z * silu_fast(g[t].z)), fabsf(u[t].w * silu_fast(g[t].w)));
+          if (scores) reinterpret_cast<float4*>(scores + (size_t)(b0 + t) * F)[q] = v;
+          s[0] += v.x; s[1] += v.y; s[2] += v.z; s[3] += v.w;
         }
       }
     } else {
-      for (int t = SHARED ? 0 : b; t < (SHARED ? B : b + 1); ++t) {
-        const float4 v = __ldcg(reinterpret_cast<const float4*>(scores + (size_t)t * F) + q);
-        s[0] += v.x; s[1] += v.y; s[2] += v.z; s[3] += v.w;
-      }
+      const float4 v = __ldcg(reinterpret_cast<const float4*>(scores + (size_t)b * F) + q);
       // (scores are magnitudes; whatever a Stage 1 that gave up has left in the buffer must order like one too, or more
       // or fewer than k2 channels would pass)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) s[e] = fabsf(s[e]);
+      s[0] = fabsf(v.x); s[1] = fabsf(v.y); s[2] = fabsf(v.z); s[3] = fabsf(v.w);
     }
     const uint4 k = make_uint4(__float_as_uint(s[0]), __float_as_uint(s[1]), __float_as_uint(s[2]), __float_as_uint(s[3]));
     skey[i] = k;

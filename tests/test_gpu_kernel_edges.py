@@ -369,3 +369,32 @@ def test_overflowed_scales_leave_nothing_behind(pb, bits, shared):
     finally:
         p.close()
         fresh.close()
+
+
+@pytest.mark.parametrize("F", [64, 1600, 4160])
+@pytest.mark.parametrize("B,bits", [(2, 4), (5, 8), (8, 4)])
+def test_batch_stage1_scores_asked_for_or_not(pb, F, B, bits):
+    """The scores that the caller asks for are the same with either mask policy and those of the tokens alone (up to the
+    16 bits to which a batch's inputs are rounded), and asking for them changes no mask."""
+    D, k1, k2 = 384, 200, F // 3
+    p = Problem(pb, *inputs.make_small(D, F, B, seed=F + B), max_batch=B)
+    try:
+        pb.prox_quantize_proxy(p.h, bits, 128)
+        got = []
+        for shared in (0, 1):
+            pb.prox_ffn_set_mask_policy(p.h, shared)
+            sel, sel1 = (torch.empty(B, k2, dtype=torch.int32, device="cuda") for _ in range(2))
+            sc = torch.full((B, F), -1.0, device="cuda")
+            pb.prox_stage1_mask(p.h, p.t_x, B, k1, k2, sel, sc)
+            pb.prox_stage1_mask(p.h, p.t_x, B, k1, k2, sel1)
+            assert torch.equal(sel, sel1)
+            got.append(sc)
+        # sums of two or three parts of a tile's units, added in any order
+        assert float((got[0] - got[1]).norm()) <= 1e-5 * float(got[0].norm())
+        alone = torch.empty(F, device="cuda")
+        for b in range(B):
+            pb.prox_stage1_mask(p.h, p.t_x[b], 1, k1, k2, sel[0], alone)
+            assert float((got[0][b] - alone).norm()) <= 2e-3 * float(alone.norm())
+        assert pb.prox_last_device_status(p.h) == 0
+    finally:
+        p.close()
