@@ -62,6 +62,7 @@ struct prox_ffn {
   int smem_optin;           // largest dynamic shared memory a block may ask for
   int debug_grid;           // test knob: blocks of the persistent kernel and of the batch gate/up ring kernel (0 = one per SM)
   int sel_unordered;        // the last forward left its mask in the persistent kernel's own order
+  bool sel_shared;          // ... or one list, in row 0, for all its tokens
   int use_fused;            // batch-1 forward runs as one persistent kernel
   int use_union;            // batch > 1 reads weights once for the union of the tokens' masks
   unsigned long long* trace;  // optional phase time stamps of the persistent kernel (debug)
@@ -191,7 +192,7 @@ int ksplit_for(const prox_ffn* h, int B, int n_rows) {
 }
 
 // Function attributes (dynamic shared memory limits) are per device: one flag per (call site, device).
-enum AttrSite { kAtGateupBatch = 0, kAtBatchS1, kAtProxyB4, kAtProxyB8, kAtMma, kAtStage2, kAtFused0, kAtTopk0, kAtRows0 = kAtTopk0 + 3, kAtSites = kAtRows0 + 4 };
+enum AttrSite { kAtGateupBatch = 0, kAtBatchS1, kAtProxyB4, kAtProxyB8, kAtMma, kAtStage2, kAtFused0, kAtTopk0, kAtRows0 = kAtTopk0 + 8, kAtSites = kAtRows0 + 4 };
 bool& attr_done(int site, int device) {
   static bool done[kAtSites][64] = {};
   return done[site][device & 63];
@@ -285,26 +286,27 @@ prox_status_t launch_proxy(prox_ffn* h, const void* x, int B, const int* idx, in
   return PROX_OK;
 }
 
-// exact top-k2 per token (or, shared, of the tokens' summed scores) by clusters of blocks
-template <int SRC>
-prox_status_t launch_channel_topk(prox_ffn* h, float* scores, int B, int k2, int* sel, int stride, unsigned* cmask, cudaStream_t st) {
-  const bool shared = SRC == kSharedSums;
+// exact top-k2 of `lists` score rows, each for `tokens` tokens, by one block or a cluster of eight per row: see prox_select.cuh
+template <int FORM>
+prox_status_t launch_channel_topk(prox_ffn* h, float* scores, int lists, int tokens, int k2, int* sel, int stride, unsigned* cmask, cudaStream_t st) {
   const int F = h->cfg.d_ff;
-  const size_t smem = (size_t)(F / 4 / kTkBlocks + 1) * 16;
-  bool& attr = attr_done(kAtTopk0 + SRC, h->device);
-  if (!attr) {                                         // (the widest layer's 32 KB and the histograms exceed the default 48 KB)
-    CK(cudaFuncSetAttribute(channel_topk_kernel<SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, 40 * 1024));
+  const bool one = F <= (lists == 1 ? kTkOneBlock : kTkOneBlockBatch);
+  const int nb = one ? 1 : kTkBlocks;
+  const auto kern = one ? channel_topk_kernel<FORM> : channel_topk_cluster_kernel<FORM>;
+  bool& attr = attr_done(kAtTopk0 + 2 * FORM + one, h->device);
+  if (!attr) {                                         // (with the histograms it can exceed the default 48 KB)
+    CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, one ? kTkOneBlock * 4 + 16 : 40 * 1024));
     attr = true;
   }
   LaunchScope ls(h, kKChannel, st);
-  CK(launch_dep(channel_topk_kernel<SRC>, dim3((shared ? 1 : B) * kTkBlocks), dim3(kTkThreads), smem, st, scores, h->pacc, B, F, k2, sel,
-                stride, cmask));
+  CK(launch_dep(kern, dim3(lists * nb), dim3(one ? 1024 : 512), (size_t)(F / 4 / nb + 1) * 16, st, scores, h->pacc, F, k2, sel, stride,
+                tokens, cmask));
   return PROX_OK;
 }
 
 prox_status_t launch_channel_select(prox_ffn* h, float* scores, int B, int k2, float tau,
                                     int use_tau, int* sel, int stride, int* cnt, cudaStream_t st) {
-  if (!use_tau && !cnt && aligned16(scores)) return launch_channel_topk<kFromScores>(h, scores, B, k2, sel, stride, nullptr, st);
+  if (!use_tau && !cnt && aligned16(scores)) return launch_channel_topk<kFromScores>(h, scores, B, 1, k2, sel, stride, nullptr, st);
   {
     LaunchScope ls(h, kKChannel, st);
     channel_select_kernel<<<B, kSelThreads, 0, st>>>(scores, h->cfg.d_ff, k2, tau, use_tau, sel, stride, cnt);
@@ -479,8 +481,19 @@ prox_status_t launch_stage1_batch(prox_ffn* h, const void* x, int B, int k1, int
     CK(cudaGetLastError());
     unsigned* const cm = mark_mask ? h->cmask : nullptr;
     float* const out = want_scores ? scores : nullptr;
-    s = h->mask_policy == 1 ? launch_channel_topk<kSharedSums>(h, out, B, k2, sel, sel_stride, cm, st)
-                            : launch_channel_topk<kFromSums>(h, out, B, k2, sel, sel_stride, cm, st);
+    if (h->mask_policy == 1) {
+      {
+        LaunchScope ls(h, kKChannel, st);
+        CK(launch_dep(shared_score_kernel, dim3((F / 4 + 127) / 128), dim3(128), 0, st, h->pacc, B, F, out, h->svals));
+      }
+      // (inside a forward call nobody reads the list but prox_ffn_last_mask, which repeats it for the tokens)
+      if (mark_mask) h->sel_shared = true;
+      s = mark_mask ? launch_channel_topk<kFromScores>(h, h->svals, 1, B, k2, sel, sel_stride, cm, st)
+                    : launch_channel_topk<kRepeated>(h, h->svals, 1, B, k2, sel, sel_stride, cm, st);
+    } else {
+      s = out ? launch_channel_topk<kFromSumsOut>(h, out, B, 1, k2, sel, sel_stride, cm, st)
+              : launch_channel_topk<kFromSums>(h, nullptr, B, 1, k2, sel, sel_stride, cm, st);
+    }
     if (s == PROX_OK && mark_mask) h->cmask_marked = 1;
     return s;
   }
@@ -792,7 +805,7 @@ prox_status_t launch_fused(prox_ffn* h, const FusedPlan& pl, const void* x, int 
 prox_status_t forward_kernels(prox_ffn* h, const void* x, int B, int k1, int k2, void* y, cudaStream_t st) {
   prox_status_t s;
   const int D = h->cfg.d_model, F = h->cfg.d_ff;
-  h->sel_unordered = 0;
+  h->sel_unordered = 0; h->sel_shared = false;
   if (B > 1 && h->mask_policy == 1 && !(h->use_union && batch_path_ok(h, B, true))) return PROX_ERR_UNSUPPORTED;
   if (h->use_union && batch_path_ok(h, B, true)) {
     if ((s = launch_stage1_batch(h, x, B, k1, k2, h->sel, F, h->scores, st, stage2_mma_ok(h), false)) != PROX_OK) return s;
@@ -1095,6 +1108,7 @@ prox_status_t prox_ffn_block_forward_threshold(prox_ffn_t* h, const float* x_res
   rmsnorm_kernel<<<B, 256, 0, st>>>(x_res, static_cast<const uint16_t*>(norm_w), rms_const(D, eps), D, h->xn);
   h->launches++;
   CK(cudaGetLastError());
+  h->sel_shared = false;
   if ((s = prox_stage1_mask_threshold(h, h->xn, B, tau_x, tau_s, h->sel, h->cnt_s, nullptr, stream)) != PROX_OK) return s;
   h->fin_resid = x_res; h->fin_out = x_res_out;          // the last kernel adds the residual stream
   s = launch_stage2(h, h->xn, B, h->sel, F, h->cnt_s, F, nullptr, st);
@@ -1152,7 +1166,7 @@ prox_status_t prox_ffn_forward_proxy_values(prox_ffn_t* h, const void* x, int B,
   if (!h->quantized) return PROX_ERR_NOT_QUANTIZED;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int D = h->cfg.d_model, F = h->cfg.d_ff;
-  h->sel_unordered = 0;
+  h->sel_unordered = 0; h->sel_shared = false;
   if ((s = launch_input_select(h, x, B, k1, 0.f, 0, h->idx_x, D, nullptr, st)) != PROX_OK) return s;
   if ((s = launch_proxy(h, x, B, h->idx_x, D, nullptr, k1, h->scores, st, h->svals)) != PROX_OK) return s;
   if ((s = launch_channel_select(h, h->scores, B, k2, 0.f, 0, h->sel, F, nullptr, st)) != PROX_OK) return s;
@@ -1337,6 +1351,10 @@ prox_status_t prox_ffn_last_mask(prox_ffn_t* h, int B, int k2, int32_t* sel_dev,
     CK(cudaGetLastError());
     return PROX_OK;
   }
+  if (B > 1 && h->sel_shared) {
+    for (int b = 0; b < B; ++b) CK(cudaMemcpyAsync(sel_dev + (size_t)b * k2, h->sel, (size_t)k2 * sizeof(int), cudaMemcpyDeviceToDevice, st));
+    return PROX_OK;
+  }
   CK(cudaMemcpy2DAsync(sel_dev, (size_t)k2 * sizeof(int), h->sel, (size_t)h->cfg.d_ff * sizeof(int),
                        (size_t)k2 * sizeof(int), (size_t)B, cudaMemcpyDeviceToDevice, st));
   return PROX_OK;
@@ -1439,6 +1457,7 @@ prox_status_t prox_ffn_forward_threshold(prox_ffn_t* h, const void* x, int B, fl
                           nullptr, nullptr, 0.0, nullptr, taus);
     }
   }
+  h->sel_shared = false;
   prox_status_t s = prox_stage1_mask_threshold(h, x, B, tau_x, tau_s, h->sel, h->cnt_s, nullptr, stream);
   if (s != PROX_OK) return s;
   return prox_stage2_ffn_var(h, x, B, h->sel, h->cnt_s, y, stream);

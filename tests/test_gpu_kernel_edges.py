@@ -398,3 +398,44 @@ def test_batch_stage1_scores_asked_for_or_not(pb, F, B, bits):
         assert pb.prox_last_device_status(p.h) == 0
     finally:
         p.close()
+
+
+def test_last_mask_of_a_shared_mask_call(pb):
+    """The one list of a shared-mask call for every token, after other calls on the handle, and per-token lists again."""
+    D, F, B, k1, k2 = 384, 4160, 5, 200, 700
+    p = Problem(pb, *inputs.make_small(D, F, B, seed=9), max_batch=B)
+    try:
+        pb.prox_quantize_proxy(p.h, 4, 128)
+        y = p.y_empty(B)
+        want = {}
+        for shared in (0, 1):
+            pb.prox_ffn_set_mask_policy(p.h, shared)
+            want[shared] = torch.empty(B, k2, dtype=torch.int32, device="cuda")
+            pb.prox_stage1_mask(p.h, p.t_x, B, k1, k2, want[shared])
+        assert all(torch.equal(want[1][0], want[1][b]) for b in range(B)) and not torch.equal(want[0][0], want[0][1])
+
+        def last():
+            got = torch.full((B, k2), -1, dtype=torch.int32, device="cuda")
+            pb.prox_ffn_last_mask(p.h, B, k2, got)
+            return got
+
+        for shared in (1, 0, 1):
+            pb.prox_ffn_set_mask_policy(p.h, shared)
+            pb.prox_ffn_forward(p.h, p.t_x, B, k1, k2, y)
+            assert torch.equal(last(), want[shared])
+            other = torch.empty(B, k2, dtype=torch.int32, device="cuda")
+            pb.prox_stage1_mask(p.h, p.t_x, B, k1, k2, other)      # Stage 1 alone leaves the forward call's mask
+            pb.prox_stage2_ffn(p.h, p.t_x, B, other, k2, y)
+            assert torch.equal(last(), want[shared])
+        pb.prox_ffn_forward_proxy_values(p.h, p.t_x, B, k1, k2, y)  # (always per token)
+        assert not torch.equal(last()[0], last()[1])
+        assert pb.prox_last_device_status(p.h) == 0
+    finally:
+        p.close()
+
+
+@pytest.mark.parametrize("F,B,shared", [(12288, 1, False), (12352, 1, False), (10240, 3, False), (10304, 3, False), (12288, 2, True),
+                                        (12352, 2, True)])
+def test_channel_mask_at_the_lines_of_its_dispatch(pb, F, B, shared):
+    """One block per list up to 12288 channels (10240 for several lists), a cluster above."""
+    test_channel_mask_is_the_exact_topk_of_the_scores(pb, F, B, shared)
