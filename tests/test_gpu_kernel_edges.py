@@ -439,3 +439,60 @@ def test_last_mask_of_a_shared_mask_call(pb):
 def test_channel_mask_at_the_lines_of_its_dispatch(pb, F, B, shared):
     """One block per list up to 12288 channels (10240 for several lists), a cluster above."""
     test_channel_mask_is_the_exact_topk_of_the_scores(pb, F, B, shared)
+
+
+@pytest.mark.parametrize("bits,group", [(4, 128), (8, 0)])
+def test_forms_mixed_on_one_handle(pb, bits, group):
+    """Plain, threshold, layer and staged calls in any order on one handle: the score histograms that some forms fill and
+    others only clear leave every mask, count and score as on a handle that saw that form alone."""
+    D, F, k1, k2 = 512, 1600, 170, 400
+    g = torch.Generator(device="cuda").manual_seed(bits)
+    w = [torch.empty(s, dtype=torch.bfloat16, device="cuda").normal_(0.0, 0.04, generator=g) for s in ((F, D), (F, D), (D, F))]
+    x = torch.randn(4, D, device="cuda", generator=g).to(torch.bfloat16)
+    nw = torch.ones(D, dtype=torch.bfloat16, device="cuda")
+
+    def call(h, form, t):
+        y, sel = torch.empty(1, D, device="cuda"), torch.empty(1, k2, dtype=torch.int32, device="cuda")
+        if form == "plain":
+            pb.prox_ffn_forward(h, x[t], 1, k1, k2, y)
+            pb.prox_ffn_last_mask(h, 1, k2, sel)
+            return [sel]
+        if form == "layer":
+            xr = x[t].float()
+            pb.prox_ffn_block_forward(h, xr, nw, 1e-6, 1, k1, k2, y)
+            pb.prox_ffn_last_mask(h, 1, k2, sel)
+            torch.cuda.synchronize()
+            return [sel]
+        if form == "threshold":
+            pb.prox_runtime_sparsity(h, reset=True)
+            pb.prox_ffn_forward_threshold(h, x[t], 1, 0.9, 0.05, y)
+            tokens, s1, s2, e = pb.prox_runtime_sparsity(h)
+            return [torch.tensor([float(tokens), s1, s2])]
+        sc = torch.empty(F, device="cuda")
+        if form == "stage1":
+            pb.prox_stage1_mask(h, x[t], 1, k1, k2, sel, sc)
+            return [sel, sc]
+        cnt, lst = torch.empty(1, dtype=torch.int32, device="cuda"), torch.zeros(1, F, dtype=torch.int32, device="cuda")
+        pb.prox_stage1_mask_threshold(h, x[t], 1, 0.9, 0.05, lst, cnt, sc)
+        n = int(cnt)
+        pb.prox_stage2_ffn_var(h, x[t], 1, lst, cnt, y)
+        return [cnt, lst[:, :n], sc]
+
+    forms = ["plain", "layer", "threshold", "stage1", "staged threshold"]
+    hs = []
+    try:
+        alone = {}
+        for f in forms + [None]:
+            hs.append(pb.prox_ffn_create(D, F, 1, 1, *w))
+            pb.prox_quantize_proxy(hs[-1], bits, group)
+            if f:
+                for t in range(4):                                 # (four calls: both sets of histograms)
+                    alone[f, t] = [v.cpu() for v in call(hs[-1], f, t)]
+        rng = np.random.default_rng(0)
+        for _ in range(60):
+            f, t = forms[rng.integers(len(forms))], int(rng.integers(4))
+            assert all(torch.equal(a, b.cpu()) for a, b in zip(alone[f, t], call(hs[-1], f, t))), (f, t)
+        assert pb.prox_last_device_status(hs[-1]) == 0
+    finally:
+        for h in hs:
+            pb.prox_ffn_destroy(h)
