@@ -129,7 +129,9 @@ prox_status_t prox_ffn_forward(prox_ffn_t* h, const void* x_dev, int B, int k1, 
  * wait between Stage 1 and Stage 2); prox_ffn_set_fused(h, 0) selects the
  * kernel-per-step path instead (always used for B > 1).  If a bounded wait
  * ever expires the kernel leaves, y is not written (undefined) and
- * prox_last_device_status reports bit 4 and returns PROX_ERR_TIMEOUT. */
+ * prox_last_device_status reports bit 4 and returns PROX_ERR_TIMEOUT.
+ * The stages called alone at B = 1 run on the same kernel (Stage 1 up to its
+ * barrier, Stage 2 from there on), and report an expired wait in the same way. */
 prox_status_t prox_ffn_set_fused(prox_ffn_t* h, int on);
 
 /* Mask policy of calls with B > 1 (the paper treats batch 1 only and names batching as future work):
@@ -137,7 +139,8 @@ prox_status_t prox_ffn_set_fused(prox_ffn_t* h, int on);
  *   1  one channel mask for the batch: the k2 channels of largest summed proxy score
  *      sum_b |s~_{b,j}| (ties: lower channel); input masks and proxy scores stay per token, and
  *      Stage 2 reads k2 rows instead of the union of B masks.  Built by the tensor-core batch
- *      path (4-bit proxies); other configurations return UNSUPPORTED from the forward calls.
+ *      path (4- and 8-bit proxies); other configurations return UNSUPPORTED from the calls that
+ *      build a mask.
  * B = 1 is not affected.  Errors: INVALID_ARG. */
 prox_status_t prox_ffn_set_mask_policy(prox_ffn_t* h, int policy);
 
@@ -278,8 +281,11 @@ prox_status_t prox_ffn_forward_proxy_values(prox_ffn_t* h, const void* x_dev, in
  *   x_res_out  dev fp32 [B, d_model]  result; may be x_res itself (in place)
  * The norm is evaluated in fp64 and rounded once to bf16, so that the FFN input,
  * on which both masks depend, is the nearest bf16 of the exact value.  At B = 1
- * norm, FFN and residual add are one launch of the persistent kernel; otherwise
- * one small norm kernel precedes the batch path and its last kernel adds x_res.
+ * norm, FFN and residual add are one launch of the persistent kernel; for B > 1 the
+ * kernel that forms the input masks also forms the norm (a small norm kernel where
+ * that path is not taken) and the last kernel adds x_res, rounding each element of
+ * the sum once.  In place at B = 1 every block adds its share of y straight to the
+ * stream: an element is rounded once per block (148 times) at the stream's magnitude.
  * The handle's out_dtype is not used.  Errors as prox_ffn_forward. */
 prox_status_t prox_ffn_block_forward(prox_ffn_t* h, const float* x_res_dev, const void* norm_w_dev,
                                      double eps, int B, int k1, int k2, float* x_res_out_dev, void* stream);
@@ -382,8 +388,8 @@ prox_status_t prox_algorithmic_bytes(const prox_ffn_t* h, int rows_in, int rows_
  * did not write its output (y is undefined); the handle's shared counters are put
  * back to their idle state here and the call returns PROX_ERR_TIMEOUT (with *code
  * filled in); the next forward call is an ordinary one.  prox_ffn_forward_host,
- * which synchronises anyway, checks for an expired wait itself and returns
- * PROX_ERR_TIMEOUT in the same way. */
+ * which synchronises anyway, checks for an expired wait of the persistent kernel
+ * (B = 1) itself and returns PROX_ERR_TIMEOUT in the same way; for B > 1 ask here. */
 prox_status_t prox_last_device_status(prox_ffn_t* h, int32_t* code, void* stream);
 
 /* Per-kernel timing hook for benchmarks.  While enabled, every kernel launched

@@ -19,7 +19,7 @@
 // the other sets.  Items = (128-byte tile of the rows, range of units); an item's partial sums
 // are added to an fp32 accumulator in global memory, from which the channel-mask kernel forms the scores.  Every block has
 // the same number of units, to one: with items of equal size dealt out in turn some blocks had 4 where 3.03 was the mean
-// (eight tokens, kernel alone: 4096 x 12288 4-bit 20.8 -> 19.8 us, 4096 x 14336 4-bit 24.2 -> 21.4 and 8-bit 27.3 -> 24.8,
+// (eight tokens, kernel alone under a one-metric capture: 4096 x 12288 4-bit 20.8 -> 19.8 us, 4096 x 14336 4-bit 24.2 -> 21.4 and 8-bit 27.3 -> 24.8,
 // 8192 x 28672 4-bit 69.3 -> 53.9: 4.5 TB/s).  A second producer lane changed nothing.
 #pragma once
 
