@@ -51,6 +51,7 @@ constexpr int kEmptyCount = 16;      // arrivals that free a ring slot
 constexpr int kChanBatch = 256;      // channels whose h values are held at once
 constexpr int kMySelCap = 512;       // channels one block may own
 constexpr int kCand2Cap = 256;       // candidates left after the second refinement
+constexpr int kRankMax = 128;        // members of the threshold bin that are ranked directly
 // Proxy ring: a loader warp owns two stages of 32 rows x 128 bytes (4 KB each), for 4-bit codes a buffer of low
 // nibbles (4 KB), and two stages of digits of x (512 bytes each).
 __host__ __device__ constexpr int proxy_warp_bytes(int bits) { return bits == 4 ? 13312 : 9216; }
@@ -71,9 +72,10 @@ struct FusedParams {
   // ppart, in the first pmore shares cgran more
   int plines, pleft0, ppart, pmore, cgran;
   float* scores; unsigned* ghist; int* sel_out;
+  unsigned* xkeys;    // [2][F] the scores' bits as the blocks hand them to each other (calls alternate); kNoKey = not there yet
   int* idx_out;       // the kept input list as this kernel built it (block 0 writes it; for checking)
   unsigned spin_limit;        // polls after which a device-side wait gives up
-  unsigned bar_bias;          // test knob (0 in normal use): added to the grid barrier's target; bit 31: see prox_debug_set_wait
+  unsigned bar_bias;          // test knob (0 in normal use): the wait for the scores does not end; bit 31: see prox_debug_set_wait
   int* host_flag;             // mapped host word set to 1 when a wait expires (NULL = none)
   float* yacc; int* status;
   unsigned long long* exits;  // grows by 256 per call, complete when all its blocks have left: the call number
@@ -93,7 +95,11 @@ struct FusedParams {
   int* cnt_x_out; int* count_out; unsigned long long* counters;
 };
 
-enum FusedCtr { kClaim1 = 0, kDone1, kClaim2, kDone2 };    // shares claimed / finished, Stage 1 and Stage 2
+constexpr unsigned kNoKey = 0xffffffffu;      // no score: those have the sign bit clear
+constexpr int kKeyQuads = 8;                   // groups of four scores that a consumer thread reads at once
+
+// shares claimed / finished, Stage 1 and Stage 2; kOut1: Stage-1 shares whose scores are on their way
+enum FusedCtr { kClaim1 = 0, kDone1, kClaim2, kDone2, kOut1 };
 
 // ---- PTX wrappers -----------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -146,6 +152,11 @@ __device__ __forceinline__ float4 lds128f(uint32_t addr) {
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint4 ld_relaxed4(const unsigned* p) {
+  uint4 v;
+  asm volatile("ld.relaxed.gpu.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
   return v;
 }
 __device__ __forceinline__ unsigned long long global_ns() {
@@ -298,13 +309,11 @@ struct FusedSmem {
   unsigned ncand2;
   unsigned prod_seq;       // rows the producers have armed so far (for the give-up path)
   unsigned next_c;         // next channel of the batch to take in the gate/up phase
-  int go;                  // the producer warps may start
   int n_mine;              // channels of this block (for the producer warps)
   int nready;              // entries of mysel that are final (the definite share first, all of them later)
-  int keys_done;           // the consumer warps no longer read the keys near the end of the big buffer
-  int c_done;              // ... nor the list of the threshold bin's members
-  int keys_s0, keys_s1;    // ring slots [s0, s1) that overlap the keys
-  int list_s0, list_s1;    // ... and the list
+  int c_done;              // the consumer warps no longer read the list of the threshold bin's members
+  int list_s0, list_s1;    // ring slots [s0, s1) that overlap it
+  unsigned poll[2][kFusedConsumerWarps];   // the warps' counts of scores (top bit: a key is missing), two rounds in turn
   unsigned slot_use[kMaxSlots];   // uses of each ring slot whose data has been seen complete
   unsigned long long pempty[kFusedConsumerWarps];   // proxy ring: the MMAs of a warp's block are complete
   unsigned long long acc_bar;            // all MMAs of a tile are complete (one arrival per loader warp)
@@ -382,7 +391,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     fence_mbar_init();
   }
   if (tid == 0) sm.soff_cnt = 0;
-  if (tid == 0) { sm.abort_flag = 0; sm.ncand2 = 0; sm.prod_seq = 0; sm.next_c = 0; sm.go = 0; }
+  if (tid == 0) { sm.abort_flag = 0; sm.ncand2 = 0; sm.prod_seq = 0; sm.next_c = 0; sm.again = 0; }
   if (tid < kMaxSlots) sm.slot_use[tid] = 0;
   // the launch may have been set up while the previous kernel of the stream was still draining: nothing of
   // global memory is touched before that kernel has completed
@@ -451,6 +460,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   tc_fence_after();
   unsigned* const ghist = p.ghist + 2048u * sm.call_par;
   unsigned* const ctr = p.ctr + 8u * sm.call_par;
+  unsigned* const xkeys = p.xkeys + (size_t)F * sm.call_par;
   // Stage-1 share of this block; the answers are first looked at after phase A.  A block that gets none and finds
   // Stage 1 complete has started late: it leaves (what it read may be a residual stream that is being added to).
   unsigned claim1 = 0, done1 = 0;
@@ -463,6 +473,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     const int per = (2048 + G - 1) / G;
     for (int i = cta * per + tid; i < min(2048, (cta + 1) * per); i += NT) other[i] = 0u;
     if (cta == 0 && tid < 8) p.ctr[8u * (sm.call_par ^ 1u) + tid] = 0u;
+    unsigned* const okeys = p.xkeys + (size_t)F * (sm.call_par ^ 1u);
+    const int perk = (F + G - 1) / G;
+    for (int i = cta * perk + tid; i < min(F, (cta + 1) * perk); i += NT) okeys[i] = kNoKey;
   }
   if (warp < 4 && MODE != kGivenList) {
     // the accumulators of the proxy GEMV start at zero: 16 columns per supergroup, two sets 256 columns apart
@@ -487,6 +500,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       reinterpret_cast<float4*>(xf)[2 * i + 1] = make_float4(bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w));
     }
   };
+  int ebase = 1;
   if (MODE == kGivenList) {
     unsigned share2 = 0;
     if (tid == 0) asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(share2) : "l"(ctr + kClaim2) : "memory");
@@ -495,7 +509,6 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     __syncthreads();
   } else {
   // ------------------------------------------------- A: input mask (top-k1 of |x|)
-  int ebase = 1;
   const bool per_row_a = p.gshift >= 31;
   {
     const uint32_t* xs32 = reinterpret_cast<const uint32_t*>(xs);
@@ -608,7 +621,18 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       if (p.counters) { atomicAdd(p.counters, 1ull); atomicAdd(p.counters + 1, (unsigned long long)k1); }
     }
   }
+  }
   PROX_TRACE(2);
+  unsigned uses = 0, acc_n = 0;                 // blocks of rows this warp has handed to the tensor core; tiles read back
+  unsigned base_seq = 0;                        // ring rows consumed so far
+  unsigned pseq = 0, puse = 0;                  // producers: rows armed or passed over, uses of the ring, ...
+  int pslot = 0;                                // ... next slot
+  // One trip per share: of Stage 1 (B) and then of Stage 2 (C to F).  Where all blocks run there is one trip; further
+  // Stage-1 shares, of blocks that are not running, come before the channel mask, further Stage-2 shares at the end.
+  bool with_b = MODE != kGivenList;
+#pragma unroll 1
+  for (bool first = true;; first = false) {
+  if (with_b) {
   // --------------------------------------- B: proxy GEMV (tensor cores), scores, score histogram
   // Per scale group g:  sum_k x_k q_kj = 2^(ebase-134) * sum_k X_k (byte_kj - offset), X_k the integer
   // form of x_k (x_digits).  A block owns a share of the packed rows' 16-byte column chunks over all kept rows: whole
@@ -625,9 +649,6 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   // segment over two lines costs two requests, and 155 MB of whole lines took less time than 116 MB of those shares);
   // 8192 x 28672 4-bit, 2458 rows: 24 us; 4096 x 12288 4-bit, 1229 rows: 8 us (the first rows arrive 3 us after phase A,
   // the last 2.5 us later).
-  unsigned uses = 0, acc_n = 0;              // blocks of rows this warp has handed to the tensor core; tiles read back
-#pragma unroll 1
-  for (bool first = true;; first = false) {
     constexpr bool LO = (BITS == 4);
     const int nchunks = F / CH;
     const int row_bytes = nchunks * 16;
@@ -639,6 +660,18 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     const int ng = per_row ? 1 : (D >> p.gshift);
     const int nsuper = (ng + 3) >> 2;
     const uint32_t tbase = sm.tmem_base;
+    if (!first) {                              // one more share: the accumulators go back to zero
+      tc_fence_after();
+      if (warp < 4) {
+        const uint32_t tz = tbase + ((uint32_t)(warp * 32) << 16);
+#pragma unroll 1
+        for (int c = 0; c < 16 * nsuper; c += 16) { tmem_st16_zero(tz + (uint32_t)c); tmem_st16_zero(tz + 256u + (uint32_t)c); }
+        tmem_st_wait();
+        tc_fence_before();
+      }
+      __syncthreads();
+      tc_fence_after();
+    }
     if (HIST && warp < kFusedConsumerWarps) {  // the block's own score histogram (used after a consumer barrier)
 #pragma unroll 1
       for (int i = tid; i < 512; i += kFusedConsumers) reinterpret_cast<uint4*>(sm.hist)[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -813,21 +846,33 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
           t0 = scalbnf(t0, ebase - 134); t1 = scalbnf(t1, ebase - 134);
           // bytes 0..7 of a chunk hold gate codes, bytes 8..15 the up codes of the same channels
           const float u0 = __shfl_xor_sync(0xffffffffu, t0, 8), u1 = __shfl_xor_sync(0xffffffffu, t1, 8);
-          if ((col & 8) == 0 && col_ok) {
+          unsigned n0 = 1u, n1 = 1u, b0 = 0u, b1 = 0u;          // (scores in front of this thread's in their bins)
+          const bool give = MODE == kScoresOnly || *abortp == 0;          // a block that has given up hands nothing on
+          if ((col & 8) == 0 && col_ok && give) {
             if (LO) {
               const int ch = chunk * 16 + 2 * (col & 7);
               const float s0 = fabsf(u0 * silu_fast(t0)), s1 = fabsf(u1 * silu_fast(t1));
+              if (MODE == kWhole) __stcg(reinterpret_cast<float2*>(xkeys + ch), make_float2(s0, s1));
               __stcg(reinterpret_cast<float2*>(p.scores + ch), make_float2(s0, s1));
               if (HIST) {
-                atomicAdd(&sm.hist[__float_as_uint(s0) >> 20], 1u);
-                atomicAdd(&sm.hist[__float_as_uint(s1) >> 20], 1u);
+                b0 = __float_as_uint(s0) >> 20; b1 = __float_as_uint(s1) >> 20;
+                n0 = atomicAdd(&sm.hist[b0], 1u); n1 = atomicAdd(&sm.hist[b1], 1u);
               }
             } else {
               const int ch = chunk * 8 + (col & 7);
               const float s0 = fabsf(u0 * silu_fast(t0));
+              if (MODE == kWhole) __stcg(reinterpret_cast<float*>(xkeys + ch), s0);
               __stcg(p.scores + ch, s0);
-              if (HIST) atomicAdd(&sm.hist[__float_as_uint(s0) >> 20], 1u);
+              if (HIST) { b0 = __float_as_uint(s0) >> 20; n0 = atomicAdd(&sm.hist[b0], 1u); }
             }
+          }
+          if (HIST) {
+            // one global atomic per occupied bin and tile (thousands of single increments on a few hot bins serialise in
+            // L2), by the thread that came first to the bin
+            __syncwarp();
+            asm volatile("bar.sync 4, 128;" ::: "memory");
+            if (n0 == 0u) { atomicAdd(ghist + b0, sm.hist[b0]); sm.hist[b0] = 0u; }
+            if (n1 == 0u) { atomicAdd(ghist + b1, sm.hist[b1]); sm.hist[b1] = 0u; }
           }
         }
         if (more) consumer_sync();             // red is free again
@@ -868,288 +913,324 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       if (first && lane == 0) { __threadfence_block(); atomicAdd(&sm.soff_cnt, 1u); }
     }
     tc_fence_before();
-    __syncthreads();
-    if (HIST && ntl > 0) {
-      // one atomic per occupied bin and block (thousands of single increments on a few hot bins serialise in L2)
-#pragma unroll 1
-      for (int i = tid; i < 2048; i += NT) { const unsigned v = sm.hist[i]; if (v) atomicAdd(ghist + i, v); }
-    }
-    PROX_TRACE(3);
-    // ------------------------------------------------------------ grid barrier
-    // Wait until all shares of Stage 1 are finished (not all blocks).  Thread 0 says that this block's is, asks for
-    // another one (there is none unless a block of the grid is not running) and for a share of Stage 2, all in flight
-    // together and with the first look at the count.
     fence_proxy_async();                        // phase B's plain accesses to the big buffer come before the ring's bulk copies
     __syncthreads();
-    if (tid == 0) {
-      const unsigned target = n1 + (p.bar_bias & 0x7fffffffu);
-      unsigned fin = 0, more1 = n1, share2 = 0;
-      bool ok = false, again = false;
-      // A block that has given up does not finish its share: without it no block gets past the barrier, and the call ends
-      // before anything is written to y or to the residual stream.
-      const bool gave_up = *abortp != 0;
-      // release (cumulative): publishes the block's writes seen through the barrier above
-      if (vid < n1 && !gave_up) {
-        asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(fin) : "l"(ctr + kDone1) : "memory");
-        asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(more1) : "l"(ctr + kClaim1) : "memory");
+    PROX_TRACE(3);
+    if (MODE == kWhole && tid == 0 && sm.vid < (unsigned)p.nshare1 && sm.abort_flag == 0)
+      asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(ctr + kOut1) : "memory");
+    if (MODE == kScoresOnly) {
+      if (tid == 0) {
+        // a block that has given up does not finish its share
+        unsigned more1 = (unsigned)p.nshare1;
+        if (sm.vid < more1 && sm.abort_flag == 0) {
+          asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ctr + kDone1) : "memory");
+          asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(more1) : "l"(ctr + kClaim1) : "memory");
+        }
+        sm.again = more1 < (unsigned)p.nshare1; sm.vid = more1;
       }
-      if (first && MODE == kWhole) asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(share2) : "l"(ctr + kClaim2) : "memory");
-      ok = vid < n1 && fin + 1u == target;
-      if (MODE == kScoresOnly) { again = more1 < n1; ok = true; }      // nobody waits
-#pragma unroll 1
-      for (unsigned it = 0; !ok && !gave_up && it < spin; ++it) {
-        unsigned cur;
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(cur) : "l"(ctr + kDone1) : "memory");
-        ok = cur >= target;
-        if (!ok && more1 < n1) { again = true; break; }
-        if (!ok && it > 64) __nanosleep(32);
-      }
-      if (first) sm.shr = share2;
-      sm.again = again; sm.vid = more1;
-      if (!ok && !again) { sm.abort_flag = 1; atomicOr(p.status, kWaitExpired); if (p.host_flag) *reinterpret_cast<volatile int*>(p.host_flag) = 1; }
-    } else if (MODE == kWhole && warp > 0) {
-      widen_x(32);                              // meanwhile
+      __syncthreads();
     }
-    __syncthreads();
-    if (!sm.again || *abortp) break;
-    // one more share: the accumulators go back to zero
-    if (warp < 4) {
-      const uint32_t tz = tbase + ((uint32_t)(warp * 32) << 16);
-#pragma unroll 1
-      for (int c = 0; c < 16 * nsuper; c += 16) { tmem_st16_zero(tz + (uint32_t)c); tmem_st16_zero(tz + 256u + (uint32_t)c); }
-      tmem_st_wait();
-      tc_fence_before();
-    }
-    __syncthreads();
-    tc_fence_after();
   }
-  }
-  if (warp == 0) tmem_free_all(sm.tmem_base);
-  const bool alive = sm.abort_flag == 0;      // block-uniform; a dead block skips to the end
-  PROX_TRACE(4);
-
   if (MODE == kScoresOnly) {
-    if (!alive && tid == 0) { atomicOr(p.status, kWaitExpired); if (p.host_flag) *reinterpret_cast<volatile int*>(p.host_flag) = 1; }
-    leave();
-    return;
-  }
-  // Stage 2: this block's share of the kept channels (and further ones if a block of the grid is not running)
-  unsigned base_seq = 0;                        // ring rows consumed so far
-  unsigned pseq = 0, puse = 0;                  // producers: rows armed or passed over, uses of the ring, ...
-  int pslot = 0;                                // ... next slot
-#pragma unroll 1
-  for (;;) {
-  const unsigned shr = sm.shr, NSH = (unsigned)p.nshare;
-  if (shr >= NSH && alive) break;
+    if (!sm.again) break;
+  } else {
   // ---------------------------------------- C: channel mask (top-k2 of the scores)
+  // The blocks wait for a count of finished shares that is not ordered behind the scores; the scores themselves say that
+  // they are there (kNoKey = not yet), and the histogram that it is complete (it counts all channels): what is missing is read
+  // again.  (Ordered by a release, i.e. behind the acknowledgement of all the block's writes, the count came one trip to L2 later.)
   // The first histogram level tells which channels are kept whatever the exact
   // threshold turns out to be (their bin lies above the threshold bin b1:
   // "definite", nd of them) and which are still open (the nb1 members of b1).
-  // The kept list is laid out as [definite, ascending][kept members of b1,
-  // ascending]; block c owns the c-th share of either part.  Its definite share
-  // is known after two passes over the scores, so its weight rows start to stream
-  // while the consumer warps still settle the threshold inside b1.
+  // The kept list is laid out as [definite][kept members of b1], either part in the order of the threads that hold the
+  // scores; block c owns the c-th share of either part.  Its definite share is known after one pass over the scores, in
+  // registers, so its weight rows start to stream while the consumer warps still settle the threshold inside b1.
   int n_mine = 0;
-  if (MODE == kGivenList) {
-    if (warp < kFusedConsumerWarps) {
-      const unsigned n = (unsigned)(p.sel_cnt ? min(max(__ldcg(p.sel_cnt), 0), F) : k2);
-      const int R0 = (int)((n * shr) / NSH);
-      n_mine = min((int)((n * (shr + 1u)) / NSH) - R0, kMySelCap);
-#pragma unroll 1
-      for (int i = tid; i < n_mine; i += kFusedConsumers) {
-        const int j = p.sel_in[R0 + i];
-        if (j < 0 || j >= F) atomicOr(p.status, kBadChannel);
-        sm.mysel[i] = (j < 0 || j >= F) ? -1 : j;
-      }
-      if (tid == 0) {
-        sm.keys_s0 = sm.keys_s1 = sm.list_s0 = sm.list_s1 = 0;
-        sm.n_mine = n_mine; sm.nready = n_mine; sm.keys_done = 1; sm.c_done = 1;
-      }
-      __threadfence_block();
-      consumer_sync();
-      if (tid == 0) *reinterpret_cast<volatile int*>(&sm.go) = 1;
+  unsigned nd = 0, b1 = 0, kk = 0, nb1 = 0;     // (THRESH: nd = the kept channels)
+  unsigned cnt = 0, ex = 0;                     // packed: definite channels (low half) and members of b1 of this thread / in front of it
+  unsigned cm[4] = {0u, 0u, 0u, 0u};            // its members of b1 as bits: see below
+  const int nw = (F / 4 + kKeyQuads * kFusedConsumers - 1) / (kKeyQuads * kFusedConsumers);
+  auto chan = [&](int w, unsigned m) {          // channel of the lowest bit set in word w of this thread's masks
+    const int bit = __ffs((int)m) - 1;
+    return 4 * (((nw - 1 - w) * kKeyQuads + (bit >> 2)) * kFusedConsumers + tid) + (bit & 3);
+  };
+  bool staged = true;                           // the same in every block
+  const int nq = F / 4;
+  const unsigned NSH = (unsigned)p.nshare;
+  int ndm = 0, ncm = 0, Rc0 = 0, Rc1 = 0;
+  uint32_t list_u32 = smem_u32(idx16);          // members of b1: 2 * D bytes, room for D / 4 of them
+  if (warp >= kFusedConsumerWarps) {
+    if (MODE == kWhole && with_b) {
+      // (in the layer form in place, the blocks wait for this count before they add to the residual stream that others read)
+      if (tid == kFusedConsumers && sm.vid < (unsigned)p.nshare1 && sm.abort_flag == 0)
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ctr + kDone1) : "memory");
+      widen_x(kFusedConsumers);
     }
-  } else if (alive && warp < kFusedConsumerWarps) {          // the producer warps wait at the ring for the go flag
-    // Shared-memory plan: the keys (score bits) sit at the END of the big buffer (the ring fills
-    // from slot 0 and reaches those slots last); the ascending list of b1's members goes where
-    // the input index list was (free since phase B), or in front of the keys if it is long.
-    const bool in_smem = (size_t)F * 4 + 256 <= (size_t)p.big_bytes;
-    const uint32_t key_off = in_smem ? (((uint32_t)p.big_bytes - (uint32_t)F * 4u) & ~127u) : 0u;
-    const uint32_t skey_u32 = big_u32 + key_off;
-    const unsigned* gkey = reinterpret_cast<const unsigned*>(p.scores);
-    auto key_at = [&](int i) -> unsigned {
-      unsigned v;
-      if (in_smem) asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(skey_u32 + (uint32_t)i * 4u));
-      else v = __ldcg(gkey + i);
-      return v;
-    };
-    auto key4_at = [&](int i) -> uint4 {                  // i % 4 == 0
-      return in_smem ? lds128(skey_u32 + (uint32_t)i * 4u) : __ldcg(reinterpret_cast<const uint4*>(gkey + i));
-    };
+  } else if (MODE == kGivenList) {
+    const unsigned shr = sm.shr;
+    const unsigned n = (unsigned)(p.sel_cnt ? min(max(__ldcg(p.sel_cnt), 0), F) : k2);
+    const int R0 = (int)((n * shr) / NSH);
+    n_mine = shr < NSH ? min((int)((n * (shr + 1u)) / NSH) - R0, kMySelCap) : 0;
+#pragma unroll 1
+    for (int i = tid; i < n_mine; i += kFusedConsumers) {
+      const int j = p.sel_in[R0 + i];
+      if (j < 0 || j >= F) atomicOr(p.status, kBadChannel);
+      sm.mysel[i] = (j < 0 || j >= F) ? -1 : j;
+    }
+    if (tid == 0) { sm.list_s0 = sm.list_s1 = 0; sm.n_mine = n_mine; sm.nready = n_mine; sm.c_done = 1; }
+  } else if (sm.abort_flag == 0) {
+    auto missing = [](const uint4& v) { return v.x == kNoKey || v.y == kNoKey || v.z == kNoKey || v.w == kNoKey; };
     uint4 hv = make_uint4(0u, 0u, 0u, 0u);
-    if (!THRESH) hv = __ldcg(reinterpret_cast<const uint4*>(ghist) + (511 - tid));
-    if (in_smem) {
+    uint4 kq[kKeyQuads];
+    unsigned hsum = 0, hbase = 0;
+    if (tid == 0) {
+      unsigned more1 = (unsigned)p.nshare1, share2 = 0, out = 0;
+      // another share of Stage 1 (there is none unless a block of the grid is not running), and one of Stage 2
+      if (with_b && sm.vid < more1) asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(more1) : "l"(ctr + kClaim1) : "memory");
+      if (with_b && first) asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(share2) : "l"(ctr + kClaim2) : "memory");
 #pragma unroll 1
-      for (int i = tid; i < F / 4; i += kFusedConsumers) cp_async16(skey_u32 + (uint32_t)i * 16u, gkey + 4 * i);
-    }
-    cp_async_commit();
-    if (tid < 256) sm.hist2[tid] = 0;
-    PROX_TRACE(16);
-    unsigned nd = 0;                                       // channels above bin b1 (THRESH: at or above tau_s)
-    unsigned b1 = 0, kk = 0, nb1 = 0;
-    if (!THRESH) {
-      const unsigned hb[4] = {hv.w, hv.z, hv.y, hv.x};
-      find_kth<4, true>(sm, hb, 2047 - 4 * tid, (unsigned)k2, lane, warp);       // (the keys are on their way meanwhile)
-      b1 = sm.res[0]; nd = sm.res[1]; nb1 = sm.res[2];
-      kk = (unsigned)k2 - nd;                              // members of b1 to keep (>= 1)
-    }
-    uint32_t list_u32 = smem_u32(idx16);                   // 2 * D bytes: room for D / 4 members
-    uint32_t list_off = 0;                                 // offset in the big buffer when it has to go there
-    bool list_in_big = false;
-    bool staged = in_smem;                                 // the same in every block
-    if (in_smem && (size_t)nb1 * 8 > (size_t)D * 2) {
-      if ((size_t)nb1 * 8 + 128 <= (size_t)key_off) {
-        list_off = (key_off - nb1 * 8u) & ~127u; list_u32 = big_u32 + list_off; list_in_big = true;
-      } else {
-        staged = false;
+      for (unsigned it = 0; it < spin; ++it) {
+        asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(out) : "l"(ctr + kOut1) : "memory");
+        if (out >= (unsigned)p.nshare1 || more1 < (unsigned)p.nshare1) break;
       }
+      sm.again = more1 < (unsigned)p.nshare1;
+      if (with_b) { sm.vid = more1; if (first) sm.shr = share2; }
+      sm.res[7] = out >= (unsigned)p.nshare1;
     }
-    const int per = ((F + 32 * kFusedConsumerWarps - 1) / (32 * kFusedConsumerWarps)) * 32;        // channels per warp run (slow path)
-    const int i0 = min(F, warp * per), i1 = min(F, i0 + per);
-    cp_async_wait<0>();
+    consumer_sync();
     PROX_TRACE(17);
-    consumer_sync();                                       // the keys are there for everyone; wsum is free again
-    if (staged) {
-      // k2 * G < 2^31 is checked on the host, so the share bounds fit 32 bits
-      // (THRESH: nd is only known after the counting pass; the bounds are set there)
-      int Rd0 = (int)((nd * shr) / NSH);
-      const int Rc0 = (int)((kk * shr) / NSH);
-      int ndm = min((int)((nd * (shr + 1u)) / NSH) - Rd0, kMySelCap);
-      const int ncm = THRESH ? 0 : min((int)((kk * (shr + 1u)) / NSH) - Rc0, kMySelCap - ndm);
-      int Rd1 = Rd0 + ndm;
-      const int Rc1 = Rc0 + ncm;
-      n_mine = ndm + ncm;
-      // pass 1: a consumer thread owns a run of 4-channel groups and counts its definite
-      // channels and its members of b1 (packed in one word); one warp scan, warp totals
-      const int nq = F / 4, qpt = (nq + kFusedConsumers - 1) / kFusedConsumers;
-      const int q0 = min(nq, tid * qpt), q1 = (tid < kFusedConsumers) ? min(nq, q0 + qpt) : q0;
-      // (with up to 64 channels per thread it also keeps them as two bit masks, so that the later
-      // passes walk set bits instead of reading and comparing the scores again)
-      const bool masks = qpt <= 16;
-      unsigned dm[2] = {0u, 0u}, cm[2] = {0u, 0u};           // channels 0..31 and 32..63 of the thread's run
-      unsigned cnt = 0;
-#pragma unroll 1
-      for (int q = q0; q < q1; ++q) {
-        const uint4 kv = key4_at(q * 4);
-        const unsigned k4[4] = {kv.x, kv.y, kv.z, kv.w};
-        unsigned d4 = 0, c4 = 0;
+    bool ok = false;
+    const bool again = sm.again != 0;
+    // (a block that has given up hands nothing on, so that the scores are never complete and the call ends before
+    // anything is written to y or to the residual stream; neither are they with the test knob)
+    const unsigned target = (p.bar_bias & 0x7fffffffu) ? ~0u : (THRESH ? 0u : (unsigned)F);
+    const unsigned tries = !again && sm.res[7] ? spin : 0u;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          if (THRESH) {
-            d4 |= ((k4[e] >= p.tkey_s) ? 1u : 0u) << e;
-          } else {
-            const unsigned bin = k4[e] >> 20;
-            d4 |= ((bin > b1) ? 1u : 0u) << e;
-            c4 |= ((bin == b1) ? 1u : 0u) << e;
+    for (int j = 0; j < kKeyQuads; ++j) kq[j] = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll 1
+    for (unsigned it = 0; it < tries; ++it) {
+      if (!THRESH) hv = ld_relaxed4(ghist + 4 * (511 - tid));
+      bool bad = false;
+#pragma unroll
+      for (int j = 0; j < kKeyQuads; ++j) {
+        const int q = j * kFusedConsumers + tid;
+        if (q < nq) kq[j] = ld_relaxed4(xkeys + 4 * q);
+      }
+#pragma unroll
+      for (int j = 0; j < kKeyQuads; ++j) bad |= missing(kq[j]);
+      hsum = hv.x + hv.y + hv.z + hv.w;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) { const unsigned t = __shfl_up_sync(0xffffffffu, hsum, o); if (lane >= o) hsum += t; }
+      bad = __any_sync(0xffffffffu, bad);
+      if (lane == 31) sm.poll[it & 1u][warp] = hsum | (bad ? 0x80000000u : 0u);
+      consumer_sync();
+      const unsigned pv = lane < kFusedConsumerWarps ? sm.poll[it & 1u][lane] : 0u;
+      const unsigned tot = __reduce_add_sync(0xffffffffu, pv & 0x7fffffffu);
+      hbase = __reduce_add_sync(0xffffffffu, lane < warp ? pv & 0x7fffffffu : 0u);
+      if (tot == target && !__any_sync(0xffffffffu, pv >> 31)) { ok = true; break; }
+    }
+    PROX_TRACE(4);
+    if (!ok) {
+      if (!again && tid == 0) { sm.abort_flag = 1; atomicOr(p.status, kWaitExpired); if (p.host_flag) *reinterpret_cast<volatile int*>(p.host_flag) = 1; }
+    } else {
+      const unsigned shr = sm.shr;
+      if (!THRESH) {
+        // the bin of the k2-th score: thread t has the counts of four bins in descending order, the threads' runs follow
+        // each other downwards
+        unsigned run = hbase + hsum - (hv.x + hv.y + hv.z + hv.w);
+        const unsigned c4[4] = {hv.w, hv.z, hv.y, hv.x};
+        if (run < (unsigned)k2 && (unsigned)k2 <= hbase + hsum) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            if (run < (unsigned)k2 && (unsigned)k2 <= run + c4[j]) { sm.res[0] = (unsigned)(2047 - 4 * tid - j); sm.res[1] = run; sm.res[2] = c4[j]; }
+            run += c4[j];
           }
         }
-        cnt += (unsigned)__popc(d4) | ((unsigned)__popc(c4) << 16);
-        if (masks) {
-          const int rel = q - q0, sh = (rel & 7) * 4;
-          if (rel < 8) { dm[0] |= d4 << sh; cm[0] |= c4 << sh; } else { dm[1] |= d4 << sh; cm[1] |= c4 << sh; }
+        if (tid < 256) sm.hist2[tid] = 0;
+        consumer_sync();
+        b1 = sm.res[0]; nd = sm.res[1]; nb1 = sm.res[2];
+        kk = (unsigned)k2 - nd;                              // members of b1 to keep (>= 1)
+      }
+      PROX_TRACE(16);
+      uint32_t list_off = 0;                                 // offset in the big buffer when the list has to go there
+      bool list_in_big = false;
+      if ((size_t)nb1 * 8 > (size_t)D * 2) {
+        if ((size_t)nb1 * 8 + 128 <= (size_t)p.big_bytes) {
+          list_off = ((uint32_t)p.big_bytes - nb1 * 8u) & ~127u; list_u32 = big_u32 + list_off; list_in_big = true;
+        } else {
+          staged = false;
         }
       }
-      const unsigned inc = warp_scan_incl(cnt, lane);
+      // a consumer thread counts its definite channels and its members of b1 and keeps them as bit masks (word 0: the last
+      // kKeyQuads groups of scores that it has read, word 1 the ones before, ...)
+      unsigned dm[4] = {0u, 0u, 0u, 0u};
+#pragma unroll 1
+      for (int w = 0;;) {
+#pragma unroll
+        for (int j = 3; j > 0; --j) { dm[j] = dm[j - 1]; cm[j] = cm[j - 1]; }
+        dm[0] = cm[0] = 0u;
+#pragma unroll
+        for (int j = 0; j < kKeyQuads; ++j) {
+          const unsigned k4[4] = {kq[j].x, kq[j].y, kq[j].z, kq[j].w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            if (THRESH) {
+              if (k4[e] >= p.tkey_s) dm[0] |= 1u << (4 * j + e);
+            } else {
+              const unsigned bin = k4[e] >> 20;
+              if (bin > b1) dm[0] |= 1u << (4 * j + e);
+              if (bin == b1) cm[0] |= 1u << (4 * j + e);
+            }
+          }
+          if ((w * kKeyQuads + j) * kFusedConsumers + tid >= nq) { dm[0] &= ~(15u << (4 * j)); cm[0] &= ~(15u << (4 * j)); }
+        }
+        if (++w * kKeyQuads * kFusedConsumers >= nq) break;
+        bool bad = true;                                     // d_ff > 16384
+#pragma unroll 1
+        for (unsigned it = 0; bad && it < spin; ++it) {      // (in the top-k form they are there: their counts are)
+          bad = false;
+#pragma unroll
+          for (int j = 0; j < kKeyQuads; ++j) {
+            const int q = (w * kKeyQuads + j) * kFusedConsumers + tid;
+            kq[j] = q < nq ? ld_relaxed4(xkeys + 4 * q) : make_uint4(0u, 0u, 0u, 0u);
+          }
+#pragma unroll
+          for (int j = 0; j < kKeyQuads; ++j) bad |= missing(kq[j]);
+        }
+        if (bad) sm.abort_flag = 1;
+      }
+      cnt = (unsigned)(__popc(dm[0]) + __popc(dm[1]) + __popc(dm[2]) + __popc(dm[3])) |
+            ((unsigned)(__popc(cm[0]) + __popc(cm[1]) + __popc(cm[2]) + __popc(cm[3])) << 16);
+      unsigned inc = cnt;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) { const unsigned t = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += t; }
       if (lane == 31) sm.wsum[warp] = inc;
+      consumer_sync();
+      PROX_TRACE(18);
+      ex = __reduce_add_sync(0xffffffffu, (lane < warp) ? sm.wsum[lane] : 0u) + inc - cnt;
       if (THRESH) {
-        consumer_sync();                                   // the warps' totals: how many channels are kept
         nd = __reduce_add_sync(0xffffffffu, (lane < kFusedConsumerWarps) ? (sm.wsum[lane] & 0xffffu) : 0u);
-        Rd0 = (int)((nd * shr) / NSH);
-        ndm = min((int)((nd * (shr + 1u)) / NSH) - Rd0, kMySelCap);
-        Rd1 = Rd0 + ndm;
-        n_mine = ndm;
         if (shr == 0 && tid == 0) {
           if (p.count_out) p.count_out[0] = (int)nd;
           if (p.counters) atomicAdd(p.counters + 2, (unsigned long long)nd);
         }
       }
-      if (tid == 0) {
-        const uint32_t rb = (uint32_t)D * 2u;
-        sm.keys_s0 = (int)(key_off / rb); sm.keys_s1 = (int)((key_off + (uint32_t)F * 4u + rb - 1u) / rb);
-        sm.list_s0 = list_in_big ? (int)(list_off / rb) : 0;
-        sm.list_s1 = list_in_big ? (int)((list_off + nb1 * 8u + rb - 1u) / rb) : 0;
-        sm.n_mine = n_mine; sm.nready = ndm; sm.keys_done = (ncm == 0) ? 1 : 0; sm.c_done = (ncm == 0) ? 1 : 0;
-      }
-      consumer_sync();
-      PROX_TRACE(18);
-      // pass 2: the threads whose definite channels meet the block's share write them out
-      const unsigned ex = __reduce_add_sync(0xffffffffu, (lane < warp) ? sm.wsum[lane] : 0u) + inc - cnt;
-      {
+      if (staged && shr < NSH) {
+        // k2 * G < 2^31 is checked on the host, so the share bounds fit 32 bits
+        const int Rd0 = (int)((nd * shr) / NSH);
+        ndm = min((int)((nd * (shr + 1u)) / NSH) - Rd0, kMySelCap);
+        Rc0 = (int)((kk * shr) / NSH);
+        ncm = THRESH ? 0 : min((int)((kk * (shr + 1u)) / NSH) - Rc0, kMySelCap - ndm);
+        Rc1 = Rc0 + ncm;
+        const int Rd1 = Rd0 + ndm;
+        n_mine = ndm + ncm;
+        if (tid == 0) {
+          const uint32_t rb = (uint32_t)D * 2u;
+          sm.list_s0 = list_in_big ? (int)(list_off / rb) : 0;
+          sm.list_s1 = list_in_big ? (int)((list_off + nb1 * 8u + rb - 1u) / rb) : 0;
+          sm.n_mine = n_mine; sm.nready = ndm; sm.c_done = (ncm == 0) ? 1 : 0;
+        }
+        // the threads whose definite channels meet the block's share write them out
         int dpos = (int)(ex & 0xffffu);
         const int cdef = (int)(cnt & 0xffffu);
-        if (masks && cdef > 0 && dpos < Rd1 && dpos + cdef > Rd0) {
+        if (cdef > 0 && dpos < Rd1 && dpos + cdef > Rd0) {
+#pragma unroll
+          for (int w = 0; w < 4; ++w) {
 #pragma unroll 1
-          for (int hw = 0; hw < 2; ++hw) {
-#pragma unroll 1
-            for (unsigned m = dm[hw]; m; m &= m - 1) {
+            for (unsigned m = dm[w]; m; m &= m - 1) {
               if (dpos >= Rd0 && dpos < Rd1) {
-                const int ch = q0 * 4 + hw * 32 + __ffs((int)m) - 1;
+                const int ch = chan(w, m);
                 sm.mysel[dpos - Rd0] = ch;
                 if (p.sel_out) p.sel_out[dpos] = ch;
               }
               ++dpos;
             }
           }
-        } else if (cdef > 0 && dpos < Rd1 && dpos + cdef > Rd0) {
+        }
+      } else if (shr < NSH) {
+        // No room in shared memory for the list of b1's members (a huge threshold bin such as an all-zero input gives):
+        // the consumer warps settle the threshold by two radix steps of 10 bits over all keys and the block keeps its
+        // share of the plain ascending list before the ring starts.
+        const int R0 = (int)(((unsigned)k2 * shr) / NSH), R1 = (int)(((unsigned)k2 * (shr + 1u)) / NSH);
+        const int per = ((F + 32 * kFusedConsumerWarps - 1) / (32 * kFusedConsumerWarps)) * 32;        // channels per warp run
+        const int i0 = min(F, warp * per), i1 = min(F, i0 + per);
+        n_mine = min(R1 - R0, kMySelCap);
+        unsigned prefix = b1, kleft = kk;
 #pragma unroll 1
-          for (int q = q0; q < q1; ++q) {
-            const uint4 kv = key4_at(q * 4);
-            const unsigned k4[4] = {kv.x, kv.y, kv.z, kv.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              if (THRESH ? (k4[e] >= p.tkey_s) : ((k4[e] >> 20) > b1)) {
-                if (dpos >= Rd0 && dpos < Rd1) {
-                  sm.mysel[dpos - Rd0] = q * 4 + e;
-                  if (p.sel_out) p.sel_out[dpos] = q * 4 + e;
-                }
-                ++dpos;
+        for (int sh = 10; sh >= 0; sh -= 10) {
+          consumer_sync();
+          for (int i = tid; i < 1024; i += kFusedConsumers) sm.hist[i] = 0;
+          consumer_sync();
+#pragma unroll 1
+          for (int i = tid; i < F; i += kFusedConsumers) {
+            const unsigned key = __ldcg(xkeys + i);
+            if ((key >> (sh + 10)) == prefix) atomicAdd(&sm.hist[(key >> sh) & 1023u], 1u);
+          }
+          consumer_sync();
+          unsigned ab;
+          const unsigned bb = kth_in_block<2, true>(sm.hist, kleft, sm.wsum, lane, warp, &ab);
+          prefix = (prefix << 10) | bb;
+          kleft -= ab;
+        }
+        const unsigned T = prefix, quota = kleft;
+        consumer_sync();
+        {
+          unsigned cg = 0, ce = 0;                 // separate words: the ties alone may be 65536
+#pragma unroll 1
+          for (int i = i0 + lane; i < i1; i += 32) {
+            const unsigned key = __ldcg(xkeys + i);
+            cg += (key > T) ? 1u : 0u; ce += (key == T) ? 1u : 0u;
+          }
+          cg = __reduce_add_sync(0xffffffffu, cg);
+          ce = __reduce_add_sync(0xffffffffu, ce);
+          if (lane == 0) { sm.wsum[warp] = cg; sm.warp_cnt[warp][1] = ce; }
+        }
+        consumer_sync();
+        {
+          unsigned bg = __reduce_add_sync(0xffffffffu, (lane < warp) ? sm.wsum[lane] : 0u);
+          unsigned be = __reduce_add_sync(0xffffffffu, (lane < warp) ? sm.warp_cnt[lane][1] : 0u);
+          const int first_pos = (int)(bg + min(be, quota));
+          const int end = (int)(bg + sm.wsum[warp] + min(be + sm.warp_cnt[warp][1], quota));
+          if (first_pos < R1 && end > R0) {
+#pragma unroll 1
+            for (int ib = i0; ib < i1; ib += 32) {
+              const int i = ib + lane;
+              const unsigned key = __ldcg(xkeys + min(i, F - 1));
+              const bool gt = i < i1 && key > T, eq = i < i1 && key == T;
+              const unsigned mg = __ballot_sync(0xffffffffu, gt), me = __ballot_sync(0xffffffffu, eq);
+              const unsigned myre = be + (unsigned)__popc(me & lt_mask);
+              const int pos = (int)(bg + (unsigned)__popc(mg & lt_mask) + min(myre, quota));
+              if ((gt || (eq && myre < quota)) && pos >= R0 && pos < R0 + n_mine) {
+                sm.mysel[pos - R0] = i;
+                if (p.sel_out) p.sel_out[pos] = i;
               }
+              bg += (unsigned)__popc(mg); be += (unsigned)__popc(me);
             }
           }
         }
+        if (tid == 0) { sm.list_s0 = sm.list_s1 = 0; sm.n_mine = n_mine; sm.nready = n_mine; sm.c_done = 1; }
       }
-      __threadfence_block();
-      consumer_sync();                          // the definite share is listed
-      if (tid == 0) *reinterpret_cast<volatile int*>(&sm.go) = 1;      // the producer warps leave for the ring
-      PROX_TRACE(21);
-      if (ncm > 0 && warp < kFusedConsumerWarps) {
-        // ---- consumer warps only (named barrier): list b1's members in channel order ...
+    }
+  }
+  __syncthreads();                              // the block's definite share is listed: the producer warps may start
+  PROX_TRACE(21);
+  const bool alive = sm.abort_flag == 0;        // block-uniform; a dead block skips to the end
+  if (MODE == kWhole && alive && with_b && sm.again) continue;      // one more share of Stage 1
+  with_b = false;
+  if (alive && sm.shr >= NSH) break;
+  if (MODE == kWhole && !THRESH && warp < kFusedConsumerWarps && ncm > 0) {
+        // ---- consumer warps only: the list of b1's members ...
         const uint32_t lkey_u32 = list_u32, lidx_u32 = lkey_u32 + nb1 * 4u;
         auto lds32 = [](uint32_t a) -> unsigned { unsigned v; asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a)); return v; };
         auto sts32 = [](uint32_t a, unsigned v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); };
-        if (masks) {
+        if (cnt >> 16) {
           unsigned cpos = ex >> 16;
-#pragma unroll 1
-          for (int hw = 0; hw < 2; ++hw) {
-#pragma unroll 1
-            for (unsigned m = cm[hw]; m; m &= m - 1) {
-              const int ch = q0 * 4 + hw * 32 + __ffs((int)m) - 1;
-              if (cpos < nb1) { sts32(lkey_u32 + cpos * 4u, key_at(ch)); sts32(lidx_u32 + cpos * 4u, (unsigned)ch); }
-              ++cpos;
-            }
-          }
-        } else if (cnt >> 16) {
-          unsigned cpos = ex >> 16;
-#pragma unroll 1
-          for (int q = q0; q < q1; ++q) {
-            const uint4 kv = key4_at(q * 4);
-            const unsigned k4[4] = {kv.x, kv.y, kv.z, kv.w};
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              if ((k4[e] >> 20) == b1) {
-                if (cpos < nb1) { sts32(lkey_u32 + cpos * 4u, k4[e]); sts32(lidx_u32 + cpos * 4u, (unsigned)(q * 4 + e)); }
-                ++cpos;
-              }
+          for (int w = 0; w < 4; ++w) {
+#pragma unroll 1
+            for (unsigned m = cm[w]; m; m &= m - 1) {
+              const int ch = chan(w, m);
+              if (cpos < nb1) { sts32(lkey_u32 + cpos * 4u, __ldcg(xkeys + ch)); sts32(lidx_u32 + cpos * 4u, (unsigned)ch); }
+              ++cpos;
             }
           }
         }
@@ -1158,9 +1239,24 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
         if (warp >= kSettlerWarps) {
           asm volatile("bar.arrive 2, %0;" ::"n"(kFusedConsumers) : "memory");
         } else {
-        asm volatile("bar.sync 2, %0;" ::"n"(kFusedConsumers) : "memory");      // the list is complete, the keys are free
-        if (tid == 0) *reinterpret_cast<volatile int*>(&sm.keys_done) = 1;
+        asm volatile("bar.sync 2, %0;" ::"n"(kFusedConsumers) : "memory");      // the list is complete
         PROX_TRACE(15);
+        if (nb1 <= (unsigned)kRankMax) {
+          // ... few of them: a member's place is its rank by (score descending, channel ascending)
+          if (tid < (int)nb1) {
+            const unsigned key = lds32(lkey_u32 + (uint32_t)tid * 4u), id = lds32(lidx_u32 + (uint32_t)tid * 4u);
+            int pos = 0;
+#pragma unroll 4
+            for (unsigned c = 0; c < nb1; ++c) {
+              const unsigned okey = lds32(lkey_u32 + c * 4u), oid = lds32(lidx_u32 + c * 4u);
+              pos += (okey > key || (okey == key && oid < id)) ? 1 : 0;
+            }
+            if (pos < (int)kk && pos >= Rc0 && pos < Rc1) {
+              sm.mysel[ndm + pos - Rc0] = (int)id;
+              if (p.sel_out) p.sel_out[(int)nd + pos] = (int)id;
+            }
+          }
+        } else {
         // ... settle the threshold inside b1: histogram of bits 19..12, then the few left ...
 #pragma unroll 1
         for (unsigned c = tid; c < nb1; c += kSettlers)
@@ -1181,56 +1277,57 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
         settler_sync();
         const unsigned n2 = sm.ncand2;
         PROX_TRACE(19);
-        unsigned T, quota;
+        unsigned T, tch;                         // score and channel of the last one kept
         if (n2 <= (unsigned)kCand2Cap) {
           // rank the few that are left by (score descending, channel ascending)
           if (tid < (int)n2) {
             const unsigned key = sm.cand2_key[tid];
             const int id = sm.cand2_idx[tid];
-            unsigned rank = 0, same_before = 0;
-#pragma unroll 1
+            unsigned rank = 0;
+#pragma unroll 4
             for (unsigned c = 0; c < n2; ++c) {
               const unsigned ok = sm.cand2_key[c];
               const int oi = sm.cand2_idx[c];
               rank += (ok > key || (ok == key && oi < id)) ? 1u : 0u;
-              same_before += (ok == key && oi < id) ? 1u : 0u;
             }
-            if (rank == kk2 - 1u) { sm.res[2] = key; sm.res[3] = same_before + 1u; }
+            if (rank == kk2 - 1u) { sm.res[2] = key; sm.res[3] = (unsigned)id; }
           }
           settler_sync();
-          T = sm.res[2]; quota = sm.res[3];
+          T = sm.res[2]; tch = sm.res[3];
         } else {
-          // many scores agree in their top 20 bits: two more radix steps of 6 bits over the list
-          unsigned prefix = pre2;
+          // many scores agree in their top 20 bits: radix steps of 7 bits over the other 12 and the inverted channel
+          unsigned prefix = 0;
 #pragma unroll 1
-          for (int sh = 6; sh >= 0; sh -= 6) {
+          for (int sh = 21; sh >= 0; sh -= 7) {
             settler_sync();                               // everyone is done with the previous histogram
-            if (tid < 64) sm.hist2[tid] = 0;
+            if (tid < 128) sm.hist2[tid] = 0;
             settler_sync();
 #pragma unroll 1
             for (unsigned c = tid; c < nb1; c += kSettlers) {
               const unsigned key = lds32(lkey_u32 + c * 4u);
-              if ((key >> (sh + 6)) == prefix) atomicAdd(&sm.hist2[(key >> sh) & 63u], 1u);
+              const unsigned low = ((key & 0xfffu) << 16) | (0xffffu ^ lds32(lidx_u32 + c * 4u));
+              if ((key >> 12) == pre2 && (low >> (sh + 7)) == prefix) atomicAdd(&sm.hist2[(low >> sh) & 127u], 1u);
             }
             settler_sync();
             unsigned ab;
-            const unsigned bb = kth_in_segment<2>(sm.hist2, 64, kk2, lane, &ab);
-            prefix = (prefix << 6) | bb;
+            const unsigned bb = kth_in_segment<4>(sm.hist2, 128, kk2, lane, &ab);
+            prefix = (prefix << 7) | bb;
             kk2 -= ab;
           }
-          T = prefix; quota = kk2;
+          T = (pre2 << 12) | (prefix >> 16); tch = 0xffffu ^ (prefix & 0xffffu);
         }
         PROX_TRACE(20);
-        // ... and keep the block's share of the members above T plus the first `quota` ties at T:
-        // a thread owns a run of the list, counts first (packed in one word), then the places
+        // ... and keep the block's share of the members down to that one: a thread owns a run of the list, counts
+        // first, then the places
         const int ept = ((int)nb1 + kSettlers - 1) / kSettlers;
         const int c0 = min((int)nb1, tid * ept), c1 = min((int)nb1, c0 + ept);
+        auto kept = [&](int c) {
+          const unsigned key = lds32(lkey_u32 + (uint32_t)c * 4u);
+          return key > T || (key == T && lds32(lidx_u32 + (uint32_t)c * 4u) <= tch);
+        };
         unsigned wt = 0;
 #pragma unroll 1
-        for (int c = c0; c < c1; ++c) {
-          const unsigned key = lds32(lkey_u32 + (uint32_t)c * 4u);
-          wt += ((key > T) ? 1u : 0u) | ((key == T) ? 0x10000u : 0u);
-        }
+        for (int c = c0; c < c1; ++c) wt += kept(c) ? 1u : 0u;
         const unsigned inc3 = warp_scan_incl(wt, lane);
         if (lane == 31) sm.warp_cnt[warp][0] = inc3;
         settler_sync();
@@ -1239,20 +1336,20 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
           unsigned bs = 0;
 #pragma unroll 1
           for (int w = 0; w < warp; ++w) bs += sm.warp_cnt[w][0];
-          const unsigned ex3 = bs + inc3 - wt;
-          unsigned ra = ex3 & 0xffffu, re = ex3 >> 16;
+          int pos = (int)(bs + inc3 - wt);
+          if (wt > 0 && pos < Rc1 && pos + (int)wt > Rc0) {
 #pragma unroll 1
-          for (int c = c0; c < c1; ++c) {
-            const unsigned key = lds32(lkey_u32 + (uint32_t)c * 4u);
-            const bool gt = key > T, eq = key == T;
-            const int pos = (int)(ra + min(re, quota));
-            if ((gt || (eq && re < quota)) && pos >= Rc0 && pos < Rc1) {
-              const int ch = (int)lds32(lidx_u32 + (uint32_t)c * 4u);
-              sm.mysel[ndm + pos - Rc0] = ch;
-              if (p.sel_out) p.sel_out[(int)nd + pos] = ch;
+            for (int c = c0; c < c1; ++c) {
+              if (!kept(c)) continue;
+              if (pos >= Rc0 && pos < Rc1) {
+                const int ch = (int)lds32(lidx_u32 + (uint32_t)c * 4u);
+                sm.mysel[ndm + pos - Rc0] = ch;
+                if (p.sel_out) p.sel_out[(int)nd + pos] = ch;
+              }
+              ++pos;
             }
-            ra += gt ? 1u : 0u; re += eq ? 1u : 0u;
           }
+        }
         }
         __threadfence_block();
         settler_sync();                          // the list is free from here on
@@ -1263,76 +1360,6 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
         }
         PROX_TRACE(6);
         }
-      }
-    } else {
-      // No room in shared memory for the keys plus the list of b1's members (a very large
-      // d_ff, or a huge threshold bin such as an all-zero input gives): the whole block
-      // settles the threshold by two radix steps of 10 bits over all keys and keeps its
-      // share of the plain ascending list before the ring starts.
-      const int R0 = (int)(((unsigned)k2 * shr) / NSH), R1 = (int)(((unsigned)k2 * (shr + 1u)) / NSH);
-      n_mine = min(R1 - R0, kMySelCap);
-      unsigned prefix = b1, kleft = kk;
-#pragma unroll 1
-      for (int sh = 10; sh >= 0; sh -= 10) {
-        consumer_sync();
-        for (int i = tid; i < 1024; i += kFusedConsumers) sm.hist[i] = 0;
-        consumer_sync();
-#pragma unroll 1
-        for (int i = tid; i < F; i += kFusedConsumers) {
-          const unsigned key = key_at(i);
-          if ((key >> (sh + 10)) == prefix) atomicAdd(&sm.hist[(key >> sh) & 1023u], 1u);
-        }
-        consumer_sync();
-        unsigned ab;
-        const unsigned bb = kth_in_block<2, true>(sm.hist, kleft, sm.wsum, lane, warp, &ab);
-        prefix = (prefix << 10) | bb;
-        kleft -= ab;
-      }
-      const unsigned T = prefix, quota = kleft;
-      consumer_sync();
-      {
-        unsigned cg = 0, ce = 0;                 // separate words: the ties alone may be 65536
-#pragma unroll 1
-        for (int i = i0 + lane; i < i1; i += 32) {
-          const unsigned key = key_at(i);
-          cg += (key > T) ? 1u : 0u; ce += (key == T) ? 1u : 0u;
-        }
-        cg = __reduce_add_sync(0xffffffffu, cg);
-        ce = __reduce_add_sync(0xffffffffu, ce);
-        if (lane == 0) { sm.wsum[warp] = cg; sm.warp_cnt[warp][1] = ce; }
-      }
-      consumer_sync();
-      {
-        unsigned bg = __reduce_add_sync(0xffffffffu, (lane < warp) ? sm.wsum[lane] : 0u);
-        unsigned be = __reduce_add_sync(0xffffffffu, (lane < warp) ? sm.warp_cnt[lane][1] : 0u);
-        const int first = (int)(bg + min(be, quota));
-        const int end = (int)(bg + sm.wsum[warp] + min(be + sm.warp_cnt[warp][1], quota));
-        if (first < R1 && end > R0) {
-#pragma unroll 1
-          for (int ib = i0; ib < i1; ib += 32) {
-            const int i = ib + lane;
-            const unsigned key = key_at(min(i, F - 1));
-            const bool gt = i < i1 && key > T, eq = i < i1 && key == T;
-            const unsigned mg = __ballot_sync(0xffffffffu, gt), me = __ballot_sync(0xffffffffu, eq);
-            const unsigned myre = be + (unsigned)__popc(me & lt_mask);
-            const int pos = (int)(bg + (unsigned)__popc(mg & lt_mask) + min(myre, quota));
-            if ((gt || (eq && myre < quota)) && pos >= R0 && pos < R0 + n_mine) {
-              sm.mysel[pos - R0] = i;
-              if (p.sel_out) p.sel_out[pos] = i;
-            }
-            bg += (unsigned)__popc(mg); be += (unsigned)__popc(me);
-          }
-        }
-      }
-      __threadfence_block();
-      consumer_sync();
-      if (tid == 0) {
-        sm.keys_s0 = sm.keys_s1 = sm.list_s0 = sm.list_s1 = 0;
-        sm.n_mine = n_mine; sm.nready = n_mine; sm.keys_done = 1; sm.c_done = 1;
-        __threadfence_block();
-        *reinterpret_cast<volatile int*>(&sm.go) = 1;
-      }
-    }
   }
 
   PROX_TRACE(5);
@@ -1352,26 +1379,14 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     // ---- producer warps: lane 0 of each feeds every kFusedProducers-th slot of
     // the ring (one thread can only start a few million bulk copies a second)
     if (lane == 0 && alive) {
-      // wait (bounded) until the consumer warps have listed the block's definite share
-      bool go = false;
-#pragma unroll 1
-      for (unsigned it = 0; it < spin; ++it) {
-        if (*reinterpret_cast<volatile int*>(&sm.go)) { go = true; break; }
-        if (*abortp) break;
-        __nanosleep(32);
-      }
-      if (!go) sm.abort_flag = 1;
-      __threadfence_block();
-      fence_proxy_async();                      // the big buffer becomes a bulk-copy target now
-      n_mine = go ? *reinterpret_cast<volatile int*>(&sm.n_mine) : 0;
+      n_mine = sm.n_mine;
       const unsigned pq = (unsigned)(warp - kFusedConsumerWarps);
       unsigned seq = pseq, use = puse;
       int slot = pslot;
       bool dead = false;
       int ready = *reinterpret_cast<volatile int*>(&sm.nready);
-      bool kdone = *reinterpret_cast<volatile int*>(&sm.keys_done) != 0;
       bool cdone = *reinterpret_cast<volatile int*>(&sm.c_done) != 0;
-      const int ks0 = sm.keys_s0, ks1 = sm.keys_s1, ls0 = sm.list_s0, ls1 = sm.list_s1;
+      const int ls0 = sm.list_s0, ls1 = sm.list_s1;
       for (int b0 = 0; b0 < n_mine && !dead; b0 += kChanBatch) {
         const int nb = min(kChanBatch, n_mine - b0);
         for (int q = 0; q < 3 * nb; ++q, ++seq) {
@@ -1380,20 +1395,19 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
           if (((unsigned)slot & (unsigned)(kFusedProducers - 1)) == pq) {
             const int mi = b0 + ((q < 2 * nb) ? (q >> 1) : (q - 2 * nb));
             // The tail of the list (the share of the threshold bin) is written late, and the ring
-            // may not touch the slots under the keys before the consumer warps are done with them.
-            auto blocked = [&]() {
-              return mi >= ready || (!kdone && slot >= ks0 && slot < ks1) || (!cdone && slot >= ls0 && slot < ls1);
-            };
+            // may not touch the slots under the list of b1's members before the consumer warps are done with it.
+            auto blocked = [&]() { return mi >= ready || (!cdone && slot >= ls0 && slot < ls1); };
             if (blocked()) {
 #pragma unroll 1
               for (unsigned it = 0; it < spin; ++it) {
                 ready = *reinterpret_cast<volatile int*>(&sm.nready);
-                kdone = *reinterpret_cast<volatile int*>(&sm.keys_done) != 0;
                 cdone = *reinterpret_cast<volatile int*>(&sm.c_done) != 0;
                 if (!blocked() || *abortp) break;
                 __nanosleep(64);
               }
               if (blocked()) { sm.abort_flag = 1; dead = true; break; }
+              __threadfence_block();
+              fence_proxy_async();
             }
             if (use > 0 && !mbar_wait(smem_u32(&sm.mbar_empty[slot]), (use - 1u) & 1u, abortp, spin)) { dead = true; break; }
             const uint16_t* src;
@@ -1423,6 +1437,17 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   } else {
     // ---- consumer warps
     const uint32_t xf_u32 = smem_u32(xf);
+    if (NORM && alive && p.xres_out == p.xres && warp == kFusedConsumerWarps - 1) {
+      // y goes straight into the residual stream below: not before all blocks with a share of Stage 1 have said that
+      // they have read it (they said so when their scores were out, which are all here: no wait in practice)
+      if (lane == 0) {
+        bool seen = false;
+#pragma unroll 1
+        for (unsigned it = 0; !seen && it < spin; ++it) seen = ld_acquire(ctr + kDone1) >= (unsigned)p.nshare1;
+        if (!seen) sm.abort_flag = 1;
+      }
+      __syncwarp();
+    }
     for (int b0 = 0; b0 < n_mine; b0 += kChanBatch) {
       const int nb = min(kChanBatch, n_mine - b0);
       // D: a warp takes the next channel of the batch that nobody has taken yet (the warps
@@ -1514,15 +1539,15 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
         }
       }
       consumer_sync();
-      for (int v4 = tid; v4 < D / 4; v4 += kFusedConsumers) {
+      for (int v4 = tid; v4 < D / 4 && !*abortp; v4 += kFusedConsumers) {       // (a block that has given up adds nothing)
         float4 s = reinterpret_cast<const float4*>(ysum)[v4];
 #pragma unroll
         for (int g2 = 1; g2 < NG; ++g2) {
           const float4 t = reinterpret_cast<const float4*>(ysum + (size_t)g2 * D)[v4];
           s.x += t.x; s.y += t.y; s.z += t.z; s.w += t.w;
         }
-        // layer form run in place on the residual stream: the block's share of y goes straight into it (every
-        // block read its input before the grid barrier), and there is nothing left to round at the end
+        // layer form run in place on the residual stream: the block's share of y goes straight into it, and there is
+        // nothing left to round at the end
         atomicAdd(reinterpret_cast<float4*>((NORM && p.xres_out == p.xres) ? p.xres_out : p.yacc) + v4, s);
       }
     }
@@ -1549,6 +1574,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       }
     }
     __syncthreads();
+    if (warp == 0) tmem_free_all(sm.tmem_base);
     leave();
     return;
   }
@@ -1596,9 +1622,12 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   }
   if (next_shr >= NSH) break;
   __syncthreads();                              // everyone has read what is reset here
-  if (tid == 0) { sm.shr = next_shr; sm.ncand2 = 0; sm.next_c = 0; sm.go = 0; sm.nready = 0; sm.n_mine = 0; sm.keys_done = 0; sm.c_done = 0; }
+  if (tid == 0) { sm.shr = next_shr; sm.ncand2 = 0; sm.next_c = 0; sm.nready = 0; sm.n_mine = 0; sm.c_done = 0; }
   __syncthreads();
   }
+  }
+  if (warp == 0) tmem_free_all(sm.tmem_base);
+  if (MODE == kScoresOnly && tid == 0 && sm.abort_flag) { atomicOr(p.status, kWaitExpired); if (p.host_flag) *reinterpret_cast<volatile int*>(p.host_flag) = 1; }
   leave();
 }
 
