@@ -59,7 +59,7 @@ struct prox_ffn {
   unsigned long long* counters;  // [0] tokens, [1] kept inputs, [2] kept channels
   unsigned* syncbuf;        // fused kernel: [0..4095] two score histograms (calls alternate), [4096..4097] 64-bit count
                             // of blocks that have left, [4104..4119] two sets of share counters
-  unsigned* xkeys;          // persistent kernel: [2][F] scores as its blocks hand them to each other, kNoKey between calls
+  uint16_t* xhalf; unsigned* xkeys;   // persistent kernel: [2][F] upper halves and all bits of the scores, as its blocks hand them to each other
   int smem_optin;           // largest dynamic shared memory a block may ask for
   int debug_grid;           // test knob: blocks of the persistent kernel and of the batch gate/up ring kernel (0 = one per SM)
   int sel_unordered;        // the last forward left its mask in the persistent kernel's own order
@@ -763,7 +763,7 @@ prox_status_t launch_fused(prox_ffn* h, const FusedPlan& pl, const void* x, int 
   prm.out_fp32 = h->cfg.out_dtype;
   prm.loaders = pl.loaders > 0 ? pl.loaders : 1;
   prm.plines = pl.plines; prm.pleft0 = pl.pleft0; prm.ppart = pl.ppart; prm.pmore = pl.pmore; prm.cgran = pl.cgran;
-  prm.scores = scores ? scores : h->scores; prm.ghist = h->syncbuf; prm.xkeys = h->xkeys; prm.idx_out = h->idx_x;
+  prm.scores = scores ? scores : h->scores; prm.ghist = h->syncbuf; prm.xkeys = h->xkeys; prm.xhalf = h->xhalf; prm.idx_out = h->idx_x;
   prm.spin_limit = h->spin_limit; prm.bar_bias = h->bar_bias; prm.host_flag = h->host_flag_dev;
   prm.sel_out = sel_out; prm.yacc = h->yacc;
   prm.exits = reinterpret_cast<unsigned long long*>(h->syncbuf + 4096); prm.ctr = h->syncbuf + 4104;
@@ -825,6 +825,7 @@ prox_status_t reset_shared_state(prox_ffn* h, cudaStream_t st) {
   const int ns_max = nstrips_for(h->cfg.d_ff, 8);
   CK(cudaMemsetAsync(h->syncbuf, 0, (4096 + 64) * sizeof(unsigned), st));
   CK(cudaMemsetAsync(h->xkeys, 0xff, (size_t)2 * h->cfg.d_ff * sizeof(unsigned), st));
+  CK(cudaMemsetAsync(h->xhalf, 0xff, (size_t)2 * h->cfg.d_ff * sizeof(uint16_t), st));
   CK(cudaMemsetAsync(h->ticket, 0, (size_t)h->cfg.max_batch * ns_max * sizeof(unsigned), st));
   CK(cudaMemsetAsync(h->yacc, 0, (size_t)h->cfg.max_batch * h->cfg.d_model * sizeof(float), st));
   if (h->gacc) {                               // accumulators of the tensor-core batch path (kept at zero between calls)
@@ -893,7 +894,7 @@ prox_status_t prox_ffn_create(const prox_ffn_config_t* cfg, const void* w_gate, 
   A(dev_alloc(&h->dev_status, (size_t)1));
   A(dev_alloc(&h->counters, (size_t)4));
   A(dev_alloc(&h->syncbuf, (size_t)4096 + 64));
-  A(dev_alloc(&h->xkeys, (size_t)2 * F));
+  A(dev_alloc(&h->xkeys, (size_t)2 * F)); A(dev_alloc(&h->xhalf, (size_t)2 * F));
   if (MB > 1) {
     A(dev_alloc(&h->u_in, (size_t)D)); A(dev_alloc(&h->u_ch, (size_t)F)); A(dev_alloc(&h->u_cnt, (size_t)4));
     A(dev_alloc(&h->xu, (size_t)D * kBT)); A(dev_alloc(&h->member, (size_t)F * kBT));
@@ -921,6 +922,7 @@ prox_status_t prox_ffn_create(const prox_ffn_config_t* cfg, const void* w_gate, 
   if (st == PROX_OK) {
     A(cudaMemset(h->syncbuf, 0, (4096 + 64) * sizeof(unsigned)));
     A(cudaMemset(h->xkeys, 0xff, (size_t)2 * F * sizeof(unsigned)));
+    A(cudaMemset(h->xhalf, 0xff, (size_t)2 * F * sizeof(uint16_t)));
   }
   A(dev_alloc(reinterpret_cast<uint16_t**>(&h->x_stage), (size_t)MB * D));
   A(dev_alloc(reinterpret_cast<float**>(&h->y_stage), (size_t)MB * D));
@@ -940,7 +942,7 @@ void prox_ffn_destroy(prox_ffn_t* h) {
   free_packed(h);
   cudaFree(h->idx_x); cudaFree(h->cnt_x); cudaFree(h->part); cudaFree(h->ticket);
   cudaFree(h->scores); cudaFree(h->svals); cudaFree(h->xn); cudaFree(h->sel); cudaFree(h->cnt_s); cudaFree(h->hbuf);
-  cudaFree(h->yacc); cudaFree(h->dev_status); cudaFree(h->counters); cudaFree(h->syncbuf); cudaFree(h->xkeys); cudaFree(h->trace);
+  cudaFree(h->yacc); cudaFree(h->dev_status); cudaFree(h->counters); cudaFree(h->syncbuf); cudaFree(h->xkeys); cudaFree(h->xhalf); cudaFree(h->trace);
   cudaFree(h->u_in); cudaFree(h->u_ch); cudaFree(h->u_cnt); cudaFree(h->xu); cudaFree(h->member); cudaFree(h->hb); cudaFree(h->gacc); cudaFree(h->pacc); cudaFree(h->tokfac); cudaFree(h->xd); cudaFree(h->soffb); cudaFree(h->cmask); cudaFree(h->umask);
   cudaFree(h->x_stage); cudaFree(h->y_stage);
   if (h->host_flag) cudaFreeHost(h->host_flag);

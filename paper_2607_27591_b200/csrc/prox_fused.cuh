@@ -50,8 +50,7 @@ constexpr int kMaxSlots = 32;
 constexpr int kEmptyCount = 16;      // arrivals that free a ring slot
 constexpr int kChanBatch = 256;      // channels whose h values are held at once
 constexpr int kMySelCap = 512;       // channels one block may own
-constexpr int kCand2Cap = 256;       // candidates left after the second refinement
-constexpr int kRankMax = 128;        // members of the threshold bin that are ranked directly
+constexpr int kCand2Cap = 256;       // members of the threshold bin that agree with the threshold in their half scores and are ranked (one per settler)
 // Proxy ring: a loader warp owns two stages of 32 rows x 128 bytes (4 KB each), for 4-bit codes a buffer of low
 // nibbles (4 KB), and two stages of digits of x (512 bytes each).
 __host__ __device__ constexpr int proxy_warp_bytes(int bits) { return bits == 4 ? 13312 : 9216; }
@@ -72,7 +71,9 @@ struct FusedParams {
   // ppart, in the first pmore shares cgran more
   int plines, pleft0, ppart, pmore, cgran;
   float* scores; unsigned* ghist; int* sel_out;
-  unsigned* xkeys;    // [2][F] the scores' bits as the blocks hand them to each other (calls alternate); kNoKey = not there yet
+  // What the blocks hand to each other, in two sets that calls take in turn (all ones = not there yet): the upper halves of
+  // the scores' bits (THRESH: per chunk of the proxy rows a word of marks, one bit per channel), and all bits.
+  uint16_t* xhalf; unsigned* xkeys;   // [2][F] each
   int* idx_out;       // the kept input list as this kernel built it (block 0 writes it; for checking)
   unsigned spin_limit;        // polls after which a device-side wait gives up
   unsigned bar_bias;          // test knob (0 in normal use): the wait for the scores does not end; bit 31: see prox_debug_set_wait
@@ -96,8 +97,6 @@ struct FusedParams {
 };
 
 constexpr unsigned kNoKey = 0xffffffffu;      // no score: those have the sign bit clear
-constexpr int kKeyQuads = 8;                   // groups of four scores that a consumer thread reads at once
-
 // shares claimed / finished, Stage 1 and Stage 2; kOut1: Stage-1 shares whose scores are on their way
 enum FusedCtr { kClaim1 = 0, kDone1, kClaim2, kDone2, kOut1 };
 
@@ -158,6 +157,11 @@ __device__ __forceinline__ uint4 ld_relaxed4(const unsigned* p) {
   uint4 v;
   asm volatile("ld.relaxed.gpu.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
   return v;
+}
+__device__ __forceinline__ unsigned every_other_bit(unsigned v) {          // bits 0..7 to bits 0, 2, .., 14
+  v = (v | (v << 4)) & 0x0f0fu;
+  v = (v | (v << 2)) & 0x3333u;
+  return (v | (v << 1)) & 0x5555u;
 }
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
@@ -220,7 +224,7 @@ __device__ __forceinline__ bool slot_wait(uint32_t bar, volatile unsigned* seen,
 // lane and trip) and the helpers below are shared between the phases.
 
 __device__ __forceinline__ unsigned warp_scan_incl(unsigned v, int lane) {
-#pragma unroll 1
+#pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const unsigned t = __shfl_up_sync(0xffffffffu, v, o);
     if (lane >= o) v += t;
@@ -311,9 +315,11 @@ struct FusedSmem {
   unsigned next_c;         // next channel of the batch to take in the gate/up phase
   int n_mine;              // channels of this block (for the producer warps)
   int nready;              // entries of mysel that are final (the definite share first, all of them later)
-  int c_done;              // the consumer warps no longer read the list of the threshold bin's members
-  int list_s0, list_s1;    // ring slots [s0, s1) that overlap it
-  unsigned poll[2][kFusedConsumerWarps];   // the warps' counts of scores (top bit: a key is missing), two rounds in turn
+  int keys_done;           // the consumer warps no longer read the keys near the end of the big buffer
+  int c_done;              // ... nor the list of the threshold bin's members
+  int keys_s0, keys_s1;    // ring slots [s0, s1) that overlap the keys
+  int list_s0, list_s1;    // ... and the list
+  unsigned poll[2][kFusedConsumerWarps];   // the warps' counts of scores in the histogram; and whether scores are missing
   unsigned slot_use[kMaxSlots];   // uses of each ring slot whose data has been seen complete
   unsigned long long pempty[kFusedConsumerWarps];   // proxy ring: the MMAs of a warp's block are complete
   unsigned long long acc_bar;            // all MMAs of a tile are complete (one arrival per loader warp)
@@ -377,6 +383,12 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   const unsigned lt_mask = (1u << lane) - 1u;
   const unsigned spin = p.spin_limit;
 
+  auto prefetch_row = [&](int i) {              // row i of the packed proxy to L2, by a warp
+    const int prow = F / CH * 16;
+    const uint8_t* src = p.P + (size_t)i * (size_t)prow;
+#pragma unroll 1
+    for (int o = lane * 32; o < prow; o += 1024) asm volatile("prefetch.global.L2 [%0];" ::"l"(src + o) : "memory");
+  };
   // ------------------------------------------------------------------ set-up
   PROX_TRACE(0);
   if (tid < kMaxSlots) {
@@ -433,6 +445,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
         }
       }
     }
+#pragma unroll 1
     for (int i = tid; i < 1024 + 32; i += NT) { if (i < 1024) sm.hist[i] = 0; else sm.hist2[i - 1024] = 0; }
     f2_warp_sum(hi, lo);
     if (lane == 0) { sm.nsum[warp][0] = hi; sm.nsum[warp][1] = lo; }
@@ -452,7 +465,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     }
   } else {
     const uint4* xg = reinterpret_cast<const uint4*>(p.x);
+#pragma unroll 1
     for (int i = tid; i < D / 8; i += NT) reinterpret_cast<uint4*>(xs)[i] = __ldg(xg + i);
+#pragma unroll 1
     for (int i = tid; i < 1024 + 32; i += NT) { if (i < 1024) sm.hist[i] = 0; else sm.hist2[i - 1024] = 0; }
   }
   tc_fence_before();
@@ -461,6 +476,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   unsigned* const ghist = p.ghist + 2048u * sm.call_par;
   unsigned* const ctr = p.ctr + 8u * sm.call_par;
   unsigned* const xkeys = p.xkeys + (size_t)F * sm.call_par;
+  uint16_t* const xhalf = p.xhalf + (size_t)F * sm.call_par;
   // Stage-1 share of this block; the answers are first looked at after phase A.  A block that gets none and finds
   // Stage 1 complete has started late: it leaves (what it read may be a residual stream that is being added to).
   unsigned claim1 = 0, done1 = 0;
@@ -471,11 +487,14 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   {
     unsigned* const other = p.ghist + 2048u * (sm.call_par ^ 1u);
     const int per = (2048 + G - 1) / G;
+#pragma unroll 1
     for (int i = cta * per + tid; i < min(2048, (cta + 1) * per); i += NT) other[i] = 0u;
     if (cta == 0 && tid < 8) p.ctr[8u * (sm.call_par ^ 1u) + tid] = 0u;
     unsigned* const okeys = p.xkeys + (size_t)F * (sm.call_par ^ 1u);
+    uint16_t* const ohalf = p.xhalf + (size_t)F * (sm.call_par ^ 1u);
     const int perk = (F + G - 1) / G;
-    for (int i = cta * perk + tid; i < min(F, (cta + 1) * perk); i += NT) okeys[i] = kNoKey;
+#pragma unroll 1
+    for (int i = cta * perk + tid; i < min(F, (cta + 1) * perk); i += NT) { okeys[i] = kNoKey; ohalf[i] = 0xffffu; }
   }
   if (warp < 4 && MODE != kGivenList) {
     // the accumulators of the proxy GEMV start at zero: 16 columns per supergroup, two sets 256 columns apart
@@ -531,80 +550,73 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       find_kth<2, false>(sm, hb, 1023 - 2 * tid, (unsigned)k1, lane, warp);
       const unsigned bin1 = sm.res[0], above1 = sm.res[1];
       PROX_TRACE(11);
-      // Inputs whose magnitude lies in a bin above the threshold bin are kept whatever the exact threshold:
-      // their packed proxy rows are pulled into L2 now (every block a share of them, one bulk prefetch per
-      // row), a few microseconds before the proxy GEMV asks for them.
-      if (warp >= kFusedConsumerWarps) {
-        const size_t prow = (size_t)(F / CH) * 16;
+      if (warp < kFusedConsumerWarps) {
 #pragma unroll 1
-        for (int i = cta + (tid - kFusedConsumers) * G; i < D; i += G * 32 * kFusedProducers)
-          if ((((unsigned)xs[i] & 0x7fffu) >> 5) > bin1)
-            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.P + (size_t)i * prow), "r"((uint32_t)prow) : "memory");
+        for (int i = tid; i < D / 2; i += kFusedConsumers) {
+          const uint32_t w = xs32[i];
+          const unsigned ka = w & 0x7fffu, kb = (w >> 16) & 0x7fffu;
+          if ((ka >> 5) == bin1) atomicAdd(&sm.hist2[ka & 31u], 1u);
+          if ((kb >> 5) == bin1) atomicAdd(&sm.hist2[kb & 31u], 1u);
+        }
+        consumer_sync();
+        PROX_TRACE(12);
+        // the exact threshold among the bin's 32 values (every warp on its own)
+        const unsigned c = sm.hist2[31 - lane], inc = warp_scan_incl(c, lane), need = (unsigned)k1 - above1;
+        const int src = __ffs((int)__ballot_sync(0xffffffffu, inc >= need)) - 1;
+        T = (bin1 << 5) | (unsigned)(31 - src);
+        quota = need - __shfl_sync(0xffffffffu, inc - c, src);      // ties at T to accept, lowest index first
+        PROX_TRACE(13);
       }
-#pragma unroll 1
-      for (int i = tid; i < D / 2; i += NT) {
-        const uint32_t w = xs32[i];
-        const unsigned ka = w & 0x7fffu, kb = (w >> 16) & 0x7fffu;
-        if ((ka >> 5) == bin1) atomicAdd(&sm.hist2[ka & 31u], 1u);
-        if ((kb >> 5) == bin1) atomicAdd(&sm.hist2[kb & 31u], 1u);
-      }
-      __syncthreads();
-      PROX_TRACE(12);
-      unsigned above2;
-      const unsigned bin2 = kth_in_segment<1>(sm.hist2, 32, (unsigned)k1 - above1, lane, &above2);
-      T = (bin1 << 5) | bin2;
-      quota = (unsigned)k1 - above1 - above2;      // ties at T to accept, lowest index first
-      PROX_TRACE(13);
     }
     // Ordered compaction: a consumer thread owns a run of 8-input groups, counts its kept
     // inputs and its ties (packed in one word), and places them behind those of the threads
     // in front (one warp scan plus the totals of the warps in front).
-    const int ngrp = D / 8, gpt = (ngrp + kFusedConsumers - 1) / kFusedConsumers;
-    const int g0 = min(ngrp, tid * gpt), g1 = (tid < kFusedConsumers) ? min(ngrp, g0 + gpt) : g0;
-    unsigned cnt = 0, mk = 0;
+    if (warp < kFusedConsumerWarps) {
+      const int ngrp = D / 8, gpt = (ngrp + kFusedConsumers - 1) / kFusedConsumers;
+      const int g0 = min(ngrp, tid * gpt), g1 = min(ngrp, g0 + gpt);
+      unsigned cnt = 0, mk = 0;
 #pragma unroll 1
-    for (int g = g0; g < g1; ++g) {
-      const uint4 kv = *reinterpret_cast<const uint4*>(xs + g * 8);
-      const uint32_t w4[4] = {kv.x, kv.y, kv.z, kv.w};
+      for (int g = g0; g < g1; ++g) {
+        const uint4 kv = *reinterpret_cast<const uint4*>(xs + g * 8);
+        const uint32_t w4[4] = {kv.x, kv.y, kv.z, kv.w};
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const unsigned key = (w4[e >> 1] >> ((e & 1) * 16)) & 0x7fffu;
-        cnt += ((all || key > T) ? 1u : 0u) | ((!all && key == T) ? 0x10000u : 0u);
-        mk = max(mk, key);
+        for (int e = 0; e < 8; ++e) {
+          const unsigned key = (w4[e >> 1] >> ((e & 1) * 16)) & 0x7fffu;
+          cnt += (all || key > T) ? 1u : 0u;
+          if (!THRESH) cnt += (!all && key == T) ? 0x10000u : 0u;
+          mk = max(mk, key);
+        }
       }
-    }
-    const unsigned inc = warp_scan_incl(cnt, lane);
-    mk = __reduce_max_sync(0xffffffffu, mk);
-    if (lane == 31) { sm.wsum[warp] = inc; sm.wmax[warp] = mk; }
-    __syncthreads();
-    PROX_TRACE(14);
-    mk = __reduce_max_sync(0xffffffffu, (lane < kFusedWarps) ? sm.wmax[lane] : 0u);
-    ebase = max(max((int)(mk >> 7), 1) - 22, 1);
-    if (THRESH) {
-      k1 = (int)__reduce_add_sync(0xffffffffu, (lane < kFusedWarps) ? (sm.wsum[lane] & 0xffffu) : 0u);
-    }
-    {
-      const unsigned ex = __reduce_add_sync(0xffffffffu, (lane < warp) ? sm.wsum[lane] : 0u) + inc - cnt;
-      unsigned rg = ex & 0xffffu, re = ex >> 16;
+      const unsigned inc = warp_scan_incl(cnt, lane);
+      mk = __reduce_max_sync(0xffffffffu, mk);
+      if (lane == 31) { sm.wsum[warp] = inc; sm.wmax[warp] = mk; }
+      consumer_sync();
+      PROX_TRACE(14);
+      const unsigned before = __reduce_add_sync(0xffffffffu, (lane < warp) ? sm.wsum[lane] : 0u) + inc - cnt;
+      unsigned re = before >> 16, at = (before & 0xffffu) + min(re, quota);
       // (also, for the proxy GEMV: where every scale group starts in the list)
       const int gmask = per_row_a ? 0x7fffffff : ((1 << p.gshift) - 1);
 #pragma unroll 1
       for (int g = g0; g < g1; ++g) {
         const uint4 kv = *reinterpret_cast<const uint4*>(xs + g * 8);
         const uint32_t w4[4] = {kv.x, kv.y, kv.z, kv.w};
-        if (((g * 8) & gmask) == 0) sm.gstart[per_row_a ? 0 : ((g * 8) >> p.gshift)] = (int)(rg + min(re, quota));
+        if (((g * 8) & gmask) == 0) sm.gstart[per_row_a ? 0 : ((g * 8) >> p.gshift)] = (int)at;
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           const unsigned key = (w4[e >> 1] >> ((e & 1) * 16)) & 0x7fffu;
-          const bool gt = all || key > T, eq = !all && key == T;
-          if (gt || (eq && re < quota)) idx16[rg + min(re, quota)] = (uint16_t)(g * 8 + e);
-          rg += gt ? 1u : 0u; re += eq ? 1u : 0u;
+          bool keep = all || key > T;
+          if (!THRESH && !all && key == T) { keep = re < quota; ++re; }
+          if (keep) idx16[at] = (uint16_t)(g * 8 + e);
+          at += keep ? 1u : 0u;
         }
       }
+      if (THRESH) k1 = (int)__reduce_add_sync(0xffffffffu, (lane < kFusedConsumerWarps) ? (sm.wsum[lane] & 0xffffu) : 0u);
+      if (tid == 0) sm.gstart[per_row_a ? 1 : (D >> p.gshift)] = k1;
     }
-    if (tid == 0) sm.gstart[per_row_a ? 1 : (D >> p.gshift)] = k1;
     if (tid == NT - 1) { sm.vid = claim1; sm.late = done1 >= (unsigned)p.nshare1 && claim1 >= (unsigned)p.nshare1; }
     __syncthreads();
+    if (THRESH && warp >= kFusedConsumerWarps) k1 = (int)__reduce_add_sync(0xffffffffu, (lane < kFusedConsumerWarps) ? (sm.wsum[lane] & 0xffffu) : 0u);
+    ebase = max(max((int)(__reduce_max_sync(0xffffffffu, (lane < kFusedConsumerWarps) ? sm.wmax[lane] : 0u) >> 7), 1) - 22, 1);
   }
   if (sm.late) {
     if (warp == 0) tmem_free_all(sm.tmem_base);
@@ -671,10 +683,6 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       }
       __syncthreads();
       tc_fence_after();
-    }
-    if (HIST && warp < kFusedConsumerWarps) {  // the block's own score histogram (used after a consumer barrier)
-#pragma unroll 1
-      for (int i = tid; i < 512; i += kFusedConsumers) reinterpret_cast<uint4*>(sm.hist)[i] = make_uint4(0u, 0u, 0u, 0u);
     }
     const uint32_t ring = (smem_u32(xf) + 1023u) & ~1023u;
     const int NL = p.loaders;
@@ -848,22 +856,29 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
           const float u0 = __shfl_xor_sync(0xffffffffu, t0, 8), u1 = __shfl_xor_sync(0xffffffffu, t1, 8);
           unsigned n0 = 1u, n1 = 1u, b0 = 0u, b1 = 0u;          // (scores in front of this thread's in their bins)
           const bool give = MODE == kScoresOnly || *abortp == 0;          // a block that has given up hands nothing on
+          const float s0 = fabsf(u0 * silu_fast(t0)), s1 = LO ? fabsf(u1 * silu_fast(t1)) : 0.f;
+          const unsigned k0 = __float_as_uint(s0), k1b = __float_as_uint(s1);
+          if (MODE == kWhole && THRESH) {
+            // marks of a chunk: bit i = its channel i (4-bit codes: a lane has channels 2 i and 2 i + 1)
+            const unsigned m0 = __ballot_sync(0xffffffffu, k0 >= p.tkey_s) >> (lane & 16), m1 = LO ? __ballot_sync(0xffffffffu, k1b >= p.tkey_s) >> (lane & 16) : 0u;
+            if ((lane & 15) == 0 && col_ok && give) __stcg(reinterpret_cast<unsigned*>(xhalf) + chunk, LO ? every_other_bit(m0 & 0xffu) | (every_other_bit(m1 & 0xffu) << 1) : m0 & 0xffu);
+          }
           if ((col & 8) == 0 && col_ok && give) {
-            if (LO) {
-              const int ch = chunk * 16 + 2 * (col & 7);
-              const float s0 = fabsf(u0 * silu_fast(t0)), s1 = fabsf(u1 * silu_fast(t1));
-              if (MODE == kWhole) __stcg(reinterpret_cast<float2*>(xkeys + ch), make_float2(s0, s1));
-              __stcg(reinterpret_cast<float2*>(p.scores + ch), make_float2(s0, s1));
-              if (HIST) {
-                b0 = __float_as_uint(s0) >> 20; b1 = __float_as_uint(s1) >> 20;
-                n0 = atomicAdd(&sm.hist[b0], 1u); n1 = atomicAdd(&sm.hist[b1], 1u);
+            const int ch = chunk * CH + (LO ? 2 : 1) * (col & 7);
+            if (MODE == kWhole && !THRESH) {
+              if (LO) {
+                __stcg(reinterpret_cast<unsigned*>(xhalf + ch), __byte_perm(k0, k1b, 0x7632));
+                __stcg(reinterpret_cast<uint2*>(xkeys + ch), make_uint2(k0, k1b));
+              } else {
+                __stcg(reinterpret_cast<unsigned short*>(xhalf + ch), (unsigned short)(k0 >> 16));
+                __stcg(xkeys + ch, k0);
               }
-            } else {
-              const int ch = chunk * 8 + (col & 7);
-              const float s0 = fabsf(u0 * silu_fast(t0));
-              if (MODE == kWhole) __stcg(reinterpret_cast<float*>(xkeys + ch), s0);
-              __stcg(p.scores + ch, s0);
-              if (HIST) { b0 = __float_as_uint(s0) >> 20; n0 = atomicAdd(&sm.hist[b0], 1u); }
+            }
+            if (LO) __stcg(reinterpret_cast<float2*>(p.scores + ch), make_float2(s0, s1));
+            else __stcg(p.scores + ch, s0);
+            if (HIST) {
+              b0 = k0 >> 20; n0 = atomicAdd(&sm.hist[b0], 1u);
+              if (LO) { b1 = k1b >> 20; n1 = atomicAdd(&sm.hist[b1], 1u); }
             }
           }
           if (HIST) {
@@ -887,13 +902,16 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       }
     }
     else {
-      // Blocks without a column pull the kept rows into L2 (whole rows, one bulk prefetch each): the loader
+      // Blocks without a column pull the kept rows into L2 (a warp a row at a time): the loader
       // warps of the other blocks then find them there instead of waiting for HBM one by one.
-      if (vid >= n1 && first && lane < 8) {
-        const int nidle = max(G - (int)n1, 1), slot_i = (int)(vid - n1) * (kFusedProducers * 8) + (warp - kFusedConsumerWarps) * 8 + lane;
+      if (vid >= n1 && first) {
+        const int nidle = max(G - (int)n1, 1);
 #pragma unroll 1
-        for (int r = slot_i; r < k1; r += nidle * kFusedProducers * 8)
-          asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.P + (size_t)idx16[r] * (size_t)row_bytes), "r"((uint32_t)row_bytes) : "memory");
+        for (int r = (int)(vid - n1) * kFusedProducers + warp - kFusedConsumerWarps; r < k1; r += nidle * kFusedProducers) prefetch_row(idx16[r]);
+      }
+      if (HIST && first) {                     // the block's own score histogram (used behind the wait for soff_cnt)
+#pragma unroll 1
+        for (int i = tid - kFusedConsumers; i < 512; i += 32 * kFusedProducers) reinterpret_cast<uint4*>(sm.hist)[i] = make_uint4(0u, 0u, 0u, 0u);
       }
       // the other four warps: per scale group, offset * sum of the kept x as integers (for the codes' offset binary)
 #pragma unroll 1
@@ -936,7 +954,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   } else {
   // ---------------------------------------- C: channel mask (top-k2 of the scores)
   // The blocks wait for a count of finished shares that is not ordered behind the scores; the scores themselves say that
-  // they are there (kNoKey = not yet), and the histogram that it is complete (it counts all channels): what is missing is read
+  // they are there (all ones = not yet), and the histogram that it is complete (it counts all channels): what is missing is read
   // again.  (Ordered by a release, i.e. behind the acknowledgement of all the block's writes, the count came one trip to L2 later.)
   // The first histogram level tells which channels are kept whatever the exact
   // threshold turns out to be (their bin lies above the threshold bin b1:
@@ -947,17 +965,27 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   int n_mine = 0;
   unsigned nd = 0, b1 = 0, kk = 0, nb1 = 0;     // (THRESH: nd = the kept channels)
   unsigned cnt = 0, ex = 0;                     // packed: definite channels (low half) and members of b1 of this thread / in front of it
-  unsigned cm[4] = {0u, 0u, 0u, 0u};            // its members of b1 as bits: see below
-  const int nw = (F / 4 + kKeyQuads * kFusedConsumers - 1) / (kKeyQuads * kFusedConsumers);
-  auto chan = [&](int w, unsigned m) {          // channel of the lowest bit set in word w of this thread's masks
-    const int bit = __ffs((int)m) - 1;
-    return 4 * (((nw - 1 - w) * kKeyQuads + (bit >> 2)) * kFusedConsumers + tid) + (bit & 3);
-  };
-  bool staged = true;                           // the same in every block
-  const int nq = F / 4;
+  const int ngrp = THRESH ? F / CH / 4 : F / 8;  // 16-byte groups of half scores (THRESH: of mark words)
   const unsigned NSH = (unsigned)p.nshare;
   int ndm = 0, ncm = 0, Rc0 = 0, Rc1 = 0;
-  uint32_t list_u32 = smem_u32(idx16);          // members of b1: 2 * D bytes, room for D / 4 of them
+  // Shared-memory plan: the half scores (THRESH: marks) sit at the END of the big buffer (the ring fills from slot 0 and
+  // reaches those slots last); the list of b1's members goes where the input index list was (free since phase B), or in
+  // front of the half scores if it is long.  Consumer thread t owns the groups t, t + 512, ... (THRESH: a run of them, so
+  // that the list is ascending)
+  const int q0 = THRESH ? tid * ((ngrp + kFusedConsumers - 1) / kFusedConsumers) : tid, qstep = THRESH ? 1 : kFusedConsumers;
+  const int qend = THRESH ? min(ngrp, q0 + (ngrp + kFusedConsumers - 1) / kFusedConsumers) : ngrp;
+  const bool in_smem = (size_t)F * 2 + 256 <= (size_t)p.big_bytes;
+  const uint32_t key_off = in_smem ? (((uint32_t)p.big_bytes - (uint32_t)ngrp * 16u) & ~127u) : 0u;
+  const uint32_t skey_u32 = big_u32 + key_off;
+  uint32_t list_u32 = smem_u32(idx16);          // 2 * D bytes: room for D / 2 members
+  unsigned klo = 0, khi = 0;                    // half scores from khi on are definite, from klo on members of b1
+  auto full_key = [&](int i) {                  // all bits of a score
+    unsigned v = kNoKey;
+#pragma unroll 1
+    for (unsigned it = 0; v == kNoKey && it < spin; ++it)
+      asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(xkeys + i) : "memory");
+    return v;
+  };
   if (warp >= kFusedConsumerWarps) {
     if (MODE == kWhole && with_b) {
       // (in the layer form in place, the blocks wait for this count before they add to the residual stream that others read)
@@ -976,11 +1004,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       if (j < 0 || j >= F) atomicOr(p.status, kBadChannel);
       sm.mysel[i] = (j < 0 || j >= F) ? -1 : j;
     }
-    if (tid == 0) { sm.list_s0 = sm.list_s1 = 0; sm.n_mine = n_mine; sm.nready = n_mine; sm.c_done = 1; }
+    if (tid == 0) { sm.keys_s0 = sm.keys_s1 = sm.list_s0 = sm.list_s1 = 0; sm.n_mine = n_mine; sm.nready = n_mine; sm.keys_done = 1; sm.c_done = 1; }
   } else if (sm.abort_flag == 0) {
-    auto missing = [](const uint4& v) { return v.x == kNoKey || v.y == kNoKey || v.z == kNoKey || v.w == kNoKey; };
     uint4 hv = make_uint4(0u, 0u, 0u, 0u);
-    uint4 kq[kKeyQuads];
     unsigned hsum = 0, hbase = 0;
     if (tid == 0) {
       unsigned more1 = (unsigned)p.nshare1, share2 = 0, out = 0;
@@ -1004,109 +1030,86 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     // anything is written to y or to the residual stream; neither are they with the test knob)
     const unsigned target = (p.bar_bias & 0x7fffffffu) ? ~0u : (THRESH ? 0u : (unsigned)F);
     const unsigned tries = !again && sm.res[7] ? spin : 0u;
-#pragma unroll
-    for (int j = 0; j < kKeyQuads; ++j) kq[j] = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll 1
     for (unsigned it = 0; it < tries; ++it) {
       if (!THRESH) hv = ld_relaxed4(ghist + 4 * (511 - tid));
-      bool bad = false;
-#pragma unroll
-      for (int j = 0; j < kKeyQuads; ++j) {
-        const int q = j * kFusedConsumers + tid;
-        if (q < nq) kq[j] = ld_relaxed4(xkeys + 4 * q);
+      if (in_smem) {
+#pragma unroll 1
+        for (int q = q0; q < qend; q += qstep) cp_async16(skey_u32 + (uint32_t)q * 16u, xhalf + 8 * q);
       }
-#pragma unroll
-      for (int j = 0; j < kKeyQuads; ++j) bad |= missing(kq[j]);
+      cp_async_commit();
+      if (tid < 256) sm.hist2[tid] = 0;
       hsum = hv.x + hv.y + hv.z + hv.w;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) { const unsigned t = __shfl_up_sync(0xffffffffu, hsum, o); if (lane >= o) hsum += t; }
-      bad = __any_sync(0xffffffffu, bad);
-      if (lane == 31) sm.poll[it & 1u][warp] = hsum | (bad ? 0x80000000u : 0u);
+      if (lane == 31) sm.poll[0][warp] = hsum;
       consumer_sync();
-      const unsigned pv = lane < kFusedConsumerWarps ? sm.poll[it & 1u][lane] : 0u;
-      const unsigned tot = __reduce_add_sync(0xffffffffu, pv & 0x7fffffffu);
-      hbase = __reduce_add_sync(0xffffffffu, lane < warp ? pv & 0x7fffffffu : 0u);
-      if (tot == target && !__any_sync(0xffffffffu, pv >> 31)) { ok = true; break; }
+      const unsigned pv = lane < kFusedConsumerWarps ? sm.poll[0][lane] : 0u;
+      const unsigned tot = __reduce_add_sync(0xffffffffu, pv);
+      hbase = __reduce_add_sync(0xffffffffu, lane < warp ? pv : 0u);
+      if (tot != target) { cp_async_wait<0>(); consumer_sync(); continue; }
+      if (!THRESH) {
+        // the bin of the k2-th score: thread t has the counts of four bins in descending order, the threads' runs follow
+        // each other downwards
+        unsigned run = hbase + hsum - (hv.x + hv.y + hv.z + hv.w);
+        if (run < (unsigned)k2 && (unsigned)k2 <= hbase + hsum) {
+          unsigned c = hv.w, bin = 2047u - 4u * (unsigned)tid;
+          if (run + c < (unsigned)k2) { run += c; c = hv.z; --bin; }
+          if (run + c < (unsigned)k2) { run += c; c = hv.y; --bin; }
+          if (run + c < (unsigned)k2) { run += c; c = hv.x; --bin; }
+          sm.res[0] = bin; sm.res[1] = run; sm.res[2] = c;
+        }
+        consumer_sync();
+        b1 = sm.res[0]; nd = sm.res[1]; nb1 = sm.res[2];
+        kk = (unsigned)k2 - nd;                              // members of b1 to keep (>= 1)
+      }
+      PROX_TRACE(16);
+      // a consumer thread counts its definite channels and its members of b1
+      klo = b1 << 4; khi = (b1 + 1u) << 4;
+      unsigned from_lo = 0, from_hi = 0, any = 0;
+      cp_async_wait<0>();
+#pragma unroll 1
+      for (int q = q0; q < qend; q += qstep) {
+        const uint4 v = in_smem ? lds128(skey_u32 + (uint32_t)q * 16u) : ld_relaxed4(reinterpret_cast<const unsigned*>(xhalf) + 4 * q);
+        any |= v.x | v.y | v.z | v.w;
+        const unsigned w4[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          if (THRESH) {
+            from_hi += (unsigned)__popc(w4[e] & 0xffffu);
+          } else {
+            from_hi += (w4[e] >= khi << 16 ? 1u : 0u) + (w4[e] << 16 >= khi << 16 ? 1u : 0u);
+            from_lo += (w4[e] >= klo << 16 ? 1u : 0u) + (w4[e] << 16 >= klo << 16 ? 1u : 0u);
+          }
+        }
+      }
+      if (THRESH) from_lo = from_hi;
+      cnt = from_hi | ((from_lo - from_hi) << 16);
+      ex = cnt;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) { const unsigned t = __shfl_up_sync(0xffffffffu, ex, o); if (lane >= o) ex += t; }
+      const bool bad = __any_sync(0xffffffffu, any & (THRESH ? 0x80000000u : 0x80008000u));     // the sign of what is not there
+      if (lane == 31) { sm.wsum[warp] = ex; sm.poll[1][warp] = bad ? 1u : 0u; }
+      consumer_sync();
+      if (!__any_sync(0xffffffffu, lane < kFusedConsumerWarps && sm.poll[1][lane] != 0u)) { ok = true; break; }
+      consumer_sync();
     }
     PROX_TRACE(4);
     if (!ok) {
       if (!again && tid == 0) { sm.abort_flag = 1; atomicOr(p.status, kWaitExpired); if (p.host_flag) *reinterpret_cast<volatile int*>(p.host_flag) = 1; }
     } else {
       const unsigned shr = sm.shr;
-      if (!THRESH) {
-        // the bin of the k2-th score: thread t has the counts of four bins in descending order, the threads' runs follow
-        // each other downwards
-        unsigned run = hbase + hsum - (hv.x + hv.y + hv.z + hv.w);
-        const unsigned c4[4] = {hv.w, hv.z, hv.y, hv.x};
-        if (run < (unsigned)k2 && (unsigned)k2 <= hbase + hsum) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            if (run < (unsigned)k2 && (unsigned)k2 <= run + c4[j]) { sm.res[0] = (unsigned)(2047 - 4 * tid - j); sm.res[1] = run; sm.res[2] = c4[j]; }
-            run += c4[j];
-          }
-        }
-        if (tid < 256) sm.hist2[tid] = 0;
-        consumer_sync();
-        b1 = sm.res[0]; nd = sm.res[1]; nb1 = sm.res[2];
-        kk = (unsigned)k2 - nd;                              // members of b1 to keep (>= 1)
-      }
-      PROX_TRACE(16);
+      ex = __reduce_add_sync(0xffffffffu, (lane < warp) ? sm.wsum[lane] : 0u) + ex - cnt;
       uint32_t list_off = 0;                                 // offset in the big buffer when the list has to go there
       bool list_in_big = false;
-      if ((size_t)nb1 * 8 > (size_t)D * 2) {
-        if ((size_t)nb1 * 8 + 128 <= (size_t)p.big_bytes) {
-          list_off = ((uint32_t)p.big_bytes - nb1 * 8u) & ~127u; list_u32 = big_u32 + list_off; list_in_big = true;
+      bool staged = in_smem;                                 // the same in every block
+      if (in_smem && (size_t)nb1 * 4 > (size_t)D * 2) {
+        if ((size_t)nb1 * 4 + 128 <= (size_t)key_off) {
+          list_off = (key_off - nb1 * 4u) & ~127u; list_u32 = big_u32 + list_off; list_in_big = true;
         } else {
           staged = false;
         }
       }
-      // a consumer thread counts its definite channels and its members of b1 and keeps them as bit masks (word 0: the last
-      // kKeyQuads groups of scores that it has read, word 1 the ones before, ...)
-      unsigned dm[4] = {0u, 0u, 0u, 0u};
-#pragma unroll 1
-      for (int w = 0;;) {
-#pragma unroll
-        for (int j = 3; j > 0; --j) { dm[j] = dm[j - 1]; cm[j] = cm[j - 1]; }
-        dm[0] = cm[0] = 0u;
-#pragma unroll
-        for (int j = 0; j < kKeyQuads; ++j) {
-          const unsigned k4[4] = {kq[j].x, kq[j].y, kq[j].z, kq[j].w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            if (THRESH) {
-              if (k4[e] >= p.tkey_s) dm[0] |= 1u << (4 * j + e);
-            } else {
-              const unsigned bin = k4[e] >> 20;
-              if (bin > b1) dm[0] |= 1u << (4 * j + e);
-              if (bin == b1) cm[0] |= 1u << (4 * j + e);
-            }
-          }
-          if ((w * kKeyQuads + j) * kFusedConsumers + tid >= nq) { dm[0] &= ~(15u << (4 * j)); cm[0] &= ~(15u << (4 * j)); }
-        }
-        if (++w * kKeyQuads * kFusedConsumers >= nq) break;
-        bool bad = true;                                     // d_ff > 16384
-#pragma unroll 1
-        for (unsigned it = 0; bad && it < spin; ++it) {      // (in the top-k form they are there: their counts are)
-          bad = false;
-#pragma unroll
-          for (int j = 0; j < kKeyQuads; ++j) {
-            const int q = (w * kKeyQuads + j) * kFusedConsumers + tid;
-            kq[j] = q < nq ? ld_relaxed4(xkeys + 4 * q) : make_uint4(0u, 0u, 0u, 0u);
-          }
-#pragma unroll
-          for (int j = 0; j < kKeyQuads; ++j) bad |= missing(kq[j]);
-        }
-        if (bad) sm.abort_flag = 1;
-      }
-      cnt = (unsigned)(__popc(dm[0]) + __popc(dm[1]) + __popc(dm[2]) + __popc(dm[3])) |
-            ((unsigned)(__popc(cm[0]) + __popc(cm[1]) + __popc(cm[2]) + __popc(cm[3])) << 16);
-      unsigned inc = cnt;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) { const unsigned t = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += t; }
-      if (lane == 31) sm.wsum[warp] = inc;
-      consumer_sync();
-      PROX_TRACE(18);
-      ex = __reduce_add_sync(0xffffffffu, (lane < warp) ? sm.wsum[lane] : 0u) + inc - cnt;
       if (THRESH) {
         nd = __reduce_add_sync(0xffffffffu, (lane < kFusedConsumerWarps) ? (sm.wsum[lane] & 0xffffu) : 0u);
         if (shr == 0 && tid == 0) {
@@ -1125,29 +1128,44 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
         n_mine = ndm + ncm;
         if (tid == 0) {
           const uint32_t rb = (uint32_t)D * 2u;
+          sm.keys_s0 = (int)(key_off / rb); sm.keys_s1 = (int)((key_off + (uint32_t)ngrp * 16u + rb - 1u) / rb);
           sm.list_s0 = list_in_big ? (int)(list_off / rb) : 0;
-          sm.list_s1 = list_in_big ? (int)((list_off + nb1 * 8u + rb - 1u) / rb) : 0;
-          sm.n_mine = n_mine; sm.nready = ndm; sm.c_done = (ncm == 0) ? 1 : 0;
+          sm.list_s1 = list_in_big ? (int)((list_off + nb1 * 4u + rb - 1u) / rb) : 0;
+          sm.n_mine = n_mine; sm.nready = ndm; sm.keys_done = sm.c_done = (ncm == 0) ? 1 : 0;
         }
-        // the threads whose definite channels meet the block's share write them out
-        int dpos = (int)(ex & 0xffffu);
-        const int cdef = (int)(cnt & 0xffffu);
-        if (cdef > 0 && dpos < Rd1 && dpos + cdef > Rd0) {
-#pragma unroll
-          for (int w = 0; w < 4; ++w) {
+        // the threads whose definite channels meet the block's share (a few neighbours): their warp lists them, one
+        // thread's channels after the other
+        const int dpos = (int)(ex & 0xffffu), cdef = (int)(cnt & 0xffffu);
+        constexpr int GC = THRESH ? 4 * CH : 8;              // channels of a group
+        const int nel = (THRESH ? (ngrp + kFusedConsumers - 1) / kFusedConsumers : (ngrp - warp * 32 + kFusedConsumers - 1) / kFusedConsumers) * GC;
 #pragma unroll 1
-            for (unsigned m = dm[w]; m; m &= m - 1) {
-              if (dpos >= Rd0 && dpos < Rd1) {
-                const int ch = chan(w, m);
-                sm.mysel[dpos - Rd0] = ch;
-                if (p.sel_out) p.sel_out[dpos] = ch;
+        for (unsigned lanes = __ballot_sync(0xffffffffu, cdef > 0 && dpos < Rd1 && dpos + cdef > Rd0); lanes; lanes &= lanes - 1) {
+          const int l = __ffs((int)lanes) - 1;
+          int at = __shfl_sync(0xffffffffu, dpos, l) - Rd0;
+          const int ql = __shfl_sync(0xffffffffu, q0, l);
+#pragma unroll 1
+          for (int i = lane; i < ((nel + 31) & ~31); i += 32) {
+            const int q = ql + (i / GC) * qstep, c = i % GC;
+            bool def = i < nel && q < ngrp;
+            if (def) {
+              unsigned v;
+              if (THRESH) {
+                asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(skey_u32 + (uint32_t)(q * 16 + (c / CH) * 4)));
+                def = (v >> (c % CH)) & 1u;
+              } else {
+                asm volatile("{\n\t.reg .u16 h;\n\tld.shared.u16 h, [%1];\n\tcvt.u32.u16 %0, h;\n\t}" : "=r"(v) : "r"(skey_u32 + (uint32_t)(q * 16 + c * 2)));
+                def = v >= khi;
               }
-              ++dpos;
             }
+            const unsigned b = __ballot_sync(0xffffffffu, def);
+            const int pos = at + __popc(b & lt_mask);
+            if (def && pos >= 0 && pos < ndm) sm.mysel[pos] = q * GC + c;
+            at += __popc(b);
           }
         }
       } else if (shr < NSH) {
-        // No room in shared memory for the list of b1's members (a huge threshold bin such as an all-zero input gives):
+        // No room in shared memory for the keys plus the list of b1's members (a very large d_ff, or a huge threshold bin such
+        // as an all-zero input gives):
         // the consumer warps settle the threshold by two radix steps of 10 bits over all keys and the block keeps its
         // share of the plain ascending list before the ring starts.
         const int R0 = (int)(((unsigned)k2 * shr) / NSH), R1 = (int)(((unsigned)k2 * (shr + 1u)) / NSH);
@@ -1158,11 +1176,12 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
 #pragma unroll 1
         for (int sh = 10; sh >= 0; sh -= 10) {
           consumer_sync();
+#pragma unroll 1
           for (int i = tid; i < 1024; i += kFusedConsumers) sm.hist[i] = 0;
           consumer_sync();
 #pragma unroll 1
           for (int i = tid; i < F; i += kFusedConsumers) {
-            const unsigned key = __ldcg(xkeys + i);
+            const unsigned key = full_key(i);
             if ((key >> (sh + 10)) == prefix) atomicAdd(&sm.hist[(key >> sh) & 1023u], 1u);
           }
           consumer_sync();
@@ -1177,7 +1196,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
           unsigned cg = 0, ce = 0;                 // separate words: the ties alone may be 65536
 #pragma unroll 1
           for (int i = i0 + lane; i < i1; i += 32) {
-            const unsigned key = __ldcg(xkeys + i);
+            const unsigned key = full_key(i);
             cg += (key > T) ? 1u : 0u; ce += (key == T) ? 1u : 0u;
           }
           cg = __reduce_add_sync(0xffffffffu, cg);
@@ -1194,7 +1213,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
 #pragma unroll 1
             for (int ib = i0; ib < i1; ib += 32) {
               const int i = ib + lane;
-              const unsigned key = __ldcg(xkeys + min(i, F - 1));
+              const unsigned key = full_key(min(i, F - 1));
               const bool gt = i < i1 && key > T, eq = i < i1 && key == T;
               const unsigned mg = __ballot_sync(0xffffffffu, gt), me = __ballot_sync(0xffffffffu, eq);
               const unsigned myre = be + (unsigned)__popc(me & lt_mask);
@@ -1207,7 +1226,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
             }
           }
         }
-        if (tid == 0) { sm.list_s0 = sm.list_s1 = 0; sm.n_mine = n_mine; sm.nready = n_mine; sm.c_done = 1; }
+        if (tid == 0) { sm.keys_s0 = sm.keys_s1 = sm.list_s0 = sm.list_s1 = 0; sm.n_mine = n_mine; sm.nready = n_mine; sm.keys_done = 1; sm.c_done = 1; }
       }
     }
   }
@@ -1217,20 +1236,29 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   if (MODE == kWhole && alive && with_b && sm.again) continue;      // one more share of Stage 1
   with_b = false;
   if (alive && sm.shr >= NSH) break;
+  if (MODE == kWhole && alive && p.sel_out && warp == kFusedConsumerWarps - 1 && ndm > 0) {       // the mask, for prox_ffn_last_mask
+    const int Rd0 = (int)((nd * sm.shr) / NSH);
+#pragma unroll 1
+    for (int i = lane; i < ndm; i += 32) p.sel_out[Rd0 + i] = sm.mysel[i];
+  }
   if (MODE == kWhole && !THRESH && warp < kFusedConsumerWarps && ncm > 0) {
-        // ---- consumer warps only: the list of b1's members ...
-        const uint32_t lkey_u32 = list_u32, lidx_u32 = lkey_u32 + nb1 * 4u;
+        // ---- consumer warps only: the list of b1's members (channel, and the four bits that its half score has below the
+        // bin's, with their histogram) ...
         auto lds32 = [](uint32_t a) -> unsigned { unsigned v; asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a)); return v; };
-        auto sts32 = [](uint32_t a, unsigned v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); };
         if (cnt >> 16) {
           unsigned cpos = ex >> 16;
-#pragma unroll
-          for (int w = 0; w < 4; ++w) {
 #pragma unroll 1
-            for (unsigned m = cm[w]; m; m &= m - 1) {
-              const int ch = chan(w, m);
-              if (cpos < nb1) { sts32(lkey_u32 + cpos * 4u, __ldcg(xkeys + ch)); sts32(lidx_u32 + cpos * 4u, (unsigned)ch); }
-              ++cpos;
+          for (int q = q0; q < qend; q += qstep) {
+            const uint4 v = lds128(skey_u32 + (uint32_t)q * 16u);
+            const unsigned w4[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              const unsigned h = e & 1 ? w4[e >> 1] >> 16 : w4[e >> 1] & 0xffffu;
+              if (h >= klo && h < khi) {
+                if (cpos < nb1) asm volatile("st.shared.u32 [%0], %1;" ::"r"(list_u32 + cpos * 4u), "r"((h & 15u) << 16 | (unsigned)(8 * q + e)) : "memory");
+                atomicAdd(&sm.hist2[h & 15u], 1u);
+                ++cpos;
+              }
             }
           }
         }
@@ -1239,47 +1267,47 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
         if (warp >= kSettlerWarps) {
           asm volatile("bar.arrive 2, %0;" ::"n"(kFusedConsumers) : "memory");
         } else {
-        asm volatile("bar.sync 2, %0;" ::"n"(kFusedConsumers) : "memory");      // the list is complete
+        asm volatile("bar.sync 2, %0;" ::"n"(kFusedConsumers) : "memory");      // the list is complete, the half scores are free
+        if (tid == 0) *reinterpret_cast<volatile int*>(&sm.keys_done) = 1;
         PROX_TRACE(15);
-        if (nb1 <= (unsigned)kRankMax) {
-          // ... few of them: a member's place is its rank by (score descending, channel ascending)
-          if (tid < (int)nb1) {
-            const unsigned key = lds32(lkey_u32 + (uint32_t)tid * 4u), id = lds32(lidx_u32 + (uint32_t)tid * 4u);
-            int pos = 0;
-#pragma unroll 4
-            for (unsigned c = 0; c < nb1; ++c) {
-              const unsigned okey = lds32(lkey_u32 + c * 4u), oid = lds32(lidx_u32 + c * 4u);
-              pos += (okey > key || (okey == key && oid < id)) ? 1 : 0;
-            }
-            if (pos < (int)kk && pos >= Rc0 && pos < Rc1) {
-              sm.mysel[ndm + pos - Rc0] = (int)id;
-              if (p.sel_out) p.sel_out[(int)nd + pos] = (int)id;
-            }
-          }
-        } else {
-        // ... settle the threshold inside b1: histogram of bits 19..12, then the few left ...
+        // ... the value of those bits at which the kk-th of them lies (every warp on its own): members above it are kept ...
+        const unsigned hc = lane < 16 ? sm.hist2[15 - lane] : 0u, hi = warp_scan_incl(hc, lane);
+        const int src = __ffs((int)__ballot_sync(0xffffffffu, hi >= kk)) - 1;
+        const unsigned sub = 15u - (unsigned)src, above = __shfl_sync(0xffffffffu, hi - hc, src), kk2 = kk - above;
+        const unsigned n2 = __shfl_sync(0xffffffffu, hc, src);
+        // ... in list order (a thread owns a run of the list), and of the n2 with that value those that rank among the first
+        // kk2 by (score descending, channel ascending), in that order
+        const int ept = ((int)nb1 + kSettlers - 1) / kSettlers;
+        const int c0 = min((int)nb1, tid * ept), c1 = min((int)nb1, c0 + ept);
+        unsigned wt = 0;
 #pragma unroll 1
-        for (unsigned c = tid; c < nb1; c += kSettlers)
-          atomicAdd(&sm.hist2[(lds32(lkey_u32 + c * 4u) >> 12) & 255u], 1u);
-        settler_sync();
-        unsigned above2;
-        const unsigned b2 = kth_in_segment<8>(sm.hist2, 256, kk, lane, &above2);     // every warp on its own
-        unsigned kk2 = kk - above2;
-        const unsigned pre2 = (b1 << 8) | b2;
-#pragma unroll 1
-        for (unsigned c = tid; c < nb1; c += kSettlers) {
-          const unsigned key = lds32(lkey_u32 + c * 4u);
-          if ((key >> 12) == pre2) {
+        for (int c = c0; c < c1; ++c) {
+          const unsigned e = lds32(list_u32 + (uint32_t)c * 4u);
+          wt += (e >> 16) > sub ? 1u : 0u;
+          if ((e >> 16) == sub && n2 <= (unsigned)kCand2Cap) {
             const unsigned slot = atomicAdd(&sm.ncand2, 1u);
-            if (slot < (unsigned)kCand2Cap) { sm.cand2_key[slot] = key; sm.cand2_idx[slot] = (int)lds32(lidx_u32 + c * 4u); }
+            sm.cand2_key[slot] = full_key((int)(e & 0xffffu)); sm.cand2_idx[slot] = (int)(e & 0xffffu);
           }
         }
+        const unsigned inc3 = warp_scan_incl(wt, lane);
+        if (lane == 31) sm.warp_cnt[warp][0] = inc3;
         settler_sync();
-        const unsigned n2 = sm.ncand2;
         PROX_TRACE(19);
-        unsigned T, tch;                         // score and channel of the last one kept
+        auto keep = [&](int pos, unsigned ch) {
+          if (pos >= Rc0 && pos < Rc1) {
+            sm.mysel[ndm + pos - Rc0] = (int)ch;
+            if (p.sel_out) p.sel_out[(int)nd + pos] = (int)ch;
+          }
+        };
+        int pos = (int)(__reduce_add_sync(0xffffffffu, lane < warp ? sm.warp_cnt[lane][0] : 0u) + inc3 - wt);
+        if (wt > 0 && pos < Rc1 && pos + (int)wt > Rc0) {
+#pragma unroll 1
+          for (int c = c0; c < c1; ++c) {
+            const unsigned e = lds32(list_u32 + (uint32_t)c * 4u);
+            if ((e >> 16) > sub) keep(pos++, e & 0xffffu);
+          }
+        }
         if (n2 <= (unsigned)kCand2Cap) {
-          // rank the few that are left by (score descending, channel ascending)
           if (tid < (int)n2) {
             const unsigned key = sm.cand2_key[tid];
             const int id = sm.cand2_idx[tid];
@@ -1290,67 +1318,47 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
               const int oi = sm.cand2_idx[c];
               rank += (ok > key || (ok == key && oi < id)) ? 1u : 0u;
             }
-            if (rank == kk2 - 1u) { sm.res[2] = key; sm.res[3] = (unsigned)id; }
+            if (rank < kk2) keep((int)(above + rank), (unsigned)id);
           }
-          settler_sync();
-          T = sm.res[2]; tch = sm.res[3];
         } else {
-          // many scores agree in their top 20 bits: radix steps of 7 bits over the other 12 and the inverted channel
-          unsigned prefix = 0;
+          // many scores agree in their upper halves: radix steps of 8 bits over the lower halves and the inverted channels
+          unsigned prefix = 0, kleft = kk2;
+          auto low = [&](unsigned ch) { return (full_key((int)ch) << 16) | (0xffffu ^ ch); };
 #pragma unroll 1
-          for (int sh = 21; sh >= 0; sh -= 7) {
+          for (int sh = 24; sh >= 0; sh -= 8) {
             settler_sync();                               // everyone is done with the previous histogram
-            if (tid < 128) sm.hist2[tid] = 0;
+            sm.hist2[tid] = 0;
             settler_sync();
 #pragma unroll 1
-            for (unsigned c = tid; c < nb1; c += kSettlers) {
-              const unsigned key = lds32(lkey_u32 + c * 4u);
-              const unsigned low = ((key & 0xfffu) << 16) | (0xffffu ^ lds32(lidx_u32 + c * 4u));
-              if ((key >> 12) == pre2 && (low >> (sh + 7)) == prefix) atomicAdd(&sm.hist2[(low >> sh) & 127u], 1u);
+            for (int c = c0; c < c1; ++c) {
+              const unsigned e = lds32(list_u32 + (uint32_t)c * 4u);
+              if ((e >> 16) != sub) continue;
+              const unsigned v = low(e & 0xffffu);
+              if (sh == 24 || (v >> (sh + 8)) == prefix) atomicAdd(&sm.hist2[(v >> sh) & 255u], 1u);
             }
             settler_sync();
             unsigned ab;
-            const unsigned bb = kth_in_segment<4>(sm.hist2, 128, kk2, lane, &ab);
-            prefix = (prefix << 7) | bb;
-            kk2 -= ab;
+            const unsigned bb = kth_in_segment<8>(sm.hist2, 256, kleft, lane, &ab);
+            prefix = (prefix << 8) | bb;
+            kleft -= ab;
           }
-          T = (pre2 << 12) | (prefix >> 16); tch = 0xffffu ^ (prefix & 0xffffu);
+          unsigned wk = 0;
+#pragma unroll 1
+          for (int c = c0; c < c1; ++c) {
+            const unsigned e = lds32(list_u32 + (uint32_t)c * 4u);
+            wk += (e >> 16) == sub && low(e & 0xffffu) >= prefix ? 1u : 0u;
+          }
+          const unsigned inck = warp_scan_incl(wk, lane);
+          if (lane == 31) sm.warp_cnt[warp][1] = inck;
+          settler_sync();
+          int at = (int)(above + __reduce_add_sync(0xffffffffu, lane < warp ? sm.warp_cnt[lane][1] : 0u) + inck - wk);
+#pragma unroll 1
+          for (int c = c0; c < c1; ++c) {
+            const unsigned e = lds32(list_u32 + (uint32_t)c * 4u);
+            if ((e >> 16) == sub && low(e & 0xffffu) >= prefix) keep(at++, e & 0xffffu);
+          }
         }
         PROX_TRACE(20);
-        // ... and keep the block's share of the members down to that one: a thread owns a run of the list, counts
-        // first, then the places
-        const int ept = ((int)nb1 + kSettlers - 1) / kSettlers;
-        const int c0 = min((int)nb1, tid * ept), c1 = min((int)nb1, c0 + ept);
-        auto kept = [&](int c) {
-          const unsigned key = lds32(lkey_u32 + (uint32_t)c * 4u);
-          return key > T || (key == T && lds32(lidx_u32 + (uint32_t)c * 4u) <= tch);
-        };
-        unsigned wt = 0;
-#pragma unroll 1
-        for (int c = c0; c < c1; ++c) wt += kept(c) ? 1u : 0u;
-        const unsigned inc3 = warp_scan_incl(wt, lane);
-        if (lane == 31) sm.warp_cnt[warp][0] = inc3;
-        settler_sync();
-        {
-          // the totals of the warps in front (every lane reads them itself: the warp may have diverged)
-          unsigned bs = 0;
-#pragma unroll 1
-          for (int w = 0; w < warp; ++w) bs += sm.warp_cnt[w][0];
-          int pos = (int)(bs + inc3 - wt);
-          if (wt > 0 && pos < Rc1 && pos + (int)wt > Rc0) {
-#pragma unroll 1
-            for (int c = c0; c < c1; ++c) {
-              if (!kept(c)) continue;
-              if (pos >= Rc0 && pos < Rc1) {
-                const int ch = (int)lds32(lidx_u32 + (uint32_t)c * 4u);
-                sm.mysel[ndm + pos - Rc0] = ch;
-                if (p.sel_out) p.sel_out[(int)nd + pos] = ch;
-              }
-              ++pos;
-            }
-          }
-        }
-        }
         __threadfence_block();
         settler_sync();                          // the list is free from here on
         if (tid == 0) {
@@ -1385,22 +1393,28 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       int slot = pslot;
       bool dead = false;
       int ready = *reinterpret_cast<volatile int*>(&sm.nready);
+      bool kdone = *reinterpret_cast<volatile int*>(&sm.keys_done) != 0;
       bool cdone = *reinterpret_cast<volatile int*>(&sm.c_done) != 0;
-      const int ls0 = sm.list_s0, ls1 = sm.list_s1;
+      const int ks0 = sm.keys_s0, ks1 = sm.keys_s1, ls0 = sm.list_s0, ls1 = sm.list_s1;
+#pragma unroll 1
       for (int b0 = 0; b0 < n_mine && !dead; b0 += kChanBatch) {
         const int nb = min(kChanBatch, n_mine - b0);
+#pragma unroll 1
         for (int q = 0; q < 3 * nb; ++q, ++seq) {
           // A slot always belongs to the same producer: its uses are then armed
           // in program order, so the parity wait below is never two phases behind.
           if (((unsigned)slot & (unsigned)(kFusedProducers - 1)) == pq) {
             const int mi = b0 + ((q < 2 * nb) ? (q >> 1) : (q - 2 * nb));
             // The tail of the list (the share of the threshold bin) is written late, and the ring
-            // may not touch the slots under the list of b1's members before the consumer warps are done with it.
-            auto blocked = [&]() { return mi >= ready || (!cdone && slot >= ls0 && slot < ls1); };
+            // may not touch the slots under the keys and the list before the consumer warps are done with them.
+            auto blocked = [&]() {
+              return mi >= ready || (!kdone && slot >= ks0 && slot < ks1) || (!cdone && slot >= ls0 && slot < ls1);
+            };
             if (blocked()) {
 #pragma unroll 1
               for (unsigned it = 0; it < spin; ++it) {
                 ready = *reinterpret_cast<volatile int*>(&sm.nready);
+                kdone = *reinterpret_cast<volatile int*>(&sm.keys_done) != 0;
                 cdone = *reinterpret_cast<volatile int*>(&sm.c_done) != 0;
                 if (!blocked() || *abortp) break;
                 __nanosleep(64);
@@ -1448,6 +1462,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       }
       __syncwarp();
     }
+#pragma unroll 1
     for (int b0 = 0; b0 < n_mine; b0 += kChanBatch) {
       const int nb = min(kChanBatch, n_mine - b0);
       // D: a warp takes the next channel of the batch that nobody has taken yet (the warps
@@ -1497,6 +1512,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       // E: group gq (TG threads) owns rows gq, gq+NG, ... ; a thread owns EV vectors of y
       {
         const int gq = tid / TG, tg = tid % TG;
+#pragma unroll 1
         for (int c = gq; c < nb; c += NG) {
           const unsigned sq = base_seq + 2u * (unsigned)nb + (unsigned)c;
           const unsigned ud = __umulhi(sq, p.nslots_rcp);
@@ -1539,6 +1555,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
         }
       }
       consumer_sync();
+#pragma unroll 1
       for (int v4 = tid; v4 < D / 4 && !*abortp; v4 += kFusedConsumers) {       // (a block that has given up adds nothing)
         float4 s = reinterpret_cast<const float4*>(ysum)[v4];
 #pragma unroll
@@ -1564,6 +1581,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       if (p.host_flag) *reinterpret_cast<volatile int*>(p.host_flag) = 1;
       const unsigned issued = sm.prod_seq;
       const unsigned first = issued > (unsigned)NS ? issued - (unsigned)NS : 0u;
+#pragma unroll 1
       for (unsigned q = first; q < issued; ++q) {        // the latest use of every slot
         const uint32_t bar = smem_u32(&sm.mbar_full[q % (unsigned)NS]);
 #pragma unroll 1
@@ -1589,6 +1607,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   }
   __syncthreads();
   if (sm.s_last) {
+#pragma unroll 1
     for (int i0 = tid * 4; i0 < D; i0 += NT * 4 * 4) {        // loads first: they must not queue behind the stores
       float4 v[4], r[4];
 #pragma unroll
@@ -1622,7 +1641,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   }
   if (next_shr >= NSH) break;
   __syncthreads();                              // everyone has read what is reset here
-  if (tid == 0) { sm.shr = next_shr; sm.ncand2 = 0; sm.next_c = 0; sm.nready = 0; sm.n_mine = 0; sm.c_done = 0; }
+  if (tid == 0) { sm.shr = next_shr; sm.ncand2 = 0; sm.next_c = 0; sm.nready = 0; sm.n_mine = 0; sm.keys_done = 0; sm.c_done = 0; }
   __syncthreads();
   }
   }
