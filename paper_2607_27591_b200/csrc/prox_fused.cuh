@@ -319,7 +319,6 @@ struct FusedSmem {
   int c_done;              // ... nor the list of the threshold bin's members
   int keys_s0, keys_s1;    // ring slots [s0, s1) that overlap the keys
   int list_s0, list_s1;    // ... and the list
-  unsigned poll[2][kFusedConsumerWarps];   // the warps' counts of scores in the histogram; and whether scores are missing
   unsigned slot_use[kMaxSlots];   // uses of each ring slot whose data has been seen complete
   unsigned long long pempty[kFusedConsumerWarps];   // proxy ring: the MMAs of a warp's block are complete
   unsigned long long acc_bar;            // all MMAs of a tile are complete (one arrival per loader warp)
@@ -329,6 +328,7 @@ struct FusedSmem {
   unsigned wmax[32];
   float nsum[kFusedWarps][2];     // RMSNorm: the warps' sums of squares (hi, lo)
   float ninv[2];                  // ... and 1 / sqrt(mean + eps) (hi, lo)
+  unsigned poll[2][kFusedConsumerWarps];   // the warps' counts of scores in the histogram; and whether scores are missing
 };
 
 // k-th largest (k >= 1) over a histogram held in registers: thread t < 512 has the counts of N bins in descending order,
@@ -686,7 +686,10 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     }
     const uint32_t ring = (smem_u32(xf) + 1023u) & ~1023u;
     const int NL = p.loaders;
-    float* red = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(xf) + (ring - smem_u32(xf)) + (uint32_t)(NL * proxy_warp_bytes(BITS)));   // [3][128][2] partial sums of warps 4..15
+    // partial sums of warps 4..15, [3][128][2], for tiles in turn: behind the ring, and over mysel and hval (not used yet)
+    float* const red0 = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(xf) + (ring - smem_u32(xf)) + (uint32_t)(NL * proxy_warp_bytes(BITS)));
+    float* const red1 = reinterpret_cast<float*>(sm.mysel);
+    static_assert(offsetof(FusedSmem, hval) == offsetof(FusedSmem, mysel) + sizeof(int) * kMySelCap && kMySelCap * 4 + kChanBatch * 4 >= 3072, "");
     PROX_TRACE(29);
     if (warp < kFusedConsumerWarps) {
       // a warp owns its stages of the ring: it fills them and issues their MMAs itself (the tensor core
@@ -845,6 +848,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
         }
         PROX_TRACE(26);
         if (more) { tmem_st_wait(); tc_fence_before(); }
+        float* const red = (tl & 1) ? red1 : red0;
         if (part > 0) { red[((part - 1) * 128 + col) * 2] = t0; red[((part - 1) * 128 + col) * 2 + 1] = t1; }
         consumer_sync();
         if (more) tc_fence_after();            // every warp's columns are back at zero before the next tile's MMAs
@@ -881,16 +885,16 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
               if (LO) { b1 = k1b >> 20; n1 = atomicAdd(&sm.hist[b1], 1u); }
             }
           }
-          if (HIST) {
-            // one global atomic per occupied bin and tile (thousands of single increments on a few hot bins serialise in
-            // L2), by the thread that came first to the bin
+          if (HIST && ntl == 1) {
+            // one global atomic per occupied bin (thousands of single increments on a few hot bins serialise in L2), by the
+            // thread that came first to the bin; with several tiles at the end of the share (done per tile, the pause between
+            // tiles cost 1.2 % of 4096 x 14336 8-bit and of 8192 x 28672)
             __syncwarp();
             asm volatile("bar.sync 4, 128;" ::: "memory");
             if (n0 == 0u) { atomicAdd(ghist + b0, sm.hist[b0]); sm.hist[b0] = 0u; }
             if (n1 == 0u) { atomicAdd(ghist + b1, sm.hist[b1]); sm.hist[b1] = 0u; }
           }
         }
-        if (more) consumer_sync();             // red is free again
       }
       // nothing may be in flight when the block frees the tensor memory (only a block whose wait expired gets here early)
       if (sm.abort_flag && lane == 0) {
@@ -933,6 +937,10 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     tc_fence_before();
     fence_proxy_async();                        // phase B's plain accesses to the big buffer come before the ring's bulk copies
     __syncthreads();
+    if (HIST && ntl > 1) {
+#pragma unroll 1
+      for (int i = tid; i < 2048; i += NT) { const unsigned v = sm.hist[i]; if (v) { atomicAdd(ghist + i, v); sm.hist[i] = 0u; } }
+    }
     PROX_TRACE(3);
     if (MODE == kWhole && tid == 0 && sm.vid < (unsigned)p.nshare1 && sm.abort_flag == 0)
       asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(ctr + kOut1) : "memory");
