@@ -25,31 +25,34 @@ __device__ __forceinline__ unsigned absmax4(const uint2& v) {   // largest of fo
   return max(m & 0xffffu, m >> 16);
 }
 
-// Codes clamp(rint(v / s)) + offset of four weights of one channel, exactly as with the IEEE quotient.  v * inv
-// (inv = 1 / s) is within 5e-5 of the quotient (|quotient| < 256, three roundings; 4-bit codes: < 16, 3e-6), so
-// its nearest integer is the quotient's unless it lies that close to a half; only then the divisions are made.
-// Rounding by adding 1.5 * 2^23 (+ the offset) leaves the code in the low mantissa bits: ten full-rate
-// instructions per weight, with rintf, clamps and conversions it was twice that and the kernel bound by them.
+// Bits of 1.5 * 2^23 + offset + rint(v / s) for four weights of one channel, from inv = 1 / s (s a normal fp16 number, or 0 and so v).
+// v has 8 significant bits and s = m 2^b has m < 2^11, so a quotient that is not a half integer itself is at least
+// 1 / (2 m) > 2^-12 away from the next one (v - (k + 1/2) s is a multiple of 2^(b-1)), and v * inv within 1e-5 of it
+// (|quotient| < 128.1): rounded to a multiple of 2^-12 first (the first addition: 3072 + quotient), what is a half
+// integer becomes exactly one and nothing else does, and the second addition rounds to the nearest integer, halves to even,
+// as the IEEE quotient would be.  No clamp: the scale is absmax / qmax to 2^-11.  With the start of the codes at bit 0 of the
+// sum's mantissa a weight takes four instructions (unpack, multiply-add, add, shift-add into the word); with the quotient's
+// distance from a half taken and divisions where it was close, clamps and masks it took eleven.
 template <int BITS>
-__device__ __forceinline__ void proxy_codes(const uint2& v, float s, float inv, uint32_t (&code)[4]) {
-  constexpr float qmax = (float)((1 << (BITS - 1)) - 1);
-  constexpr float magic = 12582912.f + (BITS == 4 ? 8.f : 128.f);
-  constexpr float close = BITS == 4 ? 0.49999f : 0.4999f;
+__device__ __forceinline__ void proxy_sums(const uint2& v, float inv, uint32_t (&t)[4]) {
+  constexpr float magic = 12582912.f + (BITS == 4 ? 8.f : 128.f), grid = 3072.f;
   const float f[4] = {bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y)};
-  float t[4], far = 0.f;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) t[e] = __float_as_uint(__fadd_rn(__fmaf_rn(f[e], inv, grid), magic - grid));
+}
+// The same with the quotients themselves and clamped, for scales that are not normal fp16 numbers (nothing but a code may
+// get into the words, whatever the weights are).
+template <int BITS>
+__device__ __noinline__ uint4 proxy_sums_small(uint2 v, float s) {
+  constexpr float qmax = (float)((1 << (BITS - 1)) - 1), magic = 12582912.f + (BITS == 4 ? 8.f : 128.f);
+  const float f[4] = {bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y)};
+  uint32_t t[4];
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
-    const float p = f[e] * inv;
-    t[e] = __fadd_rn(p, magic);
-    far = fmaxf(far, fabsf(__fsub_rn(p, __fsub_rn(t[e], magic))));
+    const float q = s != 0.f ? __fdiv_rn(f[e], s) : 0.f;
+    t[e] = __float_as_uint(fminf(fmaxf(__fadd_rn(q, magic), magic - qmax), magic + qmax));
   }
-  if (far > close) {
-#pragma unroll
-    for (int e = 0; e < 4; ++e) t[e] = __fadd_rn(__fdiv_rn(f[e], s), magic);
-  }
-#pragma unroll
-  for (int e = 0; e < 4; ++e)
-    code[e] = __float_as_uint(fminf(fmaxf(t[e], magic - qmax), magic + qmax)) & (BITS == 4 ? 0xfu : 0xffu);
+  return make_uint4(t[0], t[1], t[2], t[3]);
 }
 
 // One scale per channel row: one warp per (matrix, channel), 16-byte loads, four in flight per lane.
@@ -126,17 +129,26 @@ proxy_pack_kernel(const uint16_t* __restrict__ wg, const uint16_t* __restrict__ 
       s_mine = s_plain[(size_t)which * F + j0 + (lane & 7)];
     }
     inv_mine = s_mine != 0.f ? __fdiv_rn(1.0f, s_mine) : 0.f;     // scale 0: every code is 0
+    // the codes' words as sums of what stands in the low bits of the sums above, whose upper bits add up to a constant
+    const unsigned small = __ballot_sync(0xffffffffu, (s_mine > 0.f && s_mine < 6.103515625e-5f) || !(s_mine <= 65504.f)) & 0xffu;
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
-      uint32_t code[4];
-      proxy_codes<BITS>(v[m], __shfl_sync(0xffffffffu, s_mine, m), __shfl_sync(0xffffffffu, inv_mine, m), code);
+      uint32_t t[4];
+      proxy_sums<BITS>(v[m], __shfl_sync(0xffffffffu, inv_mine, m), t);
+      if (small && ((small >> m) & 1u)) {
+        const uint4 u = proxy_sums_small<BITS>(v[m], __shfl_sync(0xffffffffu, s_mine, m));
+        t[0] = u.x; t[1] = u.y; t[2] = u.z; t[3] = u.w;
+      }
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        if (BITS == 4) lo[e] |= code[e] << (4 * m);
-        else if (m < 4) lo[e] |= code[e] << (8 * m);
-        else hi[e] |= code[e] << (8 * (m - 4));
+        if (BITS == 4) lo[e] += t[e] << (4 * m);
+        else if (m < 4) lo[e] += t[e] << (8 * m);
+        else hi[e] += t[e] << (8 * (m - 4));
       }
     }
+    constexpr uint32_t kUpper = BITS == 4 ? 0x4b400000u + 0xb4000000u + 0x40000000u : 0x4b400000u + 0x40000000u;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) { lo[e] -= kUpper; hi[e] -= kUpper; }
     // word of the row: chunk * 4 + which * 2 + (half of the chunk's channels)
     const int col = BITS == 4 ? (grp >> 1) * 4 + which * 2 + (grp & 1) : grp * 4 + which * 2;
 #pragma unroll
