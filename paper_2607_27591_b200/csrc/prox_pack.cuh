@@ -38,7 +38,11 @@ __device__ __forceinline__ void proxy_sums(const uint2& v, float inv, uint32_t (
   constexpr float magic = 12582912.f + (BITS == 4 ? 8.f : 128.f), grid = 3072.f;
   const float f[4] = {bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y)};
 #pragma unroll
-  for (int e = 0; e < 4; ++e) t[e] = __float_as_uint(__fadd_rn(__fmaf_rn(f[e], inv, grid), magic - grid));
+  for (int e = 0; e < 4; e += 2)             // two at a time: one issue slot for two multiply-adds
+    asm("{\n\t.reg .b64 a, b, c, d;\n\t"
+        "mov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %4};\n\tmov.b64 c, {%5, %5};\n\tmov.b64 d, {%6, %6};\n\t"
+        "fma.rn.f32x2 a, a, b, c;\n\tadd.rn.f32x2 a, a, d;\n\tmov.b64 {%0, %1}, a;\n\t}"
+        : "=r"(t[e]), "=r"(t[e + 1]) : "f"(f[e]), "f"(f[e + 1]), "f"(inv), "f"(grid), "f"(magic - grid));
 }
 // The same with the quotients themselves and clamped, for scales that are not normal fp16 numbers (nothing but a code may
 // get into the words, whatever the weights are).
@@ -130,20 +134,27 @@ proxy_pack_kernel(const uint16_t* __restrict__ wg, const uint16_t* __restrict__ 
     }
     inv_mine = s_mine != 0.f ? __fdiv_rn(1.0f, s_mine) : 0.f;     // scale 0: every code is 0
     // the codes' words as sums of what stands in the low bits of the sums above, whose upper bits add up to a constant
-    const unsigned small = __ballot_sync(0xffffffffu, (s_mine > 0.f && s_mine < 6.103515625e-5f) || !(s_mine <= 65504.f)) & 0xffu;
-#pragma unroll
-    for (int m = 0; m < 8; ++m) {
-      uint32_t t[4];
-      proxy_sums<BITS>(v[m], __shfl_sync(0xffffffffu, inv_mine, m), t);
-      if (small && ((small >> m) & 1u)) {
-        const uint4 u = proxy_sums_small<BITS>(v[m], __shfl_sync(0xffffffffu, s_mine, m));
-        t[0] = u.x; t[1] = u.y; t[2] = u.z; t[3] = u.w;
-      }
+    auto add = [&](int m, const uint32_t (&t)[4]) {
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         if (BITS == 4) lo[e] += t[e] << (4 * m);
         else if (m < 4) lo[e] += t[e] << (8 * m);
         else hi[e] += t[e] << (8 * (m - 4));
+      }
+    };
+    if (!__any_sync(0xffffffffu, (s_mine > 0.f && s_mine < 6.103515625e-5f) || !(s_mine <= 65504.f))) {
+#pragma unroll
+      for (int m = 0; m < 8; ++m) {
+        uint32_t t[4];
+        proxy_sums<BITS>(v[m], __shfl_sync(0xffffffffu, inv_mine, m), t);
+        add(m, t);
+      }
+    } else {
+#pragma unroll
+      for (int m = 0; m < 8; ++m) {
+        const uint4 u = proxy_sums_small<BITS>(v[m], __shfl_sync(0xffffffffu, s_mine, m));
+        const uint32_t t[4] = {u.x, u.y, u.z, u.w};
+        add(m, t);
       }
     }
     constexpr uint32_t kUpper = BITS == 4 ? 0x4b400000u + 0xb4000000u + 0x40000000u : 0x4b400000u + 0x40000000u;
