@@ -91,13 +91,13 @@ proxy_row_scale_kernel(const uint16_t* __restrict__ wg, const uint16_t* __restri
 // takes 8 channels x 128 inputs of one matrix (eight 256-byte row pieces, 8 bytes per lane each), which give a
 // lane one word (4-bit) or two (8-bit) per input row of the packed layout; they meet in shared memory
 // (word column xor lane: no bank conflicts either way) and leave as whole 128-byte pieces of the packed rows.
-// Bound by instruction issue: 4096 x 12288, 4-bit, groups: 82 us at 2.9 instructions per clock and SM (100 MB of
-// weights and 50 MB of codes are 39 us of HBM); one scale per row: 66 us after 34 us for the scales.  With one
-// thread per packed word, its 4-byte stores a packed row apart, 2-byte loads and four cudaMalloc / cudaFree a call
-// the whole of prox_quantize_proxy took 3.4 - 5 ms; now 113 us (and 31 us of those are the W_down copy: running its
-// blocks between the packing ones in one launch gave 117 us, its small blocks want more of them per SM).
+// Bound by instruction issue (2.7 instructions per clock and SM) and the loads in flight: 4096 x 12288, 4-bit, groups: 50 us
+// (200 MB of weights and 50 MB of codes are 39 us of HBM); 82 with eleven instructions per weight (see proxy_sums), 55 with
+// single multiply-adds and a branch per channel, 52 with four blocks per SM instead of five; with the next task's rows
+// requested before one is worked on (80 registers) 54.  One scale per row: the scales are 34 us in front.  (The W_down copy is 31
+// us; running its blocks between the packing ones in one launch was slower, its small blocks want more of them per SM.)
 template <int BITS, bool GROUPED>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 5)
 proxy_pack_kernel(const uint16_t* __restrict__ wg, const uint16_t* __restrict__ wu, int D, int F,
                   __half* __restrict__ S, float* __restrict__ s_plain, uint32_t* __restrict__ P) {
   constexpr int CH = ProxyFmt<BITS>::CH;
