@@ -181,8 +181,8 @@ prox_status_t prox_ffn_last_stage1(prox_ffn_t* h, int k1, int32_t* idx_dev_or_nu
                                    void* stream);
 
 /* Test hook for the bounded device-side waits: spin_limit = polls after which a wait gives up
- * (0 = the default, about two million); barrier_bias > 0 keeps the grid barrier of the persistent
- * kernel from ever completing, so that the next B = 1 forward call runs into the limit, leaves
+ * (0 = the default, about two million); barrier_bias > 0 keeps the persistent kernel's wait for all
+ * blocks' scores from ever completing, so that the next B = 1 forward call runs into the limit, leaves
  * without writing y and reports it (see prox_last_device_status).  With bit 31 set it is a wait inside
  * Stage 1 of one block instead (the one with the first share of the columns), which Stage 1 called alone
  * has too.  Nothing hangs or faults: the blocks give up and return.  Set both back to 0 afterwards. */

@@ -68,7 +68,7 @@ struct prox_ffn {
   int use_union;            // batch > 1 reads weights once for the union of the tokens' masks
   unsigned long long* trace;  // optional phase time stamps of the persistent kernel (debug)
   unsigned spin_limit;      // polls after which a device-side wait gives up
-  unsigned bar_bias;        // test knob: keeps the grid barrier of the persistent kernel from completing
+  unsigned bar_bias;        // test knob: keeps the persistent kernel's wait for the scores from completing
   int* host_flag;           // pinned, mapped word the kernels set when a wait expires
   int* host_flag_dev;
   // batch > 1: unions of the tokens' masks (allocated when max_batch > 1)
@@ -675,8 +675,8 @@ FusedPlan plan_fused(const prox_ffn* h, int k1, int k2, bool thresh = false, int
   if (pl.big_bytes < pl.xch * D * 4) return pl;          // their partial y vectors
   if ((k2 + G - 1) / G + 2 > kMySelCap) return pl;       // a block's share: definite part + part of the threshold bin
   if (thresh) {
-    // any number of channels may pass the threshold: a block's share of all of them must fit, the scores
-    // must fit in shared memory (no radix fallback in this form), counts are kept in 16 bits
+    // any number of channels may pass the threshold: a block's share of all of them must fit, their marks must fit in
+    // shared memory (no radix fallback in this form; the line is that of whole scores), counts are kept in 16 bits
     if ((F + G - 1) / G + 2 > kMySelCap) return pl;
     if (mode == kWhole && ((size_t)F * 4 + 256 > (size_t)pl.big_bytes || F >= 65536)) return pl;
   }

@@ -7,16 +7,16 @@
 //      blocks; the rows' bytes are the A operand as they lie in memory, x enters
 //      as signed base-256 digits; the block writes the scores |u~ SiLU(g~)| of
 //      its channels and adds them to a global 2048-bin histogram
-//   -- one grid-wide barrier (bounded spin, self-resetting) --
-//   C  every block (consumer warps only; the producer warps wait at the ring):
+//   -- every block needs all scores: a bounded wait for a count of finished shares, after which the scores are read and
+//      say themselves whether they are there --
+//   C  every block (consumer warps only; the producer warps wait for them):
 //      the histogram gives the threshold bin b1; channels in bins above b1 are
 //      kept whatever the exact threshold is.  The kept list is laid out as
-//      [those channels, ascending][kept members of b1, ascending] and block c
-//      owns the c-th share of both parts.  Two passes over the scores list its
-//      share of the first part and the ring starts; half of the consumer warps
-//      then settle the exact threshold inside b1 (ordered list of its members,
-//      8-bit histogram, rank among the few left) and append the block's share
-//      of the second part, while the other half already consumes rows
+//      [those channels][kept members of b1] and block c owns the c-th share of
+//      both parts.  One pass over the upper halves of the scores finds its
+//      share of the first part, a warp lists it and the ring starts; half of the consumer warps
+//      then settle the exact threshold inside b1 (four more bits from the half scores, whole scores for the members that
+//      agree in them too) and append the block's share of the second part, while the other half already consumes rows
 //   D  gate/up rows of its channels stream through a shared-memory ring filled
 //      by bulk async copies (cp.async.bulk + mbarrier, four issuing warps); a
 //      consumer warp takes the next channel nobody has taken:
@@ -28,7 +28,7 @@
 //
 // Launch: an ordinary one, one block per SM, with programmatic stream serialization.  No block waits for a block that
 // may not be running: the shares of Stage 1 (columns) and of Stage 2 (kept channels) are claimed by tickets, a
-// running block claims again until there are none left, and the barrier counts finished shares, not blocks.  Where all
+// running block claims again until there are none left, and the wait is for finished shares, not blocks.  Where all
 // blocks run, as always on a GPU of its own, every block has one share of each.  (With the cooperative attribute
 // instead, launches of a stream did not overlap and started in steps of 2.05 us:
 // 512 x 1536 20.5 -> 19.6 us per call, 1024 x 3072 layer form 22.4 -> 20.5, 4096 x 12288 38.9 -> 37.7.)
@@ -315,9 +315,9 @@ struct FusedSmem {
   unsigned next_c;         // next channel of the batch to take in the gate/up phase
   int n_mine;              // channels of this block (for the producer warps)
   int nready;              // entries of mysel that are final (the definite share first, all of them later)
-  int keys_done;           // the consumer warps no longer read the keys near the end of the big buffer
+  int keys_done;           // the consumer warps no longer read the half scores near the end of the big buffer
   int c_done;              // ... nor the list of the threshold bin's members
-  int keys_s0, keys_s1;    // ring slots [s0, s1) that overlap the keys
+  int keys_s0, keys_s1;    // ring slots [s0, s1) that overlap them
   int list_s0, list_s1;    // ... and the list
   unsigned slot_use[kMaxSlots];   // uses of each ring slot whose data has been seen complete
   unsigned long long pempty[kFusedConsumerWarps];   // proxy ring: the MMAs of a warp's block are complete
@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   constexpr int CH = ProxyFmt<BITS>::CH;
   constexpr int NT = kFusedThreads;
   // Only the top-k form of the whole path starts its channel mask from the score histogram; filled in the threshold form as
-  // well, it cost that 0.4 us in front of the barrier (4096 x 12288 layer form: 34.5 -> 33.9 us per call).
+  // well, it cost that 0.4 us in front of the exchange (4096 x 12288 layer form: 34.5 -> 33.9 us per call).
   constexpr bool HIST = MODE == kWhole && !THRESH;
   extern __shared__ __align__(128) uint8_t smem_raw[];
   FusedSmem& sm = *reinterpret_cast<FusedSmem*>(smem_raw);
@@ -642,6 +642,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   // One trip per share: of Stage 1 (B) and then of Stage 2 (C to F).  Where all blocks run there is one trip; further
   // Stage-1 shares, of blocks that are not running, come before the channel mask, further Stage-2 shares at the end.
   bool with_b = MODE != kGivenList;
+  unsigned vid = (unsigned)p.nshare1;           // share of Stage 1 (none: the number of shares)
 #pragma unroll 1
   for (bool first = true;; first = false) {
   if (with_b) {
@@ -664,7 +665,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     constexpr bool LO = (BITS == 4);
     const int nchunks = F / CH;
     const int row_bytes = nchunks * 16;
-    const unsigned vid = sm.vid, n1 = (unsigned)p.nshare1;
+    const unsigned n1 = (unsigned)p.nshare1;
+    vid = sm.vid;
     const int lk0 = p.pleft0 + (int)vid * p.ppart + min((int)vid, p.pmore) * p.cgran;       // this block's part of the rest
     const int lk1 = min(nchunks, lk0 + p.ppart + ((int)vid < p.pmore ? p.cgran : 0));
     const int ntl = vid >= n1 ? 0 : p.plines + (lk1 > lk0 ? ((lk1 + 7) >> 3) - (lk0 >> 3) : 0);
@@ -717,6 +719,10 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
         const int sc = w > 4 ? 3 : 2, rpi = 32 >> sc;
         const int kq = lane >> sc, c = lane & ((1 << sc) - 1);
         const uint8_t* tp = p.P + (size_t)tc0 * 16 + (size_t)c * 16;
+        // copy instruction j takes the rows j * rpi + kq: where they go in a stage, for even and odd j (the chunk's place is xor-ed
+        // with the row), a step of j by two further on
+        const uint32_t sa0 = stg + (uint32_t)(kq * 128 + ((c ^ kq) << 4)), sstep = sc == 3 ? 1024u : 2048u;
+        const uint32_t sa1 = sc == 3 ? stg + (uint32_t)((kq + 4) * 128 + ((c ^ (kq + 4)) << 4)) : sa0 + 1024u;
         const int chunk = tc0 + (col >> 4);                    // chunk of this thread's byte column
         const bool col_ok = (col >> 4) < w;
         bool alive_b = true;
@@ -740,13 +746,12 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
               nrows = min(32, k1 - r0);
             }
             // rows beyond nrows and columns beyond the tile keep whatever is there: their digits are zero, their sums unused
+            const uint16_t* const ip = idx16 + r0 + kq;
+            const uint32_t so = (uint32_t)((k & 1) * 4096);
+            const int left = nrows - kq;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const int kk = j * rpi + kq;
-              if (kk < nrows)
-                cp_async16(stg + (uint32_t)((k & 1) * 4096 + (kk >> 3) * 1024 + (kk & 7) * 128 + ((c ^ (kk & 7)) << 4)),
-                           tp + (size_t)idx16[r0 + kk] * (size_t)row_bytes);
-            }
+            for (int j = 0; j < 8; ++j)
+              if (j * rpi < left) cp_async16(((j & 1) ? sa1 : sa0) + so + (uint32_t)(j >> 1) * sstep, tp + (unsigned)ip[j * rpi] * (unsigned long long)(unsigned)row_bytes);
           }
           cp_async_commit();
           if (tl == 0 && k == 0) PROX_TRACE(22);
@@ -942,13 +947,13 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       for (int i = tid; i < 2048; i += NT) { const unsigned v = sm.hist[i]; if (v) { atomicAdd(ghist + i, v); sm.hist[i] = 0u; } }
     }
     PROX_TRACE(3);
-    if (MODE == kWhole && tid == 0 && sm.vid < (unsigned)p.nshare1 && sm.abort_flag == 0)
+    if (MODE == kWhole && tid == 0 && vid < n1 && sm.abort_flag == 0)
       asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(ctr + kOut1) : "memory");
     if (MODE == kScoresOnly) {
       if (tid == 0) {
         // a block that has given up does not finish its share
         unsigned more1 = (unsigned)p.nshare1;
-        if (sm.vid < more1 && sm.abort_flag == 0) {
+        if (vid < more1 && sm.abort_flag == 0) {
           asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ctr + kDone1) : "memory");
           asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(more1) : "l"(ctr + kClaim1) : "memory");
         }
@@ -963,13 +968,17 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   // ---------------------------------------- C: channel mask (top-k2 of the scores)
   // The blocks wait for a count of finished shares that is not ordered behind the scores; the scores themselves say that
   // they are there (all ones = not yet), and the histogram that it is complete (it counts all channels): what is missing is read
-  // again.  (Ordered by a release, i.e. behind the acknowledgement of all the block's writes, the count came one trip to L2 later.)
+  // again.  (With a barrier, i.e. a count released behind the acknowledgement of all the block's writes and acquired, and with whole
+  // scores, counted by every thread in a run of its own, the first copy of phase D came 6.2 us after the last block's scores at
+  // 4096 x 12288 where it comes after 4.8, and 3.6 instead of 2.9 at 512 x 1536.  What goes to every block is 2 bytes per channel;
+  // the threshold form hands on one bit, which the block that has the score decides.  Reading histogram and scores in a loop
+  // without waiting for the count, 148 blocks on the same lines, kept the last scores from getting there: 15 % slower.)
   // The first histogram level tells which channels are kept whatever the exact
   // threshold turns out to be (their bin lies above the threshold bin b1:
   // "definite", nd of them) and which are still open (the nb1 members of b1).
   // The kept list is laid out as [definite][kept members of b1], either part in the order of the threads that hold the
-  // scores; block c owns the c-th share of either part.  Its definite share is known after one pass over the scores, in
-  // registers, so its weight rows start to stream while the consumer warps still settle the threshold inside b1.
+  // scores; block c owns the c-th share of either part.  Its definite share is known after one pass over the half scores,
+  // so its weight rows start to stream while the consumer warps still settle the threshold inside b1.
   int n_mine = 0;
   unsigned nd = 0, b1 = 0, kk = 0, nb1 = 0;     // (THRESH: nd = the kept channels)
   unsigned cnt = 0, ex = 0;                     // packed: definite channels (low half) and members of b1 of this thread / in front of it
@@ -997,7 +1006,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   if (warp >= kFusedConsumerWarps) {
     if (MODE == kWhole && with_b) {
       // (in the layer form in place, the blocks wait for this count before they add to the residual stream that others read)
-      if (tid == kFusedConsumers && sm.vid < (unsigned)p.nshare1 && sm.abort_flag == 0)
+      if (tid == kFusedConsumers && vid < (unsigned)p.nshare1 && sm.abort_flag == 0)
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ctr + kDone1) : "memory");
       widen_x(kFusedConsumers);
     }
@@ -1019,7 +1028,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     if (tid == 0) {
       unsigned more1 = (unsigned)p.nshare1, share2 = 0, out = 0;
       // another share of Stage 1 (there is none unless a block of the grid is not running), and one of Stage 2
-      if (with_b && sm.vid < more1) asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(more1) : "l"(ctr + kClaim1) : "memory");
+      if (with_b && vid < more1) asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(more1) : "l"(ctr + kClaim1) : "memory");
       if (with_b && first) asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(share2) : "l"(ctr + kClaim2) : "memory");
 #pragma unroll 1
       for (unsigned it = 0; it < spin; ++it) {
@@ -1172,7 +1181,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
           }
         }
       } else if (shr < NSH) {
-        // No room in shared memory for the keys plus the list of b1's members (a very large d_ff, or a huge threshold bin such
+        // No room in shared memory for the half scores plus the list of b1's members (a very large d_model and d_ff, or a huge threshold bin such
         // as an all-zero input gives):
         // the consumer warps settle the threshold by two radix steps of 10 bits over all keys and the block keeps its
         // share of the plain ascending list before the ring starts.
@@ -1395,6 +1404,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     // ---- producer warps: lane 0 of each feeds every kFusedProducers-th slot of
     // the ring (one thread can only start a few million bulk copies a second)
     if (lane == 0 && alive) {
+      fence_proxy_async();                      // the big buffer becomes a bulk-copy target now
       n_mine = sm.n_mine;
       const unsigned pq = (unsigned)(warp - kFusedConsumerWarps);
       unsigned seq = pseq, use = puse;
@@ -1414,7 +1424,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
           if (((unsigned)slot & (unsigned)(kFusedProducers - 1)) == pq) {
             const int mi = b0 + ((q < 2 * nb) ? (q >> 1) : (q - 2 * nb));
             // The tail of the list (the share of the threshold bin) is written late, and the ring
-            // may not touch the slots under the keys and the list before the consumer warps are done with them.
+            // may not touch the slots under the half scores and the list before the consumer warps are done with them.
             auto blocked = [&]() {
               return mi >= ready || (!kdone && slot >= ks0 && slot < ks1) || (!cdone && slot >= ls0 && slot < ls1);
             };
