@@ -496,3 +496,64 @@ def test_forms_mixed_on_one_handle(pb, bits, group):
     finally:
         for h in hs:
             pb.prox_ffn_destroy(h)
+
+
+@pytest.mark.parametrize("F,bits", [(64, 8), (512, 4), (4160, 4), (16384, 8), (16448, 8), (33344, 4), (50048, 8), (65536, 4)])
+@pytest.mark.parametrize("distinct", [0, 8, 200])
+def test_persistent_kernel_mask_is_the_exact_topk_of_its_scores(pb, F, bits, distinct):
+    """The channel mask of the whole path against the scores it was made from (ties: lower channel first): one and several
+    groups of half scores per thread, and with few distinct channels many equal scores in the threshold bin, so that its
+    members fill the index list or the ring's end and are cut by their channels; and the threshold form at the k-th score."""
+    D, k1 = 128, 50
+    g = torch.Generator(device="cuda").manual_seed(F + distinct)
+    w = [(torch.randn(F, D, device="cuda", generator=g) * 0.1).to(torch.bfloat16) for _ in range(2)]
+    if 0 < distinct < F:
+        for t in w:
+            t.copy_(t[torch.arange(F, device="cuda") % distinct])
+    wd = (torch.randn(D, F, device="cuda", generator=g) * 0.1).to(torch.bfloat16)
+    x = torch.randn(1, D, device="cuda", generator=g).to(torch.bfloat16)
+    h = pb.prox_ffn_create(D, F, 1, 1, *w, wd)
+    try:
+        pb.prox_quantize_proxy(h, bits, 128)
+        y, ref, sc = (torch.empty(n, dtype=torch.float32, device="cuda") for n in (D, D, F))
+        for k2 in (1, F // 7 + 1, F // 2 + 1, F - 1, F):
+            sel = torch.empty(1, k2, dtype=torch.int32, device="cuda")
+            pb.prox_ffn_forward(h, x, 1, k1, k2, y)
+            pb.prox_ffn_last_mask(h, 1, k2, sel)
+            pb.prox_ffn_last_stage1(h, k1, None, sc)
+            order = torch.sort(sc, descending=True, stable=True).indices[:k2]
+            assert torch.equal(sel[0].long(), order.sort().values), k2
+            pb.prox_stage2_ffn(h, x, 1, sel, k2, ref)
+            # the same products, summed in fp32 in another order
+            assert (y - ref).norm() <= 1e-5 * ref.norm(), k2
+            tau = float(sc[order[-1]])
+            n = int((sc >= tau).sum())
+            xa = float(x[0].float().abs().sort(descending=True).values[k1 - 1])
+            if int((x[0].float().abs() >= xa).sum()) == k1:         # the same inputs, hence the same scores
+                kept = torch.empty(1, n, dtype=torch.int32, device="cuda")
+                pb.prox_ffn_forward_threshold(h, x, 1, xa, tau, y)
+                pb.prox_ffn_last_mask(h, 1, n, kept)
+                assert torch.equal(kept[0].long(), (sc >= tau).nonzero()[:, 0]), k2
+        assert pb.prox_last_device_status(h) == 0
+    finally:
+        pb.prox_ffn_destroy(h)
+
+
+@pytest.mark.parametrize("bits", [4, 8])
+def test_packer_keeps_what_is_not_a_number_to_its_channel(pb, bits):
+    """A channel with an infinite weight or a scale beyond fp16 leaves the codes of the channels in the same words alone."""
+    D, F = 128, 64
+    wg, wu, wd, x = inputs.make_small(D, F, 1, seed=bits)
+    bad = wg.copy()
+    bad[5, 9] = 0x7F80                                              # inf
+    bad[6, :] = inputs.f32_to_bf16_bits(np.full(D, 1e30, dtype=np.float32))
+    p = Problem(pb, bad, wu, wd, x)
+    try:
+        pb.prox_quantize_proxy(p.h, bits, 128)
+        q, s = np.empty((F, D), dtype=np.int8), np.empty((F, 1), dtype=np.float32)
+        pb.prox_proxy_export(p.h, 0, q, s)
+        q_ref, s_ref = po.quantize_proxy(inputs.bf16_bits_to_f32(wg), bits, 128)
+        others = [j for j in range(F) if j not in (5, 6)]
+        assert np.array_equal(q[others], q_ref[others]) and np.array_equal(s[others], s_ref.astype(np.float32)[others])
+    finally:
+        p.close()
