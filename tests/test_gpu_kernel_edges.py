@@ -526,14 +526,15 @@ def test_persistent_kernel_mask_is_the_exact_topk_of_its_scores(pb, F, bits, dis
             pb.prox_stage2_ffn(h, x, 1, sel, k2, ref)
             # the same products, summed in fp32 in another order
             assert (y - ref).norm() <= 1e-5 * ref.norm(), k2
-            tau = float(sc[order[-1]])
-            n = int((sc >= tau).sum())
-            xa = float(x[0].float().abs().sort(descending=True).values[k1 - 1])
-            if int((x[0].float().abs() >= xa).sum()) == k1:         # the same inputs, hence the same scores
-                kept = torch.empty(1, n, dtype=torch.int32, device="cuda")
-                pb.prox_ffn_forward_threshold(h, x, 1, xa, tau, y)
-                pb.prox_ffn_last_mask(h, 1, n, kept)
-                assert torch.equal(kept[0].long(), (sc >= tau).nonzero()[:, 0]), k2
+            kth, xa = sc[order[-1]], float(x[0].float().abs().sort(descending=True).values[k1 - 1])
+            below = sc[sc < kth]
+            nxt = below.max() if below.numel() else torch.zeros_like(kth)
+            # between two scores (1e-5 apart or more), and with the same inputs, hence the same scores
+            if kth - nxt > 1e-5 * kth and int((x[0].float().abs() >= xa).sum()) == k1:
+                kept = torch.empty(1, int((sc >= kth).sum()), dtype=torch.int32, device="cuda")
+                pb.prox_ffn_forward_threshold(h, x, 1, xa, float((kth + nxt) / 2), y)
+                pb.prox_ffn_last_mask(h, 1, kept.shape[1], kept)
+                assert torch.equal(kept[0].long(), (sc >= kth).nonzero()[:, 0]), k2
         assert pb.prox_last_device_status(h) == 0
     finally:
         pb.prox_ffn_destroy(h)
