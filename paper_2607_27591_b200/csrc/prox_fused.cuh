@@ -258,15 +258,14 @@ __device__ __forceinline__ unsigned kth_in_segment(const unsigned* hist, int top
   return bin;
 }
 
-// Same over 512 * BPL bins with the whole block (one block barrier inside):
+// Same over 512 * BPL bins with the 16 consumer warps (one barrier of theirs inside):
 // warps 0..15 total their segment, then every warp locates the segment and
 // finishes on its own, so the result is in the registers of every thread.
-// CONSUMERS_ONLY: called by the 16 consumer warps alone (named barrier).
-template <int BPL, bool CONSUMERS_ONLY>
+template <int BPL>
 __device__ __forceinline__ unsigned kth_in_block(const unsigned* hist, unsigned k, unsigned* wsum, int lane, int warp,
                                                  unsigned* above) {
   constexpr int NB = 512 * BPL, SEG = 32 * BPL;
-  if (warp < 16) {
+  {
     const int base = NB - warp * SEG - (lane + 1) * BPL;
     unsigned s = 0;
 #pragma unroll 1
@@ -274,7 +273,7 @@ __device__ __forceinline__ unsigned kth_in_block(const unsigned* hist, unsigned 
     s = __reduce_add_sync(0xffffffffu, s);
     if (lane == 0) wsum[warp] = s;
   }
-  if (CONSUMERS_ONLY) consumer_sync(); else __syncthreads();
+  consumer_sync();
   const unsigned v = (lane < 16) ? wsum[lane] : 0u;
   const unsigned inc = warp_scan_incl(v, lane);
   const unsigned ex = inc - v;
@@ -335,14 +334,14 @@ struct FusedSmem {
 // the first of them bin `top`; the threads' runs follow each other downwards (threads from 512 on: zeros).  One scan and two
 // barriers where reading the bins segment by segment took three passes over shared memory (0.8 -> 0.4 us for 1024 bins,
 // 1.1 -> 0.6 for 2048).  res[0..2] = bin, elements above it, elements inside.
-template <int N, bool CONSUMERS_ONLY>
+template <int N>
 __device__ __forceinline__ void find_kth(FusedSmem& sm, const unsigned (&c)[N], int top, unsigned k, int lane, int warp) {
   unsigned s = 0;
 #pragma unroll
   for (int j = 0; j < N; ++j) s += c[j];
   const unsigned inc = warp_scan_incl(s, lane);
   if (lane == 31) sm.wsum[warp] = inc;
-  if (CONSUMERS_ONLY) consumer_sync(); else __syncthreads();
+  __syncthreads();
   unsigned run = __reduce_add_sync(0xffffffffu, (lane < warp) ? sm.wsum[lane] : 0u) + inc - s;
   if (run < k && k <= run + s) {
 #pragma unroll
@@ -351,7 +350,7 @@ __device__ __forceinline__ void find_kth(FusedSmem& sm, const unsigned (&c)[N], 
       run += c[j];
     }
   }
-  if (CONSUMERS_ONLY) consumer_sync(); else __syncthreads();
+  __syncthreads();
 }
 
 // NG = warp groups of the down projection (4: d_model <= 4096, 2: <= 8192, 1: <= 16384)
@@ -547,7 +546,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       PROX_TRACE(10);
       unsigned hb[2] = {0u, 0u};
       if (tid < 512) { const uint2 v = reinterpret_cast<const uint2*>(sm.hist)[511 - tid]; hb[0] = v.y; hb[1] = v.x; }
-      find_kth<2, false>(sm, hb, 1023 - 2 * tid, (unsigned)k1, lane, warp);
+      find_kth<2>(sm, hb, 1023 - 2 * tid, (unsigned)k1, lane, warp);
       const unsigned bin1 = sm.res[0], above1 = sm.res[1];
       PROX_TRACE(11);
       if (warp < kFusedConsumerWarps) {
@@ -1203,7 +1202,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
           }
           consumer_sync();
           unsigned ab;
-          const unsigned bb = kth_in_block<2, true>(sm.hist, kleft, sm.wsum, lane, warp, &ab);
+          const unsigned bb = kth_in_block<2>(sm.hist, kleft, sm.wsum, lane, warp, &ab);
           prefix = (prefix << 10) | bb;
           kleft -= ab;
         }
