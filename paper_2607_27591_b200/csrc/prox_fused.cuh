@@ -941,9 +941,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     tc_fence_before();
     fence_proxy_async();                        // phase B's plain accesses to the big buffer come before the ring's bulk copies
     __syncthreads();
-    if (HIST && ntl > 1) {
+    if (HIST && ntl > 1 && warp < kFusedConsumerWarps) {      // (only by them: phase C counts in sm.hist behind their barrier, not the block's)
 #pragma unroll 1
-      for (int i = tid; i < 2048; i += NT) { const unsigned v = sm.hist[i]; if (v) { atomicAdd(ghist + i, v); sm.hist[i] = 0u; } }
+      for (int i = tid; i < 2048; i += kFusedConsumers) { const unsigned v = sm.hist[i]; if (v) { atomicAdd(ghist + i, v); sm.hist[i] = 0u; } }
     }
     PROX_TRACE(3);
     if (MODE == kWhole && tid == 0 && vid < n1 && sm.abort_flag == 0)

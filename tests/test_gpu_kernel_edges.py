@@ -558,3 +558,42 @@ def test_packer_keeps_what_is_not_a_number_to_its_channel(pb, bits):
         assert np.array_equal(q[others], q_ref[others]) and np.array_equal(s[others], s_ref.astype(np.float32)[others])
     finally:
         p.close()
+
+
+def _mask_is_the_exact_topk(pb, D, F, bits, group, distinct, zero):
+    """Forward calls on repeated channels (`distinct` different ones, 0 = all): the mask against a stable sort of the scores
+    that it was made from, y against Stage 2 on that mask."""
+    g = torch.Generator(device="cuda").manual_seed(D + F + distinct)
+    w = [torch.empty(F, D, dtype=torch.bfloat16, device="cuda").normal_(0.0, 0.5 / D ** 0.5, generator=g) for _ in range(2)]
+    if distinct:
+        for t in w:
+            t.copy_(t[torch.arange(F, device="cuda") % distinct])
+    wd = torch.empty(D, F, dtype=torch.bfloat16, device="cuda").normal_(0.0, 0.1, generator=g)
+    x = torch.zeros(1, D, device="cuda") if zero else torch.randn(1, D, device="cuda", generator=g)
+    x, k1 = x.to(torch.bfloat16), D // 3
+    h = pb.prox_ffn_create(D, F, 1, 1, *w, wd)
+    try:
+        pb.prox_quantize_proxy(h, bits, group)
+        y, ref, sc = (torch.empty(n, dtype=torch.float32, device="cuda") for n in (D, D, F))
+        for k2 in (1, F // 3 + 1, F - 1):
+            sel = torch.empty(1, k2, dtype=torch.int32, device="cuda")
+            pb.prox_ffn_forward(h, x, 1, k1, k2, y)
+            pb.prox_ffn_last_mask(h, 1, k2, sel)
+            pb.prox_ffn_last_stage1(h, k1, None, sc)
+            order = torch.sort(sc, descending=True, stable=True).indices[:k2]
+            assert torch.equal(sel[0].long(), order.sort().values), k2
+            pb.prox_stage2_ffn(h, x, 1, sel, k2, ref)
+            # the same products, summed in fp32 in another order
+            assert (y - ref).norm() <= 1e-5 * ref.norm(), k2
+        assert pb.prox_last_device_status(h) == 0
+    finally:
+        pb.prox_ffn_destroy(h)
+
+
+@pytest.mark.parametrize("zero", [False, True])
+@pytest.mark.parametrize("D,F,bits,group,distinct", [(128, 40960, 4, 128, 1), (128, 65536, 4, 0, 2), (128, 65536, 8, 128, 1), (8192, 28672, 4, 0, 1)])
+def test_threshold_bin_too_long_for_its_list(pb, D, F, bits, group, distinct, zero):
+    """So many equal scores that the list of the threshold bin's members has no room in shared memory (20928 members at
+    128 x 65536, 33216 at 128 x 40960, 23232 at 8192 x 28672): radix steps over all channels, in blocks that have had
+    several tiles of the proxy rows each."""
+    _mask_is_the_exact_topk(pb, D, F, bits, group, distinct, zero)
