@@ -185,7 +185,7 @@ prox_status_t prox_ffn_last_stage1(prox_ffn_t* h, int k1, int32_t* idx_dev_or_nu
  * blocks' scores from ever completing, so that the next B = 1 forward call runs into the limit, leaves
  * without writing y and reports it (see prox_last_device_status).  With bit 31 set it is a wait inside
  * Stage 1 of one block instead (the one with the first share of the columns), which Stage 1 called alone
- * has too.  Nothing hangs or faults: the blocks give up and return.  Set both back to 0 afterwards. */
+ * has too; with bit 30 set the wait for whole scores while the top-k form settles its threshold.  Nothing hangs or faults: the blocks give up and return.  Set both back to 0 afterwards. */
 prox_status_t prox_debug_set_wait(prox_ffn_t* h, uint32_t spin_limit, uint32_t barrier_bias);
 
 /* Test hook: blocks the persistent kernel is launched with (0 = one per SM, at most that).  With fewer, the blocks

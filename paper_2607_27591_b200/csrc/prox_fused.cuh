@@ -76,7 +76,7 @@ struct FusedParams {
   uint16_t* xhalf; unsigned* xkeys;   // [2][F] each
   int* idx_out;       // the kept input list as this kernel built it (block 0 writes it; for checking)
   unsigned spin_limit;        // polls after which a device-side wait gives up
-  unsigned bar_bias;          // test knob (0 in normal use): the wait for the scores does not end; bit 31: see prox_debug_set_wait
+  unsigned bar_bias;          // test knob (0 in normal use): the wait for the scores does not end; bits 30 and 31: see prox_debug_set_wait
   int* host_flag;             // mapped host word set to 1 when a wait expires (NULL = none)
   float* yacc; int* status;
   unsigned long long* exits;  // grows by 256 per call, complete when all its blocks have left: the call number
@@ -97,6 +97,7 @@ struct FusedParams {
 };
 
 constexpr unsigned kNoKey = 0xffffffffu;      // no score: those have the sign bit clear
+constexpr unsigned kBiasKeys = 1u << 30;      // bar_bias: no score is there as a whole
 // shares claimed / finished, Stage 1 and Stage 2; kOut1: Stage-1 shares whose scores are on their way
 enum FusedCtr { kClaim1 = 0, kDone1, kClaim2, kDone2, kOut1 };
 
@@ -995,11 +996,14 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   const uint32_t skey_u32 = big_u32 + key_off;
   uint32_t list_u32 = smem_u32(idx16);          // 2 * D bytes: room for D / 2 members
   unsigned klo = 0, khi = 0;                    // half scores from khi on are definite, from klo on members of b1
-  auto full_key = [&](int i) {                  // all bits of a score
-    unsigned v = kNoKey;
+  auto full_key = [&](int i) {                  // all bits of a score (a bounded wait, which ends once the abort flag is up)
+    unsigned v;
 #pragma unroll 1
-    for (unsigned it = 0; v == kNoKey && it < spin; ++it)
+    for (unsigned it = 0;; ++it) {
       asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(xkeys + i) : "memory");
+      if (v != kNoKey && !(p.bar_bias & kBiasKeys)) break;
+      if (it >= spin || *abortp) { *abortp = 1; break; }
+    }
     return v;
   };
   if (warp >= kFusedConsumerWarps) {
@@ -1044,7 +1048,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
     const bool again = sm.again != 0;
     // (a block that has given up hands nothing on, so that the scores are never complete and the call ends before
     // anything is written to y or to the residual stream; neither are they with the test knob)
-    const unsigned target = (p.bar_bias & 0x7fffffffu) ? ~0u : (THRESH ? 0u : (unsigned)F);
+    const unsigned target = (p.bar_bias & (kBiasKeys - 1u)) ? ~0u : (THRESH ? 0u : (unsigned)F);
     const unsigned tries = !again && sm.res[7] ? spin : 0u;
 #pragma unroll 1
     for (unsigned it = 0; it < tries; ++it) {
@@ -1377,7 +1381,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
         PROX_TRACE(20);
         __threadfence_block();
         settler_sync();                          // the list is free from here on
-        if (tid == 0) {
+        if (tid == 0 && !*abortp) {              // (without all scores the list may have gaps: no rows are asked for by it)
           *reinterpret_cast<volatile int*>(&sm.nready) = n_mine;
           __threadfence_block();
           *reinterpret_cast<volatile int*>(&sm.c_done) = 1;

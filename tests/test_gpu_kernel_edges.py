@@ -597,3 +597,37 @@ def test_threshold_bin_too_long_for_its_list(pb, D, F, bits, group, distinct, ze
     128 x 65536, 33216 at 128 x 40960, 23232 at 8192 x 28672): radix steps over all channels, in blocks that have had
     several tiles of the proxy rows each."""
     _mask_is_the_exact_topk(pb, D, F, bits, group, distinct, zero)
+
+
+@pytest.mark.parametrize("D,F,distinct", [(512, 1536, 0), (512, 1536, 1), (128, 65536, 1)])
+def test_whole_scores_that_do_not_come_are_reported(pb, D, F, distinct):
+    """Where the threshold is settled by ranking, by radix steps over the list and by radix steps over all channels: a wait for
+    a whole score that runs out ends the call without y and with its status; the threshold form has no such wait, and the next
+    call is ordinary."""
+    g = torch.Generator(device="cuda").manual_seed(F)
+    w = [torch.empty(F, D, dtype=torch.bfloat16, device="cuda").normal_(0.0, 0.04, generator=g) for _ in range(3)]
+    if distinct:
+        for t in w[:2]:
+            t.copy_(t[torch.arange(F, device="cuda") % distinct])
+    x = torch.randn(1, D, device="cuda", generator=g).to(torch.bfloat16)
+    h = pb.prox_ffn_create(D, F, 1, 1, w[0], w[1], w[2].view(D, F))
+    try:
+        pb.prox_quantize_proxy(h, 4, 128)
+        k1, k2 = D // 3, F // 3 + 1
+        y, again = (torch.full((1, D), 7.0, device="cuda") for _ in range(2))
+        pb.prox_debug_set_wait(h, 300, 1 << 30)
+        pb.prox_ffn_forward(h, x, 1, k1, k2, y)
+        status, code = pb.prox_last_device_status_raw(h)
+        assert code & 4 and status == 6 and torch.all(y == 7.0)         # PROX_ERR_TIMEOUT
+        pb.prox_ffn_forward_threshold(h, x, 1, 0.5, 1e-3, y)
+        assert pb.prox_last_device_status(h) == 0 and not torch.any(y == 7.0)
+        pb.prox_debug_set_wait(h, 0, 0)
+        sel = torch.empty(1, k2, dtype=torch.int32, device="cuda")
+        pb.prox_ffn_forward(h, x, 1, k1, k2, y)
+        pb.prox_ffn_last_mask(h, 1, k2, sel)
+        pb.prox_stage2_ffn(h, x, 1, sel, k2, again)
+        # the same products, summed in fp32 in another order
+        assert (y - again).norm() <= 1e-5 * again.norm()
+        assert pb.prox_last_device_status(h) == 0
+    finally:
+        pb.prox_ffn_destroy(h)
