@@ -865,8 +865,10 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
           const float u0 = __shfl_xor_sync(0xffffffffu, t0, 8), u1 = __shfl_xor_sync(0xffffffffu, t1, 8);
           unsigned n0 = 1u, n1 = 1u, b0 = 0u, b1 = 0u;          // (scores in front of this thread's in their bins)
           const bool give = MODE == kScoresOnly || *abortp == 0;          // a block that has given up hands nothing on
-          const float s0 = fabsf(u0 * silu_fast(t0)), s1 = LO ? fabsf(u1 * silu_fast(t1)) : 0.f;
-          const unsigned k0 = __float_as_uint(s0), k1b = __float_as_uint(s1);
+          // (the sign is cleared as a bit: it says "not there yet" to the other blocks, and bins go by the bits behind it; fabsf
+          // need not clear it for what is not a number, as weights and inputs that are not finite make it)
+          const unsigned k0 = __float_as_uint(u0 * silu_fast(t0)) & 0x7fffffffu, k1b = LO ? __float_as_uint(u1 * silu_fast(t1)) & 0x7fffffffu : 0u;
+          const float s0 = __uint_as_float(k0), s1 = __uint_as_float(k1b);
           if (MODE == kWhole && THRESH) {
             // marks of a chunk: bit i = its channel i (4-bit codes: a lane has channels 2 i and 2 i + 1)
             const unsigned m0 = __ballot_sync(0xffffffffu, k0 >= p.tkey_s) >> (lane & 16), m1 = LO ? __ballot_sync(0xffffffffu, k1b >= p.tkey_s) >> (lane & 16) : 0u;

@@ -631,3 +631,38 @@ def test_whole_scores_that_do_not_come_are_reported(pb, D, F, distinct):
         assert pb.prox_last_device_status(h) == 0
     finally:
         pb.prox_ffn_destroy(h)
+
+
+@pytest.mark.parametrize("bits,group", [(4, 0), (4, 128), (8, 0), (8, 128)])
+def test_channels_that_are_not_finite(pb, bits, group):
+    """Weights that are infinite or not a number, of either sign: their channels rank by the bits of their scores (not a number
+    above infinity above the rest), the other channels and the call are as ever, and the threshold form keeps them."""
+    D, F, k1 = 512, 1536, 170
+    wg, wu, wd, x = inputs.make_small(D, F, 1, seed=bits + group)
+    for row, value in ((5, 0x7F80), (6, 0xFF80), (700, 0x7FC0), (1535, 0xFFC0), (40, 0x7F80)):      # inf, -inf, nan, -nan, inf
+        wg[row, :] = value
+    wu[41, 3], wu[900, :] = 0x7F80, 0xFFFF
+    h_args = [dev_bf16(t) for t in (wg, wu, wd)]
+    h = pb.prox_ffn_create(D, F, 1, 1, *h_args)
+    try:
+        pb.prox_quantize_proxy(h, bits, group)
+        t_x, y, sc = dev_bf16(x), torch.empty(1, D, device="cuda"), torch.empty(F, device="cuda")
+        for k2 in (1, 3, 8, F // 3, F):
+            sel = torch.empty(1, k2, dtype=torch.int32, device="cuda")
+            pb.prox_ffn_forward(h, t_x, 1, k1, k2, y)
+            pb.prox_ffn_last_mask(h, 1, k2, sel)
+            pb.prox_ffn_last_stage1(h, k1, None, sc)
+            keys = sc.view(torch.int32)
+            assert int(keys.min()) >= 0 and not bool(torch.isfinite(sc[[5, 6, 40, 700, 900, 1535]]).any())
+            order = torch.sort(keys, descending=True, stable=True).indices
+            assert torch.equal(sel[0].long(), order[:k2].sort().values), k2
+            tau_x = float(t_x[0].float().abs().sort(descending=True).values[k1 - 1])
+            if int((t_x[0].float().abs() >= tau_x).sum()) == k1:          # the same inputs, hence the same scores
+                kept = (keys >= torch.tensor(0.01, device="cuda").view(torch.int32)).nonzero()[:, 0]
+                got = torch.empty(1, kept.numel(), dtype=torch.int32, device="cuda")
+                pb.prox_ffn_forward_threshold(h, t_x, 1, tau_x, 0.01, y)
+                pb.prox_ffn_last_mask(h, 1, kept.numel(), got)
+                assert torch.equal(got[0].long(), kept), k2
+        assert pb.prox_last_device_status(h) == 0
+    finally:
+        pb.prox_ffn_destroy(h)
