@@ -159,6 +159,12 @@ __device__ __forceinline__ uint4 ld_relaxed4(const unsigned* p) {
   asm volatile("ld.relaxed.gpu.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
   return v;
 }
+__device__ __forceinline__ void st_relaxed(unsigned* p, unsigned v) {
+  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ void st_relaxed2(unsigned* p, unsigned a, unsigned b) {
+  asm volatile("st.relaxed.gpu.global.v2.u32 [%0], {%1,%2};" ::"l"(p), "r"(a), "r"(b) : "memory");
+}
 __device__ __forceinline__ unsigned every_other_bit(unsigned v) {          // bits 0..7 to bits 0, 2, .., 14
   v = (v | (v << 4)) & 0x0f0fu;
   v = (v | (v << 2)) & 0x3333u;
@@ -872,18 +878,16 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
           if (MODE == kWhole && THRESH) {
             // marks of a chunk: bit i = its channel i (4-bit codes: a lane has channels 2 i and 2 i + 1)
             const unsigned m0 = __ballot_sync(0xffffffffu, k0 >= p.tkey_s) >> (lane & 16), m1 = LO ? __ballot_sync(0xffffffffu, k1b >= p.tkey_s) >> (lane & 16) : 0u;
-            if ((lane & 15) == 0 && col_ok && give) __stcg(reinterpret_cast<unsigned*>(xhalf) + chunk, LO ? every_other_bit(m0 & 0xffu) | (every_other_bit(m1 & 0xffu) << 1) : m0 & 0xffu);
+            if ((lane & 15) == 0 && col_ok && give) st_relaxed(reinterpret_cast<unsigned*>(xhalf) + chunk, LO ? every_other_bit(m0 & 0xffu) | (every_other_bit(m1 & 0xffu) << 1) : m0 & 0xffu);
           }
+          const unsigned knext = LO ? k1b : (MODE == kWhole && !THRESH) ? __shfl_down_sync(0xffffffffu, k0, 1) : 0u;
           if ((col & 8) == 0 && col_ok && give) {
             const int ch = chunk * CH + (LO ? 2 : 1) * (col & 7);
             if (MODE == kWhole && !THRESH) {
-              if (LO) {
-                __stcg(reinterpret_cast<unsigned*>(xhalf + ch), __byte_perm(k0, k1b, 0x7632));
-                __stcg(reinterpret_cast<uint2*>(xkeys + ch), make_uint2(k0, k1b));
-              } else {
-                __stcg(reinterpret_cast<unsigned short*>(xhalf + ch), (unsigned short)(k0 >> 16));
-                __stcg(xkeys + ch, k0);
-              }
+              // (halves in whole words, as they are read: 8-bit codes have the odd channel's in the next lane)
+              if (LO || (lane & 1) == 0) st_relaxed(reinterpret_cast<unsigned*>(xhalf + ch), __byte_perm(k0, knext, 0x7632));
+              if (LO) st_relaxed2(xkeys + ch, k0, k1b);
+              else st_relaxed(xkeys + ch, k0);
             }
             if (LO) __stcg(reinterpret_cast<float2*>(p.scores + ch), make_float2(s0, s1));
             else __stcg(p.scores + ch, s0);
@@ -970,7 +974,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   // ---------------------------------------- C: channel mask (top-k2 of the scores)
   // The blocks wait for a count of finished shares that is not ordered behind the scores; the scores themselves say that
   // they are there (all ones = not yet), and the histogram that it is complete (it counts all channels): what is missing is read
-  // again.  (With a barrier, i.e. a count released behind the acknowledgement of all the block's writes and acquired, and with whole
+  // again.  That needs every aligned 32-bit word to be written and read as one, and a later read to see what has been written by
+  // then: relaxed stores and loads at gpu scope promise both.  The copies of the first round promise neither by the letter
+  // (they are weak); they go to L2, where the words are whole, and a word that they miss is one more round, of relaxed loads.  (With a barrier, i.e. a count released behind the acknowledgement of all the block's writes and acquired, and with whole
   // scores, counted by every thread in a run of its own, the first copy of phase D came 6.2 us after the last block's scores at
   // 4096 x 12288 where it comes after 4.8, and 3.6 instead of 2.9 at 512 x 1536.  What goes to every block is 2 bytes per channel;
   // the threshold form hands on one bit, which the block that has the score decides.  Reading histogram and scores in a loop
@@ -1057,7 +1063,14 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
       if (!THRESH) hv = ld_relaxed4(ghist + 4 * (511 - tid));
       if (in_smem) {
 #pragma unroll 1
-        for (int q = q0; q < qend; q += qstep) cp_async16(skey_u32 + (uint32_t)q * 16u, xhalf + 8 * q);
+        for (int q = q0; q < qend; q += qstep) {
+          if (it == 0) {
+            cp_async16(skey_u32 + (uint32_t)q * 16u, xhalf + 8 * q);
+          } else {
+            const uint4 v = ld_relaxed4(reinterpret_cast<const unsigned*>(xhalf) + 4 * q);
+            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(skey_u32 + (uint32_t)q * 16u), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+          }
+        }
       }
       cp_async_commit();
       if (tid < 256) sm.hist2[tid] = 0;
