@@ -360,6 +360,189 @@ __device__ __forceinline__ void find_kth(FusedSmem& sm, const unsigned (&c)[N], 
   __syncthreads();
 }
 
+// All bits of the scores of eight channels: a bounded wait, which ends once the abort flag is up.
+__device__ __forceinline__ void full_keys(const unsigned* xkeys, const int (&i)[8], unsigned (&k)[8], unsigned spin, unsigned bias, volatile int* abortp) {
+#pragma unroll 1
+  for (unsigned it = 0;; ++it) {
+    unsigned any = 0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(k[u]) : "l"(xkeys + i[u]) : "memory");
+#pragma unroll
+    for (int u = 0; u < 8; ++u) any |= k[u];
+    if (!(any >> 31) && !(bias & kBiasKeys)) break;
+    if (it >= spin || *abortp) { *abortp = 1; break; }
+  }
+}
+__device__ __forceinline__ unsigned lds32(uint32_t a) {
+  unsigned v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+  return v;
+}
+
+// Channel mask where shared memory has no room for the half scores and the list of the threshold bin b1's members (a very large
+// d_model and d_ff, or a huge bin such as an all-zero input gives): the consumer warps settle the threshold by two radix steps of
+// 10 bits over all scores, and the block gets its share of the plain ascending list of k2 channels.  Returns the share's length.
+// (A function of its own, as the next one: inside the kernel, the two cost calls that never get here 1 % of 8192 x 28672.)
+__device__ __noinline__ int settle_over_all_channels(const unsigned* xkeys, int F, unsigned k2, unsigned shr, unsigned nsh, unsigned b1, unsigned kk,
+                                                     int* sel_out, unsigned spin, unsigned bias) {
+  extern __shared__ __align__(128) uint8_t smem_raw[];
+  FusedSmem& sm = *reinterpret_cast<FusedSmem*>(smem_raw);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const unsigned lt_mask = (1u << lane) - 1u;
+  const int R0 = (int)((k2 * shr) / nsh), R1 = (int)((k2 * (shr + 1u)) / nsh);
+  const int per = ((F + 32 * kFusedConsumerWarps - 1) / (32 * kFusedConsumerWarps)) * 32;        // channels per warp run
+  const int i0 = min(F, warp * per), i1 = min(F, i0 + per);
+  const int n_mine = min(R1 - R0, kMySelCap);
+  int ch[8];
+  unsigned key[8];
+  unsigned prefix = b1, kleft = kk;
+#pragma unroll 1
+  for (int sh = 10; sh >= 0; sh -= 10) {
+    consumer_sync();
+#pragma unroll 1
+    for (int i = tid; i < 1024; i += kFusedConsumers) sm.hist[i] = 0;
+    consumer_sync();
+#pragma unroll 1
+    for (int ib = tid; ib < F; ib += 8 * kFusedConsumers) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) ch[u] = min(ib + u * kFusedConsumers, F - 1);
+      full_keys(xkeys, ch, key, spin, bias, &sm.abort_flag);
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (ib + u * kFusedConsumers < F && (key[u] >> (sh + 10)) == prefix) atomicAdd(&sm.hist[(key[u] >> sh) & 1023u], 1u);
+    }
+    consumer_sync();
+    unsigned ab;
+    const unsigned bb = kth_in_block<2>(sm.hist, kleft, sm.wsum, lane, warp, &ab);
+    prefix = (prefix << 10) | bb;
+    kleft -= ab;
+  }
+  const unsigned T = prefix, quota = kleft;
+  consumer_sync();
+  {
+    unsigned cg = 0, ce = 0;                 // separate words: the ties alone may be 65536
+#pragma unroll 1
+    for (int ib = i0 + lane; ib < i1; ib += 8 * 32) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) ch[u] = min(ib + u * 32, F - 1);
+      full_keys(xkeys, ch, key, spin, bias, &sm.abort_flag);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) { cg += (ib + u * 32 < i1 && key[u] > T) ? 1u : 0u; ce += (ib + u * 32 < i1 && key[u] == T) ? 1u : 0u; }
+    }
+    cg = __reduce_add_sync(0xffffffffu, cg);
+    ce = __reduce_add_sync(0xffffffffu, ce);
+    if (lane == 0) { sm.wsum[warp] = cg; sm.warp_cnt[warp][1] = ce; }
+  }
+  consumer_sync();
+  unsigned bg = __reduce_add_sync(0xffffffffu, (lane < warp) ? sm.wsum[lane] : 0u);
+  unsigned be = __reduce_add_sync(0xffffffffu, (lane < warp) ? sm.warp_cnt[lane][1] : 0u);
+  const int first_pos = (int)(bg + min(be, quota));
+  const int end = (int)(bg + sm.wsum[warp] + min(be + sm.warp_cnt[warp][1], quota));
+  if (first_pos < R1 && end > R0) {
+#pragma unroll 1
+    for (int ib = i0; ib < i1; ib += 8 * 32) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) ch[u] = min(ib + u * 32 + lane, F - 1);
+      full_keys(xkeys, ch, key, spin, bias, &sm.abort_flag);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int i = ib + u * 32 + lane;
+        const bool gt = i < i1 && key[u] > T, eq = i < i1 && key[u] == T;
+        const unsigned mg = __ballot_sync(0xffffffffu, gt), me = __ballot_sync(0xffffffffu, eq);
+        const unsigned myre = be + (unsigned)__popc(me & lt_mask);
+        const int pos = (int)(bg + (unsigned)__popc(mg & lt_mask) + min(myre, quota));
+        if ((gt || (eq && myre < quota)) && pos >= R0 && pos < R0 + n_mine) {
+          sm.mysel[pos - R0] = i;
+          if (sel_out) sel_out[pos] = i;
+        }
+        bg += (unsigned)__popc(mg); be += (unsigned)__popc(me);
+      }
+    }
+  }
+  return n_mine;
+}
+
+// Members of the threshold bin (list entries: four bits of the half score above the channel) of which more than kCand2Cap agree with the
+// threshold in their half scores, i.e. have `sub` there: the kk2 of them that come first by (score descending, channel
+// ascending) follow at place `above` of the members that are kept, of which the block has Rc0 .. Rc1 - 1.  Radix steps of 8 bits
+// over the lower halves and the inverted channels, which a thread puts in the place of its entries first.  By the settler warps.
+// An input of zeros at 4096 x 12288: 52 us per call; 152 with the lower halves fetched one at a time in every step, 65 when
+// all scores were whole ones in shared memory.
+__device__ __noinline__ void settle_equal_halves(uint32_t list_u32, unsigned nb1, unsigned sub, unsigned kk2, const unsigned* xkeys, int above, int Rc0,
+                                                 int Rc1, int ndm, int* sel_out, unsigned spin, unsigned bias) {
+  extern __shared__ __align__(128) uint8_t smem_raw[];
+  FusedSmem& sm = *reinterpret_cast<FusedSmem*>(smem_raw);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  unsigned mine = tid, low = ~0u, high = 0;       // end of the thread's values; lowest and highest lower half
+  settler_sync();                                 // the list is read by other threads than write it here
+#pragma unroll 1
+  for (unsigned c = tid; c < nb1; c += 8 * kSettlers) {
+    unsigned e[8], key[8];
+    int ch[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      e[u] = c + u * kSettlers < nb1 ? lds32(list_u32 + (c + u * kSettlers) * 4u) : ~0u;
+      ch[u] = (e[u] >> 16) == sub ? (int)(e[u] & 0xffffu) : 0;
+    }
+    full_keys(xkeys, ch, key, spin, bias, &sm.abort_flag);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if ((e[u] >> 16) == sub) {
+        asm volatile("st.shared.u32 [%0], %1;" ::"r"(list_u32 + mine * 4u), "r"((key[u] << 16) | (0xffffu ^ (unsigned)ch[u])) : "memory");
+        mine += kSettlers;
+        low = min(low, key[u] & 0xffffu); high = max(high, key[u] & 0xffffu);
+      }
+    }
+  }
+  // (all the same score, as where there are many: two steps less)
+  low = __reduce_min_sync(0xffffffffu, low); high = __reduce_max_sync(0xffffffffu, high);
+  if (lane == 0) { sm.cand2_key[warp] = low; sm.cand2_key[kSettlerWarps + warp] = high; }
+  settler_sync();
+  low = __reduce_min_sync(0xffffffffu, lane < kSettlerWarps ? sm.cand2_key[lane] : ~0u);
+  high = __reduce_max_sync(0xffffffffu, lane < kSettlerWarps ? sm.cand2_key[kSettlerWarps + lane] : 0u);
+  // (four entries at a time: one would wait for its load and its bin before the next)
+  unsigned prefix = low == high ? low : 0u, kleft = kk2;
+#pragma unroll 1
+  for (int sh = low == high ? 8 : 24; sh >= 0; sh -= 8) {
+    settler_sync();                               // everyone is done with the previous histogram
+    sm.hist2[tid] = 0;
+    settler_sync();
+#pragma unroll 1
+    for (unsigned c = tid; c < mine; c += 4 * kSettlers) {
+      unsigned v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[u] = c + u * kSettlers < mine ? lds32(list_u32 + (c + u * kSettlers) * 4u) : 0u;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (c + u * kSettlers < mine && (unsigned)((unsigned long long)v[u] >> (sh + 8)) == prefix) atomicAdd(&sm.hist2[(v[u] >> sh) & 255u], 1u);
+    }
+    settler_sync();
+    unsigned ab;
+    const unsigned bb = kth_in_segment<8>(sm.hist2, 256, kleft, lane, &ab);
+    prefix = (prefix << 8) | bb;
+    kleft -= ab;
+  }
+  unsigned wk = 0;
+#pragma unroll 4
+  for (unsigned c = tid; c < mine; c += kSettlers) wk += lds32(list_u32 + c * 4u) >= prefix ? 1u : 0u;
+  const unsigned inck = warp_scan_incl(wk, lane);
+  if (lane == 31) sm.warp_cnt[warp][1] = inck;
+  settler_sync();
+  int at = above + (int)(__reduce_add_sync(0xffffffffu, lane < warp ? sm.warp_cnt[lane][1] : 0u) + inck - wk);
+  if (at < Rc1 && at + (int)wk > Rc0) {
+#pragma unroll 1
+    for (unsigned c = tid; c < mine; c += kSettlers) {
+      const unsigned v = lds32(list_u32 + c * 4u);
+      if (v < prefix) continue;
+      if (at >= Rc0 && at < Rc1) {
+        sm.mysel[ndm + at - Rc0] = (int)(0xffffu ^ (v & 0xffffu));
+        if (sel_out) sel_out[at] = (int)(0xffffu ^ (v & 0xffffu));
+      }
+      ++at;
+    }
+  }
+}
+
 // NG = warp groups of the down projection (4: d_model <= 4096, 2: <= 8192, 1: <= 16384)
 // NORM = layer sub-block form (RMSNorm in the prologue, residual add at the end); THRESH = threshold
 // form of the two masks (Sec. 4.1 indicators with calibrated thresholds; no k-th element search at all).
@@ -1199,68 +1382,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
           }
         }
       } else if (shr < NSH) {
-        // No room in shared memory for the half scores plus the list of b1's members (a very large d_model and d_ff, or a huge threshold bin such
-        // as an all-zero input gives):
-        // the consumer warps settle the threshold by two radix steps of 10 bits over all keys and the block keeps its
-        // share of the plain ascending list before the ring starts.
-        const int R0 = (int)(((unsigned)k2 * shr) / NSH), R1 = (int)(((unsigned)k2 * (shr + 1u)) / NSH);
-        const int per = ((F + 32 * kFusedConsumerWarps - 1) / (32 * kFusedConsumerWarps)) * 32;        // channels per warp run
-        const int i0 = min(F, warp * per), i1 = min(F, i0 + per);
-        n_mine = min(R1 - R0, kMySelCap);
-        unsigned prefix = b1, kleft = kk;
-#pragma unroll 1
-        for (int sh = 10; sh >= 0; sh -= 10) {
-          consumer_sync();
-#pragma unroll 1
-          for (int i = tid; i < 1024; i += kFusedConsumers) sm.hist[i] = 0;
-          consumer_sync();
-#pragma unroll 1
-          for (int i = tid; i < F; i += kFusedConsumers) {
-            const unsigned key = full_key(i);
-            if ((key >> (sh + 10)) == prefix) atomicAdd(&sm.hist[(key >> sh) & 1023u], 1u);
-          }
-          consumer_sync();
-          unsigned ab;
-          const unsigned bb = kth_in_block<2>(sm.hist, kleft, sm.wsum, lane, warp, &ab);
-          prefix = (prefix << 10) | bb;
-          kleft -= ab;
-        }
-        const unsigned T = prefix, quota = kleft;
-        consumer_sync();
-        {
-          unsigned cg = 0, ce = 0;                 // separate words: the ties alone may be 65536
-#pragma unroll 1
-          for (int i = i0 + lane; i < i1; i += 32) {
-            const unsigned key = full_key(i);
-            cg += (key > T) ? 1u : 0u; ce += (key == T) ? 1u : 0u;
-          }
-          cg = __reduce_add_sync(0xffffffffu, cg);
-          ce = __reduce_add_sync(0xffffffffu, ce);
-          if (lane == 0) { sm.wsum[warp] = cg; sm.warp_cnt[warp][1] = ce; }
-        }
-        consumer_sync();
-        {
-          unsigned bg = __reduce_add_sync(0xffffffffu, (lane < warp) ? sm.wsum[lane] : 0u);
-          unsigned be = __reduce_add_sync(0xffffffffu, (lane < warp) ? sm.warp_cnt[lane][1] : 0u);
-          const int first_pos = (int)(bg + min(be, quota));
-          const int end = (int)(bg + sm.wsum[warp] + min(be + sm.warp_cnt[warp][1], quota));
-          if (first_pos < R1 && end > R0) {
-#pragma unroll 1
-            for (int ib = i0; ib < i1; ib += 32) {
-              const int i = ib + lane;
-              const unsigned key = full_key(min(i, F - 1));
-              const bool gt = i < i1 && key > T, eq = i < i1 && key == T;
-              const unsigned mg = __ballot_sync(0xffffffffu, gt), me = __ballot_sync(0xffffffffu, eq);
-              const unsigned myre = be + (unsigned)__popc(me & lt_mask);
-              const int pos = (int)(bg + (unsigned)__popc(mg & lt_mask) + min(myre, quota));
-              if ((gt || (eq && myre < quota)) && pos >= R0 && pos < R0 + n_mine) {
-                sm.mysel[pos - R0] = i;
-                if (p.sel_out) p.sel_out[pos] = i;
-              }
-              bg += (unsigned)__popc(mg); be += (unsigned)__popc(me);
-            }
-          }
-        }
+        // no room for the list: the block's share of the plain ascending mask, before the ring starts
+        n_mine = settle_over_all_channels(xkeys, F, (unsigned)k2, shr, NSH, b1, kk, p.sel_out, spin, p.bar_bias);
         if (tid == 0) { sm.keys_s0 = sm.keys_s1 = sm.list_s0 = sm.list_s1 = 0; sm.n_mine = n_mine; sm.nready = n_mine; sm.keys_done = 1; sm.c_done = 1; }
       }
     }
@@ -1279,7 +1402,6 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
   if (MODE == kWhole && !THRESH && warp < kFusedConsumerWarps && ncm > 0) {
         // ---- consumer warps only: the list of b1's members (channel, and the four bits that its half score has below the
         // bin's, with their histogram) ...
-        auto lds32 = [](uint32_t a) -> unsigned { unsigned v; asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a)); return v; };
         if (cnt >> 16) {
           unsigned cpos = ex >> 16;
 #pragma unroll 1
@@ -1356,42 +1478,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
             if (rank < kk2) keep((int)(above + rank), (unsigned)id);
           }
         } else {
-          // many scores agree in their upper halves: radix steps of 8 bits over the lower halves and the inverted channels
-          unsigned prefix = 0, kleft = kk2;
-          auto low = [&](unsigned ch) { return (full_key((int)ch) << 16) | (0xffffu ^ ch); };
-#pragma unroll 1
-          for (int sh = 24; sh >= 0; sh -= 8) {
-            settler_sync();                               // everyone is done with the previous histogram
-            sm.hist2[tid] = 0;
-            settler_sync();
-#pragma unroll 1
-            for (int c = c0; c < c1; ++c) {
-              const unsigned e = lds32(list_u32 + (uint32_t)c * 4u);
-              if ((e >> 16) != sub) continue;
-              const unsigned v = low(e & 0xffffu);
-              if (sh == 24 || (v >> (sh + 8)) == prefix) atomicAdd(&sm.hist2[(v >> sh) & 255u], 1u);
-            }
-            settler_sync();
-            unsigned ab;
-            const unsigned bb = kth_in_segment<8>(sm.hist2, 256, kleft, lane, &ab);
-            prefix = (prefix << 8) | bb;
-            kleft -= ab;
-          }
-          unsigned wk = 0;
-#pragma unroll 1
-          for (int c = c0; c < c1; ++c) {
-            const unsigned e = lds32(list_u32 + (uint32_t)c * 4u);
-            wk += (e >> 16) == sub && low(e & 0xffffu) >= prefix ? 1u : 0u;
-          }
-          const unsigned inck = warp_scan_incl(wk, lane);
-          if (lane == 31) sm.warp_cnt[warp][1] = inck;
-          settler_sync();
-          int at = (int)(above + __reduce_add_sync(0xffffffffu, lane < warp ? sm.warp_cnt[lane][1] : 0u) + inck - wk);
-#pragma unroll 1
-          for (int c = c0; c < c1; ++c) {
-            const unsigned e = lds32(list_u32 + (uint32_t)c * 4u);
-            if ((e >> 16) == sub && low(e & 0xffffu) >= prefix) keep(at++, e & 0xffffu);
-          }
+          settle_equal_halves(list_u32, nb1, sub, kk2, xkeys, (int)above, Rc0, Rc1, ndm, p.sel_out ? p.sel_out + (int)nd : nullptr, spin, p.bar_bias);
         }
         PROX_TRACE(20);
         __threadfence_block();

@@ -666,3 +666,41 @@ def test_channels_that_are_not_finite(pb, bits, group):
         assert pb.prox_last_device_status(h) == 0
     finally:
         pb.prox_ffn_destroy(h)
+
+
+@pytest.mark.parametrize("bits", [4, 8])
+def test_many_scores_that_agree_in_their_upper_halves(pb, bits):
+    """Four channels repeated, with the scale of one group a bit or none at all different: thousands of scores that share their
+    upper 16 bits, equal ones and different ones among them, are cut by their lower halves and then by their channels."""
+    D, F, base = 1024, 16384, 4
+    g = torch.Generator(device="cuda").manual_seed(bits)
+    w = [torch.empty(F, D, dtype=torch.bfloat16, device="cuda").normal_(0.0, 0.03, generator=g) for _ in range(2)]
+    ch = torch.arange(F, device="cuda")
+    for t in w:
+        t.copy_(t[ch % base])
+    up, variant = w[1].view(F, D // 128, 128), (ch // base) % 9
+    for v in range(8):                                              # the group's largest weight one step up
+        rows = (variant == v).nonzero()[:, 0]
+        at = up[rows, v].abs().argmax(dim=1)
+        up.view(torch.int16)[rows, v, at] += 1
+    wd = torch.empty(D, F, dtype=torch.bfloat16, device="cuda").normal_(0.0, 0.1, generator=g)
+    x, k1 = torch.randn(1, D, device="cuda", generator=g).to(torch.bfloat16), 341
+    h = pb.prox_ffn_create(D, F, 1, 1, *w, wd)
+    try:
+        pb.prox_quantize_proxy(h, bits, 128)
+        y, sc = torch.empty(1, D, device="cuda"), torch.empty(F, device="cuda")
+        reached = 0
+        for k2 in (500, 2048, 3000, 4097, 7000, 12000, 16000):
+            sel = torch.empty(1, k2, dtype=torch.int32, device="cuda")
+            pb.prox_ffn_forward(h, x, 1, k1, k2, y)
+            pb.prox_ffn_last_mask(h, 1, k2, sel)
+            pb.prox_ffn_last_stage1(h, k1, None, sc)
+            order = torch.sort(sc, descending=True, stable=True).indices[:k2]
+            assert torch.equal(sel[0].long(), order.sort().values), k2
+            keys = sc.view(torch.int32)
+            alike = keys[(keys >> 16) == (keys[order[-1]] >> 16)]
+            reached += int(alike.numel() > 256 and alike.unique().numel() > 1)
+        assert reached > 0
+        assert pb.prox_last_device_status(h) == 0
+    finally:
+        pb.prox_ffn_destroy(h)
