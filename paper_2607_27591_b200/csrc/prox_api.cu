@@ -43,7 +43,7 @@ struct prox_ffn {
   int* cnt_x;               // [maxB]
   float* part;              // split-K partial sums
   size_t part_floats;
-  unsigned* ticket;         // [maxB][nstrips_max]
+  unsigned* ticket;         // [maxB][strips of the narrowest format]: see ticket_count
   float* scores;            // [maxB][F]
   float* svals;             // [maxB][F] signed proxy values (proxy-values-into-down variant)
   uint16_t* xn;             // [maxB][D] bf16 FFN input of the layer sub-block form (step-wise path)
@@ -168,6 +168,9 @@ int nstrips_for(int F, int bits) {
   const int per_strip = 32 * ch_per_chunk(bits);
   return (F + per_strip - 1) / per_strip;
 }
+
+// Tickets of the step-wise proxy GEMV: one per token and strip; 16-bit strips are the narrowest (128 channels), so the most.
+size_t ticket_count(const prox_ffn_config_t& cfg) { return (size_t)cfg.max_batch * nstrips_for(cfg.d_ff, 16); }
 
 // Row split of the step-wise proxy GEMV: as many blocks as are resident at once (one wave; a few
 // blocks more would run as a second wave and double the time).
@@ -822,11 +825,10 @@ prox_status_t forward_kernels(prox_ffn* h, const void* x, int B, int k1, int k2,
 // A block gave up on a wait: counters shared between blocks may be left half-way.  Put every one of
 // them back to its idle state (the stream is idle when this runs).
 prox_status_t reset_shared_state(prox_ffn* h, cudaStream_t st) {
-  const int ns_max = nstrips_for(h->cfg.d_ff, 8);
   CK(cudaMemsetAsync(h->syncbuf, 0, (4096 + 64) * sizeof(unsigned), st));
   CK(cudaMemsetAsync(h->xkeys, 0xff, (size_t)2 * h->cfg.d_ff * sizeof(unsigned), st));
   CK(cudaMemsetAsync(h->xhalf, 0xff, (size_t)2 * h->cfg.d_ff * sizeof(uint16_t), st));
-  CK(cudaMemsetAsync(h->ticket, 0, (size_t)h->cfg.max_batch * ns_max * sizeof(unsigned), st));
+  CK(cudaMemsetAsync(h->ticket, 0, ticket_count(h->cfg) * sizeof(unsigned), st));
   CK(cudaMemsetAsync(h->yacc, 0, (size_t)h->cfg.max_batch * h->cfg.d_model * sizeof(float), st));
   if (h->gacc) {                               // accumulators of the tensor-core batch path (kept at zero between calls)
     const size_t F = (size_t)h->cfg.d_ff;
@@ -872,7 +874,7 @@ prox_status_t prox_ffn_create(const prox_ffn_config_t* cfg, const void* w_gate, 
   if (e != cudaSuccess) { delete h; return PROX_ERR_CUDA; }
 
   const int D = cfg->d_model, F = cfg->d_ff, MB = cfg->max_batch;
-  const int ns_max = nstrips_for(F, 8);            // 8-bit strips are narrower -> more of them
+  const int ns_max = nstrips_for(F, 8);            // of the integer formats (16 bits: twice as many, of a quarter of the sums each)
   h->part_floats = ((size_t)2 * h->sm_count + (size_t)MB * ns_max + 64) * 1024;
   if (MB > 1) {                                    // union path: [row split][strip][8 tokens][1024]
     const size_t need = ((size_t)h->sm_count + ns_max) * kBT * 1024;
@@ -883,7 +885,7 @@ prox_status_t prox_ffn_create(const prox_ffn_config_t* cfg, const void* w_gate, 
   A(dev_alloc(&h->idx_x, (size_t)MB * D));
   A(dev_alloc(&h->cnt_x, (size_t)MB));
   A(dev_alloc(&h->part, h->part_floats));
-  A(dev_alloc(&h->ticket, (size_t)MB * ns_max));
+  A(dev_alloc(&h->ticket, ticket_count(h->cfg)));
   A(dev_alloc(&h->scores, (size_t)MB * F));
   A(dev_alloc(&h->svals, (size_t)MB * F));      // (allocated here, not on first use: a first use may be under graph capture)
   A(dev_alloc(&h->xn, (size_t)MB * D));
@@ -927,7 +929,7 @@ prox_status_t prox_ffn_create(const prox_ffn_config_t* cfg, const void* w_gate, 
   A(dev_alloc(reinterpret_cast<uint16_t**>(&h->x_stage), (size_t)MB * D));
   A(dev_alloc(reinterpret_cast<float**>(&h->y_stage), (size_t)MB * D));
   if (st == PROX_OK) {
-    A(cudaMemset(h->ticket, 0, (size_t)MB * ns_max * sizeof(unsigned)));
+    A(cudaMemset(h->ticket, 0, ticket_count(h->cfg) * sizeof(unsigned)));
     A(cudaMemset(h->yacc, 0, (size_t)MB * D * sizeof(float)));
     A(cudaMemset(h->dev_status, 0, sizeof(int)));
     A(cudaMemset(h->counters, 0, 4 * sizeof(unsigned long long)));

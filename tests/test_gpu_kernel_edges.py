@@ -704,3 +704,26 @@ def test_many_scores_that_agree_in_their_upper_halves(pb, bits):
         assert pb.prox_last_device_status(h) == 0
     finally:
         pb.prox_ffn_destroy(h)
+
+
+@pytest.mark.parametrize("F,B", [(1536, 8), (1600, 5), (14336, 8), (19136, 1)])
+def test_sixteen_bit_scores_on_a_new_handle(pb, F, B):
+    """The split-K tickets of 16-bit proxies (strips of 128 channels, the most per token) all start at zero, whatever the memory
+    of a new handle held before."""
+    D, k1, k2 = 512, 256, F // 3
+    for words in (64, 128, 256, 1024, 4096):                        # pieces of memory that come back from the driver full of ones
+        held = [torch.full((words,), -1, dtype=torch.int32, device="cuda") for _ in range(64)]
+        del held
+    torch.cuda.empty_cache()
+    p = Problem(pb, *inputs.make_small(D, F, B, seed=F), max_batch=B)
+    try:
+        p.quantize(16, 0)
+        sel, sc = torch.empty(B, k2, dtype=torch.int32, device="cuda"), torch.empty(B, F, device="cuda")
+        for again in range(2):
+            pb.prox_stage1_mask(p.h, p.t_x, B, k1, k2, sel, sc)
+            for b in range(B):
+                _, score, _, thr = p.oracle_stage1(b, k1, k2)
+                assert float(np.max(np.abs(sc[b].cpu().numpy() - score)) / thr) < 2e-4, (again, b)      # as everywhere for scores
+        assert pb.prox_last_device_status(p.h) == 0
+    finally:
+        p.close()
