@@ -183,7 +183,7 @@ def test_batch_stage2_rows_in_sections(pb, D, F, B):
 
 @pytest.mark.parametrize("D,F,bits,group", [(128, 64, 4, 0), (640, 4992, 8, 128), (8192, 704, 4, 128), (10240, 192, 4, 128), (1024, 2048, 16, 0)])
 def test_stages_one_by_one(pb, D, F, bits, group):
-    """The stages called alone (persistent kernel up to its barrier, and on a given list; wider layers and 16-bit proxies:
+    """The stages called alone (persistent kernel up to its scores, and on a given list; wider layers and 16-bit proxies:
     step-wise kernels) against the whole path on the same masks, with repeated calls; bad channel ids are skipped."""
     wg, wu, wd, x = inputs.make_small(D, F, 2, seed=D + F)
     p = Problem(pb, wg, wu, wd, x)
@@ -503,7 +503,8 @@ def test_forms_mixed_on_one_handle(pb, bits, group):
 def test_persistent_kernel_mask_is_the_exact_topk_of_its_scores(pb, F, bits, distinct):
     """The channel mask of the whole path against the scores it was made from (ties: lower channel first): one and several
     groups of half scores per thread, and with few distinct channels many equal scores in the threshold bin, so that its
-    members fill the index list or the ring's end and are cut by their channels; and the threshold form at the k-th score."""
+    members do not fit the index list and are cut by their channels (the rows are short here: the list lies behind the ring);
+    and the threshold form at the k-th score."""
     D, k1 = 128, 50
     g = torch.Generator(device="cuda").manual_seed(F + distinct)
     w = [(torch.randn(F, D, device="cuda", generator=g) * 0.1).to(torch.bfloat16) for _ in range(2)]
@@ -576,6 +577,7 @@ def _mask_is_the_exact_topk(pb, D, F, bits, group, distinct, zero):
         pb.prox_quantize_proxy(h, bits, group)
         y, ref, sc = (torch.empty(n, dtype=torch.float32, device="cuda") for n in (D, D, F))
         for k2 in (1, F // 3 + 1, F - 1):
+            assert pb.prox_fused_kernel_info(h, k1, k2)["usable"] == 1
             sel = torch.empty(1, k2, dtype=torch.int32, device="cuda")
             pb.prox_ffn_forward(h, x, 1, k1, k2, y)
             pb.prox_ffn_last_mask(h, 1, k2, sel)
@@ -727,3 +729,17 @@ def test_sixteen_bit_scores_on_a_new_handle(pb, F, B):
         assert pb.prox_last_device_status(p.h) == 0
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("zero", [False, True])
+@pytest.mark.parametrize("D,F,bits,group,distinct", [(4096, 12288, 4, 128, 2), (4096, 14336, 8, 0, 1), (8192, 16384, 4, 0, 1)])
+def test_threshold_bin_listed_over_the_ring(pb, D, F, bits, group, distinct, zero):
+    """The list of the threshold bin's members (more than d_model / 2 of them) lies over slots of the ring that the first weight rows
+    would go to: no row may get there before the list has been read."""
+    _mask_is_the_exact_topk(pb, D, F, bits, group, distinct, zero)
+
+
+@pytest.mark.parametrize("bits,distinct", [(4, 0), (8, 3)])
+def test_half_scores_that_do_not_fit(pb, bits, distinct):
+    """65536 half scores beside a d_model of 12288: no room in shared memory, the blocks read them where the others put them."""
+    _mask_is_the_exact_topk(pb, 12288, 65536, bits, 0, distinct, False)
