@@ -125,13 +125,13 @@ prox_status_t prox_ffn_forward(prox_ffn_t* h, const void* x_dev, int B, int k1, 
                                void* y_dev, void* stream);
 
 /* For B = 1 prox_ffn_forward runs the whole path as ONE persistent kernel
- * (one block per SM, one grid-wide barrier with a bounded
- * wait between Stage 1 and Stage 2); prox_ffn_set_fused(h, 0) selects the
+ * (one block per SM; between Stage 1 and Stage 2 every block waits, with a
+ * limit, for the other blocks' scores); prox_ffn_set_fused(h, 0) selects the
  * kernel-per-step path instead (always used for B > 1).  If a bounded wait
  * ever expires the kernel leaves, y is not written (undefined) and
  * prox_last_device_status reports bit 4 and returns PROX_ERR_TIMEOUT.
- * The stages called alone at B = 1 run on the same kernel (Stage 1 up to its
- * barrier, Stage 2 from there on), and report an expired wait in the same way. */
+ * The stages called alone at B = 1 run on the same kernel (Stage 1 up to the
+ * scores, Stage 2 behind the mask), and report an expired wait in the same way. */
 prox_status_t prox_ffn_set_fused(prox_ffn_t* h, int on);
 
 /* Mask policy of calls with B > 1 (the paper treats batch 1 only and names batching as future work):
@@ -163,12 +163,12 @@ prox_status_t prox_fused_kernel_info(prox_ffn_t* h, int k1, int k2, int32_t* inf
 
 /* Debug aid: with on != 0 every block of the persistent kernel records time
  * stamps (nanoseconds of the GPU's global timer) per call.  Slots 0..9: kernel
- * entry, end of set-up, of the input mask, of the proxy GEMV, of the grid
- * barrier, of the channel mask (as seen by thread 0, which helps to settle the
+ * entry, end of set-up, of the input mask, of the proxy GEMV, of the count over
+ * all blocks' scores, of the channel mask (as seen by thread 0, which helps to settle the
  * threshold bin), slot 6 end of that settling, 7 last row consumed, 8 partial-y
  * exchange done, 9 finalize done (last block only).  Slots 10..31 are finer
- * marks inside those phases (16..21: front part of the channel mask, 21 = go
- * flag for the ring; 28 / 30: first copy / first down-projection row armed by a
+ * marks inside those phases (17, 16, 21: scores of all blocks on their way,
+ * histogram complete, definite share listed and the ring started; 15, 19, 20: settling of the threshold bin; 28 / 30: first copy / first down-projection row armed by a
  * producer warp).  If stamps_host is given, the stamps of the last call are
  * copied to it as [min(max_blocks, SM count)][32] uint64 (synchronises).
  * on = 0 frees the buffer. */

@@ -678,8 +678,10 @@ FusedPlan plan_fused(const prox_ffn* h, int k1, int k2, bool thresh = false, int
   if (pl.big_bytes < pl.xch * D * 4) return pl;          // their partial y vectors
   if ((k2 + G - 1) / G + 2 > kMySelCap) return pl;       // a block's share: definite part + part of the threshold bin
   if (thresh) {
-    // any number of channels may pass the threshold: a block's share of all of them must fit, their marks must fit in
-    // shared memory (no radix fallback in this form; the line is that of whole scores), counts are kept in 16 bits
+    // any number of channels may pass the threshold: a block's share of all of them must fit, counts are kept in 16 bits, and
+    // there is no way past shared memory for the marks (F * 4 / 16 or F * 4 / 8 bytes of them; the line is drawn at F * 4, where
+    // it was when whole scores were kept there: d_ff from 37500 at d_model 8192, from 29300 at 12288, far from any layer in
+    // use, takes the step-wise kernels as it always did)
     if ((F + G - 1) / G + 2 > kMySelCap) return pl;
     if (mode == kWhole && ((size_t)F * 4 + 256 > (size_t)pl.big_bytes || F >= 65536)) return pl;
   }
@@ -1014,7 +1016,7 @@ prox_status_t prox_stage1_mask(prox_ffn_t* h, const void* x, int B, int k1, int 
     return s;
   }
   if (B == 1) {
-    // input mask and proxy scores by the persistent kernel (up to its barrier)
+    // input mask and proxy scores by the persistent kernel (up to the scores)
     const FusedPlan pl = plan_fused(h, k1, 1, false, kScoresOnly);
     if (pl.ok) {
       float* own = aligned16(sc) ? sc : h->scores;

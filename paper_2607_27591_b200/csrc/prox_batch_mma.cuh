@@ -548,8 +548,8 @@ namespace prox {
 // With eight tokens the union of the kept inputs is nearly everything, so the proxy GEMM runs over all rows and needs
 // no union list; a dropped input contributes 0 * code.  Token slots beyond B are cleared.
 // A chain of latencies on one SM per token: the histogram's k-th bin from registers instead of three passes over shared memory,
-// and no ranking of ties that are all kept, took 0.5 us off it (4096 x 12288, eight tokens, two layers 183.4 -> 182.5 us per pass;
-// 4096 x 14336 with one mask for eight 144.2 -> 143).
+// and no ranking of ties that are all kept, took 0.5 us off it (4096 x 12288, eight tokens, two layers 185.9 -> 184.7 and 184.9 -> 183.7 us
+// per pass in two series; 4096 x 14336 with one mask for eight 143.9 -> 142.7 and 144.3 -> 143.5).
 // NORM (layer sub-block form): x is bf16(RMSNorm(xres) * norm_w), formed here and written to xn for Stage 2 (a kernel of
 // its own in front of this one took 6.6 us).
 // ----------------------------------------------------------------------------

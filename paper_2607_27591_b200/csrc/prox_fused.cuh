@@ -339,8 +339,8 @@ struct FusedSmem {
 
 // k-th largest (k >= 1) over a histogram held in registers: thread t < 512 has the counts of N bins in descending order,
 // the first of them bin `top`; the threads' runs follow each other downwards (threads from 512 on: zeros).  One scan and two
-// barriers where reading the bins segment by segment took three passes over shared memory (0.8 -> 0.4 us for 1024 bins,
-// 1.1 -> 0.6 for 2048).  res[0..2] = bin, elements above it, elements inside.
+// barriers where reading the bins segment by segment took three passes over shared memory (0.8 -> 0.4 us for 1024 bins).
+// res[0], res[1] = bin, elements above it.
 template <int N>
 __device__ __forceinline__ void find_kth(FusedSmem& sm, const unsigned (&c)[N], int top, unsigned k, int lane, int warp) {
   unsigned s = 0;
@@ -353,7 +353,7 @@ __device__ __forceinline__ void find_kth(FusedSmem& sm, const unsigned (&c)[N], 
   if (run < k && k <= run + s) {
 #pragma unroll
     for (int j = 0; j < N; ++j) {
-      if (run < k && k <= run + c[j]) { sm.res[0] = (unsigned)(top - j); sm.res[1] = run; sm.res[2] = c[j]; }
+      if (run < k && k <= run + c[j]) { sm.res[0] = (unsigned)(top - j); sm.res[1] = run; }
       run += c[j];
     }
   }

@@ -27,7 +27,8 @@ __device__ __forceinline__ unsigned absmax4(const uint2& v) {   // largest of fo
 
 // Bits of 1.5 * 2^23 + offset + rint(v / s) for four weights of one channel, from inv = 1 / s (s a normal fp16 number, or 0 and so v).
 // v has 8 significant bits and s = m 2^b has m < 2^11, so a quotient that is not a half integer itself is at least
-// 1 / (2 m) > 2^-12 away from the next one (v - (k + 1/2) s is a multiple of 2^(b-1)), and v * inv within 1e-5 of it
+// 1 / (2 m) > 2^-12 away from the next one (v - (k + 1/2) s is a multiple of 2^(b-1), unless v's last bit lies below 2^(b-1): then
+// |v| < 2^(b+6) and the quotient is below 1/16, nowhere near a half), and v * inv within 1e-5 of it
 // (|quotient| < 128.1): rounded to a multiple of 2^-12 first (the first addition: 3072 + quotient), what is a half
 // integer becomes exactly one and nothing else does, and the second addition rounds to the nearest integer, halves to even,
 // as the IEEE quotient would be.  No clamp: the scale is absmax / qmax to 2^-11.  With the start of the codes at bit 0 of the
