@@ -1381,8 +1381,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1) prox_fused_kernel(const Fuse
             at += __popc(b);
           }
         }
-      } else if (shr < NSH) {
-        // no room for the list: the block's share of the plain ascending mask, before the ring starts
+      } else if (!THRESH && shr < NSH) {
+        // no room for the list: the block's share of the plain ascending mask, before the ring starts (the threshold form has no list
+        // and is not launched where its marks do not fit; with the call in it, 3072 x 8896 8-bit took 59.5 us for two layers instead of 58.4)
         n_mine = settle_over_all_channels(xkeys, F, (unsigned)k2, shr, NSH, b1, kk, p.sel_out, spin, p.bar_bias);
         if (tid == 0) { sm.keys_s0 = sm.keys_s1 = sm.list_s0 = sm.list_s1 = 0; sm.n_mine = n_mine; sm.nready = n_mine; sm.keys_done = 1; sm.c_done = 1; }
       }
